@@ -21,9 +21,9 @@ __device__ __forceinline__ int rne_clamp(float v) {
 // binary32 exponential with a fixed operation sequence (see ssdi8.h): Cody-Waite
 // reduction by ln 2, degree-7 Taylor polynomial (Horner, fmaf), scaling by 2^n
 // through the exponent field.  0 below -80, argument clamped at +80.
-__device__ __forceinline__ float exp32(float x) {
-  if (!(x >= -80.0f)) return 0.0f;
-  x = fminf(x, 80.0f);
+// (The zero below -80 is a selection at the end: the arithmetic in front of it is harmless there.)
+__device__ __forceinline__ float exp32(float x0) {
+  const float x = fminf(x0, 80.0f);
   const float LOG2E = __uint_as_float(0x3FB8AA3Bu);
   const float LN2_HI = __uint_as_float(0x3F317200u);
   const float LN2_LO = __uint_as_float(0x35BFBE8Eu);
@@ -42,7 +42,30 @@ __device__ __forceinline__ float exp32(float x) {
   p = __fmaf_rn(p, r, 0.5f);
   p = __fmaf_rn(p, r, 1.0f);
   p = __fmaf_rn(p, r, 1.0f);
-  return __uint_as_float(__float_as_uint(p) + (__float_as_uint(nm) << 23));   // bits(nm) = 0x4B400000 + n: the shift keeps n
+  const float e = __uint_as_float(__float_as_uint(p) + (__float_as_uint(nm) << 23));   // bits(nm) = 0x4B400000 + n: the shift keeps n
+  return x0 >= -80.0f ? e : 0.0f;
+}
+// two at once, the same operations in packed form
+__device__ __forceinline__ float2 exp32x2(float x0, float x1) {
+  auto both = [](uint32_t bits) { return make_float2(__uint_as_float(bits), __uint_as_float(bits)); };
+  const float2 x = make_float2(fminf(x0, 80.0f), fminf(x1, 80.0f));
+  // (a multiply and an add that stay two operations: the packed pair would be contracted into one)
+  const float2 nm = make_float2(__fadd_rn(__fmul_rn(x.x, __uint_as_float(0x3FB8AA3Bu)), 12582912.0f),
+                                __fadd_rn(__fmul_rn(x.y, __uint_as_float(0x3FB8AA3Bu)), 12582912.0f));
+  const float2 n = __fadd2_rn(nm, make_float2(-12582912.0f, -12582912.0f));
+  float2 r = __ffma2_rn(n, both(0xBF317200u), x);
+  r = __ffma2_rn(n, both(0xB5BFBE8Eu), r);
+  float2 p = both(0x39500D01u);
+  p = __ffma2_rn(p, r, both(0x3AB60B61u));
+  p = __ffma2_rn(p, r, both(0x3C088889u));
+  p = __ffma2_rn(p, r, both(0x3D2AAAABu));
+  p = __ffma2_rn(p, r, both(0x3E2AAAABu));
+  p = __ffma2_rn(p, r, make_float2(0.5f, 0.5f));
+  p = __ffma2_rn(p, r, make_float2(1.0f, 1.0f));
+  p = __ffma2_rn(p, r, make_float2(1.0f, 1.0f));
+  const float e0 = __uint_as_float(__float_as_uint(p.x) + (__float_as_uint(nm.x) << 23));
+  const float e1 = __uint_as_float(__float_as_uint(p.y) + (__float_as_uint(nm.y) << 23));
+  return make_float2(x0 >= -80.0f ? e0 : 0.0f, x1 >= -80.0f ? e1 : 0.0f);
 }
 
 // ---- conversions that stay off the quarter-rate conversion pipe (all exact)
@@ -185,8 +208,13 @@ __device__ __forceinline__ uint64_t l2_policy_evict_last() {
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
   return pol;
 }
-__device__ __forceinline__ void st_global_hint(float* a, float v, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;" ::"l"(a), "f"(v), "l"(pol) : "memory");
+__device__ __forceinline__ void st_global_hint(float* a, float2 v, uint64_t pol) {
+  asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;" ::"l"(a), "f"(v.x), "f"(v.y), "l"(pol) : "memory");
+}
+__device__ __forceinline__ void st_global_hint(float* a, float4 v, uint64_t pol) {
+  asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;"
+               ::"l"(a), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "l"(pol)
+               : "memory");
 }
 
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

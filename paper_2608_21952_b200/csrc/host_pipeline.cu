@@ -108,11 +108,12 @@ LayerWs layer_ws(const ssdi8_dims_t& d, uint8_t* base, uint32_t flags) {
   return w;
 }
 
-// quantisers + forward on device tensors, int8 tensors and workspace given; status cleared by the caller
+// quantisers + forward on device tensors, int8 tensors and workspace given; clear_status: the status word is set
+// to 0 first (the host pipeline clears it once for all its slices)
 ssdi8_status_t layer_step(const ssdi8_dims_t& d, const ssdi8_layer_args_t& a, const float* x, const float* B,
                           const float* C, const float* dt, const float* init, float* y, float* fin,
                           int32_t* status, int8_t* xq, int8_t* Bq, int8_t* Cq, void* ws, size_t ws_bytes,
-                          uint32_t flags, cudaStream_t st) {
+                          uint32_t flags, cudaStream_t st, bool clear_status) {
   const int64_t T = (int64_t)d.batch * d.seqlen;
   ssdi8_fwd_args_t f = {};
   f.xq = xq; f.Bq = Bq; f.Cq = Cq;
@@ -132,7 +133,7 @@ ssdi8_status_t layer_step(const ssdi8_dims_t& d, const ssdi8_layer_args_t& a, co
   // ChunkCumsum complete as well.  One stream, no events.  Measured per step, this chain / ChunkCumsum on a
   // side stream / ChunkCumsum's blocks inside the quantisers' grid: 0.286 / 0.293 / 0.287 ms at batch
   // 8 x 2048 x 80 heads, 0.056 / 0.062 / 0.062 ms at 2048 x 24 heads.
-  if ((s = fwd_phases(&d, &f, fl | SSDI8_PHASE_CUMSUM, ws, ws_bytes, st, false)) != SSDI8_OK) return s;
+  if ((s = fwd_phases(&d, &f, fl | SSDI8_PHASE_CUMSUM, ws, ws_bytes, st, clear_status)) != SSDI8_OK) return s;
   if ((s = launch_quantize_xbc(x, B, C, T, d.nheads * d.headdim, d.ngroups, d.dstate, a.s_x, a.s_B, a.s_C, xq, Bq, Cq, st,
                                true)) != SSDI8_OK)
     return s;
@@ -205,9 +206,8 @@ ssdi8_status_t ssdi8_layer_fwd(const ssdi8_dims_t* dims, const ssdi8_layer_args_
     return SSDI8_ERR_ALIGN;
   const LayerWs w = layer_ws(*dims, static_cast<uint8_t*>(workspace), flags);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (a->status) SSDI8_CUDA_CHECK(cudaMemsetAsync(a->status, 0, sizeof(int32_t), st));
   return layer_step(*dims, *a, a->x, a->B, a->C, a->dt, a->init_state, a->y, a->final_state, a->status, w.xq, w.Bq,
-                    w.Cq, w.ws, w.ws_bytes, flags, st);
+                    w.Cq, w.ws, w.ws_bytes, flags, st, true);
 }
 
 size_t ssdi8_layer_fwd_host_scratch_bytes(const ssdi8_dims_t* dims, uint32_t flags) {
@@ -283,7 +283,7 @@ ssdi8_status_t ssdi8_layer_fwd_host(const ssdi8_dims_t* dims, const ssdi8_layer_
     as.s_B = a->s_B + g0; as.s_C = a->s_C + g0; as.s_cb = a->s_cb + g0;
     const size_t fin_off = (b * H + h0) * P * N;
     s = layer_step(d1, as, sb.x, sb.B, sb.C, sb.dt, a->init_state ? a->init_state + fin_off : nullptr, sb.y,
-                   a->final_state ? sb.fin : nullptr, lo.status, sb.xq, sb.Bq, sb.Cq, lo.ws, lo.ws_bytes, flags, s_cmp);
+                   a->final_state ? sb.fin : nullptr, lo.status, sb.xq, sb.Bq, sb.Cq, lo.ws, lo.ws_bytes, flags, s_cmp, false);
     if (s != SSDI8_OK) return s;
     SSDI8_CUDA_CHECK(cudaEventRecord(p->cmp_done[st], s_cmp));
     // outputs of the slice

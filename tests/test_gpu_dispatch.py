@@ -1,0 +1,61 @@
+"""The variants that the launchers choose between and the exact fast paths inside the kernels, at the sizes and values
+where they can go wrong, against the oracle.  Every comparison is bit for bit (the operation order of the library's
+binary32 and binary64 arithmetic is part of its interface), so no tolerance is needed."""
+import numpy as np
+import pytest
+
+from oracle import oracle as orc
+from paper_2608_21952_b200 import inputs
+from paper_2608_21952_b200.inputs import SSDConfig
+
+pytestmark = pytest.mark.gpu
+
+
+def _ties(dt, A):
+    # A = -1 and time steps on a grid of half binary32 units of the running sum: every prefix sum is exact in binary64
+    # and about half of them lie exactly between two binary32 numbers
+    A[:] = -1.0
+    n = np.random.default_rng(5).integers(0, 5, dt.shape).astype(np.float64)
+    dt[:] = (n * 2.0 ** -24).astype(np.float32)
+    dt[:, 0] = 1.0
+
+
+def _mixed(dt, A):
+    dt[:, 1::3] *= -1.0
+
+
+def _tiny(dt, A):
+    dt *= np.float32(1e-36)
+
+
+def _zero(dt, A):
+    dt[:] = 0.0
+
+
+def _huge(dt, A):
+    dt[:, ::7] = np.float32(3e37)
+
+
+@pytest.mark.parametrize("regime", [_ties, _mixed, _tiny, _zero, _huge], ids=lambda f: f.__name__[1:])
+@pytest.mark.parametrize("H,Q", [(1, 64), (9, 128), (12, 256)])
+def test_cumsum_scan_equals_the_sum_in_token_order(H, Q, regime):
+    import gpu_harness as gh
+    cfg = SSDConfig("cs", 2, 2 * Q, H, 64, 64, 1, Q, 0.02, 20.0, 31)
+    q = orc.prepare_quantized(cfg, inputs.make_prefill(cfg))
+    dt, A = q["dt"].reshape(2, 2 * Q, H).copy(), q["A"].copy()
+    regime(dt[:, :Q], A)
+    regime(dt[:, Q:], A)
+    q["dt"], q["A"] = dt, A
+    want = orc.chunk_cumsum(cfg, dt, A)
+    _, _, taps = gh.gpu_fwd(cfg, q, taps=("cs",))
+    assert np.array_equal(taps["cs"], want)
+
+
+def test_cumsum_on_a_grid_that_fills_the_device():
+    # 8 heads per block (the grid above takes 4), a last block with one head
+    import gpu_harness as gh
+    cfg = SSDConfig("cs_full", 2, 64 * 40, 17, 64, 64, 1, 64, 0.02, 20.0, 32)
+    q = orc.prepare_quantized(cfg, inputs.make_prefill(cfg))
+    want = orc.chunk_cumsum(cfg, q["dt"], q["A"])
+    _, _, taps = gh.gpu_fwd(cfg, q, taps=("cs",))
+    assert np.array_equal(taps["cs"], want)
