@@ -5,9 +5,9 @@
 //   Mq[i,j]       = per-row re-quantised CBq[i,j] dt_j exp(cs_i - cs_j), j <= i   (see ssdi8.h)
 //   acc_diag[i,p] = sum_j Mq[i,j] xq[j,p]                 INT8 MMA, second TMEM accumulator
 //   y = exp(cs_i) s_C s_h acc_off + (s_cb rowmax_i / 127) s_x acc_diag + D s_x xq + corr
-// Roles (28 warps): warps 0, 2, 3 issue the TMA loads (CBq K-major, the per-token scalar pack of
-// ChunkCumsum and the head's per-column vectors; Cq, hq K-major; xq MN-major, once per chunk), each
-// stream on its own ring; warp 1 issues the MMAs; warps 4-19 build Mq in place over CBq, as two
+// Roles (28 warps): warps 0 and 2 issue the TMA loads (CBq K-major, the per-token scalar pack of
+// ChunkCumsum and the head's per-column vectors; Cq, hq K-major and xq MN-major, once per chunk);
+// warps 1 and 3 issue the MMAs of the two contractions; warps 4-19 build Mq in place over CBq, as two
 // groups of 8 warps that take alternate chunks (two threads per output row in adjacent lanes, so a
 // warp owns 16 rows and needs no block barrier for the row maximum); warps 20-27 read the
 // accumulators, form y and store it through a swizzled staging tile with TMA (128-byte rows), as two
@@ -86,20 +86,24 @@ __device__ __forceinline__ uint32_t pack4_rn_product(float2 a, float2 b, float2 
 }
 
 // ---- the masked operand of one tile, in place over CBq.  Two threads per output row, in
-// adjacent lanes, so a warp owns 16 rows that share their own sub-block I16 = i / 16 (the walk
-// below is warp-uniform up to the skip tests) and the row maximum needs one shuffle, no block
-// barrier.  Chunk I16 (16 columns) is the row's own sub-block: running product of per-token
-// decays, columns split 8/8 between the two threads (the one with the lower columns first runs
-// the product through the upper ones).  Earlier chunks use the column weights woff and one
-// factor f = exp32(cs_i - cs_ce) per chunk and are dealt alternately; later chunks are zero.
+// adjacent lanes, so a warp owns 16 rows that share their own sub-block I16 = i / 16 (everything
+// below is warp-uniform up to values) and the row maximum needs one shuffle, no block barrier.  Every
+// sub-block (16 columns) is split 8/8 between the two threads.  Sub-block I16 is the row's own: running
+// product of per-token decays (the thread with the lower columns first runs the product through the upper
+// ones).  Earlier sub-blocks use the column weights woff and one factor f = fmul(dec_i, gtab[c]) each,
+// dec_i the row's decay to the end of the sub-block before its own; later ones are zero.
 //
-// Work that decides no output bit is skipped, nearest chunk first.  b127[c] bounds |cb woff| of
-// chunk c, so a chunk with fmul(b127[c], f) <= (running maximum) cannot raise the row maximum,
-// and one with fmul(b127[c], f inv) < 1/2 rounds to zero everywhere.  p127[c] bounds b127 of
-// chunks 0..c with a 1e-5 slack; where cs does not increase along the chunk, f of a farther
-// chunk is at most f of a nearer one (up to the few 1e-7 of exp32's error, inside the slack),
-// so the same two tests on p127[c] end the walk for all farther chunks at once.  (p127 is +inf
-// where cs is not monotone: the walk then visits every chunk.)
+// The own and the nearest earlier sub-block are straight-line code: they decide the row maximum of
+// nearly every row, and their products stay in registers until the codes are formed.  Of the farther
+// ones, work that decides no output bit is skipped.  bound[c] = b127[c] gtab[c], one sub-block per lane,
+// bounds |t| gtab[c] over sub-block c, so with R = the warp's largest dec_i / (row maximum so far) a
+// sub-block with bound[c] R <= 1 raises no row maximum, and with R = the warp's largest dec_i inv_i one
+// with bound[c] R < 1/2 rounds to zero in every row; both with a slack of 1e-5, far above the few
+// binary32 roundings (and the approximate reciprocal) on either side.  One ballot so names the sub-blocks
+// to visit.  Where cs increases somewhere in the chunk (p127 is +inf then) dec_i and gtab are not
+// bounded by 1, products may leave the binary32 range, and every sub-block is visited.
+// (Against a walk that tested one sub-block after the other, nearest first, 16 columns per thread: 86.5 against 97.1 M
+// warp instructions, 0.125 against 0.139 ms at batch 8 x 2048 x 80 heads.)
 template <bool TAPS>
 __device__ __forceinline__ void mask_tile(uint8_t* sCB, const float* tokbuf, float* rowbuf, int rb, int lane, int TM, uint32_t RBQ,
                                           const Tile& t, const ScanArgs& a) {
@@ -109,46 +113,63 @@ __device__ __forceinline__ void mask_tile(uint8_t* sCB, const float* tokbuf, flo
   const float* woff_s = tokbuf + 2 * Q;
   const float* atok_s = tokbuf + 3 * Q;
   const float* b127_s = tokbuf + 4 * Q;
-  const float* p127_s = b127_s + 16;
   const int r = rb * 16 + (lane >> 1), q2 = lane & 1;   // the warp's block of 16 rows
-  if (r >= TM) return;               // whole warps (TM is a multiple of 16)
+  if (rb * 16 >= TM) return;         // whole warps (TM is a multiple of 16)
   const int i = t.it * TM + r;       // row within the chunk
-  const int I16 = i >> 4, ri = i & 15;
-  const uint32_t cshift = RBQ == 128 ? 3u : 2u;  // log2(chunks per panel row)
+  const int I16 = (t.it * TM >> 4) + rb, ri = lane >> 1;
+  const uint32_t cshift = RBQ == 128 ? 3u : 2u;  // log2(sub-blocks per panel row)
   uint8_t* const rowbase = sCB + (RBQ == 128 ? (uint32_t)r * 128u : (uint32_t)r * 64u);
   const uint32_t rx = RBQ == 128 ? ((uint32_t)r & 7u) : (((uint32_t)r >> 1) & 3u);  // swizzle term of the row
-  auto chunk_ptr = [&](int c) -> uint4* {
+  auto chunk_ptr = [&](int c) -> uint8_t* {
     const uint32_t pn = (uint32_t)c >> cshift, cc = (uint32_t)c & ((1u << cshift) - 1u);
-    return reinterpret_cast<uint4*>(rowbase + pn * PANEL + ((cc ^ rx) << 4));
+    return rowbase + pn * PANEL + ((cc ^ rx) << 4);
   };
+  auto half_ptr = [&](int c) -> uint2* { return reinterpret_cast<uint2*>(chunk_ptr(c)) + q2; };   // this thread's 8 columns
+  constexpr uint32_t kAll = 0xffffffffu;
   const float cs_i = cs_s[i];
-  const int c_first = I16 - 1 - q2;  // nearest earlier chunk of this thread (may be < 0)
-  float tv[8];                       // t of this thread's half of the row's own sub-block
-  float rpart = 0.f;
-  // f of an earlier chunk c: the row's decay to the end of the chunk before its own, times the tabulated
-  // decay from there to the end of chunk c (gtab[c]; 1 for c = I16 - 1)
-  const float ri_dec = I16 > 0 ? exp32(__fsub_rn(cs_i, cs_s[I16 * 16 - 1])) : 0.f;
   const float* const gtab = b127_s + 32 + ((I16 * (I16 - 1)) >> 1);
-  uint2* const own_ptr = reinterpret_cast<uint2*>(chunk_ptr(I16)) + q2;
+  // eight products cb w of an earlier sub-block and their largest magnitude
+  auto products = [&](int c, float2 (&p)[4]) -> float {
+    const uint2 w2 = *half_ptr(c);
+    const float4* wo = reinterpret_cast<const float4*>(woff_s + c * 16 + q2 * 8);
+    const float4 o0 = wo[0], o1 = wo[1];
+    const uint32_t x0 = w2.x ^ 0x80808080u, x1 = w2.y ^ 0x80808080u;
+    p[0] = __fmul2_rn(unpack2(x0, 0), make_float2(o0.x, o0.y));
+    p[1] = __fmul2_rn(unpack2(x0, 2), make_float2(o0.z, o0.w));
+    p[2] = __fmul2_rn(unpack2(x1, 0), make_float2(o1.x, o1.y));
+    p[3] = __fmul2_rn(unpack2(x1, 2), make_float2(o1.z, o1.w));
+    float m = 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m = fmaxf(fmaxf(m, fabsf(p[k].x)), fabsf(p[k].y));
+    return m;
+  };
+  float2 tv[4], tn[4];               // t of this thread's half of the own and of the nearest earlier sub-block
+  float rmax = 0.f, dec = 0.f, bound = 0.f;
+  if (I16 > 0) {
+    dec = exp32(__fsub_rn(cs_i, cs_s[I16 * 16 - 1]));
+    rmax = __fmul_rn(products(I16 - 1, tn), dec);   // gtab[I16 - 1] = 1
+    if (lane < I16 - 1) bound = __fmul_rn(b127_s[lane], gtab[lane]);
+  }
   {
-    // own sub-block, right to left: E[i,i] = 1, E[i,j] = fmul(E[i,j+1], a_{j+1}).  Straight-line code:
-    // a step that a row does not take multiplies by 1 (exact), a column past the diagonal is
-    // selected to 0, so the 16 rows of the warp, which all stop at different columns, do not diverge.
-    const uint2 w2 = *own_ptr;
+    // own sub-block, right to left: E[i,i] = 1, E[i,j] = fmul(E[i,j+1], a_{j+1}).  Straight-line code: the
+    // product starts as 0 and is set to 1 where the row meets its diagonal, so the columns past it, which
+    // carry no weight, come out as 0 by themselves and the 16 rows of the warp do not diverge.
+    const uint2 w2 = *half_ptr(I16);
     const uint32_t ww[2] = {w2.x ^ 0x80808080u, w2.y ^ 0x80808080u};
     const float* ab = atok_s + I16 * 16;   // a_m of the sub-block at ab[m]
     const int e0 = q2 * 8;
-    float E = 1.0f;
+    float E = 0.f;
     {
-      // the thread with the lower columns first runs the product through the upper ones: a_15 .. a_9
+      // the thread with the lower columns first runs the product through the upper ones: columns 15 .. 8
       const float4 p2 = *reinterpret_cast<const float4*>(ab + 8), p3 = *reinterpret_cast<const float4*>(ab + 12);
       const float au[7] = {p2.y, p2.z, p2.w, p3.x, p3.y, p3.z, p3.w};   // a_9 .. a_15
-      const int lim = q2 ? 0 : ri;         // steps m <= lim are taken
+      const int rm = q2 ? 32 : ri;         // (the other thread keeps 0 here: its own run starts at column 15)
+      E = rm == 15 ? 1.0f : 0.f;
 #pragma unroll
-      for (int m = 15; m >= 9; --m) E = __fmul_rn(E, m <= lim ? au[m - 9] : 1.0f);
+      for (int m = 14; m >= 8; --m) E = rm == m ? 1.0f : __fmul_rn(E, au[m - 8]);
     }
     const float4 h0 = *reinterpret_cast<const float4*>(ab + e0), h1 = *reinterpret_cast<const float4*>(ab + e0 + 4);
-    const float hn[8] = {h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w, ab[e0 + 8]};   // a_{e0+k+1}; the last one is never taken when e0 = 8
+    const float hn[8] = {h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w, ab[8]};   // a_{e0+k+1}; the last one meets E = 0 when e0 = 8
     const float4 d0 = *reinterpret_cast<const float4*>(dt_s + I16 * 16 + e0);
     const float4 d1 = *reinterpret_cast<const float4*>(dt_s + I16 * 16 + e0 + 4);
     const float dv[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
@@ -156,110 +177,73 @@ __device__ __forceinline__ void mask_tile(uint8_t* sCB, const float* tokbuf, flo
     float Ev[8];
 #pragma unroll
     for (int k = 7; k >= 0; --k) {
-      E = __fmul_rn(E, k < rr ? hn[k] : 1.0f);
+      E = k == rr ? 1.0f : __fmul_rn(E, hn[k]);
       Ev[k] = E;
     }
 #pragma unroll
-    for (int k = 0; k < 8; k += 2) {
-      const float2 t2 = __fmul2_rn(unpack2(ww[k >> 2], k & 3),
-                                   __fmul2_rn(make_float2(dv[k], dv[k + 1]), make_float2(Ev[k], Ev[k + 1])));
-      tv[k] = k <= rr ? t2.x : 0.f;
-      tv[k + 1] = k + 1 <= rr ? t2.y : 0.f;
-      rpart = fmaxf(fmaxf(rpart, fabsf(tv[k])), fabsf(tv[k + 1]));
+    for (int k = 0; k < 4; ++k) {
+      tv[k] = __fmul2_rn(unpack2(ww[k >> 1], 2 * (k & 1)),
+                         __fmul2_rn(make_float2(dv[2 * k], dv[2 * k + 1]), make_float2(Ev[2 * k], Ev[2 * k + 1])));
+      rmax = fmaxf(fmaxf(rmax, fabsf(tv[k].x)), fabsf(tv[k].y));
     }
   }
-  // Both walks below are warp-uniform: every lane steps through the same iterations (chunk
-  // c_first - 2 it; the thread of a pair that starts one chunk farther runs out one step earlier) and
-  // the skip tests are taken by vote, so the 16 rows of the warp do not diverge; a lane whose own test
-  // says "skip" computes along with the others, which changes nothing (its values cannot raise the
-  // row maximum, or round to zero).
-  constexpr uint32_t kAll = 0xffffffffu;
-  const int nit = (I16 + 1) >> 1;
-  bool live = true;                  // this row has not reached its prefix bound yet
-#pragma unroll 1
-  for (int itc = 0; itc < nit; ++itc) {
-    const int c = c_first - 2 * itc;
-    live = live && c >= 0;
-    if (!__any_sync(kAll, live)) break;
-    const int cc = c < 0 ? 0 : c;
-    const float f = __fmul_rn(ri_dec, gtab[cc]);
-    if (rpart >= 1e-30f && __fmul_rn(p127_s[cc], f) <= rpart) live = false;  // nor can any farther chunk
-    const bool need = live && !(__fmul_rn(b127_s[cc], f) <= rpart);
-    if (!__any_sync(kAll, need)) continue;
-    const uint4 w4 = *chunk_ptr(cc);
-    const uint32_t ww[4] = {w4.x ^ 0x80808080u, w4.y ^ 0x80808080u, w4.z ^ 0x80808080u, w4.w ^ 0x80808080u};
-    const float4* wo = reinterpret_cast<const float4*>(woff_s + cc * 16);
-    float bmax = 0.f;
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      const float4 o = wo[w];
-      const float2 t0 = __fmul2_rn(unpack2(ww[w], 0), make_float2(o.x, o.y));
-      const float2 t1 = __fmul2_rn(unpack2(ww[w], 2), make_float2(o.z, o.w));
-      bmax = fmaxf(fmaxf(bmax, fabsf(t0.x)), fabsf(t0.y));
-      bmax = fmaxf(fmaxf(bmax, fabsf(t1.x)), fabsf(t1.y));
+  rmax = fmaxf(rmax, __shfl_xor_sync(kAll, rmax, 1));
+  const bool mono = b127_s[16] < __int_as_float(0x7f800000);
+  auto warp_max = [&](float v) { return __uint_as_float(__reduce_max_sync(kAll, __float_as_uint(v))); };   // v >= 0
+  constexpr float kSlack = 1.00001f;
+  const uint32_t all = I16 > 1 ? (1u << (I16 - 1)) - 1u : 0u;   // the farther sub-blocks
+  if (I16 > 1) {
+    float rcp;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(rcp) : "f"(rmax));
+    const float R = warp_max(__fmul_rn(dec, fminf(rcp, 3.0e38f)));   // (a row of zeros so far: any bound but 0 is above it)
+    uint32_t m = __ballot_sync(kAll, __fmul_rn(bound, R) * kSlack > 1.0f);
+    if (!mono) m = all;
+    if (m) {
+      do {
+        const int c = 31 - __clz(m);
+        m ^= 1u << c;
+        float2 p[4];
+        const float pm = products(c, p);
+        rmax = fmaxf(rmax, __fmul_rn(pm, __fmul_rn(dec, gtab[c])));
+      } while (m);
+      rmax = fmaxf(rmax, __shfl_xor_sync(kAll, rmax, 1));
     }
-    if (need) rpart = fmaxf(rpart, __fmul_rn(bmax, f));
   }
-  const float rowmax = fmaxf(rpart, __shfl_xor_sync(0xffffffffu, rpart, 1));
-  const float inv = (rowmax >= 1e-30f) ? __fdiv_rn(127.0f, rowmax) : 0.f;
+  const float inv = (rmax >= 1e-30f) ? __fdiv_rn(127.0f, rmax) : 0.f;
   int8_t* mq_tap = nullptr;
   if (TAPS && a.taps.Mq) mq_tap = a.taps.Mq + ((((i64)t.b * a.d.c + t.k) * a.d.H + t.h) * Q + i) * Q;
   if (q2 == 0) {
-    rowbuf[r] = rowmax;                 // read by the epilogue warps, with cs_i (they take its
+    rowbuf[r] = rmax;                   // read by the epilogue warps, with cs_i (they take its
     rowbuf[128 + r] = cs_i;             // exponential: the mask warps set the pace of the kernel)
-    if (TAPS && a.taps.rowmax) a.taps.rowmax[(t.tok0 + i) * a.d.H + t.h] = rowmax;
+    if (TAPS && a.taps.rowmax) a.taps.rowmax[(t.tok0 + i) * a.d.H + t.h] = rmax;
   }
-  const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
-  // (the chunks after the row's own arrive as zeros: ChunkBMM writes them so)
-  {
-    const float2 inv2 = make_float2(inv, inv);
-    uint2 v;
-    v.x = pack4_rn_product(make_float2(tv[0], tv[1]), make_float2(tv[2], tv[3]), inv2);
-    v.y = pack4_rn_product(make_float2(tv[4], tv[5]), make_float2(tv[6], tv[7]), inv2);
-    *own_ptr = v;
-    if (TAPS && mq_tap) *reinterpret_cast<uint2*>(mq_tap + I16 * 16 + q2 * 8) = v;
-  }
-  bool dead = false;                 // this chunk and every farther one round to zero in this row
-  int itc = 0;
+  // (the sub-blocks after the row's own arrive as zeros: ChunkBMM writes them so)
+  auto store = [&](int c, const float2 (&p)[4], float g) {
+    const float2 g2 = make_float2(g, g);
+    const uint2 v = make_uint2(pack4_rn_product(p[0], p[1], g2), pack4_rn_product(p[2], p[3], g2));
+    *half_ptr(c) = v;
+    if (TAPS && mq_tap) *reinterpret_cast<uint2*>(mq_tap + c * 16 + q2 * 8) = v;
+  };
+  store(I16, tv, inv);
+  const float di = __fmul_rn(dec, inv);
+  if (I16 > 0) store(I16 - 1, tn, di);
+  if (I16 > 1) {
+    uint32_t m = __ballot_sync(kAll, __fmul_rn(bound, warp_max(di)) * kSlack >= 0.5f);
+    if (!mono) m = all;
 #pragma unroll 1
-  for (; itc < nit; ++itc) {
-    const int c = c_first - 2 * itc;
-    const bool valid = c >= 0;
-    const int cc = valid ? c : 0;
-    // once no row of the warp has a chunk left that does not round to zero, what remains is zero fill
-    if (!__any_sync(kAll, valid && !dead)) break;
-    uint4* ptr = chunk_ptr(cc);
-    uint4 v = zero4;
-    {
-      const float f = __fmul_rn(ri_dec, gtab[cc]);
-      const float g = __fmul_rn(f, inv);
-      if (__fmul_rn(p127_s[cc], g) < 0.5f) dead = true;
-      const bool need = valid && !dead && __fmul_rn(b127_s[cc], g) >= 0.5f;
-      if (__any_sync(kAll, need)) {
-        const float2 g2 = make_float2(g, g);
-        const uint4 w4 = *ptr;
-        const uint32_t ww[4] = {w4.x ^ 0x80808080u, w4.y ^ 0x80808080u, w4.z ^ 0x80808080u, w4.w ^ 0x80808080u};
-        const float4* wo = reinterpret_cast<const float4*>(woff_s + cc * 16);
-        uint32_t o[4];
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          const float4 fo = wo[w];
-          o[w] = pack4_rn_product(__fmul2_rn(unpack2(ww[w], 0), make_float2(fo.x, fo.y)),
-                                  __fmul2_rn(unpack2(ww[w], 2), make_float2(fo.z, fo.w)), g2);
-        }
-        if (need) v = make_uint4(o[0], o[1], o[2], o[3]);
-      }
+    for (int c = I16 - 2 - q2; c >= 0; c -= 2) {   // 16 columns of zeros per thread, alternately
+      if ((m >> c) & 1u) continue;
+      *reinterpret_cast<uint4*>(chunk_ptr(c)) = make_uint4(0u, 0u, 0u, 0u);
+      if (TAPS && mq_tap) *reinterpret_cast<uint4*>(mq_tap + c * 16) = make_uint4(0u, 0u, 0u, 0u);
     }
-    if (valid) {
-      *ptr = v;
-      if (TAPS && mq_tap) *reinterpret_cast<uint4*>(mq_tap + c * 16) = v;
-    }
-  }
-  // the chunks farther left are zeros in every row of the warp
 #pragma unroll 1
-  for (int c = c_first - 2 * itc; c >= 0; c -= 2) {
-    *chunk_ptr(c) = zero4;
-    if (TAPS && mq_tap) *reinterpret_cast<uint4*>(mq_tap + c * 16) = zero4;
+    while (m) {
+      const int c = 31 - __clz(m);
+      m ^= 1u << c;
+      float2 p[4];
+      products(c, p);
+      store(c, p, __fmul_rn(__fmul_rn(dec, gtab[c]), inv));
+    }
   }
 }
 
@@ -293,7 +277,7 @@ chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ 
       mbar_init(&bars[B_MQ + s], kGroupWarps);
       mbar_init(&bars[B_TOK_FULL + s], 1);
       mbar_init(&bars[B_TOK_FREE + s], kGroupWarps);
-      mbar_init(&bars[B_ACC + s], 1);
+      mbar_init(&bars[B_ACC + s], 2);      // both issuers' commits
       mbar_init(&bars[B_ACC_FREE + s], kEpiGroupWarps);
     }
     for (int s = 0; s < 8; ++s) {
@@ -357,68 +341,77 @@ chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ 
       }
     }
   } else if (warp == 2) {
-    // ------------------------------------------------------------ TMA producer: Cq, hq
+    // ------------------------------------------------------------ TMA producer: xq rows, Cq, hq
     if (lane == 0) {
       Tile t = *first_tile;
 #pragma unroll 1
       for (int n = 0; n < n_end; ++n, next_tile(t, d, a.w, TM, ntpu)) {
+        if (t.it == 0) {   // the chunk's rows come with its first tile
+          const int xs = x_index(n, ntpu);
+          mbar_wait_relaxed(&bars[B_X_FREE + xs], x_phase(n, ntpu) ^ 1, a.status);
+          mbar_expect_tx(&bars[B_X_FULL + xs], (uint32_t)(Q * 64));
+          for (int j0 = 0; j0 < Q; j0 += TM)
+            tma_load_3d(smem + OFF_X + xs * 16384 + j0 * 64, &tm_x, &bars[B_X_FULL + xs], 0, t.h, (int)(t.tok0 + j0));
+        }
         mbar_wait_relaxed(&bars[B_CH_FREE], (n & 1) ^ 1, a.status);
         mbar_expect_tx(&bars[B_CH_FULL], (uint32_t)(TM * N + 64 * N));
         tma_load_3d(smem + OFF_C, &tm_C, &bars[B_CH_FULL], 0, t.h / a.w.hpg, (int)(t.tok0 + t.it * TM));
         tma_load_2d(smem + OFF_H, &tm_h, &bars[B_CH_FULL], 0, (int)((((i64)t.b * d.c + t.k) * d.H + t.h) * P));
       }
     }
-  } else if (warp == 3) {
-    // ------------------------------------------------------------ TMA producer: xq rows
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ MMA issuer: C h.  (Two issuers, one per
+    // contraction: an issue is a chain of dependent instructions of one thread, and a single thread that issued
+    // the 8 or 12 MMAs of a tile in turn took 1.0 us per tile with nothing else in its way, half of the tile's
+    // time.)
     if (lane == 0) {
-      Tile t = *first_tile;
+      const uint32_t idesc_off = idesc_s8(128, 64, 0, 0);
+      const uint32_t sbase = smem_u32(smem);
+      const uint64_t da = tile_desc(sbase + OFF_C, RBN), db = tile_desc(sbase + OFF_H, RBN);
 #pragma unroll 1
-      for (int n = 0; n < n_end; ++n, next_tile(t, d, a.w, TM, ntpu)) {
-        if (t.it != 0) continue;   // the chunk's rows were loaded with its first tile
-        const int xs = x_index(n, ntpu);
-        mbar_wait_relaxed(&bars[B_X_FREE + xs], x_phase(n, ntpu) ^ 1, a.status);
-        mbar_expect_tx(&bars[B_X_FULL + xs], (uint32_t)(Q * 64));
-        for (int j0 = 0; j0 < Q; j0 += TM)
-          tma_load_3d(smem + OFF_X + xs * 16384 + j0 * 64, &tm_x, &bars[B_X_FULL + xs], 0, t.h, (int)(t.tok0 + j0));
+      for (int n = 0; n < n_end; ++n) {
+        const int a4 = n & 3;
+        const uint32_t acc = tmem + (uint32_t)a4 * 128u;
+        mbar_wait(&bars[B_ACC_FREE + a4], ((n >> 2) & 1) ^ 1, a.status);
+        mbar_wait(&bars[B_CH_FULL], n & 1, a.status);
+        tc_fence_after();
+        // descriptors advance by a constant per 32-byte K step (their low bits are the address >> 4)
+        mma_s8_ss(acc, da, db, idesc_off, 0);
+        mma_s8_ss(acc, da + 2, db + 2, idesc_off, 1);
+        if (N == 128) {
+          mma_s8_ss(acc, da + 4, db + 4, idesc_off, 1);
+          mma_s8_ss(acc, da + 6, db + 6, idesc_off, 1);
+        }
+        mma_commit(&bars[B_CH_FREE]);
+        mma_commit(&bars[B_ACC + a4]);
       }
     }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
+  } else if (warp == 3) {
+    // ------------------------------------------------------------ MMA issuer: Mq x
     if (lane == 0) {
-      const uint32_t idesc_off = idesc_s8(128, 64, 0, 0), idesc_diag = idesc_s8(128, 64, 0, 1);
+      const uint32_t idesc_diag = idesc_s8(128, 64, 0, 1);
       const uint32_t sbase = smem_u32(smem);
 #pragma unroll 1
       for (int n = 0; n < n_end; ++n) {
         const int it = ntpu == 1 ? 0 : (n & 1);   // a CTA's first tile is the first of its unit
         const int ci = cb_index(n, it, ntpu), a4 = n & 3, xs = x_index(n, ntpu);
         const uint32_t ph4 = (n >> 2) & 1;
-        const int KJ = (it + 1) * TM;
-        const uint32_t acc = tmem + (uint32_t)a4 * 128u;
+        const uint32_t acc = tmem + (uint32_t)a4 * 128u + 64u;
+        const uint64_t da = tile_desc(sbase + cb_offset(ci), RBQ), db = tile_desc(sbase + OFF_X + xs * 16384, 64);
         mbar_wait(&bars[B_ACC_FREE + a4], ph4 ^ 1, a.status);
-        mbar_wait(&bars[B_CH_FULL], n & 1, a.status);
-        tc_fence_after();
-        // descriptors advance by a constant per 32-byte K step (their low bits are the address >> 4):
-        // this thread's issue time is on the path from a freed accumulator to the next epilogue
-        {
-          uint64_t da = tile_desc(sbase + OFF_C, RBN), db = tile_desc(sbase + OFF_H, RBN);
-#pragma unroll 1
-          for (int q = 0; q < N / 32; ++q, da += 2, db += 2) mma_s8_ss(acc, da, db, idesc_off, q > 0);
-        }
-        mma_commit(&bars[B_CH_FREE]);
-        mbar_wait(&bars[B_MQ + ci], ph4, a.status);
         mbar_wait(&bars[B_X_FULL + xs], x_phase(n, ntpu), a.status);
+        mbar_wait(&bars[B_MQ + ci], ph4, a.status);
         tc_fence_after();
-        {
-          uint64_t db = tile_desc(sbase + OFF_X + xs * 16384, 64);
-          uint32_t first = 0;
-#pragma unroll 1
-          for (uint32_t pn = 0; pn < (uint32_t)KJ / RBQ; ++pn) {     // panels of RBQ columns of Mq
-            uint64_t da = tile_desc(sbase + cb_offset(ci) + pn * PANEL, RBQ);
-#pragma unroll 1
-            for (uint32_t q = 0; q < RBQ / 32; ++q, da += 2, db += (32 * 64) >> 4) {
-              mma_s8_ss(acc + 64, da, db, idesc_diag, first);
-              first = 1;
-            }
+        constexpr uint64_t kStepX = (32 * 64) >> 4;   // 32 tokens of x
+        mma_s8_ss(acc, da, db, idesc_diag, 0);
+        mma_s8_ss(acc, da + 2, db + kStepX, idesc_diag, 1);
+        if (BIGQ) {
+          mma_s8_ss(acc, da + 4, db + 2 * kStepX, idesc_diag, 1);
+          mma_s8_ss(acc, da + 6, db + 3 * kStepX, idesc_diag, 1);
+          if (it) {   // the second panel of 128 columns
+#pragma unroll
+            for (uint32_t q = 0; q < 4; ++q)
+              mma_s8_ss(acc, da + (PANEL >> 4) + 2 * q, db + (4 + q) * kStepX, idesc_diag, 1);
           }
         }
         mma_commit(&bars[B_CB_FREE + ci]);
