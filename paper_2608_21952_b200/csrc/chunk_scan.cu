@@ -6,20 +6,27 @@
 //   acc_diag[i,p] = sum_j Mq[i,j] xq[j,p]                 INT8 MMA, second TMEM accumulator
 //   y = exp(cs_i) s_C s_h acc_off + (s_cb rowmax_i / 127) s_x acc_diag + D s_x xq + corr
 // Roles (28 warps): warps 0 and 2 issue the TMA loads (CBq K-major, the per-token scalar pack of
-// ChunkCumsum and the head's per-column vectors; Cq, hq K-major and xq MN-major, once per chunk);
-// warps 1 and 3 issue the MMAs of the two contractions; warps 4-19 build Mq in place over CBq, as two
-// groups of 8 warps that take alternate chunks (two threads per output row in adjacent lanes, so a
-// warp owns 16 rows and needs no block barrier for the row maximum); warps 20-27 read the
+// ChunkCumsum and the head's per-column vectors; hq K-major and xq MN-major, once per chunk), a
+// tile of the chunk each; warps 1 and 3 issue the MMAs of the two contractions, warp 1 loads Cq as
+// well; warps 4-19 build Mq in place over CBq, as two groups of 8 warps that take alternate chunks
+// (two threads per output row in adjacent lanes, so a warp owns 16 rows and needs no block barrier
+// for the row maximum); warps 20-27 read the
 // accumulators, form y and store it through a swizzled staging tile with TMA (128-byte rows), as two
 // groups of 4 warps on alternate tiles, so one group's per-tile bookkeeping and waits run under the
-// other's arithmetic.  Four accumulator pairs, an xq buffer per chunk (shared by the chunk's two
+// other's arithmetic.  Four accumulator pairs, an xq and an hq buffer per chunk (shared by the chunk's two
 // tiles) and an 8-deep ring for what the mask warps hand to the epilogue keep the mask and the MMAs
 // of the next tiles independent of the epilogue of the current ones.  Every buffer has its own
 // "free" barrier, released by whoever reads it last (tcgen05.commit for MMA operands), so loads run
-// several tiles ahead.  The kernel is bound by instruction issue, so it is written to issue little:
-// in each group one warp polls the mbarriers and the others wait at a hardware barrier, the wait
-// loop is one out-of-line function, the tile walk has no divisions, and the code is kept small
-// enough for the instruction cache (every role executes different code at the same time).
+// several tiles ahead.  What bounds the kernel is instruction issue (86 M warp instructions, 66 % of the
+// slots with binary32 y at batch 8 x 2048 x 80 heads, 0.113 ms; 0.104 ms with 16-bit y), so it is
+// written to issue little: in each group one warp polls the mbarriers and the others wait at a hardware
+// barrier, the wait loop is one out-of-line function, the tile walk has no divisions, and the code is kept
+// small enough for the instruction cache (every role executes different code at the same time).
+// The pipeline around it is built so that no role waits for another's order: a timeline of one CTA had the
+// mask groups waiting 2.6 us of every 6.6 for CBq buffers, which waited for in-order MMAs, which waited for
+// xq, whose buffer the epilogue gave back last; with the loads of the two tiles of a chunk on
+// two producers, the scalar pack and hq requested a chunk ahead, xq given back early and the MMA issue
+// in uniform registers the same arithmetic takes 0.113 instead of 0.125 ms.
 // No multicast; bounded waits.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -53,25 +60,28 @@ constexpr uint32_t kTmemCols = 512;  // four accumulator pairs: acc_off at 128 a
 // shared memory (bytes, from a 1024-byte aligned base)
 constexpr uint32_t OFF_CB = 0;          // ring of 4: two 2-panel buffers, two 1-panel buffers
 constexpr uint32_t OFF_C = 98304;       // [128][N]
-constexpr uint32_t OFF_H = 114688;      // [64][N]
-constexpr uint32_t OFF_X = 122880;      // ring of 2 x [256][64]: the xq rows of a chunk
-constexpr uint32_t OFF_TOK = 155648;    // ring of 4 x (5 Q floats: cs, dt, woff, atok, bounds), read by the mask warps
-constexpr uint32_t TOK_BYTES = 5120;
+constexpr uint32_t OFF_H = 114688;      // ring of 2 x [64][N], one per chunk: hq comes from HBM, requested a chunk ahead
+constexpr uint32_t H_BYTES = 8192;
+constexpr uint32_t OFF_X = 131072;      // ring of 2 x [256][64]: the xq rows of a chunk
+constexpr uint32_t OFF_YST = 163840;    // 8 warps x [32][128 B] y staging
+constexpr uint32_t OFF_TOK = OFF_YST + 32768;   // ring of 4, one per chunk, read by the mask warps: Q floats each of cs, dt, woff, atok, and what is used of the bounds row
+constexpr uint32_t TOK_BYTES = 4096 + 608;
 // ring of 8 x what the epilogue needs of a tile: [128] row maxima and [128] cs_i, written by the
 // mask warps, and the head's s_x, s_h and correction vectors ([64] each, bulk-loaded).  Eight deep so
-// that the mask of a tile never waits for the epilogue of an earlier one.
+// that the mask of a tile never waits for the epilogue of an earlier one (four deep: 0.141 against 0.125 ms).
 constexpr uint32_t OFF_ROW = OFF_TOK + 4 * TOK_BYTES;
 constexpr uint32_t ROW_BYTES = 2048, ROW_COLS = 1024, ROW_SCAL = 1792;   // scalars: s_C of the group, D of the head, s_cb
-constexpr uint32_t OFF_YST = OFF_ROW + 8 * ROW_BYTES;  // 8 warps x [32][128 B] y staging
-constexpr uint32_t OFF_BAR = OFF_YST + 32768;
-constexpr uint32_t SMEM_BYTES = OFF_BAR + 512;
+constexpr uint32_t OFF_BAR = OFF_ROW + 8 * ROW_BYTES;
+constexpr uint32_t SMEM_BYTES = OFF_BAR + 512;   // 232 320 bytes
 
 __device__ __forceinline__ uint32_t cb_offset(int idx) { return scan::cb_offset(OFF_CB, idx); }
 
-enum { B_CB_FULL = 0, B_CB_FREE = 4, B_MQ = 8, B_CH_FULL = 12, B_CH_FREE = 13, B_X_FULL = 14, B_X_FREE = 16,
-       B_TOK_FULL = 18, B_TOK_FREE = 22, B_ACC = 26, B_ACC_FREE = 30, B_ROW_FULL = 34, B_ROW_FREE = 42,
-       B_COUNT = 50 };
+enum { B_CB_FULL = 0, B_CB_FREE = 4, B_MQ = 8, B_C_FULL = 12, B_C_FREE = 13, B_X_FULL = 14, B_X_FREE = 16,
+       B_H_FULL = 18, B_H_FREE = 20, B_TOK_FULL = 22, B_TOK_FREE = 26, B_ACC = 30, B_ACC_FREE = 34, B_ROW_FULL = 38,
+       B_ROW_FREE = 46, B_COUNT = 54 };
 
+
+__device__ __forceinline__ uint32_t row_phase(int n) { return (uint32_t)(n >> 3) & 1u; }
 
 // four codes rn(a g), the exact product rounded once to the nearest integer (ties to even): for
 // |a g| < 2^22 that integer sits in the low bits of fma(a, g, 1.5 * 2^23); callers guarantee
@@ -256,19 +266,26 @@ __global__ void __launch_bounds__(kThreads, 1)
 chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ CUtensorMap tm_h,
               const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_cb,
               const __grid_constant__ CUtensorMap tm_y, const ScanArgs a) {
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  // (no padding for the 1024-byte alignment the swizzled tiles need: the kernel takes all of the SM's shared
+  // memory; the launcher checks that it uses no static shared memory, so that the dynamic part starts at the
+  // window's base, and the kernel checks the address itself)
+  uint8_t* smem = smem_raw;
+  if ((smem_u32(smem) & 1023u) != 0) {
+    if (threadIdx.x == 0 && a.status) atomicExch(a.status, (int32_t)SSDI8_ERR_ALIGN);
+    return;
+  }
   const Dims& d = a.d;
   const int Q = d.Q, N = d.N, P = d.P;
   const int TM = BIGQ ? 128 : Q;           // valid rows of a tile
   const int ntpu = BIGQ ? Q / 128 : 1;     // tiles per (batch, chunk, head)
   const uint32_t RBN = N, RBQ = BIGQ ? 128u : (uint32_t)Q;   // row bytes of the N-contracted and Q-contracted tiles
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // (the shuffle: uniform for the compiler)
   // tiles of this CTA: its units blockIdx.x, blockIdx.x + gridDim.x, ..., ntpu tiles each
   const int n_end = tiles_of_cta(a.w, (int)blockIdx.x, (int)gridDim.x, ntpu);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + OFF_BAR);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + B_COUNT);
-  Tile* first_tile = reinterpret_cast<Tile*>(bars + B_COUNT + 2);   // 416 .. 464 of the 512 bytes
+  Tile* first_tile = reinterpret_cast<Tile*>(bars + B_COUNT + 2);   // 448 .. 496 of the 512 bytes
 
   if (tid == 0) {
     for (int s = 0; s < 4; ++s) {
@@ -284,11 +301,13 @@ chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ 
       mbar_init(&bars[B_ROW_FULL + s], 1 + kGroupWarps);   // the column vectors and the mask warps' row scalars
       mbar_init(&bars[B_ROW_FREE + s], kEpiGroupWarps);
     }
-    mbar_init(&bars[B_CH_FULL], 1);
-    mbar_init(&bars[B_CH_FREE], 1);
+    mbar_init(&bars[B_C_FULL], 1);
+    mbar_init(&bars[B_C_FREE], 1);
     for (int s = 0; s < 2; ++s) {
+      mbar_init(&bars[B_H_FULL + s], 1);
+      mbar_init(&bars[B_H_FREE + s], 1);
       mbar_init(&bars[B_X_FULL + s], 1);
-      mbar_init(&bars[B_X_FREE + s], ntpu == 1 ? kEpiGroupWarps : kEpiWarps);  // the epilogues of the chunk's tiles
+      mbar_init(&bars[B_X_FREE + s], (ntpu == 1 ? kEpiGroupWarps : kEpiWarps) + 1);  // the epilogue warps of the chunk's tiles and the MMAs
     }
     fence_mbar_init();
     tma_prefetch_desc(&tm_C); tma_prefetch_desc(&tm_h); tma_prefetch_desc(&tm_x);
@@ -300,95 +319,110 @@ chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   pdl_wait();   // every role below reads or writes global memory
 
-  if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer: CBq panels + scalar pack
+  if (warp == 0 || warp == 2) {
+    // ------------------------------------------------------------ TMA producers.  Warp 0 serves the first tile of
+    // every chunk (hq, CBq panel, scalar pack), warp 2 the second (xq rows, CBq panels); each also the tile's column
+    // vectors.  The buffers of the two kinds of tile become free in an order that depends on how the mask
+    // groups happen to run, and a single in-order producer let the first tile's loads wait behind the
+    // second's: both mask groups waited 40 % of their time for CBq and the scalar pack.
     if (lane == 0) {
+      const int mine = warp >> 1;          // tile of the chunk whose loads this warp issues (warp 2: xq as well)
       Tile t = *first_tile;
+      // four rows of the pack and of the bounds row 32 + n (n - 1) / 2 entries, n = Q / 16 sub-blocks
+      const uint32_t tok_bytes = (uint32_t)(16 * Q + (((32 + (Q >> 4) * ((Q >> 4) - 1) / 2) * 4 + 15) & ~15));
 #pragma unroll 1
-      for (int n = 0; n < n_end; ++n, next_tile(t, d, a.w, TM, ntpu)) {
-        const int tg = t.h / a.w.hpg;   // group of the head (one division per tile in this one thread)
-        const int ci = cb_index(n, t.it, ntpu), t3 = n & 3;
-        const uint32_t ph4 = (n >> 2) & 1, ph3 = (n >> 2) & 1;
-        mbar_wait_relaxed(&bars[B_CB_FREE + ci], ph4 ^ 1, a.status);
-        const int npanel = t.KJ / (int)RBQ;
+      for (int n0 = 0; n0 < n_end; n0 += ntpu, next_head(t, d, a.w, TM, ntpu)) {
+        const int tg = t.h / a.w.hpg;   // group of the head (one division per chunk in this one thread)
+        const int xs = x_index(n0, ntpu);
+        const uint32_t xph = x_phase(n0, ntpu);
+        if (mine == 0) {
+          // the scalar pack of the chunk for the mask warps (four chunks deep: ahead of the wait for a CBq buffer)
+          const int u = ntpu == 1 ? n0 : n0 >> 1, ts = u & 3;
+          mbar_wait(&bars[B_TOK_FREE + ts], ((u >> 2) & 1) ^ 1, a.status);
+          mbar_expect_tx(&bars[B_TOK_FULL + ts], tok_bytes);
+          bulk_load(smem + OFF_TOK + ts * TOK_BYTES, a.pack + t.unit * kPackRows * Q, tok_bytes, &bars[B_TOK_FULL + ts]);
+          mbar_wait(&bars[B_H_FREE + xs], xph ^ 1, a.status);
+          mbar_expect_tx(&bars[B_H_FULL + xs], (uint32_t)(64 * N));
+          tma_load_2d(smem + OFF_H + xs * H_BYTES, &tm_h, &bars[B_H_FULL + xs], 0, (int)((((i64)t.b * d.c + t.k) * d.H + t.h) * P));
+        } else {
+          mbar_wait(&bars[B_X_FREE + xs], xph ^ 1, a.status);
+          mbar_expect_tx(&bars[B_X_FULL + xs], (uint32_t)(Q * 64));
+          for (int j0 = 0; j0 < Q; j0 += TM)
+            tma_load_3d(smem + OFF_X + xs * 16384 + j0 * 64, &tm_x, &bars[B_X_FULL + xs], 0, t.h, (int)(t.tok0 + j0));
+        }
+        if (mine >= ntpu) continue;
+        const int n = n0 + mine, ci = cb_index(n, mine, ntpu);
+        // the tile's three scalars, fetched here so that their latency is not in the epilogue's chain
+        const float sc0 = a.s_C[tg], sc1 = a.D ? a.D[t.h] : 0.f, sc2 = a.s_cb[tg];
+        mbar_wait(&bars[B_CB_FREE + ci], ((n >> 2) & 1) ^ 1, a.status);
+        const int npanel = BIGQ ? mine + 1 : 1;
         mbar_expect_tx(&bars[B_CB_FULL + ci], (uint32_t)(npanel * TM * RBQ));
         for (int pn = 0; pn < npanel; ++pn)
           tma_load_2d(smem + cb_offset(ci) + pn * PANEL, &tm_cb, &bars[B_CB_FULL + ci], pn * (int)RBQ,
-                      (int)((((i64)t.b * d.c + t.k) * d.G + tg) * Q + t.it * TM));
-        mbar_wait_relaxed(&bars[B_TOK_FREE + t3], ph3 ^ 1, a.status);
-        // the scalar pack of the chunk for the mask warps
-        mbar_expect_tx(&bars[B_TOK_FULL + t3], (uint32_t)(5 * Q * 4));
-        bulk_load(smem + OFF_TOK + t3 * TOK_BYTES, a.pack + t.unit * kPackRows * Q, (uint32_t)(5 * Q * 4),
-                  &bars[B_TOK_FULL + t3]);
+                      (int)((((i64)t.b * d.c + t.k) * d.G + tg) * Q + mine * TM));
         // the head's per-column vectors for the epilogue (read once per 8-column piece: from global
         // memory each read would be a long-latency load in its chain)
         const int r8 = n & 7;
-        mbar_wait_relaxed(&bars[B_ROW_FREE + r8], ((n >> 3) & 1) ^ 1, a.status);
+        mbar_wait(&bars[B_ROW_FREE + r8], row_phase(n) ^ 1, a.status);
         uint8_t* cols = smem + OFF_ROW + r8 * ROW_BYTES + ROW_COLS;
-        {   // the tile's three scalars, fetched here so that their latency is not in the epilogue's chain
-          float* sc = reinterpret_cast<float*>(smem + OFF_ROW + r8 * ROW_BYTES + ROW_SCAL);
-          sc[0] = a.s_C[tg];
-          sc[1] = a.D ? a.D[t.h] : 0.f;
-          sc[2] = a.s_cb[tg];
-        }
+        float* sc = reinterpret_cast<float*>(smem + OFF_ROW + r8 * ROW_BYTES + ROW_SCAL);
+        sc[0] = sc0;
+        sc[1] = sc1;
+        sc[2] = sc2;
         mbar_expect_tx(&bars[B_ROW_FULL + r8], (uint32_t)((CORR ? 3 : 2) * P * 4));   // (an arrival: releases the stores above)
         bulk_load(cols, a.s_x + t.h * P, (uint32_t)(P * 4), &bars[B_ROW_FULL + r8]);
         bulk_load(cols + 256, a.s_h + t.h * P, (uint32_t)(P * 4), &bars[B_ROW_FULL + r8]);
         if (CORR) bulk_load(cols + 512, a.corr + t.h * P, (uint32_t)(P * 4), &bars[B_ROW_FULL + r8]);
       }
     }
-  } else if (warp == 2) {
-    // ------------------------------------------------------------ TMA producer: xq rows, Cq, hq
-    if (lane == 0) {
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ C h: this thread loads the one Cq buffer itself,
+    // as soon as its MMAs of the tile before have read it, and issues the MMAs.  (The MMAs of the two
+    // contractions have an issuer each: an issue is a chain of dependent instructions of one thread, and a single
+    // thread that issued the 8 or 12 MMAs of a tile in turn took 1.0 us per tile with nothing else in its way,
+    // half of the tile's time.)
+    {   // (the whole warp runs the loop, see elect_one: one lane alone kept every descriptor in per-thread registers, 80 ns per MMA)
+      const uint32_t idesc_off = idesc_s8(128, 64, 0, 0);
+      const uint32_t sbase = smem_u32(smem);
+      const uint64_t da = tile_desc(sbase + OFF_C, RBN);
       Tile t = *first_tile;
 #pragma unroll 1
       for (int n = 0; n < n_end; ++n, next_tile(t, d, a.w, TM, ntpu)) {
-        if (t.it == 0) {   // the chunk's rows come with its first tile
-          const int xs = x_index(n, ntpu);
-          mbar_wait_relaxed(&bars[B_X_FREE + xs], x_phase(n, ntpu) ^ 1, a.status);
-          mbar_expect_tx(&bars[B_X_FULL + xs], (uint32_t)(Q * 64));
-          for (int j0 = 0; j0 < Q; j0 += TM)
-            tma_load_3d(smem + OFF_X + xs * 16384 + j0 * 64, &tm_x, &bars[B_X_FULL + xs], 0, t.h, (int)(t.tok0 + j0));
-        }
-        mbar_wait_relaxed(&bars[B_CH_FREE], (n & 1) ^ 1, a.status);
-        mbar_expect_tx(&bars[B_CH_FULL], (uint32_t)(TM * N + 64 * N));
-        tma_load_3d(smem + OFF_C, &tm_C, &bars[B_CH_FULL], 0, t.h / a.w.hpg, (int)(t.tok0 + t.it * TM));
-        tma_load_2d(smem + OFF_H, &tm_h, &bars[B_CH_FULL], 0, (int)((((i64)t.b * d.c + t.k) * d.H + t.h) * P));
-      }
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer: C h.  (Two issuers, one per
-    // contraction: an issue is a chain of dependent instructions of one thread, and a single thread that issued
-    // the 8 or 12 MMAs of a tile in turn took 1.0 us per tile with nothing else in its way, half of the tile's
-    // time.)
-    if (lane == 0) {
-      const uint32_t idesc_off = idesc_s8(128, 64, 0, 0);
-      const uint32_t sbase = smem_u32(smem);
-      const uint64_t da = tile_desc(sbase + OFF_C, RBN), db = tile_desc(sbase + OFF_H, RBN);
-#pragma unroll 1
-      for (int n = 0; n < n_end; ++n) {
-        const int a4 = n & 3;
+        const int a4 = n & 3, xs = x_index(n, ntpu);
+        const uint64_t db = tile_desc(sbase + OFF_H + xs * H_BYTES, RBN);
         const uint32_t acc = tmem + (uint32_t)a4 * 128u;
-        mbar_wait(&bars[B_ACC_FREE + a4], ((n >> 2) & 1) ^ 1, a.status);
-        mbar_wait(&bars[B_CH_FULL], n & 1, a.status);
-        tc_fence_after();
-        // descriptors advance by a constant per 32-byte K step (their low bits are the address >> 4)
-        mma_s8_ss(acc, da, db, idesc_off, 0);
-        mma_s8_ss(acc, da + 2, db + 2, idesc_off, 1);
-        if (N == 128) {
-          mma_s8_ss(acc, da + 4, db + 4, idesc_off, 1);
-          mma_s8_ss(acc, da + 6, db + 6, idesc_off, 1);
+        const int tg = t.h / a.w.hpg;
+        mbar_wait(&bars[B_C_FREE], (n & 1) ^ 1, a.status);
+        if (elect_one()) {
+          mbar_expect_tx(&bars[B_C_FULL], (uint32_t)(TM * N));
+          tma_load_3d(smem + OFF_C, &tm_C, &bars[B_C_FULL], 0, tg, (int)(t.tok0 + t.it * TM));
         }
-        mma_commit(&bars[B_CH_FREE]);
-        mma_commit(&bars[B_ACC + a4]);
+        __syncwarp();
+        mbar_wait(&bars[B_ACC_FREE + a4], ((n >> 2) & 1) ^ 1, a.status);
+        mbar_wait(&bars[B_H_FULL + xs], x_phase(n, ntpu), a.status);
+        mbar_wait(&bars[B_C_FULL], n & 1, a.status);
+        tc_fence_after();
+        if (elect_one()) {
+          // descriptors advance by a constant per 32-byte K step (their low bits are the address >> 4)
+          mma_s8_ss(acc, da, db, idesc_off, 0);
+          mma_s8_ss(acc, da + 2, db + 2, idesc_off, 1);
+          if (N == 128) {
+            mma_s8_ss(acc, da + 4, db + 4, idesc_off, 1);
+            mma_s8_ss(acc, da + 6, db + 6, idesc_off, 1);
+          }
+          mma_commit(&bars[B_C_FREE]);
+          if (t.it + 1 == ntpu) mma_commit(&bars[B_H_FREE + xs]);   // the chunk's last tile
+          mma_commit(&bars[B_ACC + a4]);
+        }
+        __syncwarp();
       }
     }
   } else if (warp == 3) {
     // ------------------------------------------------------------ MMA issuer: Mq x
-    if (lane == 0) {
+    {
       const uint32_t idesc_diag = idesc_s8(128, 64, 0, 1);
       const uint32_t sbase = smem_u32(smem);
 #pragma unroll 1
@@ -403,19 +437,23 @@ chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ 
         mbar_wait(&bars[B_MQ + ci], ph4, a.status);
         tc_fence_after();
         constexpr uint64_t kStepX = (32 * 64) >> 4;   // 32 tokens of x
-        mma_s8_ss(acc, da, db, idesc_diag, 0);
-        mma_s8_ss(acc, da + 2, db + kStepX, idesc_diag, 1);
-        if (BIGQ) {
-          mma_s8_ss(acc, da + 4, db + 2 * kStepX, idesc_diag, 1);
-          mma_s8_ss(acc, da + 6, db + 3 * kStepX, idesc_diag, 1);
-          if (it) {   // the second panel of 128 columns
+        if (elect_one()) {
+          mma_s8_ss(acc, da, db, idesc_diag, 0);
+          mma_s8_ss(acc, da + 2, db + kStepX, idesc_diag, 1);
+          if (BIGQ) {
+            mma_s8_ss(acc, da + 4, db + 2 * kStepX, idesc_diag, 1);
+            mma_s8_ss(acc, da + 6, db + 3 * kStepX, idesc_diag, 1);
+            if (it) {   // the second panel of 128 columns
 #pragma unroll
-            for (uint32_t q = 0; q < 4; ++q)
-              mma_s8_ss(acc, da + (PANEL >> 4) + 2 * q, db + (4 + q) * kStepX, idesc_diag, 1);
+              for (uint32_t q = 0; q < 4; ++q)
+                mma_s8_ss(acc, da + (PANEL >> 4) + 2 * q, db + (4 + q) * kStepX, idesc_diag, 1);
+            }
           }
+          mma_commit(&bars[B_CB_FREE + ci]);
+          mma_commit(&bars[B_ACC + a4]);
+          if (it + 1 == ntpu) mma_commit(&bars[B_X_FREE + xs]);   // the chunk's last tile
         }
-        mma_commit(&bars[B_CB_FREE + ci]);
-        mma_commit(&bars[B_ACC + a4]);
+        __syncwarp();
       }
     }
   } else if (warp < kEpiWarp0) {
@@ -429,22 +467,24 @@ chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ 
     if (g) next_head(t, d, a.w, TM, ntpu);
 #pragma unroll 1
     for (int n = g * ntpu; n < n_end; ++n) {
-      const int ci = cb_index(n, t.it, ntpu), t3 = n & 3, r8 = n & 7;
+      const int ci = cb_index(n, t.it, ntpu), r8 = n & 7;
+      const int u = ntpu == 1 ? n : n >> 1, ts = u & 3;   // the chunk's scalar pack
       const uint32_t ph4 = (n >> 2) & 1;
       const int rb = t.it ? kGroupWarps - 1 - w : w;
       // one warp of the group polls (the scalar pack, the CBq tile, and the epilogue of the tile that
       // used the row slot); the others wait at a hardware barrier, which costs no issue slots
       if (w == 0 && lane < 3) {
-        const int bi = lane == 0 ? B_TOK_FULL + t3 : lane == 1 ? B_CB_FULL + ci : B_ROW_FREE + r8;
-        mbar_wait_relaxed(&bars[bi], lane == 2 ? (((n >> 3) & 1) ^ 1) : ph4, a.status);
+        const int bi = lane == 0 ? B_TOK_FULL + ts : lane == 1 ? B_CB_FULL + ci : B_ROW_FREE + r8;
+        mbar_wait(&bars[bi], lane == 2 ? (row_phase(n) ^ 1) : lane == 1 ? ph4 : ((u >> 2) & 1), a.status);
       }
       named_bar_sync(1 + g, kGroupWarps * 32);
-      mask_tile<TAPS>(smem + cb_offset(ci), reinterpret_cast<const float*>(smem + OFF_TOK + t3 * TOK_BYTES),
+      mask_tile<TAPS>(smem + cb_offset(ci), reinterpret_cast<const float*>(smem + OFF_TOK + ts * TOK_BYTES),
                       reinterpret_cast<float*>(smem + OFF_ROW + r8 * ROW_BYTES), rb, lane, TM, RBQ, t, a);
       fence_async_smem();
       __syncwarp();
-      if (lane < 3) mbar_arrive(&bars[lane == 0 ? B_MQ + ci : lane == 1 ? B_TOK_FREE + t3 : B_ROW_FULL + r8]);
-      if (t.it + 1 < ntpu) {   // the chunk's second tile
+      const bool last = t.it + 1 == ntpu;   // the scalar pack serves both tiles of the chunk
+      if (lane < (last ? 3 : 2)) mbar_arrive(&bars[lane == 0 ? B_MQ + ci : lane == 1 ? B_ROW_FULL + r8 : B_TOK_FREE + ts]);
+      if (!last) {             // the chunk's second tile
         t.it = 1;
         t.KJ = 2 * TM;
       } else {                 // skip the other group's chunk (or tile)
@@ -474,61 +514,71 @@ chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ 
       const float4* ssx = reinterpret_cast<const float4*>(row + ROW_COLS / 4);
       const float4* ssh = ssx + 16;
       const float4* sco = ssx + 32;
-      // three lanes of one warp of the group poll side by side, one barrier each: the accumulators, the
-      // xq rows (skip term), and the row slot (the head's column vectors and the row scalars written by
-      // the mask warps; not the mask barrier of the CBq buffer, which may complete a second time before
-      // this group gets here); the other warps wait at a hardware barrier, which costs no issue slots
-      if (q == 0 && lane < 3) {
-        const int bi = lane == 0 ? B_ACC + a4 : lane == 1 ? B_X_FULL + xs : B_ROW_FULL + (n & 7);
-        const uint32_t bp = lane == 0 ? ph4 : lane == 1 ? x_phase(n, ntpu) : ((n >> 3) & 1);
-        mbar_wait_relaxed(&bars[bi], bp, a.status);
-      }
-      named_bar_sync(3 + eg, kEpiGroupWarps * 32);
-      tc_fence_after();
       const bool ok = er < TM;
       const int ei = t.it * TM + er;
+      // The row of x for the skip term goes to registers before the accumulators are waited for, and the warp
+      // hands its share of the buffer back: were it read (and released) with the accumulators, the load of the
+      // chunk after next would wait for the end of this epilogue, and with it the MMAs, the CBq buffers and the
+      // mask of that chunk.
+      uint4 xr[4];
+      mbar_wait(&bars[B_X_FULL + xs], x_phase(n, ntpu), a.status);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        xr[j] = ok ? *reinterpret_cast<const uint4*>(sX + swz_off((uint32_t)ei, (uint32_t)j, 64)) : make_uint4(0u, 0u, 0u, 0u);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars[B_X_FREE + xs]);
+      // two lanes of one warp of the group poll side by side, one barrier each: the accumulators and the row
+      // slot (the head's column vectors and the row scalars written by the mask warps; not the mask barrier of
+      // the CBq buffer, which may complete a second time before this group gets here); the other warps wait at
+      // a hardware barrier, which costs no issue slots
+      if (q == 0 && lane < 2) mbar_wait(&bars[lane == 0 ? B_ACC + a4 : B_ROW_FULL + (n & 7)], lane == 0 ? ph4 : row_phase(n), a.status);
+      named_bar_sync(3 + eg, kEpiGroupWarps * 32);
+      tc_fence_after();
       const float sC = row[ROW_SCAL / 4], Dh = row[ROW_SCAL / 4 + 1], scb = row[ROW_SCAL / 4 + 2];
       const float dec = ok ? exp32(row[128 + er]) * sC : 0.f;
       const float sm = ok ? scb * row[er] * (1.0f / 127.0f) : 0.f;
       const float2 dec2 = make_float2(dec, dec), sm2 = make_float2(sm, sm), Dh2 = make_float2(Dh, Dh);
       const uint32_t tbase = tmem + (uint32_t)a4 * 128u + ((uint32_t)(q * 32) << 16);
-#pragma unroll 4                           // (a round of 32 columns per iteration: the piece index folds into addresses)
+#pragma unroll                             // (the piece index folds into addresses and registers)
       for (int pc = 0; pc < 8; ++pc) {       // 8 columns at a time (keeps the accumulators in registers)
         int acc_o[8], acc_d[8];
         tmem_ld8(tbase + pc * 8, acc_o);
         tmem_ld8(tbase + 64 + pc * 8, acc_d);
-        if ((pc & (PPR - 1)) == 0) {         // the last store has finished reading the staging tile
+        const uint4& x4 = xr[pc >> 1];
+        const uint32_t xw[2] = {(pc & 1 ? x4.z : x4.x) ^ 0x80808080u, (pc & 1 ? x4.w : x4.y) ^ 0x80808080u};
+        float2 v[4];
+        tmem_ld_wait();
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc) {
+          const float4 sx4 = ssx[pc * 2 + cc], sh4 = ssh[pc * 2 + cc];
+          const float4 co4 = CORR ? sco[pc * 2 + cc] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int e2 = 0; e2 < 2; ++e2) {
+            const int pp = cc * 4 + e2 * 2;
+            const float2 sx2 = e2 ? make_float2(sx4.z, sx4.w) : make_float2(sx4.x, sx4.y);
+            const float2 sh2 = e2 ? make_float2(sh4.z, sh4.w) : make_float2(sh4.x, sh4.y);
+            const float2 co2 = e2 ? make_float2(co4.z, co4.w) : make_float2(co4.x, co4.y);
+            const float2 xv = unpack2(xw[cc], e2 * 2);
+            const float2 ao = make_float2((float)acc_o[pp], (float)acc_o[pp + 1]);
+            const float2 ad = make_float2((float)acc_d[pp], (float)acc_d[pp + 1]);
+            // y = s_x (s_M acc_diag + D x) + s_h (dec acc_off) + corr: five packed operations
+            const float2 u2 = __ffma2_rn(sm2, ad, __fmul2_rn(Dh2, xv));
+            const float2 r2 = __ffma2_rn(sx2, u2, co2);
+            v[cc * 2 + e2] = __ffma2_rn(sh2, __fmul2_rn(dec2, ao), r2);
+          }
+        }
+        // the staging tile must have been read by the last store: waited for here, with this piece's arithmetic done
+        if ((pc & (PPR - 1)) == 0) {
           if (lane == 3) tma_store_wait_read();
           __syncwarp();
         }
-        tmem_ld_wait();
         if (ok) {
-          const uint2 xr = *reinterpret_cast<const uint2*>(sX + swz_off((uint32_t)ei, (uint32_t)(pc >> 1), 64) + (pc & 1) * 8);
-          const uint32_t xw[2] = {xr.x ^ 0x80808080u, xr.y ^ 0x80808080u};
-          float2 v[4];
+          if (YT == 0) {  // 4 values = one 16-byte chunk
 #pragma unroll
-          for (int cc = 0; cc < 2; ++cc) {
-            const float4 sx4 = ssx[pc * 2 + cc], sh4 = ssh[pc * 2 + cc];
-            const float4 co4 = CORR ? sco[pc * 2 + cc] : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int e2 = 0; e2 < 2; ++e2) {
-              const int pp = cc * 4 + e2 * 2;
-              const float2 sx2 = e2 ? make_float2(sx4.z, sx4.w) : make_float2(sx4.x, sx4.y);
-              const float2 sh2 = e2 ? make_float2(sh4.z, sh4.w) : make_float2(sh4.x, sh4.y);
-              const float2 co2 = e2 ? make_float2(co4.z, co4.w) : make_float2(co4.x, co4.y);
-              const float2 xv = unpack2(xw[cc], e2 * 2);
-              const float2 ao = make_float2((float)acc_o[pp], (float)acc_o[pp + 1]);
-              const float2 ad = make_float2((float)acc_d[pp], (float)acc_d[pp + 1]);
-              // y = s_x (s_M acc_diag + D x) + s_h (dec acc_off) + corr: five packed operations
-              const float2 u2 = __ffma2_rn(sm2, ad, __fmul2_rn(Dh2, xv));
-              const float2 r2 = __ffma2_rn(sx2, u2, co2);
-              v[cc * 2 + e2] = __ffma2_rn(sh2, __fmul2_rn(dec2, ao), r2);
-            }
-            if (YT == 0)   // 4 values = one 16-byte chunk
+            for (int cc = 0; cc < 2; ++cc)
               *reinterpret_cast<float4*>(srow + ((((pc & 3) * 2 + cc) ^ (lane & 7)) << 4)) =
                   make_float4(v[cc * 2].x, v[cc * 2].y, v[cc * 2 + 1].x, v[cc * 2 + 1].y);
-          }
-          if (YT != 0) {  // 8 values = one 16-byte chunk
+          } else {        // 8 values = one 16-byte chunk
             uint32_t h[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -555,8 +605,8 @@ chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ 
           if (pc == 7) tc_fence_before();
           fence_async_smem();
           __syncwarp();
-          if (pc == 7 && lane < 3) {         // one release each, side by side
-            mbar_arrive(&bars[lane == 0 ? B_ACC_FREE + a4 : lane == 1 ? B_X_FREE + xs : B_ROW_FREE + (n & 7)]);
+          if (pc == 7 && lane < 2) {         // one release each, side by side
+            mbar_arrive(&bars[lane == 0 ? B_ACC_FREE + a4 : B_ROW_FREE + (n & 7)]);
           } else if (lane == 3 && q * 32 < TM) {
             tma_store_3d(&tm_y, ystage, (pc / PPR) * 32, t.h, (int)(t.tok0 + t.it * TM + q * 32));
             tma_store_commit();
@@ -633,10 +683,13 @@ ssdi8_status_t launch_chunk_scan(const Dims& d, const int8_t* xq, const int8_t* 
   int grid_i = 0;
   if (!make_unit_walk(d, TM, sms, &walk, &grid_i)) return SSDI8_ERR_SHAPE;
   ScanArgs a = {s_x, s_C, s_cb, s_h, pack, D, corr, static_cast<uint8_t*>(y), status, taps, d, walk};
-  const size_t smem = SMEM_BYTES + 1024;
+  const size_t smem = SMEM_BYTES;
   const unsigned grid = (unsigned)grid_i;
   const bool tp = taps.acc_off || taps.rowmax || taps.Mq || taps.acc_diag;
   auto launch = [&](auto kernel) -> ssdi8_status_t {
+    cudaFuncAttributes fa;
+    SSDI8_CUDA_CHECK(cudaFuncGetAttributes(&fa, kernel));
+    if (fa.sharedSizeBytes != 0) return SSDI8_ERR_CUDA;   // the dynamic part must start at the window's base
     SSDI8_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     return launch_pdl(kernel, dim3(grid), dim3(kThreads), smem, st, tm_C, tm_h, tm_x, tm_cb, tm_y, a) == cudaSuccess ? SSDI8_OK : SSDI8_ERR_CUDA;
   };

@@ -106,6 +106,14 @@ __device__ __forceinline__ void mbar_wait_inline(uint64_t* bar, uint32_t parity,
   if (status) atomicExch(status, (int32_t)SSDI8_ERR_DEVICE_TIMEOUT);
 }
 
+// One lane of the (converged) warp.  Issue loops run with the whole warp and elect the issuing lane only around
+// the instructions themselves, so that descriptors and addresses stay in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // ------------------------------------------------------------------ proxies and fences
 __device__ __forceinline__ void fence_async_smem() {  // generic-proxy smem writes -> async proxy
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
