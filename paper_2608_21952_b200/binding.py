@@ -1,9 +1,10 @@
-"""Thin ctypes binding of libssdi8 (argument marshalling only).
+"""Thin binding of libssdi8 (argument marshalling only).
 
 The functions carry the names of the C entry points declared in include/ssdi8.h
 and take torch CUDA tensors; every step of the computation runs inside the
-library's kernels.  There is no fallback: if the library cannot be loaded the
-import raises.
+library's kernels.  The calls that enqueue work go through the native marshalling
+module (csrc/marshal.cpp), the rest through ctypes.  There is no fallback: if either
+cannot be loaded the import raises.
 """
 from __future__ import annotations
 
@@ -20,6 +21,9 @@ if not os.path.exists(_LIB_PATH):
         f"{_LIB_PATH} is missing: build it with `python -m paper_2608_21952_b200.build` "
         "(nvcc, sm_100a); there is no CPU or PyTorch fallback")
 _lib = C.CDLL(_LIB_PATH)
+if not os.path.exists(_build.MARSHAL):
+    raise ImportError(f"{_build.MARSHAL} is missing: build it with `python -m paper_2608_21952_b200.build`")
+from . import _marshal as _m  # noqa: E402  (linked against the library loaded above)
 
 OK = 0
 ERR_NULL, ERR_SHAPE, ERR_ALIGN, ERR_WORKSPACE, ERR_ARCH, ERR_CUDA, ERR_DEVICE_TIMEOUT, ERR_UNSUPPORTED = \
@@ -134,8 +138,9 @@ def ssdi8_workspace_bytes(dims: Dims, flags: int = 0) -> int:
 
 
 def ssdi8_quantize_act(inp, R: int, Ch: int, I: int, scale, mode: int, out, stream=None) -> None:
-    _check(_lib.ssdi8_quantize_act(_ptr(inp), R, Ch, I, _ptr(scale), mode, _ptr(out), _stream(stream)),
-           "ssdi8_quantize_act")
+    code = _m.quantize_act(inp, R, Ch, I, scale, mode, out, stream)
+    if code:
+        _check(code, "ssdi8_quantize_act")
 
 
 def make_fwd_args(**tensors) -> FwdArgs:
@@ -149,23 +154,24 @@ def make_fwd_args(**tensors) -> FwdArgs:
 
 
 def ssdi8_chunk_scan_fwd(dims: Dims, args: FwdArgs, workspace, flags: int = 0, stream=None) -> None:
-    _check(_lib.ssdi8_chunk_scan_fwd(C.byref(dims), C.byref(args), flags, _ptr(workspace),
-                                     workspace.numel() * workspace.element_size(), _stream(stream)),
-           "ssdi8_chunk_scan_fwd")
+    code = _m.chunk_scan_fwd(dims, args, workspace, flags, stream)
+    if code:
+        _check(code, "ssdi8_chunk_scan_fwd")
 
 
 def ssdi8_chunk_scan_fwd_static(dims: Dims, args: FwdArgs, flags: int = 0, stream=None) -> None:
     """Forward pass on the library's built-in scratch: no workspace argument, no allocation.
     For callers that cannot allocate device memory; raises SSDi8Error(ERR_WORKSPACE) when the
     dimensions need more than STATIC_WORKSPACE_BYTES."""
-    _check(_lib.ssdi8_chunk_scan_fwd_static(C.byref(dims), C.byref(args), flags, _stream(stream)),
-           "ssdi8_chunk_scan_fwd_static")
+    code = _m.chunk_scan_fwd_static(dims, args, flags, stream)
+    if code:
+        _check(code, "ssdi8_chunk_scan_fwd_static")
 
 
 def ssdi8_calibrate(dims: Dims, args: FwdArgs, s_xs, s_cb, s_h, workspace, stream=None) -> None:
-    _check(_lib.ssdi8_calibrate(C.byref(dims), C.byref(args), _ptr(s_xs), _ptr(s_cb), _ptr(s_h),
-                                _ptr(workspace), workspace.numel() * workspace.element_size(),
-                                _stream(stream)), "ssdi8_calibrate")
+    code = _m.calibrate(dims, args, s_xs, s_cb, s_h, workspace, stream)
+    if code:
+        _check(code, "ssdi8_calibrate")
 
 
 _lib.ssdi8_layer_fwd_host_scratch_bytes.restype = C.c_size_t
@@ -205,9 +211,9 @@ def ssdi8_layer_fwd_workspace_bytes(dims: Dims, flags: int = 0) -> int:
 
 
 def ssdi8_layer_fwd(dims: Dims, args: LayerArgs, workspace, flags: int = 0, stream=None) -> None:
-    _check(_lib.ssdi8_layer_fwd(C.byref(dims), C.byref(args), _ptr(workspace),
-                                workspace.numel() * workspace.element_size(), flags, _stream(stream)),
-           "ssdi8_layer_fwd")
+    code = _m.layer_fwd(dims, args, workspace, flags, stream)
+    if code:
+        _check(code, "ssdi8_layer_fwd")
 
 
 def ssdi8_layer_fwd_host_scratch_bytes(dims: Dims, flags: int = 0) -> int:
@@ -215,18 +221,18 @@ def ssdi8_layer_fwd_host_scratch_bytes(dims: Dims, flags: int = 0) -> int:
 
 
 def ssdi8_layer_fwd_host(dims: Dims, args: LayerArgs, scratch, flags: int = 0, stream=None) -> None:
-    _check(_lib.ssdi8_layer_fwd_host(C.byref(dims), C.byref(args), _ptr(scratch),
-                                     scratch.numel() * scratch.element_size(), flags, _stream(stream)),
-           "ssdi8_layer_fwd_host")
+    code = _m.layer_fwd_host(dims, args, scratch, flags, stream)
+    if code:
+        _check(code, "ssdi8_layer_fwd_host")
 
 
 _ENTRY_DTYPES = {torch.float32: 0, torch.float16: 1, torch.bfloat16: 2}
 
 
 def ssdi8_quantize_entry(xBC, T: int, D: int, G: int, N: int, s_x, s_B, s_C, xq, Bq, Cq, stream=None) -> None:
-    _check(_lib.ssdi8_quantize_entry(_ptr(xBC), _ENTRY_DTYPES[xBC.dtype], T, D, G, N, _ptr(s_x), _ptr(s_B),
-                                     _ptr(s_C), _ptr(xq), _ptr(Bq), _ptr(Cq), _stream(stream)),
-           "ssdi8_quantize_entry")
+    code = _m.quantize_entry(xBC, _ENTRY_DTYPES[xBC.dtype], T, D, G, N, s_x, s_B, s_C, xq, Bq, Cq, stream)
+    if code:
+        _check(code, "ssdi8_quantize_entry")
 
 
 def ssdi8_mean_correction_workspace_bytes(Ch: int) -> int:
@@ -234,22 +240,22 @@ def ssdi8_mean_correction_workspace_bytes(Ch: int) -> int:
 
 
 def ssdi8_mean_correction(y_ref, y_q, R: int, Ch: int, eta: float, corr, workspace, stream=None) -> None:
-    _check(_lib.ssdi8_mean_correction(_ptr(y_ref), _ptr(y_q), R, Ch, eta, _ptr(corr), _ptr(workspace),
-                                      workspace.numel() * workspace.element_size(), _stream(stream)),
-           "ssdi8_mean_correction")
+    code = _m.mean_correction(y_ref, y_q, R, Ch, eta, corr, workspace, stream)
+    if code:
+        _check(code, "ssdi8_mean_correction")
 
 
 def ssdi8_state_passing(dims: Dims, loc, gamma, init_state, prev, final_state, hq, s_h,
                         stream=None) -> None:
-    _check(_lib.ssdi8_state_passing(C.byref(dims), _ptr(loc), _ptr(gamma), _ptr(init_state), _ptr(prev),
-                                    _ptr(final_state), _ptr(hq), _ptr(s_h), _stream(stream)),
-           "ssdi8_state_passing")
+    code = _m.state_passing(dims, loc, gamma, init_state, prev, final_state, hq, s_h, stream)
+    if code:
+        _check(code, "ssdi8_state_passing")
 
 
 def ssdi8_ssd_step(dims: Dims, xq, s_x, Bq, s_B, Cq, s_C, dt, A, D, corr, state, y, stream=None) -> None:
-    _check(_lib.ssdi8_ssd_step(C.byref(dims), _ptr(xq), _ptr(s_x), _ptr(Bq), _ptr(s_B), _ptr(Cq),
-                               _ptr(s_C), _ptr(dt), _ptr(A), _ptr(D), _ptr(corr), _ptr(state), _ptr(y),
-                               _stream(stream)), "ssdi8_ssd_step")
+    code = _m.ssd_step(dims, xq, s_x, Bq, s_B, Cq, s_C, dt, A, D, corr, state, y, stream)
+    if code:
+        _check(code, "ssdi8_ssd_step")
 
 
 _lib.ssdi8_int8_mma_peak.restype = C.c_int32
@@ -263,8 +269,9 @@ _lib.ssdi8_softplus_dt.argtypes = [C.c_void_p, C.c_void_p, C.c_int64, C.c_int32,
 
 
 def ssdi8_softplus_dt(dt_raw, dt_bias, rows: int, H: int, dt, stream=None) -> None:
-    _check(_lib.ssdi8_softplus_dt(_ptr(dt_raw), _ptr(dt_bias), rows, H, _ptr(dt), _stream(stream)),
-           "ssdi8_softplus_dt")
+    code = _m.softplus_dt(dt_raw, dt_bias, rows, H, dt, stream)
+    if code:
+        _check(code, "ssdi8_softplus_dt")
 
 
 def ssdi8_int8_mma_peak(mma_per_sm: int, status=None, stream=None) -> float:

@@ -1,4 +1,5 @@
-"""Builds libssdi8.so (the C-ABI CUDA library) in-tree for sm_100a with nvcc."""
+"""Builds libssdi8.so (the C-ABI CUDA library) in-tree for sm_100a with nvcc, and _marshal.so (the argument marshalling of
+the Python binding) with the host compiler against the installed torch."""
 from __future__ import annotations
 
 import glob
@@ -8,9 +9,11 @@ import subprocess
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libssdi8.so")
+MARSHAL_SRC = os.path.join(CSRC, "marshal.cpp")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17", "--threads", "0",
-              "-Xcompiler", "-fPIC", "-shared"]
+              "-Xcompiler", "-fPIC", "-shared", "-Xlinker", "-soname=libssdi8.so"]
 
 
 def sources():
@@ -26,7 +29,32 @@ def _stale() -> bool:
     return any(os.path.getmtime(p) > t for p in deps)
 
 
+def build_marshal(force: bool = False) -> str:
+    header = os.path.join(os.path.dirname(HERE), "include", "ssdi8.h")
+    if not force and os.path.exists(MARSHAL) and \
+            os.path.getmtime(MARSHAL) >= max(os.path.getmtime(MARSHAL_SRC), os.path.getmtime(header)):
+        return MARSHAL
+    import sysconfig
+    import torch
+    from torch.utils.cpp_extension import include_paths, library_paths
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd += ["-I" + p for p in (*include_paths(), sysconfig.get_paths()["include"], os.path.join(cuda, "include"))]
+    cmd += ["-o", MARSHAL, MARSHAL_SRC]
+    cmd += ["-L" + p for p in library_paths()]
+    cmd += ["-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10", LIB, "-Wl,-rpath,$ORIGIN"]
+    subprocess.run(cmd, check=True)
+    return MARSHAL
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    lib = build_library(force, verbose)
+    build_marshal(force)
+    return lib
+
+
+def build_library(force: bool = False, verbose: bool = False) -> str:
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
