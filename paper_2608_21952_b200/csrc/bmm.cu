@@ -177,11 +177,8 @@ ssdi8_status_t launch_bmm(const Dims& d, const int8_t* Cq, const int8_t* Bq, con
   }
   BmmArgs a = {s_C, s_B, s_cb, tap_acc, absmax_acc, status, d, store ? 1 : 0, after_state_kernel ? 1 : 0};
   const size_t smem = SMEM_BYTES + 1024;
-  SSDI8_CUDA_CHECK(cudaFuncSetAttribute(bmm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const unsigned grid = (unsigned)((i64)d.b * d.c * d.G * (d.Q / TM));
-  if (launch_pdl(bmm_tc, dim3(grid), dim3(kThreads), smem, st, tm_C, tm_B, tm_o, a) != cudaSuccess) return SSDI8_ERR_CUDA;
-  SSDI8_LAUNCH_CHECK();
-  return SSDI8_OK;
+  return launch_configured(bmm_tc, dim3(grid), dim3(kThreads), smem, -1, false, st, tm_C, tm_B, tm_o, a);
 }
 
 }  // namespace ssdi8

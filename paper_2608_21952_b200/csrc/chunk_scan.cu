@@ -676,9 +676,8 @@ ssdi8_status_t launch_chunk_scan(const Dims& d, const int8_t* xq, const int8_t* 
     uint32_t box[3] = {ydt ? 64u : 32u, 1, 32};   // 128 bytes of a row per store
     if (!encode_tensor_map(&tm_y, y, (int)eb, 3, dims, str, box, 128)) return SSDI8_ERR_CUDA;
   }
-  int dev = 0, sms = 0;
-  SSDI8_CUDA_CHECK(cudaGetDevice(&dev));
-  SSDI8_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int sms = sm_count();
+  if (sms == 0) return SSDI8_ERR_CUDA;
   UnitWalk walk;
   int grid_i = 0;
   if (!make_unit_walk(d, TM, sms, &walk, &grid_i)) return SSDI8_ERR_SHAPE;
@@ -687,11 +686,7 @@ ssdi8_status_t launch_chunk_scan(const Dims& d, const int8_t* xq, const int8_t* 
   const unsigned grid = (unsigned)grid_i;
   const bool tp = taps.acc_off || taps.rowmax || taps.Mq || taps.acc_diag;
   auto launch = [&](auto kernel) -> ssdi8_status_t {
-    cudaFuncAttributes fa;
-    SSDI8_CUDA_CHECK(cudaFuncGetAttributes(&fa, kernel));
-    if (fa.sharedSizeBytes != 0) return SSDI8_ERR_CUDA;   // the dynamic part must start at the window's base
-    SSDI8_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    return launch_pdl(kernel, dim3(grid), dim3(kThreads), smem, st, tm_C, tm_h, tm_x, tm_cb, tm_y, a) == cudaSuccess ? SSDI8_OK : SSDI8_ERR_CUDA;
+    return launch_configured(kernel, dim3(grid), dim3(kThreads), smem, -1, true, st, tm_C, tm_h, tm_x, tm_cb, tm_y, a);
   };
   if (tp && ydt) return SSDI8_ERR_UNSUPPORTED;  // the taps come with binary32 y only
   const bool big = d.Q >= 128;

@@ -576,9 +576,8 @@ ssdi8_status_t launch_chunk_scan_f16(const Dims& d, const int8_t* xq, const int8
     uint32_t box[3] = {ydt ? 32u : 16u, 1, 32};
     if (!encode_tensor_map(&tm_y, y, (int)eb, 3, dims, str, box, 64)) return SSDI8_ERR_CUDA;
   }
-  int dev = 0, sms = 0;
-  SSDI8_CUDA_CHECK(cudaGetDevice(&dev));
-  SSDI8_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int sms = sm_count();
+  if (sms == 0) return SSDI8_ERR_CUDA;
   UnitWalk walk;
   int grid_i = 0;
   if (!make_unit_walk(d, TM, sms, &walk, &grid_i)) return SSDI8_ERR_SHAPE;
@@ -586,8 +585,7 @@ ssdi8_status_t launch_chunk_scan_f16(const Dims& d, const int8_t* xq, const int8
   const size_t smem = SMEM_BYTES + 1024;
   const unsigned grid = (unsigned)grid_i;
   auto launch = [&](auto kernel) -> ssdi8_status_t {
-    SSDI8_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    return launch_pdl(kernel, dim3(grid), dim3(kThreads), smem, st, tm_C, tm_h, tm_x, tm_cb, tm_y, a) == cudaSuccess ? SSDI8_OK : SSDI8_ERR_CUDA;
+    return launch_configured(kernel, dim3(grid), dim3(kThreads), smem, -1, false, st, tm_C, tm_h, tm_x, tm_cb, tm_y, a);
   };
   const bool big = d.Q >= 128;
   auto pick = [&](auto corr_c, auto big_c) -> ssdi8_status_t {

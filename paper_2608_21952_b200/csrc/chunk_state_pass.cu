@@ -475,9 +475,8 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
   // units, and the units of a last, partly filled wave as four quarter-width CTAs each, which pack
   // into that wave's free slots (a quarter costs about a third of a whole unit: the operand tiles
   // and the MMA stay full width)
-  int dev = 0, sms = 0;
-  SSDI8_CUDA_CHECK(cudaGetDevice(&dev));
-  SSDI8_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int sms = sm_count();
+  if (sms == 0) return SSDI8_ERR_CUDA;
   const int units = d.H * d.b, slots = 3 * sms;
   // Whole (batch, head) units wherever the device is filled: with three CTAs per SM the kernel is bound
   // by instruction issue, so a partly filled last wave of whole units runs faster per CTA and costs less
@@ -494,11 +493,7 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
   const unsigned grid = (unsigned)(n_full + split * (units - n_full));
   const bool taps = tap_loc || tap_prev || tap_Xsq || tap_acc;
   auto launch = [&](auto kernel) -> ssdi8_status_t {
-    cudaFuncAttributes fa;
-    SSDI8_CUDA_CHECK(cudaFuncGetAttributes(&fa, kernel));
-    if (fa.sharedSizeBytes != 0) return SSDI8_ERR_CUDA;   // the dynamic part must start at the window's base
-    SSDI8_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    return launch_pdl(kernel, dim3(grid), dim3(kThreads), smem, st, tm_B, tm_x, tm_hq, a) == cudaSuccess ? SSDI8_OK : SSDI8_ERR_CUDA;
+    return launch_configured(kernel, dim3(grid), dim3(kThreads), smem, -1, true, st, tm_B, tm_x, tm_hq, a);
   };
   ssdi8_status_t ls;
   if (int8_state)

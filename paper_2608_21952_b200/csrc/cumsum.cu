@@ -236,17 +236,15 @@ ssdi8_status_t launch_softplus_dt(const float* dt_raw, const float* dt_bias, flo
 
 ssdi8_status_t launch_cumsum(const Dims& d, const float* dt, const float* A, float* pack, float* gamma, float* tap_cs,
                              cudaStream_t st, const float* dt_bias, bool softplus, int32_t* clear_status) {
-  int dev = 0, sms = 0;
-  SSDI8_CUDA_CHECK(cudaGetDevice(&dev));
-  SSDI8_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int sms = sm_count();
+  if (sms == 0) return SSDI8_ERR_CUDA;
   // a grid that leaves SMs empty takes half the heads per block: one warp per scheduler, twice the SMs
   int hpb = kMaxHeads;
   if ((i64)((d.H + hpb - 1) / hpb) * d.c * d.b <= sms) hpb /= 2;
   const dim3 grid((d.H + hpb - 1) / hpb, d.c, d.b);
   auto launch = [&](auto kernel) -> ssdi8_status_t {
-    SSDI8_CUDA_CHECK(prefer_l1(kernel));
-    return launch_pdl(kernel, grid, dim3(32 * hpb), 0, st, dt, A, pack, gamma, tap_cs, d, dt_bias, clear_status) == cudaSuccess
-               ? SSDI8_OK : SSDI8_ERR_CUDA;
+    return launch_configured(kernel, grid, dim3(32 * hpb), 0, kStreamCarveout, false, st, dt, A, pack, gamma, tap_cs, d,
+                             dt_bias, clear_status);
   };
   ssdi8_status_t ls;
   if (d.Q == 256)

@@ -24,6 +24,26 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// Launch attributes of a kernel (largest dynamic shared memory, preferred share of shared memory in percent or -1),
+// set at its first launch on a device and remembered per kernel and device (launch_state.cu; set on
+// every call they are 1.2 us of the 14.7 us of host time of a layer call).  check_static: fail if the
+// kernel uses static shared memory (kernels that need their dynamic part at the window's base).
+cudaError_t kernel_ready(const void* kernel, size_t smem, int carveout, bool check_static);
+void kernel_forget(const void* kernel);   // the device was reset under us: set the attributes again
+template <typename... KArgs, typename... Args>
+inline ssdi8_status_t launch_configured(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, int carveout,
+                                        bool check_static, cudaStream_t st, Args&&... args) {
+  const void* k = reinterpret_cast<const void*>(kernel);
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    if (kernel_ready(k, smem, carveout, check_static) != cudaSuccess) break;
+    if (launch_pdl(kernel, grid, block, smem, st, args...) == cudaSuccess) return SSDI8_OK;
+    kernel_forget(k);
+  }
+  (void)cudaGetLastError();
+  return SSDI8_ERR_CUDA;
+}
+int sm_count();   // of the current device (0 on failure)
+
 // L1 / shared memory split of the streaming kernels that lead a layer (ChunkCumsum, the quantisers), in percent
 // of shared memory: 64 KB of 228.  Launched through programmatic dependent launch right behind ChunkScan they
 // would otherwise inherit its split (28 KB of L1), too little for the loads a streaming kernel keeps in flight
@@ -31,10 +51,6 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 // 0.300 ms without and 0.279 ms with the preference (1.03 and 0.94 ms at batch 4 x 8192 x 128 heads); 0, 14, 44
 // and 58 percent are within 2 % of it.
 constexpr int kStreamCarveout = 28;
-template <typename K>
-inline cudaError_t prefer_l1(K kernel) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, kStreamCarveout);
-}
 
 ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* scale, int mode,
                                int8_t* out, cudaStream_t st);

@@ -273,10 +273,7 @@ ssdi8_status_t launch_quantize_xbc(const float* x, const float* B, const float* 
   nb = fill(a.job[1], C, s_C, Cq, G * N, shift, nb);
   nb = fill(a.job[2], x, s_x, xq, D, 0, nb);
   a.late_wait = after_cumsum ? 1 : 0;
-  SSDI8_CUDA_CHECK(prefer_l1(quant_jobs));
-  if (launch_pdl(quant_jobs, dim3((unsigned)nb), dim3(128), 0, st, a) != cudaSuccess) return SSDI8_ERR_CUDA;
-  SSDI8_LAUNCH_CHECK();
-  return SSDI8_OK;
+  return launch_configured(quant_jobs, dim3((unsigned)nb), dim3(128), 0, kStreamCarveout, false, st, a);
 }
 
 // bits[k] holds either a binary32 absmax or (bits_are_int) an int32 absmax; the step size is

@@ -17,6 +17,8 @@ __global__ void __launch_bounds__(ST_T) ssd_step_kernel(
     const float* __restrict__ s_B, const uint32_t* __restrict__ Cq, const float* __restrict__ s_C,
     const float* __restrict__ dt, const float* __restrict__ A, const float* __restrict__ D,
     const float* __restrict__ corr, float4* __restrict__ state, float* __restrict__ y, Dims d) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int lane = threadIdx.x % N4;
   const i64 grp = ((i64)blockIdx.x * ST_T + threadIdx.x) / N4;  // over b*H*P/ROWS
   const int pgroups = d.P / ROWS;
@@ -77,12 +79,11 @@ ssdi8_status_t launch_ssd_step(const Dims& d, const int8_t* xq, const float* s_x
   auto Bw = reinterpret_cast<const uint32_t*>(Bq);
   auto Cw = reinterpret_cast<const uint32_t*>(Cq);
   auto S4 = reinterpret_cast<float4*>(state);
-  if (N4 == 32)
-    ssd_step_kernel<32><<<grid, ST_T, 0, st>>>(xq, s_x, Bw, s_B, Cw, s_C, dt, A, D, corr, S4, y, d);
-  else
-    ssd_step_kernel<16><<<grid, ST_T, 0, st>>>(xq, s_x, Bw, s_B, Cw, s_C, dt, A, D, corr, S4, y, d);
-  SSDI8_LAUNCH_CHECK();
-  return SSDI8_OK;
+  auto launch = [&](auto kernel) -> ssdi8_status_t {
+    return launch_configured(kernel, dim3(grid), dim3(ST_T), 0, kStreamCarveout, false, st, xq, s_x, Bw, s_B, Cw, s_C, dt, A,
+                             D, corr, S4, y, d);
+  };
+  return N4 == 32 ? launch(ssd_step_kernel<32>) : launch(ssd_step_kernel<16>);
 }
 
 }  // namespace ssdi8
