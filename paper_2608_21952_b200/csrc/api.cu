@@ -183,11 +183,11 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
   } else {
     if ((ph & SSDI8_PHASE_CHUNK_STATE) &&
         (s = launch_chunk_state(d, a->xq, a->Bq, a->s_x, a->s_xs, a->s_B, pack, loc, a->tap_Xsq,
-                                a->tap_acc_st, nullptr, a->status, st)) != SSDI8_OK)
+                                a->tap_acc_st, a->status, st)) != SSDI8_OK)
       return s;
     if ((ph & SSDI8_PHASE_STATE_PASSING) &&
         (s = launch_state_passing(d, loc, gamma, a->init_state, a->s_h, a->tap_prev, a->final_state,
-                                  hq, nullptr, st)) != SSDI8_OK)
+                                  hq, st)) != SSDI8_OK)
       return s;
   }
   if ((ph & SSDI8_PHASE_SCAN) && f16op)
@@ -225,28 +225,21 @@ ssdi8_status_t ssdi8_calibrate(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t*
   char* ws = static_cast<char*>(workspace);
   float* pack = reinterpret_cast<float*>(ws + w.pack);
   float* gamma = reinterpret_cast<float*>(ws + w.gamma);
-  float* loc = reinterpret_cast<float*>(ws + w.loc);
   const i64 nhp = (i64)d.H * d.P;
-  // the outputs double as the running maxima (bit patterns), finalised in place
-  SSDI8_CUDA_CHECK(cudaMemsetAsync(s_xs, 0, sizeof(float) * nhp, st));
-  SSDI8_CUDA_CHECK(cudaMemsetAsync(s_cb, 0, sizeof(float) * d.G, st));
-  SSDI8_CUDA_CHECK(cudaMemsetAsync(s_h, 0, sizeof(float) * nhp, st));
+  // The outputs double as the running maxima (bit patterns), finalised in place.  Eight launches, chained by
+  // programmatic dependent launch; the chunk-local states stay on the chip (see the state kernel's calibration pass).
+  if ((s = launch_clear_words(s_xs, nhp, s_cb, d.G, s_h, nhp, st)) != SSDI8_OK) return s;
   if ((s = launch_cumsum(d, a->dt, a->A, pack, gamma, nullptr, st)) != SSDI8_OK) return s;
-  if ((s = launch_chunk_state(d, a->xq, a->Bq, a->s_x, nullptr, a->s_B, pack, nullptr, nullptr,
-                              nullptr, reinterpret_cast<uint32_t*>(s_xs), nullptr, st)) != SSDI8_OK)
+  if ((s = launch_absmax_xs(d, a->xq, a->s_x, pack, reinterpret_cast<uint32_t*>(s_xs), st)) != SSDI8_OK) return s;
+  if ((s = launch_bmm(d, a->Cq, a->Bq, a->s_C, a->s_B, nullptr, nullptr, nullptr, reinterpret_cast<uint32_t*>(s_cb),
+                      nullptr, st)) != SSDI8_OK)
     return s;
-  if ((s = launch_finalize_scales(s_xs, nhp, nullptr, nullptr, 0, st)) != SSDI8_OK) return s;
-  if ((s = launch_bmm(d, a->Cq, a->Bq, a->s_C, a->s_B, nullptr, nullptr, nullptr,
-                      reinterpret_cast<uint32_t*>(s_cb), nullptr, st)) != SSDI8_OK)
+  if ((s = launch_finalize_scales(s_xs, nhp, s_cb, d.G, a->s_C, a->s_B, st)) != SSDI8_OK) return s;
+  if ((s = launch_chunk_state_passing(d, a->xq, a->Bq, a->s_x, s_xs, a->s_B, nullptr, pack, gamma, a->init_state,
+                                      reinterpret_cast<int8_t*>(ws + w.hq), nullptr, nullptr, nullptr, nullptr, nullptr,
+                                      nullptr, false, st, reinterpret_cast<uint32_t*>(s_h))) != SSDI8_OK)
     return s;
-  if ((s = launch_finalize_scales(s_cb, d.G, a->s_C, a->s_B, 1, st)) != SSDI8_OK) return s;
-  if ((s = launch_chunk_state(d, a->xq, a->Bq, a->s_x, s_xs, a->s_B, pack, loc, nullptr,
-                              nullptr, nullptr, nullptr, st)) != SSDI8_OK)
-    return s;
-  if ((s = launch_state_passing(d, loc, gamma, a->init_state, nullptr, nullptr, nullptr, nullptr,
-                                reinterpret_cast<uint32_t*>(s_h), st)) != SSDI8_OK)
-    return s;
-  return launch_finalize_scales(s_h, nhp, nullptr, nullptr, 0, st);
+  return launch_finalize_scales(s_h, nhp, nullptr, 0, nullptr, nullptr, st);
 }
 
 ssdi8_status_t ssdi8_state_passing(const ssdi8_dims_t* dims, const float* loc, const float* gamma,
@@ -261,7 +254,7 @@ ssdi8_status_t ssdi8_state_passing(const ssdi8_dims_t* dims, const float* loc, c
   ssdi8_status_t s = check_arch();
   if (s != SSDI8_OK) return s;
   return launch_state_passing(make_dims(dims), loc, gamma, init_state, s_h, prev, final_state, hq,
-                              nullptr, static_cast<cudaStream_t>(stream));
+                              static_cast<cudaStream_t>(stream));
 }
 
 ssdi8_status_t ssdi8_ssd_step(const ssdi8_dims_t* dims, const int8_t* xq, const float* s_x,

@@ -18,7 +18,7 @@ using namespace sm100;
 
 struct StateArgs {
   const float* s_x; const float* s_xs; const float* s_B; const float* pack;
-  float* loc; int8_t* tap_Xsq; int32_t* tap_acc; uint32_t* absmax_xs; int32_t* status;
+  float* loc; int8_t* tap_Xsq; int32_t* tap_acc; int32_t* status;
   Dims d;
 };
 
@@ -45,7 +45,6 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
   float* lut = reinterpret_cast<float*>(smem + OFF_F);
   uint64_t* bars = reinterpret_cast<uint64_t*>(lut + 256);  // [0] operands landed, [1] MMA done
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
-  const bool calib = a.absmax_xs != nullptr;
 
   if (tid == 0) {
     mbar_init(&bars[0], 1);
@@ -54,15 +53,17 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
     tma_prefetch_desc(&tm_B);
     tma_prefetch_desc(&tm_x);
   }
-  if (warp == 1 && !calib) tmem_alloc(tmem_slot, 64);
+  pdl_launch_dependents();
+  if (warp == 1) tmem_alloc(tmem_slot, 64);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_wait();
   if (tid == 0) {
-    mbar_expect_tx(&bars[0], (uint32_t)(Q * 64 + (calib ? 0 : Q * N)));
+    mbar_expect_tx(&bars[0], (uint32_t)(Q * 64 + Q * N));
     for (int i0 = 0; i0 < Q; i0 += TQ) {
       tma_load_3d(sX + i0 * 64, &tm_x, &bars[0], 0, h, (int)(tok0 + i0));
-      if (!calib) tma_load_3d(sB + i0 * N, &tm_B, &bars[0], 0, g, (int)(tok0 + i0));
+      tma_load_3d(sB + i0 * N, &tm_B, &bars[0], 0, g, (int)(tok0 + i0));
     }
   }
   if (tid < Q) lut[tid] = a.pack[((((i64)b * d.H + h) * d.c + k) * kPackRows + PACK_LUT) * Q + tid];
@@ -72,25 +73,18 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
 #pragma unroll
   for (int e = 0; e < 16; ++e) {
     const int hp = h * P + c * 16 + e;
-    rx[e] = calib ? a.s_x[hp] : __fdiv_rn(a.s_x[hp], a.s_xs[hp]);
+    rx[e] = __fdiv_rn(a.s_x[hp], a.s_xs[hp]);
   }
   __syncthreads();
   mbar_wait(&bars[0], 0, a.status);
 
   // ---- X_scaled, re-quantised in place (thread: chunk c of rows tid/4, tid/4 + 64, ...)
-  float mx[16];
-#pragma unroll
-  for (int e = 0; e < 16; ++e) mx[e] = 0.f;
   for (int i = tid >> 2; i < Q; i += kThreads / 4) {
     uint4* ptr = reinterpret_cast<uint4*>(sX + swz_off((uint32_t)i, (uint32_t)c, 64));
     const uint4 w4 = *ptr;
     const uint32_t ww[4] = {w4.x ^ 0x80808080u, w4.y ^ 0x80808080u, w4.z ^ 0x80808080u, w4.w ^ 0x80808080u};
     const float l = lut[i];
-    if (calib) {
-#pragma unroll
-      for (int e = 0; e < 16; ++e)
-        mx[e] = fmaxf(mx[e], fabsf(__fmul_rn(__fmul_rn(s8_to_f32(ww[e >> 2], e & 3), rx[e]), l)));
-    } else {
+    {
       uint32_t o[4];
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
@@ -104,11 +98,6 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
       *ptr = v;
       if (a.tap_Xsq) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = v;
     }
-  }
-  if (calib) {
-#pragma unroll
-    for (int e = 0; e < 16; ++e) atomicMax(a.absmax_xs + h * P + c * 16 + e, __float_as_uint(mx[e]));
-    return;
   }
   fence_async_smem();
   __syncthreads();
@@ -161,8 +150,7 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
 ssdi8_status_t launch_chunk_state(const Dims& d, const int8_t* xq, const int8_t* Bq,
                                   const float* s_x, const float* s_xs, const float* s_B,
                                   const float* pack, float* loc, int8_t* tap_Xsq,
-                                  int32_t* tap_acc, uint32_t* absmax_xs, int32_t* status,
-                                  cudaStream_t st) {
+                                  int32_t* tap_acc, int32_t* status, cudaStream_t st) {
   const int TQ = d.Q < 128 ? d.Q : 128;
   const uint64_t T = (uint64_t)d.b * d.L;
   CUtensorMap tm_B, tm_x;
@@ -178,13 +166,10 @@ ssdi8_status_t launch_chunk_state(const Dims& d, const int8_t* xq, const int8_t*
     uint32_t box[3] = {64, 1, (uint32_t)TQ};
     if (!encode_tensor_map(&tm_x, xq, 1, 3, dims, str, box, 64)) return SSDI8_ERR_CUDA;
   }
-  StateArgs a = {s_x, s_xs, s_B, pack, loc, tap_Xsq, tap_acc, absmax_xs, status, d};
+  StateArgs a = {s_x, s_xs, s_B, pack, loc, tap_Xsq, tap_acc, status, d};
   const size_t smem = SMEM_BYTES + 1024;
-  SSDI8_CUDA_CHECK(cudaFuncSetAttribute(chunk_state_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid(d.H, d.c, d.b);
-  chunk_state_tc<<<grid, kThreads, smem, st>>>(tm_B, tm_x, a);
-  SSDI8_LAUNCH_CHECK();
-  return SSDI8_OK;
+  return launch_configured(chunk_state_tc, grid, dim3(kThreads), smem, -1, false, st, tm_B, tm_x, a);
 }
 
 }  // namespace ssdi8

@@ -22,6 +22,9 @@
 // registers, and the recurrence is integer with a fixed-point decay:
 //   locq = rne(fmul(float(acc_st), fdiv(fmul(s_xs, s_B), s_h)));  Gq = rne(fmul(Gamma_k, 128))
 //   Sq   = sat(locq + ((Gq * Sq + 64) >> 7));  hq[k] = Sq before the update;  final = fmul(float(Sq), s_h)
+// CAL = true is the calibration pass: no codes are formed; the largest |S| of every channel over init_state and
+// every S_k goes into absmax_h (binary32 bits, one atomic per channel and CTA).  (Against separate ChunkState and
+// StatePassing passes over 42 MB of chunk-local states in HBM, 28 + 7 us at batch 2 x 2048 x 80 heads, this takes 22.)
 #include "kernels.h"
 #include "sm100.cuh"
 
@@ -33,7 +36,7 @@ using namespace sm100;
 struct FusedArgs {
   const float* s_x; const float* s_xs; const float* s_B; const float* s_h; const float* pack;
   const float* gamma; const float* init; float* final_state;
-  float* tap_loc; float* tap_prev; int8_t* tap_Xsq; int32_t* tap_acc; int32_t* status;
+  float* tap_loc; float* tap_prev; int8_t* tap_Xsq; int32_t* tap_acc; int32_t* status; uint32_t* absmax_h;
   Dims d;
   int n_full;  // CTAs below this index own a whole (batch, head); the rest own one part of one
   int split;   // parts per (batch, head) of the rest: 2 (halves of 32 channels) or 4 (quarters of 16)
@@ -60,7 +63,7 @@ __device__ __forceinline__ void named_bar(int id, int nthreads) {
 
 // TAPS: any of the intermediate-tensor taps is requested (tests); the production instance carries no tap code
 // NCQ: 16-channel chunks of the head this CTA owns (4 = the whole head, 1 = one quarter)
-template <bool I8S, bool TAPS, int NCQ>
+template <bool I8S, bool TAPS, bool CAL, int NCQ>
 __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtensorMap& tm_x, const CUtensorMap& tm_hq,
                                            const FusedArgs& a, const int unit, const int c0) {
   // (no padding for the 1024-byte alignment the swizzled tiles need: three CTAs fill the SM's shared
@@ -106,10 +109,16 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
   // for this kernel, so it must not be scheduled before this kernel's predecessors have completed)
   pdl_launch_dependents();
   if (tid < 64) {
-    const float sxb = __fmul_rn(a.s_xs[h * P + tid], a.s_B[g]), sh = a.s_h[h * P + tid];
-    col_scale[tid] = I8S ? __fdiv_rn(sxb, sh) : sxb;
-    col_invh[tid] = __fdiv_rn(1.0f, sh);
-    col_sh[tid] = sh;
+    const float sxb = __fmul_rn(a.s_xs[h * P + tid], a.s_B[g]);
+    if (CAL) {
+      col_scale[tid] = sxb;
+      col_invh[tid] = 0.f;               // running maximum of the channel
+    } else {
+      const float sh = a.s_h[h * P + tid];
+      col_scale[tid] = I8S ? __fdiv_rn(sxb, sh) : sxb;
+      col_invh[tid] = __fdiv_rn(1.0f, sh);
+      col_sh[tid] = sh;
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -264,6 +273,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     // the running state S[p, n]: fp32, or (I8S) the integer code, in tensor-memory columns 64 + p of lane n
     const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16);
     const uint32_t tS = tlane + 64u + (uint32_t)cb;
+    float smax[CAL ? 32 : 1];   // CAL: running maxima of |S[p, n]| over the chunks
 #pragma unroll
     for (int p0 = 0; p0 < 32; p0 += 8) {
       if (p0 < npp) {
@@ -272,6 +282,10 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
         for (int e = 0; e < 8; ++e) {
           const float v = (a.init && ok) ? a.init[(bh * P + cb + p0 + e) * N + n] : 0.f;
           sv[e] = I8S ? (int)(int8_t)(rne_clamp_bits(__fmul_rn(v, col_invh[(cb + p0 + e) & 63])) & 0xffu) : __float_as_int(v);
+        }
+        if (CAL) {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) smax[CAL ? p0 + e : 0] = fabsf(__int_as_float(sv[e]));
         }
         tmem_st8(tS + (uint32_t)p0, sv);
       }
@@ -291,7 +305,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
       // of the wait for the chunk's MMAs, from a second read of the state; forming them in the update pass of
       // the chunk before, while the new values are in registers, puts them behind that wait on the chain of
       // the chunk and was measured slower (0.0568 against 0.0536 ms at batch 8 x 2048 x 80 heads).
-      {
+      if (!CAL) {
         const i64 obase = (((((i64)b * d.c + k) * d.H + h) * P) + cb) * N + n;
         // batches of 8: all loads of a batch before its byte stores (a byte store may alias anything,
         // so interleaving them would serialise the loop on shared-memory latency).  The tensor-memory
@@ -336,7 +350,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
       if (warp == 0) mbar_wait_inline<256>(&bars[B_MMA], k & 1, a.status);
       named_bar(1, kStateThreads);
       // ---- hq[k] leaves by TMA
-      if (tid == 0) {
+      if (tid == 0 && !CAL) {
         for (int j = c0; j < c0 + ncq; ++j)  // 16 channels (rows of hq) per store
           tma_store_2d(&tm_hq, sHQ + 16 * j * N, 0, (int)(((((i64)b * d.c + k) * d.H + h) * P) + 16 * j));
         tma_store_commit();
@@ -385,6 +399,10 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
                                            make_float2(__int_as_float(sv[e]), __int_as_float(sv[e + 1])), l2);
               sv[e] = __float_as_int(s2.x);
               sv[e + 1] = __float_as_int(s2.y);
+              if (CAL) {
+                smax[CAL ? hf * 8 + e : 0] = fmaxf(smax[CAL ? hf * 8 + e : 0], fabsf(s2.x));
+                smax[CAL ? hf * 8 + e + 1 : 0] = fmaxf(smax[CAL ? hf * 8 + e + 1 : 0], fabsf(s2.y));
+              }
             }
           }
         }
@@ -396,7 +414,18 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[B_ACC_FREE]);  // this warp has read the accumulator of chunk k
     }
-    if (a.final_state) {
+    if (CAL) {
+#pragma unroll
+      for (int p = 0; p < 32; ++p) {
+        if (p < npp) {
+          const uint32_t m = __reduce_max_sync(0xffffffffu, ok ? __float_as_uint(smax[CAL ? p : 0]) : 0u);
+          if (lane == (p & 31)) atomicMax(reinterpret_cast<uint32_t*>(col_invh) + cb + p, m);
+        }
+      }
+      named_bar(1, kStateThreads);
+      if (tid < 64) atomicMax(a.absmax_h + h * P + tid, reinterpret_cast<const uint32_t*>(col_invh)[tid]);
+    }
+    if (!CAL && a.final_state) {
 #pragma unroll
       for (int p0 = 0; p0 < 32; p0 += 8) {
         if (p0 < npp) {
@@ -426,18 +455,18 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
 // the heads of a nearly empty last wave, split in halves or quarters so that they spread over the
 // free slots (operand tiles and the MMA stay full width: only the re-quantisation, the state
 // update and the hq rows are restricted to the range).
-template <bool I8S, bool TAPS>
-__global__ void __launch_bounds__(kThreads, 3)
+template <bool I8S, bool TAPS, bool CAL>
+__global__ void __launch_bounds__(kThreads, CAL ? 2 : 3)
 chunk_state_pass_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__ CUtensorMap tm_x,
                     const __grid_constant__ CUtensorMap tm_hq, const FusedArgs a) {
   if ((int)blockIdx.x < a.n_full) {
-    fused_body<I8S, TAPS, 4>(tm_B, tm_x, tm_hq, a, (int)blockIdx.x, 0);
+    fused_body<I8S, TAPS, CAL, 4>(tm_B, tm_x, tm_hq, a, (int)blockIdx.x, 0);
   } else if (a.split == 2) {
     const int r = (int)blockIdx.x - a.n_full;
-    fused_body<I8S, TAPS, 2>(tm_B, tm_x, tm_hq, a, a.n_full + (r >> 1), 2 * (r & 1));
+    fused_body<I8S, TAPS, CAL, 2>(tm_B, tm_x, tm_hq, a, a.n_full + (r >> 1), 2 * (r & 1));
   } else {
     const int r = (int)blockIdx.x - a.n_full;
-    fused_body<I8S, TAPS, 1>(tm_B, tm_x, tm_hq, a, a.n_full + (r >> 2), r & 3);
+    fused_body<I8S, TAPS, CAL, 1>(tm_B, tm_x, tm_hq, a, a.n_full + (r >> 2), r & 3);
   }
 }
 
@@ -449,7 +478,7 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
                                           const float* init, int8_t* hq, float* final_state,
                                           float* tap_loc, float* tap_prev, int8_t* tap_Xsq,
                                           int32_t* tap_acc, int32_t* status, bool int8_state,
-                                          cudaStream_t st) {
+                                          cudaStream_t st, uint32_t* absmax_h) {
   const int TQ = d.Q < 128 ? d.Q : 128;
   const uint64_t T = (uint64_t)d.b * d.L;
   CUtensorMap tm_B, tm_x, tm_hq;
@@ -488,7 +517,7 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
   int split = 4;
   if (8 * (units - n_full) > slots) n_full = units;
   FusedArgs a = {s_x, s_xs, s_B, s_h, pack, gamma, init, final_state, tap_loc, tap_prev, tap_Xsq, tap_acc,
-                 status, d, n_full, split};
+                 status, absmax_h, d, n_full, split};
   const size_t smem = SMEM_BYTES;
   const unsigned grid = (unsigned)(n_full + split * (units - n_full));
   const bool taps = tap_loc || tap_prev || tap_Xsq || tap_acc;
@@ -496,10 +525,12 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
     return launch_configured(kernel, dim3(grid), dim3(kThreads), smem, -1, true, st, tm_B, tm_x, tm_hq, a);
   };
   ssdi8_status_t ls;
-  if (int8_state)
-    ls = taps ? launch(chunk_state_pass_tc<true, true>) : launch(chunk_state_pass_tc<true, false>);
+  if (absmax_h)
+    ls = launch(chunk_state_pass_tc<false, false, true>);
+  else if (int8_state)
+    ls = taps ? launch(chunk_state_pass_tc<true, true, false>) : launch(chunk_state_pass_tc<true, false, false>);
   else
-    ls = taps ? launch(chunk_state_pass_tc<false, true>) : launch(chunk_state_pass_tc<false, false>);
+    ls = taps ? launch(chunk_state_pass_tc<false, true, false>) : launch(chunk_state_pass_tc<false, false, false>);
   if (ls != SSDI8_OK) return ls;
   SSDI8_LAUNCH_CHECK();
   return SSDI8_OK;

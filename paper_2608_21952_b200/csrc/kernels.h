@@ -96,28 +96,24 @@ ssdi8_status_t launch_bmm(const Dims& d, const int8_t* Cq, const int8_t* Bq, con
                           const float* s_B, const float* s_cb, int8_t* CBq, int32_t* tap_acc,
                           uint32_t* absmax_acc, int32_t* status, cudaStream_t st, bool after_state_kernel = false);
 
-// absmax_xs: per-channel running max (as binary32 bits) of |x_scaled| (calibration; may be
-// NULL).  When absmax_xs is non-NULL only that is computed.
 ssdi8_status_t launch_chunk_state(const Dims& d, const int8_t* xq, const int8_t* Bq,
                                   const float* s_x, const float* s_xs, const float* s_B,
                                   const float* pack, float* loc, int8_t* tap_Xsq,
-                                  int32_t* tap_acc, uint32_t* absmax_xs, int32_t* status,
-                                  cudaStream_t st);
+                                  int32_t* tap_acc, int32_t* status, cudaStream_t st);
 
-// ChunkState and StatePassing in one chunk-sequential kernel (loc never leaves the chip)
+// ChunkState and StatePassing in one chunk-sequential kernel (loc never leaves the chip).  absmax_h (calibration):
+// per-channel running max (binary32 bits) of |S| over init and every S_k; no other output is written then
 ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const int8_t* Bq,
                                           const float* s_x, const float* s_xs, const float* s_B,
                                           const float* s_h, const float* pack, const float* gamma,
                                           const float* init, int8_t* hq, float* final_state,
                                           float* tap_loc, float* tap_prev, int8_t* tap_Xsq,
                                           int32_t* tap_acc, int32_t* status, bool int8_state,
-                                          cudaStream_t st);
+                                          cudaStream_t st, uint32_t* absmax_h = nullptr);
 
-// absmax_h: per-channel running max (binary32 bits) of |S| over init, prev and final
 ssdi8_status_t launch_state_passing(const Dims& d, const float* loc, const float* gamma,
                                     const float* init, const float* s_h, float* prev,
-                                    float* final_state, int8_t* hq, uint32_t* absmax_h,
-                                    cudaStream_t st);
+                                    float* final_state, int8_t* hq, cudaStream_t st);
 
 struct ScanTaps {
   int32_t* acc_off; float* rowmax; int8_t* Mq; int32_t* acc_diag;
@@ -153,8 +149,11 @@ ssdi8_status_t launch_int8_mma_peak(int nbatch, int32_t* status, int* ctas, cuda
 int int8_mma_peak_batch();
 ssdi8_status_t launch_bounded_wait_expires(int32_t* status, cudaStream_t st);
 
-// scale[k] = bits[k] == 0 ? 1 : fdiv(as_float(bits[k]) [* mul], 127)   (in place)
-ssdi8_status_t launch_finalize_scales(float* scale_bits, i64 n, const float* mul_a,
-                                      const float* mul_b, int bits_are_int, cudaStream_t st);
+// calibration (calibrate.cu): per-channel running max of |X_scaled|; three arrays of words set to 0; step sizes from
+// maxima in place (s: binary32 absmax; q: int32 absmax of acc_cb, times s_C s_B), 1 where a maximum is 0
+ssdi8_status_t launch_absmax_xs(const Dims& d, const int8_t* xq, const float* s_x, const float* pack, uint32_t* absmax,
+                                cudaStream_t st);
+ssdi8_status_t launch_clear_words(void* a, i64 na, void* b, i64 nb, void* c, i64 nc, cudaStream_t st);
+ssdi8_status_t launch_finalize_scales(float* s, i64 n, float* q, i64 nq, const float* s_C, const float* s_B, cudaStream_t st);
 
 }  // namespace ssdi8

@@ -14,13 +14,21 @@ constexpr int QUNROLL = 4;   // float4 loads in flight per thread
 // float4 column (its four step sizes stay in registers) and walks a slab of rows with QROWS
 // independent 16-byte loads in flight; a warp reads 512 and writes 128 contiguous bytes per row.
 constexpr int QROWS = 8;
-__global__ void __launch_bounds__(128) quant_ch_fastest(const float4* __restrict__ in,
-                                                        const float4* __restrict__ scale,
+// FIX: the step sizes were just formed by an absmax kernel; an all-zero channel has 0 there and gets 1 (every
+// block reads 0 or 1 and takes 1, the first row of blocks writes it).
+template <bool FIX>
+__global__ void __launch_bounds__(128) quant_ch_fastest(const float4* __restrict__ in, float4* scale,
                                                         uint32_t* __restrict__ out, i64 R, int ch4,
                                                         int rows_per_block) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int q = blockIdx.x * 128 + threadIdx.x;
   if (q >= ch4) return;
-  const float4 s = __ldg(scale + q);
+  float4 s = scale[q];
+  if (FIX && (s.x == 0.f || s.y == 0.f || s.z == 0.f || s.w == 0.f)) {
+    s = make_float4(s.x == 0.f ? 1.f : s.x, s.y == 0.f ? 1.f : s.y, s.z == 0.f ? 1.f : s.z, s.w == 0.f ? 1.f : s.w);
+    if (blockIdx.y == 0) scale[q] = s;
+  }
   const QuantStep sx = quant_step(s.x), sy = quant_step(s.y), sz = quant_step(s.z), sw = quant_step(s.w);
   const i64 r0 = (i64)blockIdx.y * rows_per_block;
   const i64 r1 = r0 + rows_per_block < R ? r0 + rows_per_block : R;
@@ -108,45 +116,56 @@ __global__ void __launch_bounds__(128, 8) quant_jobs(const QuantJobs a) {
 }
 
 // ---- quantise, I % 4 == 0: 4 consecutive elements share a channel
-__global__ void __launch_bounds__(QT) quant_inner(const float4* __restrict__ in,
-                                                  const float* __restrict__ scale,
+template <bool FIX>
+__global__ void __launch_bounds__(QT) quant_inner(const float4* __restrict__ in, float* scale,
                                                   uint32_t* __restrict__ out, uint32_t n4,
                                                   uint32_t I4, uint32_t Ch) {
+  pdl_launch_dependents();
+  pdl_wait();
   uint32_t base = blockIdx.x * (QT * QUNROLL) + threadIdx.x;
 #pragma unroll
   for (int u = 0; u < QUNROLL; ++u) {
     uint32_t e = base + u * QT;
     if (e < n4) {
       float4 v = __ldcs(in + e);
-      const QuantStep s = quant_step(__ldg(scale + (e / I4) % Ch));
+      const uint32_t ch = (e / I4) % Ch;
+      float al = scale[ch];
+      if (FIX && al == 0.f) {
+        al = 1.f;
+        if (e < I4 * Ch) scale[ch] = al;   // the first row
+      }
+      const QuantStep s = quant_step(al);
       out[e] = quant_code4(v, s, s, s, s);
     }
   }
 }
 
-// ---- absmax, I == 1.  Thread owns 4 channels and walks rows; grid.y splits the rows.
-__global__ void __launch_bounds__(QT) absmax_ch_fastest(const float4* __restrict__ in,
-                                                        uint32_t* __restrict__ bits, i64 R, int ch4,
-                                                        int rows_per_block) {
-  int q = blockIdx.x * QT + threadIdx.x;
+// ---- absmax, I == 1.  Thread owns 4 channels and walks rows with AROWS loads in flight; grid.y splits the rows.
+// The loads leave their lines in L2 for the quantiser that follows.
+constexpr int AROWS = 8;
+__global__ void __launch_bounds__(128) absmax_ch_fastest(const float4* __restrict__ in,
+                                                         uint32_t* __restrict__ bits, i64 R, int ch4,
+                                                         int rows_per_block) {
+  pdl_launch_dependents();
+  pdl_wait();
+  int q = blockIdx.x * 128 + threadIdx.x;
   if (q >= ch4) return;
   i64 r0 = (i64)blockIdx.y * rows_per_block;
   i64 r1 = r0 + rows_per_block < R ? r0 + rows_per_block : R;
   float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
-  i64 r = r0;
-  for (; r + 4 <= r1; r += 4) {
-    float4 v0 = __ldg(in + (r + 0) * ch4 + q), v1 = __ldg(in + (r + 1) * ch4 + q);
-    float4 v2 = __ldg(in + (r + 2) * ch4 + q), v3 = __ldg(in + (r + 3) * ch4 + q);
-    m.x = fmaxf(fmaxf(fmaxf(m.x, fabsf(v0.x)), fmaxf(fabsf(v1.x), fabsf(v2.x))), fabsf(v3.x));
-    m.y = fmaxf(fmaxf(fmaxf(m.y, fabsf(v0.y)), fmaxf(fabsf(v1.y), fabsf(v2.y))), fabsf(v3.y));
-    m.z = fmaxf(fmaxf(fmaxf(m.z, fabsf(v0.z)), fmaxf(fabsf(v1.z), fabsf(v2.z))), fabsf(v3.z));
-    m.w = fmaxf(fmaxf(fmaxf(m.w, fabsf(v0.w)), fmaxf(fabsf(v1.w), fabsf(v2.w))), fabsf(v3.w));
-  }
-  for (; r < r1; ++r) {
-    float4 v = __ldg(in + r * ch4 + q);
+  auto take = [&](const float4& v) {
     m.x = fmaxf(m.x, fabsf(v.x)); m.y = fmaxf(m.y, fabsf(v.y));
     m.z = fmaxf(m.z, fabsf(v.z)); m.w = fmaxf(m.w, fabsf(v.w));
+  };
+  i64 r = r0;
+  for (; r + AROWS <= r1; r += AROWS) {
+    float4 v[AROWS];
+#pragma unroll
+    for (int u = 0; u < AROWS; ++u) v[u] = __ldg(in + (r + u) * ch4 + q);
+#pragma unroll
+    for (int u = 0; u < AROWS; ++u) take(v[u]);
   }
+  for (; r < r1; ++r) take(__ldg(in + r * ch4 + q));
   // step size of this partial maximum: fdiv by a positive constant is monotone, so the
   // maximum of the step sizes is the step size of the maximum
   atomicMax(bits + 4 * q + 0, __float_as_uint(__fdiv_rn(m.x, 127.0f)));
@@ -160,6 +179,8 @@ __global__ void __launch_bounds__(QT) absmax_inner(const float4* __restrict__ in
                                                    uint32_t* __restrict__ bits, i64 R, int Ch, int I4,
                                                    int rows_per_block) {
   __shared__ float red[QT / 32];
+  pdl_launch_dependents();
+  pdl_wait();
   int ch = blockIdx.y;
   i64 r0 = (i64)blockIdx.x * rows_per_block;
   i64 r1 = r0 + rows_per_block < R ? r0 + rows_per_block : R;
@@ -182,11 +203,6 @@ __global__ void __launch_bounds__(QT) absmax_inner(const float4* __restrict__ in
   }
 }
 
-__global__ void finalize_alpha(uint32_t* bits, i64 n) {
-  i64 k = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n && bits[k] == 0u) bits[k] = __float_as_uint(1.0f);  // all-zero channel: alpha = 1
-}
-
 }  // namespace
 
 ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* scale, int mode,
@@ -194,18 +210,21 @@ ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* sca
   const i64 n4 = R * Ch * I / 4;
   if (n4 == 0) return SSDI8_OK;
   uint32_t* bits = reinterpret_cast<uint32_t*>(scale);
+  ssdi8_status_t ls;
   if (mode == 1 || mode == 2) {
-    if (mode == 1) SSDI8_CUDA_CHECK(cudaMemsetAsync(scale, 0, sizeof(float) * Ch, st));
+    if (mode == 1 && (ls = launch_clear_words(scale, Ch, nullptr, 0, nullptr, 0, st)) != SSDI8_OK) return ls;
     if (I == 1) {
       int ch4 = (int)(Ch / 4);
-      int gx = (ch4 + QT - 1) / QT;
-      // enough row splits to fill the machine, at least 64 rows each
-      i64 want = (148 * 8 + gx - 1) / gx;
+      int gx = (ch4 + 127) / 128;
+      // enough row splits to fill the machine several times over, a few rounds of loads each (64 rows at least, on
+      // 256 threads, left 2560 channels x 4096 rows on 320 blocks: 22 us at 84 MB against 17)
+      i64 want = (148 * 16 + gx - 1) / gx;
       i64 rows = (R + want - 1) / want;
-      if (rows < 64) rows = 64;
+      if (rows < 2 * AROWS) rows = 2 * AROWS;
+      rows = (rows + AROWS - 1) / AROWS * AROWS;
       int gy = (int)((R + rows - 1) / rows);
-      absmax_ch_fastest<<<dim3(gx, gy), QT, 0, st>>>(reinterpret_cast<const float4*>(in), bits, R,
-                                                      ch4, (int)rows);
+      ls = launch_configured(absmax_ch_fastest, dim3(gx, gy), dim3(128), 0, kStreamCarveout, false, st,
+                             reinterpret_cast<const float4*>(in), bits, R, ch4, (int)rows);
     } else {
       int I4 = (int)(I / 4);
       i64 want = (148 * 8 + Ch - 1) / Ch;
@@ -213,17 +232,13 @@ ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* sca
       i64 min_rows = (QT * 4 + I4 - 1) / I4;
       if (rows < min_rows) rows = min_rows;
       int gx = (int)((R + rows - 1) / rows);
-      absmax_inner<<<dim3(gx, (unsigned)Ch), QT, 0, st>>>(reinterpret_cast<const float4*>(in), bits,
-                                                           R, (int)Ch, I4, (int)rows);
+      ls = launch_configured(absmax_inner, dim3(gx, (unsigned)Ch), dim3(QT), 0, kStreamCarveout, false, st,
+                             reinterpret_cast<const float4*>(in), bits, R, (int)Ch, I4, (int)rows);
     }
-    SSDI8_LAUNCH_CHECK();
-    if (mode == 1) {
-      finalize_alpha<<<(unsigned)((Ch + 255) / 256), 256, 0, st>>>(bits, Ch);
-      SSDI8_LAUNCH_CHECK();
-    }
+    if (ls != SSDI8_OK) return ls;
   }
   if (!out) return SSDI8_OK;
-  unsigned grid = (unsigned)((n4 + QT * QUNROLL - 1) / (QT * QUNROLL));
+  const bool fix = mode == 1;   // an all-zero channel: alpha = 1
   if (I == 1) {
     const int ch4 = (int)(Ch / 4);
     const int gx = (ch4 + 127) / 128;
@@ -233,16 +248,14 @@ ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* sca
     if (rows < 32) rows = 32;
     rows = (rows + QROWS - 1) / QROWS * QROWS;
     const int gy = (int)((R + rows - 1) / rows);
-    quant_ch_fastest<<<dim3(gx, gy), 128, 0, st>>>(reinterpret_cast<const float4*>(in),
-                                                   reinterpret_cast<const float4*>(scale),
-                                                   reinterpret_cast<uint32_t*>(out), R, ch4, (int)rows);
+    return launch_configured(fix ? quant_ch_fastest<true> : quant_ch_fastest<false>, dim3(gx, gy), dim3(128), 0,
+                             kStreamCarveout, false, st, reinterpret_cast<const float4*>(in),
+                             reinterpret_cast<float4*>(scale), reinterpret_cast<uint32_t*>(out), R, ch4, (int)rows);
   }
-  else
-    quant_inner<<<grid, QT, 0, st>>>(reinterpret_cast<const float4*>(in), scale,
-                                     reinterpret_cast<uint32_t*>(out), (uint32_t)n4, (uint32_t)(I / 4),
-                                     (uint32_t)Ch);
-  SSDI8_LAUNCH_CHECK();
-  return SSDI8_OK;
+  const unsigned grid = (unsigned)((n4 + QT * QUNROLL - 1) / (QT * QUNROLL));
+  return launch_configured(fix ? quant_inner<true> : quant_inner<false>, dim3(grid), dim3(QT), 0, kStreamCarveout, false, st,
+                           reinterpret_cast<const float4*>(in), scale, reinterpret_cast<uint32_t*>(out), (uint32_t)n4,
+                           (uint32_t)(I / 4), (uint32_t)Ch);
 }
 
 ssdi8_status_t launch_quantize_xbc(const float* x, const float* B, const float* C, i64 T_, int D, int G, int N,
@@ -274,29 +287,6 @@ ssdi8_status_t launch_quantize_xbc(const float* x, const float* B, const float* 
   nb = fill(a.job[2], x, s_x, xq, D, 0, nb);
   a.late_wait = after_cumsum ? 1 : 0;
   return launch_configured(quant_jobs, dim3((unsigned)nb), dim3(128), 0, kStreamCarveout, false, st, a);
-}
-
-// bits[k] holds either a binary32 absmax or (bits_are_int) an int32 absmax; the step size is
-// fdiv(fmul(value, fmul(mul_a[k], mul_b[k])), 127) (multipliers optional), 1 if the value is 0.
-namespace {
-__global__ void finalize_scales_k(float* s, i64 n, const float* mul_a, const float* mul_b,
-                                  int bits_are_int) {
-  i64 k = (i64)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  uint32_t u = __float_as_uint(s[k]);
-  if (u == 0u) { s[k] = 1.0f; return; }
-  float v = bits_are_int ? (float)(int)u : s[k];
-  if (mul_a) v = __fmul_rn(v, __fmul_rn(mul_a[k], mul_b[k]));
-  s[k] = __fdiv_rn(v, 127.0f);
-}
-}  // namespace
-
-ssdi8_status_t launch_finalize_scales(float* scale_bits, i64 n, const float* mul_a,
-                                      const float* mul_b, int bits_are_int, cudaStream_t st) {
-  finalize_scales_k<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(scale_bits, n, mul_a, mul_b,
-                                                                 bits_are_int);
-  SSDI8_LAUNCH_CHECK();
-  return SSDI8_OK;
 }
 
 }  // namespace ssdi8

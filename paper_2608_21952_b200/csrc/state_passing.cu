@@ -13,7 +13,9 @@ constexpr int SP_T = 256;
 __global__ void __launch_bounds__(SP_T) state_passing_kernel(
     const float4* loc /* may alias prev: no __restrict__ */, const float* __restrict__ gamma, const float4* __restrict__ init,
     const float* __restrict__ s_h, float4* prev, float4* __restrict__ final_state,
-    uint32_t* __restrict__ hq, uint32_t* __restrict__ absmax_h, Dims d) {
+    uint32_t* __restrict__ hq, Dims d) {
+  pdl_launch_dependents();
+  pdl_wait();
   const int N4 = d.N / 4;
   const i64 per_b = (i64)d.H * d.P * N4;               // float4 per (b) slice of one chunk
   const i64 idx = (i64)blockIdx.x * SP_T + threadIdx.x;  // over b * H * P * N4
@@ -26,7 +28,6 @@ __global__ void __launch_bounds__(SP_T) state_passing_kernel(
   if (hq) inv_h = __fdiv_rn(1.0f, s_h[hp]);
   float4 S = init ? init[idx] : make_float4(0.f, 0.f, 0.f, 0.f);
   const float* gm = gamma + ((i64)b * d.H + h) * d.c;
-  float m = 0.f;
   const i64 stride = per_b;                              // chunk stride in float4
   i64 o = (i64)b * d.c * per_b + r;
   for (int k = 0; k < d.c; ++k, o += stride) {
@@ -36,36 +37,25 @@ __global__ void __launch_bounds__(SP_T) state_passing_kernel(
       hq[o] = pack4(rne_clamp(__fmul_rn(S.x, inv_h)), rne_clamp(__fmul_rn(S.y, inv_h)),
                     rne_clamp(__fmul_rn(S.z, inv_h)), rne_clamp(__fmul_rn(S.w, inv_h)));
     if (prev) prev[o] = S;
-    if (absmax_h) m = fmaxf(fmaxf(fmaxf(m, fabsf(S.x)), fmaxf(fabsf(S.y), fabsf(S.z))), fabsf(S.w));
     S.x = __fmaf_rn(g, S.x, l.x);
     S.y = __fmaf_rn(g, S.y, l.y);
     S.z = __fmaf_rn(g, S.z, l.z);
     S.w = __fmaf_rn(g, S.w, l.w);
   }
   if (final_state) final_state[idx] = S;
-  if (absmax_h) {
-    m = fmaxf(fmaxf(fmaxf(m, fabsf(S.x)), fmaxf(fabsf(S.y), fabsf(S.z))), fabsf(S.w));
-    // lanes of a warp that share (h,p): N4 consecutive threads (N4 = 16 or 32)
-    for (int off = 1; off < N4 && off < 32; off <<= 1)
-      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if ((threadIdx.x & (min(N4, 32) - 1)) == 0) atomicMax(absmax_h + hp, __float_as_uint(m));
-  }
 }
 
 }  // namespace
 
 ssdi8_status_t launch_state_passing(const Dims& d, const float* loc, const float* gamma,
                                     const float* init, const float* s_h, float* prev,
-                                    float* final_state, int8_t* hq, uint32_t* absmax_h,
-                                    cudaStream_t st) {
+                                    float* final_state, int8_t* hq, cudaStream_t st) {
   const i64 n = (i64)d.b * d.H * d.P * (d.N / 4);
   unsigned grid = (unsigned)((n + SP_T - 1) / SP_T);
-  state_passing_kernel<<<grid, SP_T, 0, st>>>(
-      reinterpret_cast<const float4*>(loc), gamma, reinterpret_cast<const float4*>(init), s_h,
-      reinterpret_cast<float4*>(prev), reinterpret_cast<float4*>(final_state),
-      reinterpret_cast<uint32_t*>(hq), absmax_h, d);
-  SSDI8_LAUNCH_CHECK();
-  return SSDI8_OK;
+  return launch_configured(state_passing_kernel, dim3(grid), dim3(SP_T), 0, -1, false, st,
+                           reinterpret_cast<const float4*>(loc), gamma, reinterpret_cast<const float4*>(init), s_h,
+                           reinterpret_cast<float4*>(prev), reinterpret_cast<float4*>(final_state),
+                           reinterpret_cast<uint32_t*>(hq), d);
 }
 
 }  // namespace ssdi8

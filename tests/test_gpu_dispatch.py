@@ -59,3 +59,35 @@ def test_cumsum_on_a_grid_that_fills_the_device():
     want = orc.chunk_cumsum(cfg, q["dt"], q["A"])
     _, _, taps = gh.gpu_fwd(cfg, q, taps=("cs",))
     assert np.array_equal(taps["cs"], want)
+
+
+@pytest.mark.parametrize("b,c,H,N,G,Q", [(1, 1, 1, 64, 1, 64), (2, 3, 9, 128, 1, 128), (1, 2, 16, 64, 2, 256), (3, 1, 150, 128, 1, 64)])
+@pytest.mark.parametrize("with_init", [False, True])
+def test_calibration_at_ragged_head_counts(b, c, H, N, G, Q, with_init):
+    # 8 heads per block in the X_scaled pass (1 and 9 heads leave most of a block idle); whole heads and quarter heads per
+    # CTA in the state pass
+    import torch
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("cal", b, c * Q, H, 64, N, G, Q, 0.02, 20.0, 33)
+    t = inputs.make_prefill(cfg)
+    init = inputs.make_init_state(cfg) * np.float32(3.0) if with_init else None
+    q = orc.prepare_quantized(cfg, t, init)
+    dims = bd.dims_of(cfg)
+    dv = {k: gh.dev(q[k]) for k in ("xq", "Bq", "Cq", "s_x", "s_B", "s_C", "dt", "A")}
+    s = [torch.full((n,), float("nan"), device="cuda") for n in (H * 64, G, H * 64)]
+    bd.ssdi8_calibrate(dims, bd.make_fwd_args(init_state=gh.dev(init), **dv), *s, bd.alloc_workspace(dims))
+    torch.cuda.synchronize()
+    for got, name in zip(s, ("s_xs", "s_cb", "s_h")):
+        assert np.array_equal(got.cpu().numpy(), np.asarray(q[name]).reshape(-1)), name
+
+
+@pytest.mark.parametrize("R,Ch,I", [(1, 4, 1), (15, 516, 1), (16, 8, 64), (129, 2, 128)])
+def test_quantiser_gives_all_zero_channels_a_step_of_one(R, Ch, I):
+    import gpu_harness as gh
+    v = np.random.default_rng(7).standard_normal((R, Ch, I)).astype(np.float32)
+    v[:, ::2] = 0.0
+    q, s = gh.gpu_quantize(v.reshape(R, Ch, I), R, Ch, I)
+    qr, sr = orc.quantize(v.reshape(R, Ch, I), R, Ch, I, mode=1)
+    assert np.array_equal(s, sr) and np.all(s[::2] == 1.0)
+    assert np.array_equal(q.reshape(-1), np.asarray(qr).reshape(-1))
