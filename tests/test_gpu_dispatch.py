@@ -91,3 +91,41 @@ def test_quantiser_gives_all_zero_channels_a_step_of_one(R, Ch, I):
     qr, sr = orc.quantize(v.reshape(R, Ch, I), R, Ch, I, mode=1)
     assert np.array_equal(s, sr) and np.all(s[::2] == 1.0)
     assert np.array_equal(q.reshape(-1), np.asarray(qr).reshape(-1))
+
+
+@pytest.mark.parametrize("b,c,H,G", [(9, 1, 80, 1), (5, 2, 129, 1), (2, 7, 130, 2), (6, 3, 40, 8), (1, 9, 256, 1), (14, 1, 8, 1)],
+                         ids=lambda v: str(v))
+@pytest.mark.parametrize("flags", [0, 2 | 4], ids=["default", "int8_state_y_fp16"])
+def test_host_pipeline_cuts_equal_the_device_call(b, c, H, G, flags):
+    # several whole elements per slice with a ragged last one, one element per slice, elements in two, three and more
+    # slices (a short last one among them), B, C and dt in one piece per element and in several: bit for bit
+    import torch
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("host_cut", b, c * 128, H, 64, 64, G, 128, 0.02, 20.0, 34)
+    dims = bd.dims_of(cfg)
+    g = torch.Generator().manual_seed(3)
+    T, HP = cfg.tokens, cfg.channels
+    r = lambda *s: torch.randn(*s, generator=g)
+    host = {"x": r(T, HP), "B": r(T, G * 64), "C": r(T, G * 64), "dt": torch.nn.functional.softplus(r(T, H) - 3.0)}
+    host = {k: v.pin_memory() for k, v in host.items()}
+    dv = {k: v.cuda() for k, v in host.items()}
+    init = r(b, H, 64, 64).cuda()
+    par = {"A": -torch.exp(r(H)).cuda(), "D": r(H).cuda(), "s_x": torch.full((HP,), 0.03), "s_B": torch.full((G,), 0.03),
+           "s_C": torch.full((G,), 0.03), "s_xs": torch.full((HP,), 0.002), "s_cb": torch.full((G,), 0.4),
+           "s_h": torch.full((HP,), 0.02)}
+    par = {k: v.cuda() for k, v in par.items()}
+    ydt = torch.float16 if flags & 4 else torch.float32
+    y_d, fin_d = torch.empty(T, HP, dtype=ydt, device="cuda"), torch.empty_like(init)
+    lws = torch.empty(bd.ssdi8_layer_fwd_workspace_bytes(dims, flags), dtype=torch.uint8, device="cuda")
+    bd.ssdi8_layer_fwd(dims, bd.make_layer_args(y=y_d, final_state=fin_d, init_state=init, **dv, **par), lws, flags=flags)
+    scratch = torch.empty(bd.ssdi8_layer_fwd_host_scratch_bytes(dims, flags), dtype=torch.uint8, device="cuda")
+    for with_state in (True, False, True):
+        y_h = torch.full((T, HP), float("nan"), dtype=ydt).pin_memory()
+        fin_h = torch.full(init.shape, float("nan")).pin_memory()
+        st = torch.full((1,), -99, dtype=torch.int32).pin_memory()
+        bd.ssdi8_layer_fwd_host(dims, bd.make_host_args(y=y_h, final_state=fin_h if with_state else None, status=st,
+                                                        init_state=init, **host, **par), scratch, flags=flags)
+        torch.cuda.synchronize()
+        assert int(st[0]) == 0
+        assert torch.equal(y_h, y_d.cpu())
+        assert not with_state or torch.equal(fin_h, fin_d.cpu())
