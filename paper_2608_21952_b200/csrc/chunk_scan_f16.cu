@@ -237,7 +237,7 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
   const int TM = BIGQ ? 128 : Q;           // valid rows of a tile
   const int ntpu = BIGQ ? Q / 128 : 1;     // tiles per (batch, chunk, head)
   const uint32_t RBN = N, RBQ = BIGQ ? 128u : (uint32_t)Q;        // row bytes of the N-contracted and Q-contracted int8 tiles
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // (the shuffle: uniform for the compiler)
   // tiles of this CTA: its units blockIdx.x, blockIdx.x + gridDim.x, ..., ntpu tiles each
   const int n_end = tiles_of_cta(a.w, (int)blockIdx.x, (int)gridDim.x, ntpu);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + OFF_BAR);
@@ -272,7 +272,7 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   pdl_wait();   // every role below reads or writes global memory
 
   if (warp == 0) {
@@ -296,13 +296,13 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
         const int tg = t.h / a.w.hpg;   // group of the head
         const int ci = cb_index(n, t.it, ntpu), t3 = n & 3;
         const uint32_t ph4 = (n >> 2) & 1;
-        mbar_wait_relaxed(&bars[B_CB_FREE + ci], ph4 ^ 1, a.status);
+        mbar_wait(&bars[B_CB_FREE + ci], ph4 ^ 1, a.status);
         const int npanel = t.KJ / (int)RBQ;
         mbar_expect_tx(&bars[B_CB_FULL + ci], (uint32_t)(npanel * TM * RBQ));
         for (int pn = 0; pn < npanel; ++pn)
           tma_load_2d(smem + cb_offset(ci) + pn * PANEL, &tm_cb, &bars[B_CB_FULL + ci], pn * (int)RBQ,
                       (int)((((i64)t.b * d.c + t.k) * d.G + tg) * Q + t.it * TM));
-        mbar_wait_relaxed(&bars[B_TOK_FREE + t3], ph4 ^ 1, a.status);
+        mbar_wait(&bars[B_TOK_FREE + t3], ph4 ^ 1, a.status);
         // the scalar pack of the chunk and the head's per-column vectors (the epilogue reads them once per
         // 8-column piece: from global memory each read would be a long-latency load in its chain)
         uint8_t* slot = smem + OFF_TOK + t3 * TOK_BYTES;
@@ -325,7 +325,7 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
 #pragma unroll 1
       for (int n = 0; n < n_end; ++n, next_tile(t, d, a.w, TM, ntpu)) {
         // the MMAs of tile n - 1 (the other issuer's) have read the buffer
-        if (n > 0) mbar_wait_relaxed(&bars[B_CH_FREE + ((n - 1) & 1)], ((n - 1) >> 1) & 1, a.status);
+        if (n > 0) mbar_wait(&bars[B_CH_FREE + ((n - 1) & 1)], ((n - 1) >> 1) & 1, a.status);
         uint64_t* full = &bars[B_CH_FULL + (n & 1)];
         mbar_expect_tx(full, (uint32_t)(TM * N + 64 * N));
         tma_load_3d(smem + OFF_C, &tm_C, full, 0, t.h / a.w.hpg, (int)(t.tok0 + t.it * TM));
@@ -336,36 +336,52 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
     // ------------------------------------------------------------ MMA issuers: warp 1 takes the even tiles of
     // this CTA, warp 3 the odd ones (a tile is 12 to 20 instructions of 16 tokens each, and issuing one
     // takes a thread about 0.1 us: one issuer alone would set the pace of the kernel)
-    if (lane == 0) {
+    {   // (the whole warp runs the loop, see elect_one)
       const int par = warp == 3 ? 1 : 0;
       const uint32_t idesc_off = idesc_s8(128, 64, 0, 0), idesc_diag = idesc_f16(128, 64, 1);
       const uint32_t sbase = smem_u32(smem);
+      const uint64_t dc = tile_desc(sbase + OFF_C, RBN), dh = tile_desc(sbase + OFF_H, RBN);
 #pragma unroll 1
       for (int n = par; n < n_end; n += 2) {
         const int it = ntpu == 1 ? 0 : (n & 1);   // a CTA's first tile is the first of its unit
         const int ci = cb_index(n, it, ntpu), s2 = n & 1, xs = x_index(n, ntpu);
         const uint32_t ph4 = (n >> 2) & 1, ph2 = (n >> 1) & 1;
-        const int KJ = (it + 1) * TM;
         const uint32_t acc = tmem + (uint32_t)s2 * 128u;
         mbar_wait(&bars[B_ACC_FREE + s2], ph2 ^ 1, a.status);
         mbar_wait(&bars[B_CH_FULL + par], ph2, a.status);
         tc_fence_after();
-#pragma unroll 1
-        for (int q = 0; q < N / 32; ++q)
-          mma_s8_ss(acc, tile_desc(sbase + OFF_C + 32 * q, RBN), tile_desc(sbase + OFF_H + 32 * q, RBN),
-                    idesc_off, q > 0);
-        mma_commit(&bars[B_CH_FREE + par]);
-        mbar_wait(&bars[B_MQ + ci], ph4, a.status);        // the operand of this tile is in tensor memory
+        if (elect_one()) {
+          mma_s8_ss(acc, dc, dh, idesc_off, 0);
+          mma_s8_ss(acc, dc + 2, dh + 2, idesc_off, 1);
+          if (N == 128) {
+            mma_s8_ss(acc, dc + 4, dh + 4, idesc_off, 1);
+            mma_s8_ss(acc, dc + 6, dh + 6, idesc_off, 1);
+          }
+          mma_commit(&bars[B_CH_FREE + par]);
+        }
+        __syncwarp();
         mbar_wait(&bars[B_X_FULL + xs], x_phase(n, ntpu), a.status);
+        mbar_wait(&bars[B_MQ + ci], ph4, a.status);        // the operand of this tile is in tensor memory
         tc_fence_after();
-        // 16 tokens per instruction: 8 operand columns and 16 rows of 128 bytes of x
-        uint64_t bd = smem_desc(sbase + OFF_X + xs * X_BYTES, 16, 1024, SWZ_128B);
-        const uint32_t a_op = tmem + 256u + (uint32_t)s2 * 128u;
-#pragma unroll 1
-        for (int q = 0; q < KJ / 16; ++q, bd += (16 * 128) >> 4)
-          mma_f16_ts(acc + 64, a_op + (uint32_t)(q * 8), bd, idesc_diag, q > 0);
-        mma_commit(&bars[B_AFREE + s2]);
-        mma_commit(&bars[B_ACC + s2]);
+        if (elect_one()) {
+          // 16 tokens per instruction: 8 operand columns and 16 rows of 128 bytes of x
+          const uint64_t bd = smem_desc(sbase + OFF_X + xs * X_BYTES, 16, 1024, SWZ_128B);
+          const uint32_t a_op = tmem + 256u + (uint32_t)s2 * 128u;
+          constexpr uint64_t kStepX = (16 * 128) >> 4;
+#pragma unroll
+          for (uint32_t q = 0; q < 4; ++q) mma_f16_ts(acc + 64, a_op + q * 8, bd + q * kStepX, idesc_diag, q > 0);
+          if (BIGQ) {
+#pragma unroll
+            for (uint32_t q = 4; q < 8; ++q) mma_f16_ts(acc + 64, a_op + q * 8, bd + q * kStepX, idesc_diag, 1);
+            if (it) {
+#pragma unroll
+              for (uint32_t q = 8; q < 16; ++q) mma_f16_ts(acc + 64, a_op + q * 8, bd + q * kStepX, idesc_diag, 1);
+            }
+          }
+          mma_commit(&bars[B_AFREE + s2]);
+          mma_commit(&bars[B_ACC + s2]);
+        }
+        __syncwarp();
       }
     }
   } else if (warp < kEpiWarp0) {
@@ -388,9 +404,9 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
       // which costs no issue slots
       if (wg == 0 && lane < 3) {
         const int bi = lane == 0 ? B_TOK_FULL + t3 : lane == 1 ? B_CB_FULL + ci : B_AFREE + ob;
-        mbar_wait_relaxed(&bars[bi], lane == 2 ? (((n >> 1) & 1) ^ 1) : ph4, a.status);
+        mbar_wait(&bars[bi], lane == 2 ? (((n >> 1) & 1) ^ 1) : ph4, a.status);
       } else if (wg == 0 && lane == 3 && t.it == 0) {
-        mbar_wait_relaxed(&bars[B_X_RAW + x_index(n, ntpu)], x_phase(n, ntpu), a.status);   // the chunk's xq codes
+        mbar_wait(&bars[B_X_RAW + x_index(n, ntpu)], x_phase(n, ntpu), a.status);   // the chunk's xq codes
       }
       named_bar_sync(1 + g, kGroupWarps * 32);
       if (t.it == 0) {   // first tile of a chunk: the group expands the chunk's xq rows to FP16, a row per thread
@@ -438,7 +454,7 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
       // three lanes wait side by side: the accumulators, the x rows (skip term), the scalar pack (cs)
       if (ew == 0 && lane < 3) {   // one warp polls, the others wait at a hardware barrier
         const int bi = lane == 0 ? B_ACC + s2 : lane == 1 ? B_X_FULL + xs : B_TOK_FULL + t3;
-        mbar_wait_relaxed(&bars[bi], lane == 2 ? ph4 : lane == 1 ? x_phase(n, ntpu) : ph2, a.status);
+        mbar_wait(&bars[bi], lane == 2 ? ph4 : lane == 1 ? x_phase(n, ntpu) : ph2, a.status);
       }
       named_bar_sync(3, kEpiWarps * 32);
       tc_fence_after();
