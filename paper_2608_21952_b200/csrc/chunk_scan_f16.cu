@@ -9,11 +9,9 @@
 //  * the mask warps write M16 straight into tensor memory (tcgen05.st, thread = row), from where
 //    tcgen05.mma.kind::f16 takes it as its A operand: the operand never exists in shared memory,
 //    there is no row maximum, no second pass and no zero fill of shared memory;
-//  * X enters the MMA as the exact FP16 image of its int8 codes: the codes of a chunk arrive by TMA in
-//    the upper half of the chunk's x buffer and the mask group that takes the chunk expands them in
-//    place, a row per thread, into the MN-major tile with 128-byte swizzled rows that the MMA reads;
-//    the epilogue warps request the codes of the chunk after next when they hand a buffer back;
-//    ChunkScan1 stays an int8 MMA;
+//  * X enters the MMA as the exact FP16 image of its int8 codes: the codes of the next chunk arrive by TMA in a
+//    buffer of their own and the epilogue warps expand them, a row per thread, into the MN-major tile with
+//    128-byte swizzled rows that the MMA reads; ChunkScan1 stays an int8 MMA;
 //  * tensor memory: two accumulator pairs (INT32 C h, FP32 M16 x) and two operand buffers, 512 columns.
 // One factor per 16-column sub-block as in chunk_scan.cu: own sub-block by the running product of
 // per-token decays, earlier ones woff_j f with f the row's decay to the end of the sub-block before its own
@@ -48,7 +46,10 @@ constexpr int kMaskWarp0 = 4, kGroupWarps = 8;
 constexpr int kEpiWarp0 = 20, kEpiWarps = 8;
 constexpr uint32_t kTmemCols = 512;  // accumulator pair a at 128 a (+0 INT32 C h, +64 FP32 M16 x); operand buffer g at 256 + 128 g
 // shared memory (bytes, from a 1024-byte aligned base)
-constexpr uint32_t OFF_CB = 0;          // ring of 4: two 2-panel buffers, two 1-panel buffers
+// CBq: with two tiles per chunk two 2-panel buffers for the second tiles and one 1-panel buffer for the first
+// ones (a first tile is read in a quarter of a chunk's time); with one tile per chunk a ring of 4 panels
+constexpr uint32_t OFF_CB = 0;
+constexpr uint32_t OFF_XRAW = 81920;    // [256][64] int8 codes of the chunk after next
 constexpr uint32_t OFF_C = 98304;       // [128][N]
 constexpr uint32_t OFF_H = 114688;      // [64][N]
 constexpr uint32_t OFF_X = 122880;      // ring of 2 x [256][64] fp16 (128-byte rows)
@@ -61,13 +62,15 @@ constexpr uint32_t OFF_YST = OFF_TOK + 4 * TOK_BYTES;  // 8 warps x [32][64 B] y
 constexpr uint32_t OFF_BAR = OFF_YST + 16384;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 512;
 
-__device__ __forceinline__ uint32_t cb_offset(int idx) { return scan::cb_offset(OFF_CB, idx); }
+__device__ __forceinline__ uint32_t cb_offset(int n, int it, int ntpu) {
+  return ntpu == 1 ? (uint32_t)(n & 3) * PANEL : it ? (uint32_t)((n >> 1) & 1) * 2 * PANEL : 4 * PANEL;
+}
 
 // The Cq/hq buffer is single, but its barriers come in pairs indexed by the parity of the tile: the two
 // MMA issuers take alternate tiles, and a barrier polled by parity must be seen phase by phase by its
 // one waiter (an issuer that skipped a phase would pass its first wait at once).
-enum { B_CB_FULL = 0, B_CB_FREE = 4, B_MQ = 8, B_CH_FULL = 12, B_X_FULL = 14, B_X_FREE = 16,
-       B_TOK_FULL = 18, B_TOK_FREE = 22, B_ACC = 26, B_ACC_FREE = 28, B_AFREE = 30, B_CH_FREE = 32, B_X_RAW = 34, B_COUNT = 36 };
+enum { B_CB_FULL = 0, B_CB_FREE = 4, B_MQ = 8, B_CH_FULL = 12, B_X_FULL = 14,
+       B_TOK_FULL = 18, B_TOK_FREE = 22, B_ACC = 26, B_ACC_FREE = 28, B_AFREE = 30, B_CH_FREE = 32, B_X_RAW = 34, B_RAW_FREE = 35, B_COUNT = 36 };
 
 __device__ __forceinline__ uint32_t half2_bits(float2 v) {
   const __half2 h = __floats2half2_rn(v.x, v.y);
@@ -196,18 +199,18 @@ __device__ __forceinline__ void mask_tile_f16(const uint8_t* sCB, const float* t
   tmem_st_wait();
 }
 
-// The xq rows of a chunk arrive as int8 codes in the upper half of the chunk's x buffer (rows of 64
-// bytes from byte 64 Q on) and are expanded in place into the MMA's FP16 operand (rows of 128 bytes,
-// 128-byte swizzle, from byte 0) by the mask group that takes the chunk: one row per thread, every
-// thread reads its codes, the group meets at its hardware barrier, every thread writes its row.  With
+// A row of x, from its int8 codes (64 plain bytes) to the MMA's FP16 operand (128 bytes, 128-byte swizzle).  With
 // u = code ^ 0x80 the half with bits 0x6400 | u is 1024 + u exactly, and subtracting 1152 gives the
-// code (one byte permute and one packed subtraction per two codes).
-__device__ __forceinline__ void x_row_to_half(uint8_t* xb, int r, const uint4 (&w)[4]) {
+// code (one byte permute and one packed subtraction per two codes).  (The 16-byte pieces are taken in an order
+// that depends on the row, which spreads the rows' equal offsets over the banks.)
+__device__ __forceinline__ void x_row_to_half(const uint8_t* raw, uint8_t* xb, int r) {
   const __half2 off = __floats2half2_rn(1152.f, 1152.f);
   uint8_t* row = xb + r * 128;
 #pragma unroll
-  for (int qd = 0; qd < 4; ++qd) {
-    const uint32_t ww[4] = {w[qd].x ^ 0x80808080u, w[qd].y ^ 0x80808080u, w[qd].z ^ 0x80808080u, w[qd].w ^ 0x80808080u};
+  for (int j = 0; j < 4; ++j) {
+    const int qd = (j + (r >> 1)) & 3;
+    const uint4 w = *reinterpret_cast<const uint4*>(raw + r * 64 + qd * 16);
+    const uint32_t ww[4] = {w.x ^ 0x80808080u, w.y ^ 0x80808080u, w.z ^ 0x80808080u, w.w ^ 0x80808080u};
     uint32_t o[8];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -256,13 +259,13 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
       mbar_init(&bars[B_CH_FREE + s], 1);
     }
     for (int s = 0; s < 2; ++s) {
-      mbar_init(&bars[B_X_FULL + s], kGroupWarps);   // the warps of the mask group that expands the rows
-      mbar_init(&bars[B_X_RAW + s], 1);
-      mbar_init(&bars[B_X_FREE + s], kEpiWarps * ntpu);   // the epilogues of the chunk's tiles
+      mbar_init(&bars[B_X_FULL + s], kEpiWarps);   // the warps that expand the rows
       mbar_init(&bars[B_ACC + s], 1);
       mbar_init(&bars[B_ACC_FREE + s], kEpiWarps);
       mbar_init(&bars[B_AFREE + s], 1);
     }
+    mbar_init(&bars[B_X_RAW], 1);
+    mbar_init(&bars[B_RAW_FREE], kEpiWarps);
     fence_mbar_init();
     tma_prefetch_desc(&tm_C); tma_prefetch_desc(&tm_h); tma_prefetch_desc(&tm_x);
     tma_prefetch_desc(&tm_cb); tma_prefetch_desc(&tm_y);
@@ -276,31 +279,25 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
   pdl_wait();   // every role below reads or writes global memory
 
   if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer: CBq panels, scalar pack, and the
-    // int8 xq rows of each chunk (the mask group that takes the chunk expands them to FP16)
+    // ------------------------------------------------------------ TMA producer: CBq panels, scalar pack
     if (lane == 0) {
       Tile t = decode_unit((int)blockIdx.x, d, TM);
-      {   // the int8 xq rows of the first two chunks (both buffers are free); later requests come from the
-          // epilogue warps, the moment they have finished with a buffer
-        Tile tn = t;
-        for (int kc = 0; kc < 2 && kc * ntpu < n_end; ++kc) {
-          uint8_t* xb = smem + OFF_X + kc * X_BYTES;
-          mbar_expect_tx(&bars[B_X_RAW + kc], (uint32_t)(Q * 64));
-          for (int j0 = 0; j0 < Q; j0 += TM)
-            tma_load_3d(xb + Q * 64 + j0 * 64, &tm_x, &bars[B_X_RAW + kc], 0, tn.h, (int)(tn.tok0 + j0));
-          next_head(tn, d, a.w, TM, ntpu);
-        }
-      }
 #pragma unroll 1
       for (int n = 0; n < n_end; ++n, next_tile(t, d, a.w, TM, ntpu)) {
         const int tg = t.h / a.w.hpg;   // group of the head
         const int ci = cb_index(n, t.it, ntpu), t3 = n & 3;
         const uint32_t ph4 = (n >> 2) & 1;
-        mbar_wait(&bars[B_CB_FREE + ci], ph4 ^ 1, a.status);
+        if (BIGQ && ntpu == 2 && t.it == 0) {
+          // the first tiles share one buffer; their barriers come in pairs by the parity of the chunk (see below), so
+          // the chunk before has the other pair
+          if (n > 0) mbar_wait(&bars[B_CB_FREE + (ci ^ 1)], ((n - 2) >> 2) & 1, a.status);
+        } else {
+          mbar_wait(&bars[B_CB_FREE + ci], ph4 ^ 1, a.status);
+        }
         const int npanel = t.KJ / (int)RBQ;
         mbar_expect_tx(&bars[B_CB_FULL + ci], (uint32_t)(npanel * TM * RBQ));
         for (int pn = 0; pn < npanel; ++pn)
-          tma_load_2d(smem + cb_offset(ci) + pn * PANEL, &tm_cb, &bars[B_CB_FULL + ci], pn * (int)RBQ,
+          tma_load_2d(smem + OFF_CB + cb_offset(n, t.it, ntpu) + pn * PANEL, &tm_cb, &bars[B_CB_FULL + ci], pn * (int)RBQ,
                       (int)((((i64)t.b * d.c + t.k) * d.G + tg) * Q + t.it * TM));
         mbar_wait(&bars[B_TOK_FREE + t3], ph4 ^ 1, a.status);
         // the scalar pack of the chunk and the head's per-column vectors (the epilogue reads them once per
@@ -319,9 +316,15 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
       }
     }
   } else if (warp == 2) {
-    // ------------------------------------------------------------ TMA producer: Cq, hq
+    // ------------------------------------------------------------ TMA producer: Cq, hq, and the int8 xq rows a chunk ahead
     if (lane == 0) {
       Tile t = decode_unit((int)blockIdx.x, d, TM);
+      auto load_x = [&](const Tile& x) {
+        mbar_expect_tx(&bars[B_X_RAW], (uint32_t)(Q * 64));
+        for (int j0 = 0; j0 < Q; j0 += TM)
+          tma_load_3d(smem + OFF_XRAW + j0 * 64, &tm_x, &bars[B_X_RAW], 0, x.h, (int)(x.tok0 + j0));
+      };
+      load_x(t);
 #pragma unroll 1
       for (int n = 0; n < n_end; ++n, next_tile(t, d, a.w, TM, ntpu)) {
         // the MMAs of tile n - 1 (the other issuer's) have read the buffer
@@ -330,6 +333,13 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
         mbar_expect_tx(full, (uint32_t)(TM * N + 64 * N));
         tma_load_3d(smem + OFF_C, &tm_C, full, 0, t.h / a.w.hpg, (int)(t.tok0 + t.it * TM));
         tma_load_2d(smem + OFF_H, &tm_h, full, 0, (int)((((i64)t.b * d.c + t.k) * d.H + t.h) * P));
+        if (t.it == 0 && n + ntpu < n_end) {   // the rows of the next chunk, once those of this one have been expanded
+          const int u = ntpu == 1 ? n : n >> 1;
+          mbar_wait(&bars[B_RAW_FREE], (uint32_t)u & 1u, a.status);
+          Tile tn = t;
+          next_unit(tn, d, a.w);
+          load_x(tn);
+        }
       }
     }
   } else if (warp == 1 || warp == 3) {
@@ -405,26 +415,10 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
       if (wg == 0 && lane < 3) {
         const int bi = lane == 0 ? B_TOK_FULL + t3 : lane == 1 ? B_CB_FULL + ci : B_AFREE + ob;
         mbar_wait(&bars[bi], lane == 2 ? (((n >> 1) & 1) ^ 1) : ph4, a.status);
-      } else if (wg == 0 && lane == 3 && t.it == 0) {
-        mbar_wait(&bars[B_X_RAW + x_index(n, ntpu)], x_phase(n, ntpu), a.status);   // the chunk's xq codes
       }
       named_bar_sync(1 + g, kGroupWarps * 32);
-      if (t.it == 0) {   // first tile of a chunk: the group expands the chunk's xq rows to FP16, a row per thread
-        uint8_t* xb = smem + OFF_X + x_index(n, ntpu) * X_BYTES;
-        const int r = wg * 32 + lane;
-        uint4 w[4];
-        if (r < Q) {
-#pragma unroll
-          for (int qd = 0; qd < 4; ++qd) w[qd] = *reinterpret_cast<const uint4*>(xb + Q * 64 + r * 64 + qd * 16);
-        }
-        named_bar_sync(1 + g, kGroupWarps * 32);   // every code is in a register: the rows may be overwritten
-        if (r < Q) x_row_to_half(xb, r, w);
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars[B_X_FULL + x_index(n, ntpu)]);
-      }
       tc_fence_after();
-      mask_tile_f16(smem + cb_offset(ci), reinterpret_cast<const float*>(smem + OFF_TOK + t3 * TOK_BYTES),
+      mask_tile_f16(smem + OFF_CB + cb_offset(n, t.it, ntpu), reinterpret_cast<const float*>(smem + OFF_TOK + t3 * TOK_BYTES),
                     tmem + 256u + (uint32_t)ob * 128u, rq, q2, lane, TM, RBQ, t, a);
       tc_fence_before();
       __syncwarp();
@@ -441,6 +435,20 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
     const int er = q * 32 + lane;           // row of the tile
     uint8_t* ystage = smem + OFF_YST + ew * 2048;   // [32][64 B], 64-byte swizzle
     uint8_t* srow = ystage + lane * 64;
+    // These warps also expand the xq rows of a chunk to FP16, a row per thread, one chunk ahead of its MMAs and at the
+    // start of a chunk, when they would wait for its accumulators anyway.  (The mask groups, which set the pace,
+    // waited 2 us per chunk for the codes and spent 1 us on them.)
+    const int nunits = n_end / ntpu;
+    auto expand_x = [&](int u) {
+      mbar_wait(&bars[B_X_RAW], (uint32_t)u & 1u, a.status);
+      const int r = ew * 32 + lane;
+      if (r < Q) x_row_to_half(smem + OFF_XRAW, smem + OFF_X + (u & 1) * X_BYTES, r);
+      fence_async_smem();
+      __syncwarp();
+      if (lane < 2) mbar_arrive(&bars[lane == 0 ? B_X_FULL + (u & 1) : B_RAW_FREE]);
+    };
+    expand_x(0);
+    if (nunits > 1) expand_x(1);
     Tile t = decode_unit((int)blockIdx.x, d, TM);
 #pragma unroll 1
     for (int n = 0; n < n_end; ++n, next_tile(t, d, a.w, TM, ntpu)) {
@@ -451,11 +459,18 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
       const float4* gsx = reinterpret_cast<const float4*>(smem + OFF_TOK + t3 * TOK_BYTES + TOK_COLS) + ch * 8;
       const float4* gsh = gsx + 16;
       const float4* gco = gsx + 32;
-      // three lanes wait side by side: the accumulators, the x rows (skip term), the scalar pack (cs)
-      if (ew == 0 && lane < 3) {   // one warp polls, the others wait at a hardware barrier
-        const int bi = lane == 0 ? B_ACC + s2 : lane == 1 ? B_X_FULL + xs : B_TOK_FULL + t3;
-        mbar_wait(&bars[bi], lane == 2 ? ph4 : lane == 1 ? x_phase(n, ntpu) : ph2, a.status);
+      if (t.it == 0 && n > 0) {
+        // every warp is through with the chunk before (its MMAs have completed, and no one reads its rows any
+        // more): its x buffer takes the next chunk
+        const int u = ntpu == 1 ? n : n >> 1;
+        if (u + 1 < nunits) {
+          named_bar_sync(3, kEpiWarps * 32);
+          expand_x(u + 1);
+        }
       }
+      // two lanes wait side by side: the accumulators, the scalar pack (cs)
+      if (ew == 0 && lane < 2)   // one warp polls, the others wait at a hardware barrier
+        mbar_wait(&bars[lane == 0 ? B_ACC + s2 : B_TOK_FULL + t3], lane == 0 ? ph2 : ph4, a.status);
       named_bar_sync(3, kEpiWarps * 32);
       tc_fence_after();
       const bool ok = er < TM;
@@ -518,21 +533,8 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
           if (pc == 3) tc_fence_before();
           fence_async_smem();
           __syncwarp();
-          if (pc == 3 && lane < 3) {
-            mbar_arrive(&bars[lane == 0 ? B_ACC_FREE + s2 : lane == 1 ? B_X_FREE + xs : B_TOK_FREE + t3]);
-            // the chunk's last tile: once every epilogue warp is through, its x buffer takes the codes of
-            // the chunk after next
-            const int n2 = n - (ntpu - 1) + 2 * ntpu;   // first tile of that chunk
-            if (ew == 0 && lane == 1 && t.it == ntpu - 1 && n2 < n_end) {
-              mbar_wait(&bars[B_X_FREE + xs], x_phase(n, ntpu), a.status);
-              Tile tn = t;
-              next_unit(tn, d, a.w);
-              next_unit(tn, d, a.w);
-              uint8_t* xb = smem + OFF_X + xs * X_BYTES;
-              mbar_expect_tx(&bars[B_X_RAW + xs], (uint32_t)(Q * 64));
-              for (int j0 = 0; j0 < Q; j0 += TM)
-                tma_load_3d(xb + Q * 64 + j0 * 64, &tm_x, &bars[B_X_RAW + xs], 0, tn.h, (int)(tn.tok0 + j0));
-            }
+          if (pc == 3 && lane < 2) {
+            mbar_arrive(&bars[lane == 0 ? B_ACC_FREE + s2 : B_TOK_FREE + t3]);
           } else if (lane == 3 && q * 32 < TM) {
             tma_store_3d(&tm_y, ystage, ch * 32 + (YT != 0 ? 0 : (pc >> 1) * 16), t.h,
                          (int)(t.tok0 + t.it * TM + q * 32));
