@@ -10,7 +10,7 @@
 //    tcgen05.mma.kind::f16 takes it as its A operand: the operand never exists in shared memory,
 //    there is no row maximum, no second pass and no zero fill of shared memory;
 //  * X enters the MMA as the exact FP16 image of its int8 codes: the codes of the next chunk arrive by TMA in a
-//    buffer of their own and the epilogue warps expand them, a row per thread, into the MN-major tile with
+//    buffer of their own and the mask group that has the chunk expands them, a row per thread, into the MN-major tile with
 //    128-byte swizzled rows that the MMA reads; ChunkScan1 stays an int8 MMA;
 //  * tensor memory: two accumulator pairs (INT32 C h, FP32 M16 x) and two operand buffers, 512 columns.
 // One factor per 16-column sub-block as in chunk_scan.cu: own sub-block by the running product of
@@ -70,7 +70,7 @@ __device__ __forceinline__ uint32_t cb_offset(int n, int it, int ntpu) {
 // MMA issuers take alternate tiles, and a barrier polled by parity must be seen phase by phase by its
 // one waiter (an issuer that skipped a phase would pass its first wait at once).
 enum { B_CB_FULL = 0, B_CB_FREE = 4, B_MQ = 8, B_CH_FULL = 12, B_X_FULL = 14,
-       B_TOK_FULL = 18, B_TOK_FREE = 22, B_ACC = 26, B_ACC_FREE = 28, B_AFREE = 30, B_CH_FREE = 32, B_X_RAW = 34, B_RAW_FREE = 35, B_COUNT = 36 };
+       B_TOK_FULL = 18, B_TOK_FREE = 22, B_ACC = 26, B_ACC_FREE = 28, B_AFREE = 30, B_CH_FREE = 32, B_X_RAW = 34, B_X_FREE = 36, B_RAW_FREE = 38, B_COUNT = 39 };
 
 __device__ __forceinline__ uint32_t half2_bits(float2 v) {
   const __half2 h = __floats2half2_rn(v.x, v.y);
@@ -199,17 +199,16 @@ __device__ __forceinline__ void mask_tile_f16(const uint8_t* sCB, const float* t
   tmem_st_wait();
 }
 
-// A row of x, from its int8 codes (64 plain bytes) to the MMA's FP16 operand (128 bytes, 128-byte swizzle).  With
+// A row of x, from its int8 codes (64 bytes, 64-byte swizzle) to the MMA's FP16 operand (128 bytes, 128-byte swizzle:
+// neither side has bank conflicts; with plain rows the expansion of a chunk took 1.4 us).  With
 // u = code ^ 0x80 the half with bits 0x6400 | u is 1024 + u exactly, and subtracting 1152 gives the
-// code (one byte permute and one packed subtraction per two codes).  (The 16-byte pieces are taken in an order
-// that depends on the row, which spreads the rows' equal offsets over the banks.)
+// code (one byte permute and one packed subtraction per two codes).
 __device__ __forceinline__ void x_row_to_half(const uint8_t* raw, uint8_t* xb, int r) {
   const __half2 off = __floats2half2_rn(1152.f, 1152.f);
   uint8_t* row = xb + r * 128;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int qd = (j + (r >> 1)) & 3;
-    const uint4 w = *reinterpret_cast<const uint4*>(raw + r * 64 + qd * 16);
+  for (int qd = 0; qd < 4; ++qd) {
+    const uint4 w = *reinterpret_cast<const uint4*>(raw + swz_off((uint32_t)r, (uint32_t)qd, 64));
     const uint32_t ww[4] = {w.x ^ 0x80808080u, w.y ^ 0x80808080u, w.z ^ 0x80808080u, w.w ^ 0x80808080u};
     uint32_t o[8];
 #pragma unroll
@@ -259,13 +258,14 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
       mbar_init(&bars[B_CH_FREE + s], 1);
     }
     for (int s = 0; s < 2; ++s) {
-      mbar_init(&bars[B_X_FULL + s], kEpiWarps);   // the warps that expand the rows
+      mbar_init(&bars[B_X_FULL + s], kGroupWarps);   // the warps of the mask group that expands the rows
+      mbar_init(&bars[B_X_RAW + s], 1);
+      mbar_init(&bars[B_X_FREE + s], kEpiWarps);     // the epilogue of the chunk's last tile (its MMAs are done by then)
       mbar_init(&bars[B_ACC + s], 1);
       mbar_init(&bars[B_ACC_FREE + s], kEpiWarps);
       mbar_init(&bars[B_AFREE + s], 1);
     }
-    mbar_init(&bars[B_X_RAW], 1);
-    mbar_init(&bars[B_RAW_FREE], kEpiWarps);
+    mbar_init(&bars[B_RAW_FREE], kGroupWarps);
     fence_mbar_init();
     tma_prefetch_desc(&tm_C); tma_prefetch_desc(&tm_h); tma_prefetch_desc(&tm_x);
     tma_prefetch_desc(&tm_cb); tma_prefetch_desc(&tm_y);
@@ -287,18 +287,6 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
         const int tg = t.h / a.w.hpg;   // group of the head
         const int ci = cb_index(n, t.it, ntpu), t3 = n & 3;
         const uint32_t ph4 = (n >> 2) & 1;
-        if (BIGQ && ntpu == 2 && t.it == 0) {
-          // the first tiles share one buffer; their barriers come in pairs by the parity of the chunk (see below), so
-          // the chunk before has the other pair
-          if (n > 0) mbar_wait(&bars[B_CB_FREE + (ci ^ 1)], ((n - 2) >> 2) & 1, a.status);
-        } else {
-          mbar_wait(&bars[B_CB_FREE + ci], ph4 ^ 1, a.status);
-        }
-        const int npanel = t.KJ / (int)RBQ;
-        mbar_expect_tx(&bars[B_CB_FULL + ci], (uint32_t)(npanel * TM * RBQ));
-        for (int pn = 0; pn < npanel; ++pn)
-          tma_load_2d(smem + OFF_CB + cb_offset(n, t.it, ntpu) + pn * PANEL, &tm_cb, &bars[B_CB_FULL + ci], pn * (int)RBQ,
-                      (int)((((i64)t.b * d.c + t.k) * d.G + tg) * Q + t.it * TM));
         mbar_wait(&bars[B_TOK_FREE + t3], ph4 ^ 1, a.status);
         // the scalar pack of the chunk and the head's per-column vectors (the epilogue reads them once per
         // 8-column piece: from global memory each read would be a long-latency load in its chain)
@@ -313,18 +301,30 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
         bulk_load(slot + TOK_COLS, a.s_x + t.h * P, (uint32_t)(P * 4), &bars[B_TOK_FULL + t3]);
         bulk_load(slot + TOK_COLS + 256, a.s_h + t.h * P, (uint32_t)(P * 4), &bars[B_TOK_FULL + t3]);
         if (CORR) bulk_load(slot + TOK_COLS + 512, a.corr + t.h * P, (uint32_t)(P * 4), &bars[B_TOK_FULL + t3]);
+        if (BIGQ && ntpu == 2 && t.it == 0) {
+          // the first tiles share one buffer; their barriers come in pairs by the parity of the chunk (see below), so
+          // the chunk before has the other pair
+          if (n > 0) mbar_wait(&bars[B_CB_FREE + (ci ^ 1)], ((n - 2) >> 2) & 1, a.status);
+        } else {
+          mbar_wait(&bars[B_CB_FREE + ci], ph4 ^ 1, a.status);
+        }
+        const int npanel = t.KJ / (int)RBQ;
+        mbar_expect_tx(&bars[B_CB_FULL + ci], (uint32_t)(npanel * TM * RBQ));
+        for (int pn = 0; pn < npanel; ++pn)
+          tma_load_2d(smem + OFF_CB + cb_offset(n, t.it, ntpu) + pn * PANEL, &tm_cb, &bars[B_CB_FULL + ci], pn * (int)RBQ,
+                      (int)((((i64)t.b * d.c + t.k) * d.G + tg) * Q + t.it * TM));
       }
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------ TMA producer: Cq, hq, and the int8 xq rows a chunk ahead
     if (lane == 0) {
       Tile t = decode_unit((int)blockIdx.x, d, TM);
-      auto load_x = [&](const Tile& x) {
-        mbar_expect_tx(&bars[B_X_RAW], (uint32_t)(Q * 64));
+      auto load_x = [&](const Tile& x, int u) {
+        mbar_expect_tx(&bars[B_X_RAW + (u & 1)], (uint32_t)(Q * 64));
         for (int j0 = 0; j0 < Q; j0 += TM)
-          tma_load_3d(smem + OFF_XRAW + j0 * 64, &tm_x, &bars[B_X_RAW], 0, x.h, (int)(x.tok0 + j0));
+          tma_load_3d(smem + OFF_XRAW + j0 * 64, &tm_x, &bars[B_X_RAW + (u & 1)], 0, x.h, (int)(x.tok0 + j0));
       };
-      load_x(t);
+      load_x(t, 0);
 #pragma unroll 1
       for (int n = 0; n < n_end; ++n, next_tile(t, d, a.w, TM, ntpu)) {
         // the MMAs of tile n - 1 (the other issuer's) have read the buffer
@@ -338,7 +338,7 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
           mbar_wait(&bars[B_RAW_FREE], (uint32_t)u & 1u, a.status);
           Tile tn = t;
           next_unit(tn, d, a.w);
-          load_x(tn);
+          load_x(tn, u + 1);
         }
       }
     }
@@ -426,6 +426,21 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
         mbar_arrive(&bars[B_MQ + ci]);
         mbar_arrive(&bars[B_CB_FREE + ci]);
       }
+      if (t.it == 0) {
+        // The chunk's xq rows, a row per thread: behind the first tile's operand, when the epilogue of the chunk
+        // before last has long given the buffer back.  (By the epilogue warps instead, one chunk ahead: 0.154 against
+        // 0.151 ms at batch 8 x 2048 x 80 heads; ahead of the first tile, with the codes in the same buffer, the
+        // groups waited 2 us per chunk.)
+        const int xs = x_index(n, ntpu);
+        const uint32_t xp = x_phase(n, ntpu);
+        if (wg == 0 && lane < 2) mbar_wait(&bars[lane == 0 ? B_X_RAW + xs : B_X_FREE + xs], lane == 0 ? xp : xp ^ 1, a.status);
+        named_bar_sync(1 + g, kGroupWarps * 32);
+        const int r = wg * 32 + lane;
+        if (r < Q) x_row_to_half(smem + OFF_XRAW, smem + OFF_X + xs * X_BYTES, r);
+        fence_async_smem();
+        __syncwarp();
+        if (lane < 2) mbar_arrive(&bars[lane == 0 ? B_X_FULL + xs : B_RAW_FREE]);
+      }
     }
   } else {
     // ------------------------------------------------------------ epilogue warps: rows 32 q .., columns 32 ch ..
@@ -435,20 +450,6 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
     const int er = q * 32 + lane;           // row of the tile
     uint8_t* ystage = smem + OFF_YST + ew * 2048;   // [32][64 B], 64-byte swizzle
     uint8_t* srow = ystage + lane * 64;
-    // These warps also expand the xq rows of a chunk to FP16, a row per thread, one chunk ahead of its MMAs and at the
-    // start of a chunk, when they would wait for its accumulators anyway.  (The mask groups, which set the pace,
-    // waited 2 us per chunk for the codes and spent 1 us on them.)
-    const int nunits = n_end / ntpu;
-    auto expand_x = [&](int u) {
-      mbar_wait(&bars[B_X_RAW], (uint32_t)u & 1u, a.status);
-      const int r = ew * 32 + lane;
-      if (r < Q) x_row_to_half(smem + OFF_XRAW, smem + OFF_X + (u & 1) * X_BYTES, r);
-      fence_async_smem();
-      __syncwarp();
-      if (lane < 2) mbar_arrive(&bars[lane == 0 ? B_X_FULL + (u & 1) : B_RAW_FREE]);
-    };
-    expand_x(0);
-    if (nunits > 1) expand_x(1);
     Tile t = decode_unit((int)blockIdx.x, d, TM);
 #pragma unroll 1
     for (int n = 0; n < n_end; ++n, next_tile(t, d, a.w, TM, ntpu)) {
@@ -459,18 +460,11 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
       const float4* gsx = reinterpret_cast<const float4*>(smem + OFF_TOK + t3 * TOK_BYTES + TOK_COLS) + ch * 8;
       const float4* gsh = gsx + 16;
       const float4* gco = gsx + 32;
-      if (t.it == 0 && n > 0) {
-        // every warp is through with the chunk before (its MMAs have completed, and no one reads its rows any
-        // more): its x buffer takes the next chunk
-        const int u = ntpu == 1 ? n : n >> 1;
-        if (u + 1 < nunits) {
-          named_bar_sync(3, kEpiWarps * 32);
-          expand_x(u + 1);
-        }
+      // three lanes wait side by side: the accumulators, the x rows (skip term), the scalar pack (cs)
+      if (ew == 0 && lane < 3) {   // one warp polls, the others wait at a hardware barrier
+        const int bi = lane == 0 ? B_ACC + s2 : lane == 1 ? B_X_FULL + xs : B_TOK_FULL + t3;
+        mbar_wait(&bars[bi], lane == 2 ? ph4 : lane == 1 ? x_phase(n, ntpu) : ph2, a.status);
       }
-      // two lanes wait side by side: the accumulators, the scalar pack (cs)
-      if (ew == 0 && lane < 2)   // one warp polls, the others wait at a hardware barrier
-        mbar_wait(&bars[lane == 0 ? B_ACC + s2 : B_TOK_FULL + t3], lane == 0 ? ph2 : ph4, a.status);
       named_bar_sync(3, kEpiWarps * 32);
       tc_fence_after();
       const bool ok = er < TM;
@@ -533,8 +527,9 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
           if (pc == 3) tc_fence_before();
           fence_async_smem();
           __syncwarp();
-          if (pc == 3 && lane < 2) {
-            mbar_arrive(&bars[lane == 0 ? B_ACC_FREE + s2 : B_TOK_FREE + t3]);
+          if (pc == 3 && lane < 3) {
+            if (lane < 2 || t.it + 1 == ntpu)
+              mbar_arrive(&bars[lane == 0 ? B_ACC_FREE + s2 : lane == 1 ? B_TOK_FREE + t3 : B_X_FREE + xs]);
           } else if (lane == 3 && q * 32 < TM) {
             tma_store_3d(&tm_y, ystage, ch * 32 + (YT != 0 ? 0 : (pc >> 1) * 16), t.h,
                          (int)(t.tok0 + t.it * TM + q * 32));
@@ -578,8 +573,8 @@ ssdi8_status_t launch_chunk_scan_f16(const Dims& d, const int8_t* xq, const int8
   {
     uint64_t dims[3] = {(uint64_t)d.P, (uint64_t)d.H, T};
     uint64_t str[2] = {(uint64_t)d.P, (uint64_t)d.H * d.P};
-    uint32_t box[3] = {64, 1, (uint32_t)TM};   // int8 codes, plain rows of 64 bytes
-    if (!encode_tensor_map(&tm_x, xq, 1, 3, dims, str, box, 0)) return SSDI8_ERR_CUDA;
+    uint32_t box[3] = {64, 1, (uint32_t)TM};   // int8 codes
+    if (!encode_tensor_map(&tm_x, xq, 1, 3, dims, str, box, 64)) return SSDI8_ERR_CUDA;
   }
   {
     uint64_t dims[2] = {(uint64_t)d.Q, (uint64_t)d.b * d.c * d.G * d.Q};
