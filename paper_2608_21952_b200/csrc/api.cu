@@ -163,15 +163,31 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
   if ((ph & SSDI8_PHASE_CUMSUM) && (s = launch_cumsum(d, a->dt, a->A, pack, gamma, a->tap_cs, st, a->dt_bias,
                                                      (flags & SSDI8_FLAG_DT_SOFTPLUS) != 0, to_clear)) != SSDI8_OK)
     return s;
-  // ChunkBMM depends on neither ChunkCumsum nor the state kernel and is needed by ChunkScan only.  When the
-  // fused state kernel runs in this call, ChunkBMM is launched after it and works beside its last wave.
+  // ChunkBMM depends on neither ChunkCumsum nor the state kernels and is needed by ChunkScan only.  When both
+  // state modules run in this call, ChunkBMM is launched after the first state kernel and works beside it.
   const bool fused_state = (ph & SSDI8_PHASE_CHUNK_STATE) && (ph & SSDI8_PHASE_STATE_PASSING);
   const bool bmm_late = (ph & SSDI8_PHASE_BMM) && fused_state;
+  // Few sequences with several chunks: the fused kernel walks a (batch, head)'s chunks one after the other, about 1.9 us
+  // each however few CTAs there are, while ChunkState takes all chunks at once (states through L2) and StatePassing
+  // is a short elementwise pass.  Algorithm 2 with the fused kernel / with the two, us: 1 x 512 tokens x 4
+  // heads 23 / 19, 2048 x 24 40 / 35, 8192 x 24 90 / 60, 8192 x 8 (N 64, chunks of 64) 198 / 59, 4 x 2048 x 24
+  // 57 / 56; but 2 x 2048 x 80 72 / 76, 3 x 1408 x 50 60 / 63, and with two chunks 24 / 25.
+  const int sms = fused_state ? sm_count() : 0;
+  const bool split_state = fused_state && !i8s && d.c >= 4 && (i64)d.b * d.H * 4 <= (i64)3 * sms;
   if ((ph & SSDI8_PHASE_BMM) && !bmm_late &&
       (s = launch_bmm(d, a->Cq, a->Bq, a->s_C, a->s_B, a->s_cb, cbq, a->tap_acc_cb, nullptr, a->status, st)) !=
           SSDI8_OK)
     return s;
-  if ((ph & SSDI8_PHASE_CHUNK_STATE) && (ph & SSDI8_PHASE_STATE_PASSING)) {
+  if (split_state) {
+    if ((s = launch_chunk_state(d, a->xq, a->Bq, a->s_x, a->s_xs, a->s_B, pack, loc, a->tap_Xsq, a->tap_acc_st, a->status,
+                                st)) != SSDI8_OK)
+      return s;
+    if (bmm_late && (s = launch_bmm(d, a->Cq, a->Bq, a->s_C, a->s_B, a->s_cb, cbq, a->tap_acc_cb, nullptr, a->status,
+                                    st, true)) != SSDI8_OK)
+      return s;
+    if ((s = launch_state_passing(d, loc, gamma, a->init_state, a->s_h, a->tap_prev, a->final_state, hq, st)) != SSDI8_OK)
+      return s;
+  } else if (fused_state) {
     // both modules: the fused chunk-sequential kernel (the fp32 chunk-local states stay on chip)
     if ((s = launch_chunk_state_passing(d, a->xq, a->Bq, a->s_x, a->s_xs, a->s_B, a->s_h, pack, gamma,
                                         a->init_state, hq, a->final_state, a->tap_loc, a->tap_prev,

@@ -8,6 +8,8 @@
 // as they are and the MMA reads them through MN-major descriptors (no transposes anywhere).
 // The accumulator is held with the state index n on the TMEM lanes, so that each warp store
 // of the epilogue writes 32 consecutive n of one p: full 128-byte lines of loc[p][n].
+// The forward pass takes this kernel where there are too few (batch, head) pairs to fill the device with
+// chunk-sequential ones (see fwd_phases).
 #include "kernels.h"
 #include "sm100.cuh"
 
@@ -25,8 +27,8 @@ struct StateArgs {
 constexpr int kThreads = 256;
 constexpr uint32_t OFF_B = 0;        // [Q][N]  Bq rows (token-major)
 constexpr uint32_t OFF_X = 32768;    // [Q][64] xq rows -> Xs_q in place
-constexpr uint32_t OFF_F = 49152;    // lut[256], bars, tmem slot
-constexpr uint32_t SMEM_BYTES = OFF_F + 256 * 4 + 64;
+constexpr uint32_t OFF_F = 49152;    // lut[256], s_x / s_xs [64], bars, tmem slot
+constexpr uint32_t SMEM_BYTES = OFF_F + 256 * 4 + 64 * 4 + 64;
 
 __global__ void __launch_bounds__(kThreads, 3)
 chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__ CUtensorMap tm_x,
@@ -43,7 +45,8 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
   uint8_t* sB = smem + OFF_B;
   uint8_t* sX = smem + OFF_X;
   float* lut = reinterpret_cast<float*>(smem + OFF_F);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(lut + 256);  // [0] operands landed, [1] MMA done
+  float* rxs = lut + 256;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(rxs + 64);  // [0] operands landed, [1] MMA done
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
 
   if (tid == 0) {
@@ -53,12 +56,14 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
     tma_prefetch_desc(&tm_B);
     tma_prefetch_desc(&tm_x);
   }
-  pdl_launch_dependents();
   if (warp == 1) tmem_alloc(tmem_slot, 64);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // (the wait ahead of the trigger: ChunkBMM, launched next, reads and writes global memory without waiting for this
+  // kernel, so it must not be scheduled before this kernel's predecessors have completed)
   pdl_wait();
+  pdl_launch_dependents();
   if (tid == 0) {
     mbar_expect_tx(&bars[0], (uint32_t)(Q * 64 + Q * N));
     for (int i0 = 0; i0 < Q; i0 += TQ) {
@@ -67,37 +72,58 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
     }
   }
   if (tid < Q) lut[tid] = a.pack[((((i64)b * d.H + h) * d.c + k) * kPackRows + PACK_LUT) * Q + tid];
+  if (tid >= kThreads - 64) {   // one division per channel (each thread's own sixteen were a third of the kernel's instructions)
+    const int p = tid - (kThreads - 64);
+    rxs[p] = __fdiv_rn(a.s_x[h * P + p], a.s_xs[h * P + p]);
+  }
+  __syncthreads();
   // per-column factors of this thread's 16 channels (16-byte chunk c of every row it visits)
   const int c = tid & 3;
   float rx[16];
 #pragma unroll
-  for (int e = 0; e < 16; ++e) {
-    const int hp = h * P + c * 16 + e;
-    rx[e] = __fdiv_rn(a.s_x[hp], a.s_xs[hp]);
+  for (int e = 0; e < 16; e += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(rxs + c * 16 + e);
+    rx[e] = v.x; rx[e + 1] = v.y; rx[e + 2] = v.z; rx[e + 3] = v.w;
   }
-  __syncthreads();
+  // rows that re-quantise to zero, by the bound of the fused kernel (chunk_state_pass.cu): stored as zeros
+  // without the arithmetic, and a 32-token slab of such rows issues no MMA
+  float rxm = 0.f;
+#pragma unroll
+  for (int e = 0; e < 16; ++e) rxm = fmaxf(rxm, fabsf(rx[e]));
+  rxm = fmaxf(rxm, __shfl_xor_sync(0xffffffffu, rxm, 1));
+  rxm = fmaxf(rxm, __shfl_xor_sync(0xffffffffu, rxm, 2));
+  const float b127 = __fmul_rn(127.0f, rxm);
+  uint32_t live = 0;   // slabs with a row that does not (in the issuing warp)
+  if (warp == 0) {
+    for (int sl = 0; sl < Q / 32; ++sl)
+      if (__any_sync(0xffffffffu, !(__fmul_rn(b127, fabsf(lut[sl * 32 + lane])) < 0.5f))) live |= 1u << sl;
+    if (live == 0) live = 1u;
+  }
   mbar_wait(&bars[0], 0, a.status);
 
   // ---- X_scaled, re-quantised in place (thread: chunk c of rows tid/4, tid/4 + 64, ...)
   for (int i = tid >> 2; i < Q; i += kThreads / 4) {
     uint4* ptr = reinterpret_cast<uint4*>(sX + swz_off((uint32_t)i, (uint32_t)c, 64));
+    const float l = lut[i];
+    if (__fmul_rn(b127, fabsf(l)) < 0.5f) {
+      *ptr = make_uint4(0u, 0u, 0u, 0u);
+      if (a.tap_Xsq) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = make_uint4(0u, 0u, 0u, 0u);
+      continue;
+    }
     const uint4 w4 = *ptr;
     const uint32_t ww[4] = {w4.x ^ 0x80808080u, w4.y ^ 0x80808080u, w4.z ^ 0x80808080u, w4.w ^ 0x80808080u};
-    const float l = lut[i];
-    {
-      uint32_t o[4];
+    uint32_t o[4];
 #pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        uint32_t q4[4];
+    for (int w = 0; w < 4; ++w) {
+      uint32_t q4[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          q4[e] = rne_clamp_bits(__fmul_rn(__fmul_rn(s8_to_f32(ww[w], e), rx[w * 4 + e]), l));
-        o[w] = pack4_bits(q4[0], q4[1], q4[2], q4[3]);
-      }
-      const uint4 v = make_uint4(o[0], o[1], o[2], o[3]);
-      *ptr = v;
-      if (a.tap_Xsq) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = v;
+      for (int e = 0; e < 4; ++e)
+        q4[e] = rne_clamp_bits(__fmul_rn(__fmul_rn(s8_to_f32(ww[w], e), rx[w * 4 + e]), l));
+      o[w] = pack4_bits(q4[0], q4[1], q4[2], q4[3]);
     }
+    const uint4 v = make_uint4(o[0], o[1], o[2], o[3]);
+    *ptr = v;
+    if (a.tap_Xsq) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = v;
   }
   fence_async_smem();
   __syncthreads();
@@ -107,9 +133,13 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
   if (tid == 0) {
     tc_fence_after();
     const uint32_t idesc = idesc_s8(N, 64, 1, 1);
-    for (int s = 0; s < Q / 32; ++s)
+    uint32_t first = 0;
+    for (int s = 0; s < Q / 32; ++s) {
+      if (!((live >> s) & 1u)) continue;
       mma_s8_ss(tmem, tile_desc(smem_u32(sB) + 32 * s * N, (uint32_t)N),
-                tile_desc(smem_u32(sX) + 32 * s * 64, 64), idesc, s > 0);
+                tile_desc(smem_u32(sX) + 32 * s * 64, 64), idesc, first);
+      first = 1;
+    }
     mma_commit(&bars[1]);
   }
   __syncwarp();

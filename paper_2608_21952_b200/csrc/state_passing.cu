@@ -10,6 +10,9 @@ namespace {
 
 constexpr int SP_T = 256;
 
+// PREV: the entering states are written (they may go over loc, so a chunk's load cannot be moved ahead of the store
+// of the one before); without them the loads of eight chunks are in flight at once.
+template <bool PREV>
 __global__ void __launch_bounds__(SP_T) state_passing_kernel(
     const float4* loc /* may alias prev: no __restrict__ */, const float* __restrict__ gamma, const float4* __restrict__ init,
     const float* __restrict__ s_h, float4* prev, float4* __restrict__ final_state,
@@ -30,18 +33,31 @@ __global__ void __launch_bounds__(SP_T) state_passing_kernel(
   const float* gm = gamma + ((i64)b * d.H + h) * d.c;
   const i64 stride = per_b;                              // chunk stride in float4
   i64 o = (i64)b * d.c * per_b + r;
-  for (int k = 0; k < d.c; ++k, o += stride) {
-    const float4 l = loc[o];  // read before prev[o] is written: prev may alias loc
-    const float g = gm[k];
+  auto step = [&](const float4& l, float g) {
     if (hq)
       hq[o] = pack4(rne_clamp(__fmul_rn(S.x, inv_h)), rne_clamp(__fmul_rn(S.y, inv_h)),
                     rne_clamp(__fmul_rn(S.z, inv_h)), rne_clamp(__fmul_rn(S.w, inv_h)));
-    if (prev) prev[o] = S;
+    if (PREV) prev[o] = S;
     S.x = __fmaf_rn(g, S.x, l.x);
     S.y = __fmaf_rn(g, S.y, l.y);
     S.z = __fmaf_rn(g, S.z, l.z);
     S.w = __fmaf_rn(g, S.w, l.w);
+    o += stride;
+  };
+  constexpr int K = PREV ? 1 : 8;
+  int k = 0;
+  for (; k + K <= d.c; k += K) {
+    float4 l[K];
+    float g[K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      l[j] = loc[o + j * stride];  // (read before prev[o] is written: prev may alias loc)
+      g[j] = gm[k + j];
+    }
+#pragma unroll
+    for (int j = 0; j < K; ++j) step(l[j], g[j]);
   }
+  for (; k < d.c; ++k) step(loc[o], gm[k]);
   if (final_state) final_state[idx] = S;
 }
 
@@ -52,7 +68,7 @@ ssdi8_status_t launch_state_passing(const Dims& d, const float* loc, const float
                                     float* final_state, int8_t* hq, cudaStream_t st) {
   const i64 n = (i64)d.b * d.H * d.P * (d.N / 4);
   unsigned grid = (unsigned)((n + SP_T - 1) / SP_T);
-  return launch_configured(state_passing_kernel, dim3(grid), dim3(SP_T), 0, -1, false, st,
+  return launch_configured(prev ? state_passing_kernel<true> : state_passing_kernel<false>, dim3(grid), dim3(SP_T), 0, -1, false, st,
                            reinterpret_cast<const float4*>(loc), gamma, reinterpret_cast<const float4*>(init), s_h,
                            reinterpret_cast<float4*>(prev), reinterpret_cast<float4*>(final_state),
                            reinterpret_cast<uint32_t*>(hq), d);
