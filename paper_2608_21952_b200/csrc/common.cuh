@@ -101,54 +101,51 @@ __device__ __forceinline__ uint32_t pack4_bits(uint32_t a, uint32_t b, uint32_t 
   return __byte_perm(__byte_perm(a, b, 0x0040u), __byte_perm(c, d, 0x0040u), 0x5410u);
 }
 
-// Eq. 1 codes without a division per element.  With rcp = frcp_rn(alpha), t = fmul(v, rcp) and
-// d = fdiv_rn(v, alpha) differ by at most 1.5 * 2^-23 |v / alpha| < 2.3e-5 wherever the code is not
-// saturated, so rne(t) = rne(d) unless t lies that close to a rounding boundary k + 1/2 (ties
-// included).  Those elements (about one in 10^4) take the division, and so does every element of a
-// step size whose reciprocal may not be a normal number, so the code always equals
-// rne(fdiv_rn(v, alpha)) saturated.  quant_code_bits returns bits whose low byte is the code.
-struct QuantStep {
-  float alpha, rcp, thr;
+// Eq. 1 codes, rne(fdiv_rn(v, alpha)) saturated, four as one word, without a division and without a branch: with y =
+// frcp_rn(alpha), q = fmul(v, y) is within two units in the last place of v / alpha, its residual fmaf(-q, alpha, v) is
+// exact, and fmaf(residual, y, q) is the quotient up to 2^-22 unit before it is rounded (Markstein's scheme, IBM J. Res.
+// Dev. 34, 1990).  It can differ from fdiv_rn only where v / alpha lies that close to the midpoint of two binary32
+// numbers, and the code then only where one of the two is k + 1/2: an equation M A - V 2^s = j with M that midpoint's
+// 25 bits, A and V the significands and |j| < 8, which has one A for each (k, j, s).  All its solutions up to |j| =
+// 200 round as the division does (35 696 pairs; the nearest are in the tests).  |v| is limited to 127.25 alpha first,
+// so the code saturates by itself and nothing overflows; quotients below 1/2, whose residuals may underflow, round to 0
+// either way.  Step sizes outside [1e-30, 1e30] (`usable` false) take the divisions.
+// (Products with y and a division where one came close to a rounding boundary cost 56 instructions per 128 codes, and
+// 16-bit inputs under a step size of absmax / 127 are ties in one code of 500, so that a quarter of the warps divided.
+// Entry quantiser, bf16, 8960 x 5376: 33.5 -> 22.0 us (6.6 TB/s); 16384 x 5376: 58.9 -> 45.0 us.  A second correction
+// step, which needs no such enumeration, with a loop that waited for `usable`: 35.3 and 64.5 us.)
+struct Step4 {
+  float2 y01, y23, n01, n23;   // reciprocals and negatives of four step sizes
+  float4 lim;                  // 127.25 of them
+  bool usable;
 };
-__device__ __forceinline__ QuantStep quant_step(float alpha) {
-  QuantStep s;
-  s.alpha = alpha;
-  s.rcp = __frcp_rn(alpha);
-  s.thr = (alpha >= 1e-30f && alpha <= 1e30f) ? 0.49994f : -1.0f;
+__device__ __forceinline__ Step4 step4(const float4& a) {
+  auto normal = [](float x) { return x >= 1e-30f && x <= 1e30f; };
+  Step4 s;
+  s.y01 = make_float2(__frcp_rn(a.x), __frcp_rn(a.y));
+  s.y23 = make_float2(__frcp_rn(a.z), __frcp_rn(a.w));
+  s.n01 = make_float2(-a.x, -a.y);
+  s.n23 = make_float2(-a.z, -a.w);
+  s.lim = make_float4(__fmul_rn(a.x, 127.25f), __fmul_rn(a.y, 127.25f), __fmul_rn(a.z, 127.25f), __fmul_rn(a.w, 127.25f));
+  s.usable = normal(a.x) && normal(a.y) && normal(a.z) && normal(a.w);
   return s;
 }
-__device__ __forceinline__ uint32_t quant_code_bits(float v, const QuantStep& s) {
-  const float tc = fminf(fmaxf(__fmul_rn(v, s.rcp), -127.0f), 127.0f);
-  const float m = __fadd_rn(tc, kMagicOut);
-  const float e = __fsub_rn(tc, __fsub_rn(m, kMagicOut));
-  if (fabsf(e) > s.thr) return rne_clamp_bits(__fdiv_rn(v, s.alpha));
-  return __float_as_uint(m);
+__device__ __forceinline__ uint32_t code4(const float4& v, const Step4& s) {
+  float2 v01, v23;   // min(|v|, lim) with the sign of v
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(v01.x) : "f"(v.x), "f"(s.lim.x));
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(v01.y) : "f"(v.y), "f"(s.lim.y));
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(v23.x) : "f"(v.z), "f"(s.lim.z));
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(v23.y) : "f"(v.w), "f"(s.lim.w));
+  float2 q01 = __fmul2_rn(v01, s.y01), q23 = __fmul2_rn(v23, s.y23);
+  q01 = __ffma2_rn(__ffma2_rn(q01, s.n01, v01), s.y01, q01);
+  q23 = __ffma2_rn(__ffma2_rn(q23, s.n23, v23), s.y23, q23);
+  const float2 mg = make_float2(kMagicOut, kMagicOut);
+  const float2 m01 = __fadd2_rn(q01, mg), m23 = __fadd2_rn(q23, mg);
+  return pack4_bits(__float_as_uint(m01.x), __float_as_uint(m01.y), __float_as_uint(m23.x), __float_as_uint(m23.y));
 }
-// Four codes as one word.  The common path is packed arithmetic and one branch for the four elements:
-// products, clamp (min(|t|, 127) with the sign of t), the magic addition, the rounded value and the distance
-// of the product from it; only a word with an element near a rounding boundary (or an abnormal step size)
-// goes through the divisions, element by element.
-__device__ __forceinline__ uint32_t quant_code4(const float4& v, const QuantStep& a, const QuantStep& b,
-                                                const QuantStep& c, const QuantStep& d) {
-  const float2 t01 = __fmul2_rn(make_float2(v.x, v.y), make_float2(a.rcp, b.rcp));
-  const float2 t23 = __fmul2_rn(make_float2(v.z, v.w), make_float2(c.rcp, d.rcp));
-  float2 c01, c23;
-  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(c01.x) : "f"(t01.x), "f"(127.0f));
-  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(c01.y) : "f"(t01.y), "f"(127.0f));
-  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(c23.x) : "f"(t23.x), "f"(127.0f));
-  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(c23.y) : "f"(t23.y), "f"(127.0f));
-  const float2 mg = make_float2(kMagicOut, kMagicOut), ng = make_float2(-kMagicOut, -kMagicOut);
-  const float2 m01 = __fadd2_rn(c01, mg), m23 = __fadd2_rn(c23, mg);
-  const float2 m1 = make_float2(-1.0f, -1.0f);   // e = c - (m - magic): both differences are exact
-  const float2 e01 = __ffma2_rn(__fadd2_rn(m01, ng), m1, c01), e23 = __ffma2_rn(__fadd2_rn(m23, ng), m1, c23);
-  uint32_t b0 = __float_as_uint(m01.x), b1 = __float_as_uint(m01.y), b2 = __float_as_uint(m23.x), b3 = __float_as_uint(m23.y);
-  if (fabsf(e01.x) > a.thr || fabsf(e01.y) > b.thr || fabsf(e23.x) > c.thr || fabsf(e23.y) > d.thr) {
-    if (fabsf(e01.x) > a.thr) b0 = rne_clamp_bits(__fdiv_rn(v.x, a.alpha));
-    if (fabsf(e01.y) > b.thr) b1 = rne_clamp_bits(__fdiv_rn(v.y, b.alpha));
-    if (fabsf(e23.x) > c.thr) b2 = rne_clamp_bits(__fdiv_rn(v.z, c.alpha));
-    if (fabsf(e23.y) > d.thr) b3 = rne_clamp_bits(__fdiv_rn(v.w, d.alpha));
-  }
-  return pack4_bits(b0, b1, b2, b3);
+__device__ __forceinline__ uint32_t code4_by_division(const float4& v, const float4& a) {
+  return pack4_bits(rne_clamp_bits(__fdiv_rn(v.x, a.x)), rne_clamp_bits(__fdiv_rn(v.y, a.y)),
+                    rne_clamp_bits(__fdiv_rn(v.z, a.z)), rne_clamp_bits(__fdiv_rn(v.w, a.w)));
 }
 
 __device__ __forceinline__ uint32_t pack4(int a, int b, int c, int d) {

@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(128) quant_ch_fastest(const float4* __restrict
     s = make_float4(s.x == 0.f ? 1.f : s.x, s.y == 0.f ? 1.f : s.y, s.z == 0.f ? 1.f : s.z, s.w == 0.f ? 1.f : s.w);
     if (blockIdx.y == 0) scale[q] = s;
   }
-  const QuantStep sx = quant_step(s.x), sy = quant_step(s.y), sz = quant_step(s.z), sw = quant_step(s.w);
+  const Step4 st = step4(s);
   const i64 r0 = (i64)blockIdx.y * rows_per_block;
   const i64 r1 = r0 + rows_per_block < R ? r0 + rows_per_block : R;
   i64 r = r0;
@@ -37,14 +37,15 @@ __global__ void __launch_bounds__(128) quant_ch_fastest(const float4* __restrict
     float4 v[QROWS];
 #pragma unroll
     for (int u = 0; u < QROWS; ++u) v[u] = __ldcs(in + (r + u) * ch4 + q);
+    if (st.usable) {
 #pragma unroll
-    for (int u = 0; u < QROWS; ++u)
-      __stcs(out + (r + u) * ch4 + q, quant_code4(v[u], sx, sy, sz, sw));
+      for (int u = 0; u < QROWS; ++u) __stcs(out + (r + u) * ch4 + q, code4(v[u], st));
+    } else {
+#pragma unroll 1
+      for (int u = 0; u < QROWS; ++u) __stcs(out + (r + u) * ch4 + q, code4_by_division(in[(r + u) * ch4 + q], s));
+    }
   }
-  for (; r < r1; ++r) {
-    const float4 v = __ldcs(in + r * ch4 + q);
-    __stcs(out + r * ch4 + q, quant_code4(v, sx, sy, sz, sw));
-  }
+  for (; r < r1; ++r) __stcs(out + r * ch4 + q, code4_by_division(__ldcs(in + r * ch4 + q), s));
 }
 
 // ---- the layer's three static quantisers (x per channel; B and C per group) as one launch.  Every
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(128, 8) quant_jobs(const QuantJobs a) {
     const float g = __ldg(j.scale + ((q * 4) >> j.shift));   // 4 consecutive channels share a group
     s = make_float4(g, g, g, g);
   }
-  const QuantStep sx = quant_step(s.x), sy = quant_step(s.y), sz = quant_step(s.z), sw = quant_step(s.w);
+  const Step4 st = step4(s);
   const i64 r0 = (i64)by * j.rows + tr;
   const i64 r1 = (i64)(by + 1) * j.rows < a.R ? (i64)(by + 1) * j.rows : a.R;
   if (r0 >= r1) return;
@@ -109,10 +110,15 @@ __global__ void __launch_bounds__(128, 8) quant_jobs(const QuantJobs a) {
     float4 v[QROWS];
 #pragma unroll
     for (int u = 0; u < QROWS; ++u) v[u] = __ldcs(in + (e + u * stride));
+    if (st.usable) {
 #pragma unroll
-    for (int u = 0; u < QROWS; ++u) out[e + u * stride] = quant_code4(v[u], sx, sy, sz, sw);
+      for (int u = 0; u < QROWS; ++u) out[e + u * stride] = code4(v[u], st);
+    } else {
+#pragma unroll 1
+      for (int u = 0; u < QROWS; ++u) out[e + u * stride] = code4_by_division(in[e + u * stride], s);
+    }
   }
-  for (; left > 0; --left, e += stride) out[e] = quant_code4(__ldcs(in + e), sx, sy, sz, sw);
+  for (; left > 0; --left, e += stride) out[e] = code4_by_division(__ldcs(in + e), s);
 }
 
 // ---- quantise, I % 4 == 0: 4 consecutive elements share a channel
@@ -134,8 +140,9 @@ __global__ void __launch_bounds__(QT) quant_inner(const float4* __restrict__ in,
         al = 1.f;
         if (e < I4 * Ch) scale[ch] = al;   // the first row
       }
-      const QuantStep s = quant_step(al);
-      out[e] = quant_code4(v, s, s, s, s);
+      const float4 a4 = make_float4(al, al, al, al);
+      const Step4 st = step4(a4);
+      out[e] = st.usable ? code4(v, st) : code4_by_division(v, a4);
     }
   }
 }

@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(128) quant_entry_kernel(const typename Vec4<T>
     s = make_float4(a, a, a, a);
     out = Cq; ow4 = GN / 4; oq = (col - D - GN) / 4;
   }
-  const QuantStep sx = quant_step(s.x), sy = quant_step(s.y), sz = quant_step(s.z), sw = quant_step(s.w);
+  const Step4 st = step4(s);
   const i64 r0 = (i64)blockIdx.y * rows_per_block;
   const i64 r1 = r0 + rows_per_block < T_ ? r0 + rows_per_block : T_;
   i64 r = r0;
@@ -74,16 +74,15 @@ __global__ void __launch_bounds__(128) quant_entry_kernel(const typename Vec4<T>
     typename Vec4<T>::raw v[EROWS];
 #pragma unroll
     for (int u = 0; u < EROWS; ++u) v[u] = __ldcs(in + (r + u) * W4 + q);
+    if (st.usable) {
 #pragma unroll
-    for (int u = 0; u < EROWS; ++u) {
-      const float4 f = Vec4<T>::cvt(v[u]);
-      __stcs(out + (r + u) * ow4 + oq, quant_code4(f, sx, sy, sz, sw));
+      for (int u = 0; u < EROWS; ++u) out[(r + u) * ow4 + oq] = code4(Vec4<T>::cvt(v[u]), st);
+    } else {
+#pragma unroll 1
+      for (int u = 0; u < EROWS; ++u) out[(r + u) * ow4 + oq] = code4_by_division(Vec4<T>::cvt(in[(r + u) * W4 + q]), s);
     }
   }
-  for (; r < r1; ++r) {
-    const float4 f = Vec4<T>::cvt(__ldcs(in + r * W4 + q));
-    __stcs(out + r * ow4 + oq, quant_code4(f, sx, sy, sz, sw));
-  }
+  for (; r < r1; ++r) out[r * ow4 + oq] = code4_by_division(Vec4<T>::cvt(__ldcs(in + r * W4 + q)), s);
 }
 
 }  // namespace

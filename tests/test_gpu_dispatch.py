@@ -148,3 +148,62 @@ def test_state_kernels_on_both_sides_of_the_dispatch(cfg, fast):
         t["A"] *= np.float32(60.0)
 
     check_fwd(cfg, init=inputs.make_init_state(cfg, 0.5), mutate=decay if fast else None)
+
+
+def _near_ties():
+    # Pairs (v, alpha) whose quotient lies within 8 / alpha's significand of the midpoint between k + 1/2 and a neighbour
+    # in binary32: where a quotient formed from a reciprocal could fall on the other side.
+    v, a = [], []
+    for k in range(128):
+        h = np.float32(k + 0.5)
+        for nb in (np.nextafter(h, np.float32(np.inf)), np.nextafter(h, np.float32(0))):
+            mid = (float(h) + float(nb)) / 2
+            M = int(np.ldexp(np.frexp(mid)[0], 25))
+            for s in (24, 25):
+                for j in range(-8, 9):
+                    A = j * pow(M, -1, 1 << s) % (1 << s)
+                    V = (M * A - j) >> s
+                    if 1 << 23 <= A < 1 << 24 and 1 << 23 <= V < 1 << 24:
+                        a.append(A)
+                        v.append(np.ldexp(V, int(np.rint(np.log2(mid * A / V)))))
+    return np.float32(v), np.float32(a)
+
+
+@pytest.mark.parametrize("dtype", ["float32", "float16", "bfloat16", "near ties"])
+def test_entry_quantiser_codes_are_those_of_the_division(dtype):
+    # Every finite 16-bit pattern (and the same values as binary32, with their neighbours) under step sizes where quotients
+    # are ties, near-ties, saturated, overflowing or underflowing, and under step sizes that take the divisions.  The
+    # reference is the definition, rne(fdiv(v, alpha)) saturated: numpy's binary32 division is correctly rounded.
+    import torch
+    from paper_2608_21952_b200 import binding as bd
+    pat = np.arange(65536, dtype=np.uint16)
+    if dtype == "bfloat16":
+        vals = (pat.astype(np.uint32) << 16).view(np.float32)
+    else:
+        vals = pat.view(np.float16).astype(np.float32)
+    vals = vals[np.isfinite(vals)]
+    if dtype == "float32":
+        vals = np.concatenate([vals, np.nextafter(vals, np.float32(np.inf)), np.nextafter(vals, np.float32(-np.inf))])
+    vals = vals[np.isfinite(vals)]
+    rng = np.random.default_rng(9)
+    alpha = np.concatenate([np.float32([1.0, 0.5, 2.0 ** -5, 3.0, 1.0 / 127, 1.0 / 3, 0.1, 1e-30, 9e-31, 1e30, 1.1e30, 1e-38, 1e-42,
+                                        1e-20, 5e4, 2.0 ** -9 / 127]),
+                            np.abs(rng.choice(vals[vals != 0], 32)).astype(np.float32) / np.float32(127),
+                            np.exp(rng.uniform(-9, 3, 80)).astype(np.float32)]).astype(np.float32)
+    if dtype == "near ties":
+        dtype, (vals, alpha) = "float32", _near_ties()
+        n = alpha.size // 16 * 16
+        vals, alpha = vals[:n], alpha[:n]
+    D, T = alpha.size, (vals.size + 7) // 8 * 8 + 3          # a ragged last round
+    col = np.resize(vals, T)
+    x = np.repeat(col[:, None], D, axis=1)
+    t = torch.from_numpy(np.concatenate([x, np.zeros((T, 32), np.float32)], axis=1)).to(getattr(torch, dtype)).cuda()
+    s_x = torch.from_numpy(alpha).cuda()
+    one = torch.ones(1, device="cuda")
+    out = [torch.empty(T, w, dtype=torch.int8, device="cuda") for w in (D, 16, 16)]
+    bd.ssdi8_quantize_entry(t, T, D, 1, 16, s_x, one, one, *out)
+    with np.errstate(all="ignore"):
+        want = np.clip(np.rint(x / alpha), -127, 127).astype(np.int8)
+    got = out[0].cpu().numpy()
+    bad = np.argwhere(got != want)
+    assert bad.size == 0, (len(bad), col[bad[0][0]], alpha[bad[0][1]], got[tuple(bad[0])], want[tuple(bad[0])])
