@@ -10,11 +10,9 @@
 // 32 channels p; the state itself is kept in tensor memory beside the accumulator (64 more columns,
 // read and written 8 columns at a time), which leaves the threads with few registers so that three CTAs
 // fit an SM: the kernel is a chain of short dependent steps per chunk, and what fills an SM is other
-// CTAs' chains.  The xq tiles arrive by TMA double-buffered across chunks, the Bq tile of a chunk is
-// single-buffered (requested when the MMAs of the chunk before have finished, needed only when the
-// accumulator is free again); each re-quantisation
-// warp owns whole 32-token slabs and issues their MMAs itself (the accumulator is opened by the warp
-// that owns slab 0, the others order their MMAs after it through an mbarrier); hq leaves through
+// CTAs' chains.  Three warps re-quantise the xq rows up to two chunks ahead, a fourth issues the MMAs
+// and requests the tiles by TMA: xq double-buffered across chunks, Bq single-buffered (requested
+// when the MMAs of the chunk before have finished); hq leaves through
 // a shared-memory tile and one TMA store per chunk.  Same arithmetic, operation for operation,
 // as the separate kernels (chunk_state.cu, state_passing.cu).
 // I8S = true selects the paper's own state format (Section 4.2, Eq. 4 and Eq. 7): the state is an
@@ -42,9 +40,10 @@ struct FusedArgs {
   int split;   // parts per (batch, head) of the rest: 2 (halves of 32 channels) or 4 (quarters of 16)
 };
 
-constexpr int kStateThreads = 256;   // warps 0-7: running state, hq, MMA issue, TMA
-constexpr int kQuantThreads = 128;   // warps 8-11: Q(X_scaled) of the next chunk, one chunk ahead
+constexpr int kStateThreads = 256;   // warps 0-7: running state, hq and its TMA stores
+constexpr int kQuantThreads = 128;   // warps 8-10: Q(X_scaled), up to two chunks ahead; warp 11: MMA issue, TMA loads
 constexpr int kThreads = kStateThreads + kQuantThreads;
+constexpr int kRowWarps = 3;
 constexpr uint32_t XSTAGE = 16384;                // xq rows [Q][64] of one chunk
 constexpr uint32_t OFF_X = 0;                     // two stages
 constexpr uint32_t OFF_B = 2 * XSTAGE;            // Bq rows [Q][N] of one chunk (single buffer)
@@ -55,10 +54,13 @@ constexpr uint32_t OFF_BAR = OFF_COL + 768;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 64;     // 76 608 bytes: three CTAs per SM
 constexpr uint32_t kTmemCols = 128;               // accumulator in columns 0..63, running state in 64..127
 
-enum { B_XFULL = 0, B_BFULL = 2, B_OPEN = 3, B_MMA = 4, B_ACC_FREE = 5, B_COUNT = 6 };
+enum { B_XFULL = 0, B_BFULL = 2, B_MMA = 3, B_ACC_FREE = 4, B_COUNT = 5 };
 
 __device__ __forceinline__ void named_bar(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+__device__ __forceinline__ void named_bar_arrive(int id, int nthreads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
 // TAPS: any of the intermediate-tensor taps is requested (tests); the production instance carries no tap code
@@ -78,10 +80,9 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
   }
   const Dims& d = a.d;
   const int Q = d.Q, N = d.N, P = d.P;
-  const int TQ = Q < 128 ? Q : 128;  // rows per TMA box
   const int h = unit % d.H, b = unit / d.H;
   const int g = h / (d.H / d.G);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // (the shuffle: uniform for the compiler)
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + OFF_BAR);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + B_COUNT);
   uint8_t* sHQ = smem + OFF_HQ;
@@ -95,8 +96,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     mbar_init(&bars[B_XFULL], 1);
     mbar_init(&bars[B_XFULL + 1], 1);
     mbar_init(&bars[B_BFULL], 1);
-    mbar_init(&bars[B_OPEN], 1);
-    mbar_init(&bars[B_MMA], Q / 32 < kQuantThreads / 32 ? Q / 32 : kQuantThreads / 32);   // one commit per issuing warp
+    mbar_init(&bars[B_MMA], 1);
     mbar_init(&bars[B_ACC_FREE], kStateThreads / 32);
     fence_mbar_init();
     tma_prefetch_desc(&tm_B);
@@ -125,25 +125,37 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  auto issue_x = [&](int k) {  // thread 0 only: xq rows and LUT_state of chunk k
+  // One warp: the slabs of 32 tokens named by m of the xq rows (with LUT_state of the chunk: a global
+  // load there would sit on the re-quantisation group's critical path) or of the Bq rows of chunk k
+  auto issue_x = [&](int k, uint32_t m) {
     const int s = k & 1;
-    const i64 tok0 = (i64)b * d.L + (i64)k * Q;
-    mbar_expect_tx(&bars[B_XFULL + s], (uint32_t)(Q * 64 + Q * 4));
-    // LUT_state of the chunk arrives with the tile (a global load here would sit on the
-    // re-quantisation group's critical path)
-    bulk_load(smem + OFF_LUT + s * 1024, a.pack + ((unit0 + k) * kPackRows + PACK_LUT) * Q, (uint32_t)(Q * 4),
-              &bars[B_XFULL + s]);
-    for (int i0 = 0; i0 < Q; i0 += TQ)
-      tma_load_3d(smem + OFF_X + s * XSTAGE + i0 * 64, &tm_x, &bars[B_XFULL + s], 0, h, (int)(tok0 + i0));
+    const int tok0 = (int)((i64)b * d.L + (i64)k * Q);
+    if (elect_one()) {
+      mbar_expect_tx(&bars[B_XFULL + s], (uint32_t)(__popc(m) * 32 * 64 + Q * 4));
+      bulk_load(smem + OFF_LUT + s * 1024, a.pack + ((unit0 + k) * kPackRows + PACK_LUT) * Q, (uint32_t)(Q * 4),
+                &bars[B_XFULL + s]);
+#pragma unroll 1
+      for (; m; m &= m - 1) {
+        const int i0 = (__ffs((int)m) - 1) * 32;
+        tma_load_3d(smem + OFF_X + s * XSTAGE + i0 * 64, &tm_x, &bars[B_XFULL + s], 0, h, tok0 + i0);
+      }
+    }
+    __syncwarp();
   };
-  auto issue_B = [&](int k) {  // thread 0 only: Bq rows of chunk k, once the MMAs of chunk k-1 have finished
-    const i64 tok0 = (i64)b * d.L + (i64)k * Q;
-    mbar_expect_tx(&bars[B_BFULL], (uint32_t)(Q * N));
-    for (int i0 = 0; i0 < Q; i0 += TQ)
-      tma_load_3d(smem + OFF_B + i0 * N, &tm_B, &bars[B_BFULL], 0, g, (int)(tok0 + i0));
+  auto issue_B = [&](int k, uint32_t m) {   // once the MMAs of chunk k - 1 have finished
+    const int tok0 = (int)((i64)b * d.L + (i64)k * Q);
+    if (elect_one()) {
+      mbar_expect_tx(&bars[B_BFULL], (uint32_t)(__popc(m) * 32 * N));
+#pragma unroll 1
+      for (; m; m &= m - 1) {
+        const int i0 = (__ffs((int)m) - 1) * 32;
+        tma_load_3d(smem + OFF_B + i0 * N, &tm_B, &bars[B_BFULL], 0, g, tok0 + i0);
+      }
+    }
+    __syncwarp();
   };
 
-  if (tid >= kStateThreads) {
+  if (warp >= kStateThreads / 32) {
     // ------------------------------------------------------------ Q(X_scaled), one chunk ahead of the state warps
     const int qt = tid - kStateThreads;
     constexpr int lq = ncq == 4 ? 2 : ncq == 2 ? 1 : 0;  // log2(chunks per row in this CTA's range)
@@ -165,101 +177,129 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     if (ncq >= 2) rxm = fmaxf(rxm, __shfl_xor_sync(0xffffffffu, rxm, 1));
     if (ncq == 4) rxm = fmaxf(rxm, __shfl_xor_sync(0xffffffffu, rxm, 2));
     const float b127 = __fmul_rn(127.0f, rxm);
+    // Three of the warps share the live rows of a chunk evenly, up to two chunks ahead; the fourth requests the tiles, the
+    // live slabs of them only, and issues the MMAs.  The live slabs are the last ones of a chunk, often two or three: with
+    // whole slabs dealt out by position the warp that had most of them was the time of a chunk, and with all of xq
+    // and Bq loaded (48 KB per chunk and CTA) the loads of three CTAs took 1.4 us.  The row warps only arrive at
+    // the barrier that releases the MMAs, one of two in turn: they are held back by the xq tile of the chunk after next,
+    // which is requested when this chunk's MMAs have finished.
+    // (Batch 8 x 2048 x 80 heads: 48.9 us with slabs dealt out by position, 41.0 this way; 4 x 8192 x 128 151 and 118.)
+    const int qw = warp - kStateThreads / 32, nsl = Q / 32;
+    // live slabs of a chunk from its LUT_state: nsl consecutive tokens per lane, 32 / nsl lanes per slab.  A chunk
+    // without a live slab opens the accumulator with its last one, all rows of it stored as zeros.
+    struct Lut { float4 a, b; };
+    auto lut_of_lane = [&](const float* l) -> Lut {
+      Lut v = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+      if (nsl == 2) {
+        const float2 u = reinterpret_cast<const float2*>(l)[lane];
+        v.a.x = u.x;
+        v.a.y = u.y;
+      } else {
+        v.a = reinterpret_cast<const float4*>(l + lane * nsl)[0];
+        if (nsl == 8) v.b = reinterpret_cast<const float4*>(l + lane * nsl)[1];
+      }
+      return v;
+    };
+    auto live_slabs = [&](const Lut& v) -> uint32_t {
+      auto alive = [&](float l) { return !(__fmul_rn(b127, fabsf(l)) < 0.5f); };
+      const bool any = alive(v.a.x) | alive(v.a.y) | alive(v.a.z) | alive(v.a.w) | alive(v.b.x) | alive(v.b.y) | alive(v.b.z) | alive(v.b.w);
+      const uint32_t bal = __ballot_sync(0xffffffffu, any);
+      const int lps = 32 / nsl;
+      const uint32_t m = __ballot_sync(0xffffffffu, lane < nsl && ((bal >> ((lane * lps) & 31)) & ((1u << lps) - 1u)) != 0);
+      return m ? m : 1u << (nsl - 1);
+    };
+    constexpr int kRowStep = 32 * kRowWarps >> lq;
+    const float* const lut0 = a.pack + (unit0 * kPackRows + PACK_LUT) * Q;   // LUT_state of chunk 0; the next one kPackRows Q floats on
+    const i64 lut_step = (i64)kPackRows * Q;
+    if (qw == kRowWarps) {
+      issue_x(0, (1u << nsl) - 1u);    // (all of the first chunk: its LUT_state would have to come first)
+      issue_B(0, (1u << nsl) - 1u);
+      uint32_t cur = live_slabs(lut_of_lane(lut0)), next = 0;
+      if (d.c > 1) {
+        next = live_slabs(lut_of_lane(lut0 + lut_step));
+        issue_x(1, next);
+      }
+      const uint32_t idesc = idesc_s8(N, 64, 1, 1);
+#pragma unroll 1
+      for (int k = 0; k < d.c; ++k) {
+        Lut v = {};
+        if (k + 2 < d.c) v = lut_of_lane(lut0 + (k + 2) * lut_step);     // (its latency under the waits)
+        named_bar(2 + (k & 1), kQuantThreads);                           // the rows are re-quantised
+        mbar_wait_inline<0>(&bars[B_ACC_FREE], (k & 1) ^ 1, a.status);   // the state warps have read the accumulator of chunk k-1
+        mbar_wait_inline<0>(&bars[B_BFULL], k & 1, a.status);            // the chunk's Bq rows have landed
+        tc_fence_after();
+        const uint32_t sBa = smem_u32(smem + OFF_B), sXa = smem_u32(smem + OFF_X + (k & 1) * XSTAGE);
+        if (elect_one()) {
+#pragma unroll 1
+          for (uint32_t m = cur; m; m &= m - 1) {
+            const int sl = __ffs((int)m) - 1;
+            mma_s8_ss(tmem, tile_desc(sBa + 32 * sl * N, (uint32_t)N), tile_desc(sXa + 32 * sl * 64, 64), idesc, m != cur);
+          }
+          mma_commit(&bars[B_MMA]);
+        }
+        __syncwarp();
+        if (k + 1 < d.c) {
+          mbar_wait_inline<0>(&bars[B_MMA], k & 1, a.status);   // the MMAs of chunk k have read the Bq buffer and its xq stage
+          issue_B(k + 1, next);
+          cur = next;
+          if (k + 2 < d.c) {
+            next = live_slabs(v);
+            issue_x(k + 2, next);
+          }
+        }
+      }
+    } else {
 #pragma unroll 1
     for (int k = 0; k < d.c; ++k) {
       const int s = k & 1;
       uint8_t* sX = smem + OFF_X + s * XSTAGE;
       float* lut = reinterpret_cast<float*>(smem + OFF_LUT) + s * 256;
       const i64 tok0 = (i64)b * d.L + (i64)k * Q;
-      // one warp polls for the tiles; the others wait at a hardware barrier, which costs no issue slots
-      if (qt < 32) mbar_wait_inline<256>(&bars[B_XFULL + s], (k >> 1) & 1, a.status);
-      named_bar(2, kQuantThreads);
-      // a warp owns whole 32-token slabs (slab = one MMA): rows of a slab are split over the lanes,
-      // and the warp's lane 0 issues the slab's MMA as soon as the warp has re-quantised it, so no
-      // warp waits for another.  The accumulator is opened by the MMA of the first live slab
-      // (accumulate = 0); the other issuing threads order their first MMA of the chunk after it
-      // through B_OPEN.  A chunk without a live slab opens with its last slab stored as zeros.
-      const int qw = qt >> 5;
-      const int nsl = Q / 32;
-      uint32_t lm = 0;   // live slabs of the chunk (every warp computes the same mask)
-      for (int sl = 0; sl < nsl; ++sl) {
-        const bool dead = __fmul_rn(b127, fabsf(lut[sl * 32 + lane])) < 0.5f;
-        if (!__all_sync(0xffffffffu, dead)) lm |= 1u << sl;
-      }
-      const bool zero_open = lm == 0;
-      if (zero_open) lm = 1u << (nsl - 1);
-      const int first = __ffs((int)lm) - 1;
-      const uint32_t sBa = smem_u32(smem + OFF_B), sXa = smem_u32(sX);
-      const uint32_t idesc = idesc_s8(N, 64, 1, 1);
+      mbar_wait_inline<256>(&bars[B_XFULL + s], (k >> 1) & 1, a.status);
+      const uint32_t lm = live_slabs(lut_of_lane(lut));   // (every warp computes the same mask)
       const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
-      bool mine = false;   // this warp owns a live slab
+      if (TAPS && a.tap_Xsq) {
+        for (int i = qt >> lq; i < Q; i += kRowStep)
+          if (!((lm >> (i >> 5)) & 1u)) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = zero4;
+      }
 #pragma unroll 1
-      for (int sl = qw; sl < nsl; sl += kQuantThreads / 32) {
-        if (!((lm >> sl) & 1u)) {
-          if (TAPS && a.tap_Xsq) {
-            for (int i = sl * 32 + (lane >> lq); i < sl * 32 + 32; i += 32 >> lq)
-              *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = zero4;
-          }
+      for (int r = qt >> lq, m = (int)lm;; r += kRowStep) {   // r: row among the live ones
+        for (; r >= 32; r -= 32) m &= m - 1;
+        if (m == 0) break;
+        const int i = (__ffs(m) - 1) * 32 + r;
+        uint4* ptr = reinterpret_cast<uint4*>(sX + swz_off((uint32_t)i, (uint32_t)c, 64));
+        const float l = lut[i];
+        if (__fmul_rn(b127, fabsf(l)) < 0.5f) {
+          *ptr = zero4;
+          if (TAPS && a.tap_Xsq) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = zero4;
           continue;
         }
-        mine = true;
-#pragma unroll 1
-        for (int i = sl * 32 + (lane >> lq); i < sl * 32 + 32; i += 32 >> lq) {
-          uint4* ptr = reinterpret_cast<uint4*>(sX + swz_off((uint32_t)i, (uint32_t)c, 64));
-          const float l = lut[i];
-          if (zero_open || __fmul_rn(b127, fabsf(l)) < 0.5f) {
-            *ptr = zero4;
-            if (TAPS && a.tap_Xsq) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = zero4;
-            continue;
-          }
-          const uint4 w4 = *ptr;
-          const uint32_t ww[4] = {w4.x ^ 0x80808080u, w4.y ^ 0x80808080u, w4.z ^ 0x80808080u, w4.w ^ 0x80808080u};
-          const float2 l2 = make_float2(l, l);
-          uint32_t o[4];
+        const uint4 w4 = *ptr;
+        const uint32_t ww[4] = {w4.x ^ 0x80808080u, w4.y ^ 0x80808080u, w4.z ^ 0x80808080u, w4.w ^ 0x80808080u};
+        const float2 l2 = make_float2(l, l);
+        uint32_t o[4];
 #pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            uint32_t q4[4];
+        for (int w = 0; w < 4; ++w) {
+          uint32_t q4[4];
 #pragma unroll
-            for (int e = 0; e < 4; e += 2) {
-              const float2 xf = __fadd2_rn(
-                  make_float2(__uint_as_float(__byte_perm(ww[w], 0x4B400000u, 0x7650u + e)),
-                              __uint_as_float(__byte_perm(ww[w], 0x4B400000u, 0x7651u + e))),
-                  make_float2(-kMagicIn, -kMagicIn));
-              const uint2 c2 = rne_clamp_bits2(__fmul2_rn(__fmul2_rn(xf, make_float2(rx[w * 4 + e], rx[w * 4 + e + 1])), l2));
-              q4[e] = c2.x;
-              q4[e + 1] = c2.y;
-            }
-            o[w] = pack4_bits(q4[0], q4[1], q4[2], q4[3]);
+          for (int e = 0; e < 4; e += 2) {
+            const float2 xf = __fadd2_rn(
+                make_float2(__uint_as_float(__byte_perm(ww[w], 0x4B400000u, 0x7650u + e)),
+                            __uint_as_float(__byte_perm(ww[w], 0x4B400000u, 0x7651u + e))),
+                make_float2(-kMagicIn, -kMagicIn));
+            const uint2 c2 = rne_clamp_bits2(__fmul2_rn(__fmul2_rn(xf, make_float2(rx[w * 4 + e], rx[w * 4 + e + 1])), l2));
+            q4[e] = c2.x;
+            q4[e + 1] = c2.y;
           }
-          const uint4 v = make_uint4(o[0], o[1], o[2], o[3]);
-          *ptr = v;
-          if (TAPS && a.tap_Xsq) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = v;
+          o[w] = pack4_bits(q4[0], q4[1], q4[2], q4[3]);
         }
+        const uint4 v = make_uint4(o[0], o[1], o[2], o[3]);
+        *ptr = v;
+        if (TAPS && a.tap_Xsq) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = v;
       }
       fence_async_smem();
-      __syncwarp();
-      if (lane == 0 && qw < nsl) {
-        if (mine) {
-          if ((first & (kQuantThreads / 32 - 1)) == qw) {
-            mbar_wait_inline<0>(&bars[B_ACC_FREE], (k & 1) ^ 1, a.status);   // the state warps have read chunk k-1
-          } else {
-            mbar_wait_inline<0>(&bars[B_OPEN], k & 1, a.status);
-          }
-          mbar_wait_inline<0>(&bars[B_BFULL], k & 1, a.status);   // the chunk's Bq rows have landed
-          tc_fence_after();
-#pragma unroll 1
-          for (int sl = qw; sl < nsl; sl += kQuantThreads / 32) {
-            if (!((lm >> sl) & 1u)) continue;
-            mma_s8_ss(tmem, tile_desc(sBa + 32 * sl * N, (uint32_t)N), tile_desc(sXa + 32 * sl * 64, 64), idesc, sl != first);
-            if (sl == first) {
-              tc_fence_before();
-              mbar_arrive(&bars[B_OPEN]);
-            }
-          }
-        }
-        mma_commit(&bars[B_MMA]);   // arrives when this thread's MMAs are done (at once if it issued none)
-      }
-      __syncwarp();
+      named_bar_arrive(2 + (k & 1), kQuantThreads);
+    }
     }
   } else {
     // ------------------------------------------------------------ state warps
@@ -291,15 +331,10 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
       }
     }
     tmem_st_wait();
-    if (tid == 0) {
-      issue_x(0);
-      issue_B(0);
-      if (d.c > 1) issue_x(1);
-    }
 #pragma unroll 1
     for (int k = 0; k < d.c; ++k) {
       const float gam = a.gamma[unit0 + k];
-      if (tid == 0 && k > 0) tma_store_wait_read();  // last chunk's hq store has read the staging tile
+      if (tid < ncq && k > 0) tma_store_wait_read();  // last chunk's hq store has read the staging tile
       named_bar(1, kStateThreads);  // also: every state thread has read the accumulator of chunk k-1
       // ---- hq[k] = codes of the state entering this chunk (and the prev tap).  They are formed here, ahead
       // of the wait for the chunk's MMAs, from a second read of the state; forming them in the update pass of
@@ -350,17 +385,13 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
       if (warp == 0) mbar_wait_inline<256>(&bars[B_MMA], k & 1, a.status);
       named_bar(1, kStateThreads);
       // ---- hq[k] leaves by TMA
-      if (tid == 0 && !CAL) {
-        for (int j = c0; j < c0 + ncq; ++j)  // 16 channels (rows of hq) per store
-          tma_store_2d(&tm_hq, sHQ + 16 * j * N, 0, (int)(((((i64)b * d.c + k) * d.H + h) * P) + 16 * j));
+      if (tid < ncq && !CAL) {
+        const int j = c0 + tid;              // 16 channels (rows of hq) per store
+        tma_store_2d(&tm_hq, sHQ + 16 * j * N, 0, (int)(((((i64)b * d.c + k) * d.H + h) * P) + 16 * j));
         tma_store_commit();
       }
       // ---- epilogue of the MMA: S = fmaf(Gamma_k, S, loc), 8 channels at a time
       tc_fence_after();
-      if (tid == 0) {   // the MMAs of chunk k have finished reading the Bq buffer and xq stage s
-        if (k + 1 < d.c) issue_B(k + 1);
-        if (k + 2 < d.c) issue_x(k + 2);
-      }
 #pragma unroll
       for (int hf = 0; hf < 4; ++hf) {       // 8 channels at a time
         if (hf < ncq) {
@@ -441,7 +472,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
         }
       }
     }
-    if (tid == 0) tma_store_wait_read();
+    if (tid < ncq) tma_store_wait_read();
   }
   drain_after_timeout(a.status);
   __syncthreads();
@@ -479,19 +510,18 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
                                           float* tap_loc, float* tap_prev, int8_t* tap_Xsq,
                                           int32_t* tap_acc, int32_t* status, bool int8_state,
                                           cudaStream_t st, uint32_t* absmax_h) {
-  const int TQ = d.Q < 128 ? d.Q : 128;
   const uint64_t T = (uint64_t)d.b * d.L;
   CUtensorMap tm_B, tm_x, tm_hq;
   {
     uint64_t dims[3] = {(uint64_t)d.N, (uint64_t)d.G, T};
     uint64_t str[2] = {(uint64_t)d.N, (uint64_t)d.G * d.N};
-    uint32_t box[3] = {(uint32_t)d.N, 1, (uint32_t)TQ};
+    uint32_t box[3] = {(uint32_t)d.N, 1, 32};
     if (!encode_tensor_map(&tm_B, Bq, 1, 3, dims, str, box, d.N)) return SSDI8_ERR_CUDA;
   }
   {
     uint64_t dims[3] = {(uint64_t)d.P, (uint64_t)d.H, T};
     uint64_t str[2] = {(uint64_t)d.P, (uint64_t)d.H * d.P};
-    uint32_t box[3] = {64, 1, (uint32_t)TQ};
+    uint32_t box[3] = {64, 1, 32};
     if (!encode_tensor_map(&tm_x, xq, 1, 3, dims, str, box, 64)) return SSDI8_ERR_CUDA;
   }
   {
