@@ -49,7 +49,7 @@ constexpr uint32_t OFF_X = 0;                     // two stages
 constexpr uint32_t OFF_B = 2 * XSTAGE;            // Bq rows [Q][N] of one chunk (single buffer)
 constexpr uint32_t OFF_HQ = OFF_B + 32768;        // [64 p][N] int8 staging of hq
 constexpr uint32_t OFF_LUT = OFF_HQ + 8192;       // 2 x [256] floats
-constexpr uint32_t OFF_COL = OFF_LUT + 2048;      // [64] loc scale, [64] 1 / s_h, [64] s_h
+constexpr uint32_t OFF_COL = OFF_LUT + 2048;      // [64] loc scale, [64] 1 / s_h, [64] s_x / s_xs
 constexpr uint32_t OFF_BAR = OFF_COL + 768;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 64;     // 76 608 bytes: three CTAs per SM
 constexpr uint32_t kTmemCols = 128;               // accumulator in columns 0..63, running state in 64..127
@@ -88,42 +88,9 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
   uint8_t* sHQ = smem + OFF_HQ;
   float* col_scale = reinterpret_cast<float*>(smem + OFF_COL);
   float* col_invh = col_scale + 64;
-  float* col_sh = col_invh + 64;
+  float* col_rx = col_invh + 64;
   const i64 bh = (i64)b * d.H + h;
   const i64 unit0 = bh * d.c;
-
-  if (tid == 0) {
-    mbar_init(&bars[B_XFULL], 1);
-    mbar_init(&bars[B_XFULL + 1], 1);
-    mbar_init(&bars[B_BFULL], 1);
-    mbar_init(&bars[B_MMA], 1);
-    mbar_init(&bars[B_ACC_FREE], kStateThreads / 32);
-    fence_mbar_init();
-    tma_prefetch_desc(&tm_B);
-    tma_prefetch_desc(&tm_x);
-    tma_prefetch_desc(&tm_hq);
-  }
-  if (warp == 1) tmem_alloc(tmem_slot, kTmemCols);
-  pdl_wait();   // everything below reads global memory
-  // (after the wait, not before it: ChunkBMM, launched next, reads and writes global memory without waiting
-  // for this kernel, so it must not be scheduled before this kernel's predecessors have completed)
-  pdl_launch_dependents();
-  if (tid < 64) {
-    const float sxb = __fmul_rn(a.s_xs[h * P + tid], a.s_B[g]);
-    if (CAL) {
-      col_scale[tid] = sxb;
-      col_invh[tid] = 0.f;               // running maximum of the channel
-    } else {
-      const float sh = a.s_h[h * P + tid];
-      col_scale[tid] = I8S ? __fdiv_rn(sxb, sh) : sxb;
-      col_invh[tid] = __fdiv_rn(1.0f, sh);
-      col_sh[tid] = sh;
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
 
   // One warp: the slabs of 32 tokens named by m of the xq rows (with LUT_state of the chunk: a global
   // load there would sit on the re-quantisation group's critical path) or of the Bq rows of chunk k
@@ -155,6 +122,48 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     __syncwarp();
   };
 
+  constexpr int kLoadWarp = kStateThreads / 32 + kRowWarps;
+  if (warp == kLoadWarp) {
+    if (lane == 0) {
+      mbar_init(&bars[B_XFULL], 1);
+      mbar_init(&bars[B_XFULL + 1], 1);
+      mbar_init(&bars[B_BFULL], 1);
+      mbar_init(&bars[B_MMA], 1);
+      mbar_init(&bars[B_ACC_FREE], kStateThreads / 32);
+      fence_mbar_init();
+      tma_prefetch_desc(&tm_B);
+      tma_prefetch_desc(&tm_x);
+      tma_prefetch_desc(&tm_hq);
+    }
+    __syncwarp();
+  }
+  if (warp == 1) tmem_alloc(tmem_slot, kTmemCols);
+  pdl_wait();   // everything below reads global memory
+  // (after the wait, not before it: ChunkBMM, launched next, reads and writes global memory without waiting
+  // for this kernel, so it must not be scheduled before this kernel's predecessors have completed)
+  pdl_launch_dependents();
+  if (warp == kLoadWarp) {   // all slabs of the first chunk: its LUT_state would have to come first
+    issue_x(0, (1u << (Q / 32)) - 1u);
+    issue_B(0, (1u << (Q / 32)) - 1u);
+  }
+  if (tid < 64) {
+    const float sxb = __fmul_rn(a.s_xs[h * P + tid], a.s_B[g]);
+    if (CAL) {
+      col_scale[tid] = sxb;
+      col_invh[tid] = 0.f;               // running maximum of the channel
+    } else {
+      const float sh = a.s_h[h * P + tid];
+      col_scale[tid] = I8S ? __fdiv_rn(sxb, sh) : sxb;
+      col_invh[tid] = __fdiv_rn(1.0f, sh);
+    }
+  } else if (tid < 128) {
+    col_rx[tid - 64] = __fdiv_rn(a.s_x[h * P + tid - 64], a.s_xs[h * P + tid - 64]);
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
   if (warp >= kStateThreads / 32) {
     // ------------------------------------------------------------ Q(X_scaled), one chunk ahead of the state warps
     const int qt = tid - kStateThreads;
@@ -162,10 +171,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     const int c = c0 + (qt & (ncq - 1));  // 16-byte chunk (16 channels) of every row this thread visits
     float rx[16];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-      const int hp = h * P + c * 16 + e;
-      rx[e] = __fdiv_rn(a.s_x[hp], a.s_xs[hp]);
-    }
+    for (int e = 0; e < 16; ++e) rx[e] = col_rx[c * 16 + e];
     // Rows that re-quantise to zero (the sparsity Eq. 3 rests on: LUT_state decays towards the start
     // of a chunk).  fmul is monotone, so with rxm >= |rx| of every channel of this CTA's range,
     // fmul(fmul(127, rxm), |LUT_state[i]|) < 1/2 implies |fmul(fmul(x, rx), LUT_state[i])| < 1/2 for every
@@ -183,7 +189,8 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     // and Bq loaded (48 KB per chunk and CTA) the loads of three CTAs took 1.4 us.  The row warps only arrive at
     // the barrier that releases the MMAs, one of two in turn: they are held back by the xq tile of the chunk after next,
     // which is requested when this chunk's MMAs have finished.
-    // (Batch 8 x 2048 x 80 heads: 48.9 us with slabs dealt out by position, 41.0 this way; 4 x 8192 x 128 151 and 118.)
+    // (Batch 8 x 2048 x 80 heads: 48.9 us with slabs dealt out by position, 41.0 this way, 38.7 with the first tiles requested
+    // ahead of all other set-up and s_x / s_xs divided once per channel; 4 x 8192 x 128 151, 118, 115.)
     const int qw = warp - kStateThreads / 32, nsl = Q / 32;
     // live slabs of a chunk from its LUT_state: nsl consecutive tokens per lane, 32 / nsl lanes per slab.  A chunk
     // without a live slab opens the accumulator with its last one, all rows of it stored as zeros.
@@ -212,8 +219,6 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     const float* const lut0 = a.pack + (unit0 * kPackRows + PACK_LUT) * Q;   // LUT_state of chunk 0; the next one kPackRows Q floats on
     const i64 lut_step = (i64)kPackRows * Q;
     if (qw == kRowWarps) {
-      issue_x(0, (1u << nsl) - 1u);    // (all of the first chunk: its LUT_state would have to come first)
-      issue_B(0, (1u << nsl) - 1u);
       uint32_t cur = live_slabs(lut_of_lane(lut0)), next = 0;
       if (d.c > 1) {
         next = live_slabs(lut_of_lane(lut0 + lut_step));
@@ -467,7 +472,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
 #pragma unroll
             for (int e = 0; e < 8; ++e)
               a.final_state[(bh * P + cb + p0 + e) * N + n] =
-                  I8S ? __fmul_rn((float)sv[e], col_sh[cb + p0 + e]) : __int_as_float(sv[e]);
+                  I8S ? __fmul_rn((float)sv[e], a.s_h[h * P + cb + p0 + e]) : __int_as_float(sv[e]);
           }
         }
       }
