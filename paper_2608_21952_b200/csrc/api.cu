@@ -167,13 +167,15 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
   // state modules run in this call, ChunkBMM is launched after the first state kernel and works beside it.
   const bool fused_state = (ph & SSDI8_PHASE_CHUNK_STATE) && (ph & SSDI8_PHASE_STATE_PASSING);
   const bool bmm_late = (ph & SSDI8_PHASE_BMM) && fused_state;
-  // Few sequences with several chunks: the fused kernel walks a (batch, head)'s chunks one after the other, about 1.9 us
+  // Few sequences of many chunks: the fused kernel walks a (batch, head)'s chunks one after the other, about 1.3 us
   // each however few CTAs there are, while ChunkState takes all chunks at once (states through L2) and StatePassing
-  // is a short elementwise pass.  Algorithm 2 with the fused kernel / with the two, us: 1 x 512 tokens x 4
-  // heads 23 / 19, 2048 x 24 40 / 35, 8192 x 24 90 / 60, 8192 x 8 (N 64, chunks of 64) 198 / 59, 4 x 2048 x 24
-  // 57 / 56; but 2 x 2048 x 80 72 / 76, 3 x 1408 x 50 60 / 63, and with two chunks 24 / 25.
+  // is a short elementwise pass.  Algorithm 2 with the fused kernel / with the two, us: 8192 tokens x 8 heads (N 64,
+  // chunks of 64) 128 / 58, 8192 x 24 75 / 62, 4096 x 80 81 / 78, 8192 x 80 144 / 136; with eight chunks and few enough
+  // of them for two CTAs per SM at once 512 x 4 (chunks of 64) 19 / 18 and the whole layer at 2048 x 24 34.6 / 33.5; but
+  // 8192 x 110 143 / 175, 3 x 8192 x 50 213 / 239, 2 x 2048 x 40 51 / 52, with four chunks 1024 x 24 26 / 28.
   const int sms = fused_state ? sm_count() : 0;
-  const bool split_state = fused_state && !i8s && d.c >= 4 && (i64)d.b * d.H * 4 <= (i64)3 * sms;
+  const i64 seqs = (i64)d.b * d.H;
+  const bool split_state = fused_state && !i8s && (d.c >= 12 ? 3 * seqs <= 2 * sms : d.c >= 8 && seqs * d.c <= 2 * sms);
   if ((ph & SSDI8_PHASE_BMM) && !bmm_late &&
       (s = launch_bmm(d, a->Cq, a->Bq, a->s_C, a->s_B, a->s_cb, cbq, a->tap_acc_cb, nullptr, a->status, st)) !=
           SSDI8_OK)
