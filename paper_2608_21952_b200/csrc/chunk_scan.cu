@@ -17,7 +17,7 @@
 // tiles) and an 8-deep ring for what the mask warps hand to the epilogue keep the mask and the MMAs
 // of the next tiles independent of the epilogue of the current ones.  Every buffer has its own
 // "free" barrier, released by whoever reads it last (tcgen05.commit for MMA operands), so loads run
-// several tiles ahead.  What bounds the kernel is instruction issue (86 M warp instructions, 66 % of the
+// several tiles ahead.  What bounds the kernel is instruction issue (78 M warp instructions, 66 % of the
 // slots with binary32 y at batch 8 x 2048 x 80 heads, 0.113 ms; 0.104 ms with 16-bit y), so it is
 // written to issue little: in each group one warp polls the mbarriers and the others wait at a hardware
 // barrier, the wait loop is one out-of-line function, the tile walk has no divisions, and the code is kept
