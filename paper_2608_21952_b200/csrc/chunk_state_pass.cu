@@ -542,15 +542,18 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
   const int sms = sm_count();
   if (sms == 0) return SSDI8_ERR_CUDA;
   const int units = d.H * d.b, slots = 3 * sms;
-  // Whole (batch, head) units wherever the device is filled: with three CTAs per SM the kernel is bound
-  // by instruction issue, so a partly filled last wave of whole units runs faster per CTA and costs less
-  // than the same units cut into more CTAs (measured at 640 units on 444 slots: 0.054 ms whole, 0.056 ms
-  // in halves, 0.067 ms in quarters).  Only a workload that leaves most slots empty (fewer units than an
-  // eighth of a wave beyond the full waves) is cut into quarter-width CTAs, which spreads it over more
-  // SMs (24 units: 0.0225 ms in quarters against 0.0265 ms whole).
+  // Whole (batch, head) units wherever the device is filled: a partly filled last wave of whole units runs faster per
+  // CTA and costs less than the same units cut into more CTAs (592 units on 444 slots: 36.7 us whole, 41.9 with the last
+  // 148 in quarters).  Quarter-width CTAs have the shorter chain per chunk (a quarter of the state per thread), so they
+  // take a remainder of less than an eighth of a wave (512 tokens x 24 heads: 5.1 us, 7.1 whole) and, where all
+  // of them fit the device beside the next kernel's first CTAs and a chain has four chunks or more, the whole workload
+  // (Algorithm 2, us, whole / quarters: 2048 tokens x 80 heads 50.4 / 47.6, 2 x 2048 x 50 54.0 / 52.0, 1408 x 70 in chunks of
+  // 128 43.8 / 40.4, 1024 x 80 36.6 / 35.5; but with one or two chunks 3 x 256 x 37 24.4 / 26.0, 512 x 100 29.9 / 30.5, and
+  // 2048 x 111 55.8 / 56.7).
   int n_full = units / slots * slots;
   int split = 4;
-  if (8 * (units - n_full) > slots) n_full = units;
+  const bool quarters = 8 * (units - n_full) <= slots || (n_full == 0 && d.c >= 4 && 4 * units <= slots - slots / 10);
+  if (!quarters) n_full = units;
   FusedArgs a = {s_x, s_xs, s_B, s_h, pack, gamma, init, final_state, tap_loc, tap_prev, tap_Xsq, tap_acc,
                  status, absmax_h, d, n_full, split};
   const size_t smem = SMEM_BYTES;

@@ -139,7 +139,9 @@ def test_host_pipeline_cuts_equal_the_device_call(b, c, H, G, flags):
                                  SSDConfig("fused_eight", 2, 8 * 64, 19, 64, 128, 1, 64, 0.02, 20.0, 41),
                                  SSDConfig("fused_short", 1, 3 * 128, 2, 64, 128, 1, 128, 0.02, 20.0, 40),
                                  SSDConfig("fused_one", 2, 256, 30, 64, 128, 2, 256, 0.02, 20.0, 42),
-                                 SSDConfig("fused_q256", 1, 4 * 256, 60, 64, 64, 1, 256, 0.02, 20.0, 43)], ids=lambda c: c.name)
+                                 SSDConfig("fused_q256", 1, 4 * 256, 60, 64, 64, 1, 256, 0.02, 20.0, 43),
+                                 SSDConfig("quarters_last", 2, 4 * 64, 50, 64, 64, 1, 64, 0.02, 20.0, 44),
+                                 SSDConfig("whole_first", 1, 4 * 64, 101, 64, 64, 1, 64, 0.02, 20.0, 45)], ids=lambda c: c.name)
 @pytest.mark.parametrize("fast", [False, True])
 def test_state_kernels_on_both_sides_of_the_dispatch(cfg, fast):
     # With 12 chunks 98 (batch, head) pairs are the last that take ChunkState + StatePassing on 148 SMs, 99 the first that do
