@@ -167,15 +167,15 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
   // state modules run in this call, ChunkBMM is launched after the first state kernel and works beside it.
   const bool fused_state = (ph & SSDI8_PHASE_CHUNK_STATE) && (ph & SSDI8_PHASE_STATE_PASSING);
   const bool bmm_late = (ph & SSDI8_PHASE_BMM) && fused_state;
-  // Few sequences of many chunks: the fused kernel walks a (batch, head)'s chunks one after the other, about 1.3 us
+  // Few sequences of many chunks: the fused kernel walks a (batch, head)'s chunks one after the other, about 1.2 us
   // each however few CTAs there are, while ChunkState takes all chunks at once (states through L2) and StatePassing
   // is a short elementwise pass.  Algorithm 2 with the fused kernel / with the two, us: 8192 tokens x 8 heads (N 64,
-  // chunks of 64) 128 / 58, 8192 x 24 75 / 62, 4096 x 80 81 / 78, 8192 x 80 144 / 136; with eight chunks and few enough
-  // of them for two CTAs per SM at once 512 x 4 (chunks of 64) 19 / 18 and the whole layer at 2048 x 24 34.6 / 33.5; but
-  // 8192 x 110 143 / 175, 3 x 8192 x 50 213 / 239, 2 x 2048 x 40 51 / 52, with four chunks 1024 x 24 26 / 28.
+  // chunks of 64) 128 / 58, 8192 x 48 98.5 / 92.5, 4096 x 48 58.8 / 57.6, 4096 x 24 44.2 / 42.7, 512 x 4 (chunks of 64)
+  // 18.0 / 16.0; but 8192 x 60 104.7 / 109.2, 8192 x 80 119 / 136, 4096 x 80 74 / 78.  With eight to eleven chunks the line
+  // lies where two CTAs per SM take all of them at once (2048 x 24: even).
   const int sms = fused_state ? sm_count() : 0;
   const i64 seqs = (i64)d.b * d.H;
-  const bool split_state = fused_state && !i8s && (d.c >= 12 ? 3 * seqs <= 2 * sms : d.c >= 8 && seqs * d.c <= 2 * sms);
+  const bool split_state = fused_state && !i8s && (d.c >= 12 ? 3 * seqs <= sms : d.c >= 8 && seqs * d.c <= 2 * sms);
   if ((ph & SSDI8_PHASE_BMM) && !bmm_late &&
       (s = launch_bmm(d, a->Cq, a->Bq, a->s_C, a->s_B, a->s_cb, cbq, a->tap_acc_cb, nullptr, a->status, st)) !=
           SSDI8_OK)

@@ -134,8 +134,8 @@ def test_host_pipeline_cuts_equal_the_device_call(b, c, H, G, flags):
 @pytest.mark.parametrize("cfg", [SSDConfig("split_small", 1, 8 * 64, 1, 64, 128, 1, 64, 0.02, 20.0, 35),
                                  SSDConfig("split_deep", 2, 17 * 64, 3, 64, 64, 1, 64, 0.02, 20.0, 36),
                                  SSDConfig("split_q256", 1, 9 * 256, 5, 64, 128, 1, 256, 0.02, 20.0, 37),
-                                 SSDConfig("split_edge", 2, 12 * 64, 49, 64, 64, 7, 64, 0.02, 20.0, 38),
-                                 SSDConfig("fused_edge", 3, 12 * 64, 33, 64, 64, 3, 64, 0.02, 20.0, 39),
+                                 SSDConfig("split_edge", 1, 12 * 64, 49, 64, 64, 7, 64, 0.02, 20.0, 38),
+                                 SSDConfig("fused_edge", 2, 12 * 64, 25, 64, 64, 5, 64, 0.02, 20.0, 39),
                                  SSDConfig("fused_eight", 2, 8 * 64, 19, 64, 128, 1, 64, 0.02, 20.0, 41),
                                  SSDConfig("fused_short", 1, 3 * 128, 2, 64, 128, 1, 128, 0.02, 20.0, 40),
                                  SSDConfig("fused_one", 2, 256, 30, 64, 128, 2, 256, 0.02, 20.0, 42),
@@ -144,7 +144,7 @@ def test_host_pipeline_cuts_equal_the_device_call(b, c, H, G, flags):
                                  SSDConfig("whole_first", 1, 4 * 64, 101, 64, 64, 1, 64, 0.02, 20.0, 45)], ids=lambda c: c.name)
 @pytest.mark.parametrize("fast", [False, True])
 def test_state_kernels_on_both_sides_of_the_dispatch(cfg, fast):
-    # With 12 chunks 98 (batch, head) pairs are the last that take ChunkState + StatePassing on 148 SMs, 99 the first that do
+    # With 12 chunks 49 (batch, head) pairs are the last that take ChunkState + StatePassing on 148 SMs, 50 the first that do
     # not; with 8 chunks 37 and 38; 17 and 9 chunks leave one after two and one batches of eight.  The fused kernel shares
     # the live rows of a chunk among its warps: heads of different decay have any number of live slabs, and with very
     # fast decay whole slabs and whole chunks re-quantise to zero
