@@ -525,6 +525,10 @@ chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ 
 #pragma unroll
       for (int j = 0; j < 4; ++j)
         xr[j] = ok ? *reinterpret_cast<const uint4*>(sX + swz_off((uint32_t)ei, (uint32_t)j, 64)) : make_uint4(0u, 0u, 0u, 0u);
+      // (the fence: nothing has consumed the loads yet, and an arrival alone does not order them ahead of the next TMA
+      // load into the buffer, which is another proxy's write.  Behind a warp's own backlog of global stores they were still
+      // waiting when that load landed, and the skip term was that of the chunk after next.)
+      fence_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[B_X_FREE + xs]);
       // two lanes of one warp of the group poll side by side, one barrier each: the accumulators and the row
