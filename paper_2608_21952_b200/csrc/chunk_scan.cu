@@ -163,7 +163,7 @@ __device__ __forceinline__ void mask_tile(uint8_t* sCB, const float* tokbuf, flo
   {
     // own sub-block, right to left: E[i,i] = 1, E[i,j] = fmul(E[i,j+1], a_{j+1}).  Straight-line code: the
     // product starts as 0 and is set to 1 where the row meets its diagonal, so the columns past it, which
-    // carry no weight, come out as 0 by themselves and the 16 rows of the warp do not diverge.
+    // carry no weight, raise no row maximum and the 16 rows of the warp do not diverge.
     const uint2 w2 = *half_ptr(I16);
     const uint32_t ww[2] = {w2.x ^ 0x80808080u, w2.y ^ 0x80808080u};
     const float* ab = atok_s + I16 * 16;   // a_m of the sub-block at ab[m]
@@ -228,13 +228,18 @@ __device__ __forceinline__ void mask_tile(uint8_t* sCB, const float* tokbuf, flo
     if (TAPS && a.taps.rowmax) a.taps.rowmax[(t.tok0 + i) * a.d.H + t.h] = rmax;
   }
   // (the sub-blocks after the row's own arrive as zeros: ChunkBMM writes them so)
-  auto store = [&](int c, const float2 (&p)[4], float g) {
+  auto store = [&](int c, const float2 (&p)[4], float g, uint32_t keep0 = ~0u, uint32_t keep1 = ~0u) {
     const float2 g2 = make_float2(g, g);
-    const uint2 v = make_uint2(pack4_rn_product(p[0], p[1], g2), pack4_rn_product(p[2], p[3], g2));
+    const uint2 v = make_uint2(pack4_rn_product(p[0], p[1], g2) & keep0, pack4_rn_product(p[2], p[3], g2) & keep1);
     *half_ptr(c) = v;
     if (TAPS && mq_tap) *reinterpret_cast<uint2*>(mq_tap + c * 16 + q2 * 8) = v;
   };
-  store(I16, tv, inv);
+  {
+    // Codes past the diagonal are cleared by their bytes: their E is 0, but 0 times a dt that is not finite is not, and a
+    // token must not reach the rows before it whatever its dt.
+    const int live = 8 * (ri - q2 * 8 + 1);   // bits of this thread's columns on or below the diagonal
+    store(I16, tv, inv, __funnelshift_lc(~0u, 0u, max(live, 0)), __funnelshift_lc(~0u, 0u, max(live - 32, 0)));
+  }
   const float di = __fmul_rn(dec, inv);
   if (I16 > 0) store(I16 - 1, tn, di);
   if (I16 > 1) {

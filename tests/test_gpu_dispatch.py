@@ -239,3 +239,18 @@ def test_output_does_not_depend_on_the_pace_of_the_epilogue(Q, taps):
     for _ in range(3):
         y, fin, _ = gh.gpu_fwd(cfg, q, taps=taps)
         assert np.array_equal(y, want[0]) and np.array_equal(fin, want[1])
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("Q", [64, 256])
+def test_a_time_step_that_is_not_finite_does_not_reach_earlier_tokens(Q, value):
+    import gpu_harness as gh
+    cfg = SSDConfig("causal", 1, 2 * Q, 3, 64, 64, 1, Q, 0.02, 20.0, 47)
+    q = _random_codes(cfg, 47)
+    want = gh.gpu_fwd(cfg, q, taps=())[0]
+    for j in (0, 5, 15, Q - 1, Q + 8, 2 * Q - 10):
+        dt = q["dt"].copy()
+        dt[j, 1] = value
+        y = gh.gpu_fwd(cfg, dict(q, dt=dt), taps=())[0]
+        assert np.array_equal(y[:, :j], want[:, :j]), j
+        assert np.array_equal(y[:, :, ::2], want[:, :, ::2])
