@@ -45,7 +45,10 @@ __global__ void __launch_bounds__(128) quant_ch_fastest(const float4* __restrict
       for (int u = 0; u < QROWS; ++u) __stcs(out + (r + u) * ch4 + q, code4_by_division(in[(r + u) * ch4 + q], s));
     }
   }
-  for (; r < r1; ++r) __stcs(out + r * ch4 + q, code4_by_division(__ldcs(in + r * ch4 + q), s));
+  for (; r < r1; ++r) {
+    const float4 v = __ldcs(in + r * ch4 + q);
+    __stcs(out + r * ch4 + q, st.usable ? code4(v, st) : code4_by_division(v, s));
+  }
 }
 
 // ---- the layer's three static quantisers (x per channel; B and C per group) as one launch.  Every
@@ -118,7 +121,10 @@ __global__ void __launch_bounds__(128, 8) quant_jobs(const QuantJobs a) {
       for (int u = 0; u < QROWS; ++u) out[e + u * stride] = code4_by_division(in[e + u * stride], s);
     }
   }
-  for (; left > 0; --left, e += stride) out[e] = code4_by_division(__ldcs(in + e), s);
+  for (; left > 0; --left, e += stride) {
+    const float4 v = __ldcs(in + e);
+    out[e] = st.usable ? code4(v, st) : code4_by_division(v, s);
+  }
 }
 
 // ---- quantise, I % 4 == 0: 4 consecutive elements share a channel

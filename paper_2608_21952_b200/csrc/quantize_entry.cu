@@ -82,7 +82,10 @@ __global__ void __launch_bounds__(128) quant_entry_kernel(const typename Vec4<T>
       for (int u = 0; u < EROWS; ++u) out[(r + u) * ow4 + oq] = code4_by_division(Vec4<T>::cvt(in[(r + u) * W4 + q]), s);
     }
   }
-  for (; r < r1; ++r) out[r * ow4 + oq] = code4_by_division(Vec4<T>::cvt(__ldcs(in + r * W4 + q)), s);
+  for (; r < r1; ++r) {
+    const float4 v = Vec4<T>::cvt(__ldcs(in + r * W4 + q));
+    out[r * ow4 + oq] = st.usable ? code4(v, st) : code4_by_division(v, s);
+  }
 }
 
 }  // namespace

@@ -254,3 +254,31 @@ def test_a_time_step_that_is_not_finite_does_not_reach_earlier_tokens(Q, value):
         y = gh.gpu_fwd(cfg, dict(q, dt=dt), taps=())[0]
         assert np.array_equal(y[:, :j], want[:, :j]), j
         assert np.array_equal(y[:, :, ::2], want[:, :, ::2])
+
+
+@pytest.mark.parametrize("dtype", ["float32", "float16", "bfloat16"])
+def test_codes_do_not_depend_on_the_row(dtype):
+    # The same values in every row, in full rounds of eight rows and in the remainder: NaNs of both signs, infinities,
+    # values beyond the range of the quotient among them
+    import torch
+    from paper_2608_21952_b200 import binding as bd
+    v = np.array([0x7fc00000, 0xffc00000, 0x7f800000, 0xff800000, 0x7f7fffff, 0xff7fffff, 0, 0x80000000], np.uint32).view(np.float32)
+    D, T = 64, 8 + 7
+    row = np.concatenate([np.resize(v, D), np.zeros(32, np.float32)])
+    bits = row.view(np.int32)
+    t = torch.from_numpy(np.tile(bits, (T, 1))).cuda().view(torch.float32)
+    if dtype == "bfloat16":    # (torch's conversion drops the sign of a NaN)
+        t = torch.from_numpy(np.tile((bits >> 16).astype(np.int16), (T, 1))).cuda().view(torch.bfloat16)
+    elif dtype == "float16":
+        t = t.half()
+        t[:, 1::8].view(torch.int16).fill_(-512)   # 0xfe00: a negative NaN
+    one = torch.ones(1, device="cuda")
+    out = [torch.empty(T, w, dtype=torch.int8, device="cuda") for w in (D, 16, 16)]
+    s_x = torch.from_numpy(np.repeat(np.float32([0.03, 1.0, 1e-42, 3e-30, 7e29, np.inf, 0.5, 127.0]), 8)).cuda()
+    bd.ssdi8_quantize_entry(t.contiguous(), T, D, 1, 16, s_x, one, one, *out)
+    got = out[0].cpu().numpy()
+    assert np.array_equal(got, np.tile(got[8:9], (T, 1)))
+    if dtype == "float32":
+        q = torch.empty(T, D, dtype=torch.int8, device="cuda")
+        bd.ssdi8_quantize_act(t[:, :D].contiguous(), T, D, 1, s_x, 0, q)
+        assert np.array_equal(q.cpu().numpy(), got)
