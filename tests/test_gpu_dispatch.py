@@ -278,6 +278,7 @@ def test_codes_do_not_depend_on_the_row(dtype):
     bd.ssdi8_quantize_entry(t.contiguous(), T, D, 1, 16, s_x, one, one, *out)
     got = out[0].cpu().numpy()
     assert np.array_equal(got, np.tile(got[8:9], (T, 1)))
+    assert np.all(got[:, 0::8] == 127) and np.all(got[:, 1::8] == 127)   # a NaN of either sign, as by division
     if dtype == "float32":
         q = torch.empty(T, D, dtype=torch.int8, device="cuda")
         bd.ssdi8_quantize_act(t[:, :D].contiguous(), T, D, 1, s_x, 0, q)
