@@ -17,7 +17,7 @@ constexpr int QROWS = 8;
 // FIX: the step sizes were just formed by an absmax kernel; an all-zero channel has 0 there and gets 1 (every
 // block reads 0 or 1 and takes 1, the first row of blocks writes it).
 template <bool FIX>
-__global__ void __launch_bounds__(128) quant_ch_fastest(const float4* __restrict__ in, float4* scale,
+__global__ void __launch_bounds__(128, 8) quant_ch_fastest(const float4* __restrict__ in, float4* scale,
                                                         uint32_t* __restrict__ out, i64 R, int ch4,
                                                         int rows_per_block) {
   pdl_launch_dependents();
@@ -32,22 +32,26 @@ __global__ void __launch_bounds__(128) quant_ch_fastest(const float4* __restrict
   const Step4 st = step4(s);
   const i64 r0 = (i64)blockIdx.y * rows_per_block;
   const i64 r1 = r0 + rows_per_block < R ? r0 + rows_per_block : R;
+  if (!st.usable) {   // abnormal step sizes: row by row
+    for (i64 r = r0; r < r1; ++r) __stcs(out + r * ch4 + q, code4_by_division(__ldcs(in + r * ch4 + q), s));
+    return;
+  }
   i64 r = r0;
   for (; r + QROWS <= r1; r += QROWS) {
     float4 v[QROWS];
 #pragma unroll
     for (int u = 0; u < QROWS; ++u) v[u] = __ldcs(in + (r + u) * ch4 + q);
-    if (st.usable) {
 #pragma unroll
-      for (int u = 0; u < QROWS; ++u) __stcs(out + (r + u) * ch4 + q, code4(v[u], st));
-    } else {
-#pragma unroll 1
-      for (int u = 0; u < QROWS; ++u) __stcs(out + (r + u) * ch4 + q, code4_by_division(in[(r + u) * ch4 + q], s));
-    }
+    for (int u = 0; u < QROWS; ++u) __stcs(out + (r + u) * ch4 + q, code4(v[u], st));
   }
-  for (; r < r1; ++r) {
-    const float4 v = __ldcs(in + r * ch4 + q);
-    __stcs(out + r * ch4 + q, st.usable ? code4(v, st) : code4_by_division(v, s));
+  if (r < r1) {   // the last rows, their loads in flight together too
+    float4 v[QROWS];
+#pragma unroll
+    for (int u = 0; u < QROWS - 1; ++u)
+      if (r + u < r1) v[u] = __ldcs(in + (r + u) * ch4 + q);
+#pragma unroll
+    for (int u = 0; u < QROWS - 1; ++u)
+      if (r + u < r1) __stcs(out + (r + u) * ch4 + q, code4(v[u], st));
   }
 }
 
