@@ -8,12 +8,10 @@
 namespace ssdi8 {
 namespace {
 
-constexpr int SP_T = 256;
-
-// PREV: the entering states are written (they may go over loc, so a chunk's load cannot be moved ahead of the store
-// of the one before); without them the loads of eight chunks are in flight at once.
-template <bool PREV>
-__global__ void __launch_bounds__(SP_T) state_passing_kernel(
+// K chunks' loads are in flight at once; AHEAD: the next K too, requested before the present ones are used.  PREV: the entering
+// states are written; prev may be loc (or start before it): a chunk's load is ahead of the store that goes over it either way.
+template <bool PREV, int K, bool AHEAD, int THREADS>
+__global__ void __launch_bounds__(THREADS) state_passing_kernel(
     const float4* loc /* may alias prev: no __restrict__ */, const float* __restrict__ gamma, const float4* __restrict__ init,
     const float* __restrict__ s_h, float4* prev, float4* __restrict__ final_state,
     uint32_t* __restrict__ hq, Dims d) {
@@ -21,7 +19,7 @@ __global__ void __launch_bounds__(SP_T) state_passing_kernel(
   pdl_wait();
   const int N4 = d.N / 4;
   const i64 per_b = (i64)d.H * d.P * N4;               // float4 per (b) slice of one chunk
-  const i64 idx = (i64)blockIdx.x * SP_T + threadIdx.x;  // over b * H * P * N4
+  const i64 idx = (i64)blockIdx.x * THREADS + threadIdx.x;  // over b * H * P * N4
   if (idx >= per_b * d.b) return;
   const int b = (int)(idx / per_b);
   const i64 r = idx % per_b;                             // (h, p, n4)
@@ -33,6 +31,17 @@ __global__ void __launch_bounds__(SP_T) state_passing_kernel(
   const float* gm = gamma + ((i64)b * d.H + h) * d.c;
   const i64 stride = per_b;                              // chunk stride in float4
   i64 o = (i64)b * d.c * per_b + r;
+  struct Batch {
+    float4 l[K];
+    float g[K];
+  };
+  auto fetch = [&](Batch& v, i64 at, int k) {
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      v.l[j] = loc[at + j * stride];
+      v.g[j] = gm[k + j];
+    }
+  };
   auto step = [&](const float4& l, float g) {
     if (hq)
       hq[o] = pack4(rne_clamp(__fmul_rn(S.x, inv_h)), rne_clamp(__fmul_rn(S.y, inv_h)),
@@ -44,20 +53,36 @@ __global__ void __launch_bounds__(SP_T) state_passing_kernel(
     S.w = __fmaf_rn(g, S.w, l.w);
     o += stride;
   };
-  constexpr int K = PREV ? 1 : 8;
+  auto steps = [&](const Batch& v) {
+#pragma unroll
+    for (int j = 0; j < K; ++j) step(v.l[j], v.g[j]);
+  };
   int k = 0;
-  for (; k + K <= d.c; k += K) {
-    float4 l[K];
-    float g[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) {
-      l[j] = loc[o + j * stride];  // (read before prev[o] is written: prev may alias loc)
-      g[j] = gm[k + j];
+  if (AHEAD) {
+    Batch v0, v1;
+    if (K <= d.c) fetch(v0, o, 0);
+    for (; k + K <= d.c; k += 2 * K) {
+      const bool second = k + 2 * K <= d.c;
+      if (second) fetch(v1, o + K * stride, k + K);
+      steps(v0);
+      if (!second) {
+        k += K;
+        break;
+      }
+      if (k + 3 * K <= d.c) fetch(v0, o + K * stride, k + 2 * K);
+      steps(v1);
     }
-#pragma unroll
-    for (int j = 0; j < K; ++j) step(l[j], g[j]);
+  } else {
+    for (; k + K <= d.c; k += K) {
+      Batch v;
+      fetch(v, o, k);
+      steps(v);
+    }
   }
-  for (; k < d.c; ++k) step(loc[o], gm[k]);
+  for (; k < d.c; ++k) {
+    const float4 l = loc[o];   // (a copy: prev[o] may be the same place)
+    step(l, gm[k]);
+  }
   if (final_state) final_state[idx] = S;
 }
 
@@ -67,11 +92,25 @@ ssdi8_status_t launch_state_passing(const Dims& d, const float* loc, const float
                                     const float* init, const float* s_h, float* prev,
                                     float* final_state, int8_t* hq, cudaStream_t st) {
   const i64 n = (i64)d.b * d.H * d.P * (d.N / 4);
-  unsigned grid = (unsigned)((n + SP_T - 1) / SP_T);
-  return launch_configured(prev ? state_passing_kernel<true> : state_passing_kernel<false>, dim3(grid), dim3(SP_T), 0, -1, false, st,
-                           reinterpret_cast<const float4*>(loc), gamma, reinterpret_cast<const float4*>(init), s_h,
-                           reinterpret_cast<float4*>(prev), reinterpret_cast<float4*>(final_state),
-                           reinterpret_cast<uint32_t*>(hq), d);
+  auto launch = [&](auto kernel, int threads) -> ssdi8_status_t {
+    return launch_configured(kernel, dim3((unsigned)((n + threads - 1) / threads)), dim3(threads), 0, -1, false, st,
+                             reinterpret_cast<const float4*>(loc), gamma, reinterpret_cast<const float4*>(init), s_h,
+                             reinterpret_cast<float4*>(prev), reinterpret_cast<float4*>(final_state),
+                             reinterpret_cast<uint32_t*>(hq), d);
+  };
+  // Loads in flight per thread against how many threads the registers leave room for.  With eight chunks and more, eight at a
+  // time; from sixteen on, where few threads are all there is, the next eight ahead as well.  us, one batch of eight / the
+  // next ahead: 8192 tokens x 24 heads 9.2 / 7.2, 32768 x 4 (chunks of 64) 54 / 36, but 8192 x 80 16.9 / 20.3.  Where prev is
+  // written, one at a time / four / eight and the next ahead: 64 sequences of one chunk x 80 heads 89 / 118 / -, 2048 x 80 8.8 /
+  // 6.8 / 7.0, 8192 x 80 38 / 36 / 33, 8192 x 24 9.1 / 11.6 / 8.5.
+  if (prev) {
+    if (d.c < 4) return launch(state_passing_kernel<true, 1, false, 256>, 256);
+    if (d.c < 16) return launch(state_passing_kernel<true, 4, false, 256>, 256);
+    return launch(state_passing_kernel<true, 8, true, 128>, 128);
+  }
+  if (d.c < 8) return launch(state_passing_kernel<false, 4, false, 256>, 256);
+  if (d.c < 16 || n > 96 * 1024) return launch(state_passing_kernel<false, 8, false, 256>, 256);
+  return launch(state_passing_kernel<false, 8, true, 128>, 128);
 }
 
 }  // namespace ssdi8

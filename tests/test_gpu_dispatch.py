@@ -283,3 +283,48 @@ def test_codes_do_not_depend_on_the_row(dtype):
         q = torch.empty(T, D, dtype=torch.int8, device="cuda")
         bd.ssdi8_quantize_act(t[:, :D].contiguous(), T, D, 1, s_x, 0, q)
         assert np.array_equal(q.cpu().numpy(), got)
+
+
+@pytest.mark.parametrize("chunks", [1, 3, 4, 5, 7, 8, 15, 16, 17, 24, 25, 31, 32, 33, 40])
+@pytest.mark.parametrize("prev", [None, "own", "loc", "before loc"])
+def test_state_passing_batches(chunks, prev):
+    # every remainder of the batches of four and eight chunks and of the batch ahead; prev absent, of its own, over loc, and
+    # starting one chunk before loc
+    import torch
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("batches", 1, 64 * chunks, 3, 64, 64, 1, 64, 0.02, 20.0, 48)
+    rng = np.random.default_rng(chunks)
+    per = 3 * 64 * 64
+    loc = rng.standard_normal((1, chunks, 3, 64, 64)).astype(np.float32)
+    gamma = rng.uniform(0, 1, (1, 3, chunks)).astype(np.float32)
+    init = rng.standard_normal((1, 3, 64, 64)).astype(np.float32)
+    s_h = rng.uniform(0.01, 0.05, cfg.channels).astype(np.float32)
+    want = orc.state_passing(cfg, loc, gamma, init, s_h)
+    buf = torch.zeros((chunks + 1) * per, device="cuda")
+    dl = buf[per:]
+    dl.copy_(gh.dev(loc).reshape(-1))
+    dp = {None: None, "own": torch.empty_like(dl), "loc": dl, "before loc": buf[:-per]}[prev]
+    fin, hq = torch.empty(init.shape, device="cuda"), torch.empty(loc.shape, dtype=torch.int8, device="cuda")
+    bd.ssdi8_state_passing(bd.dims_of(cfg), dl, gh.dev(gamma), gh.dev(init), dp, fin, hq, gh.dev(s_h))
+    torch.cuda.synchronize()
+    assert prev is None or np.array_equal(dp.cpu().numpy(), np.asarray(want[0]).reshape(-1))
+    assert np.array_equal(fin.cpu().numpy(), want[1]) and np.array_equal(hq.cpu().numpy(), want[2])
+
+
+@pytest.mark.parametrize("b,H", [(1, 23), (1, 25), (2, 33)])
+def test_state_passing_on_either_side_of_the_thread_limit(b, H):
+    # 16 chunks: up to 98 304 threads (48 heads of 64 x 128 states) keep the next batch ahead
+    import torch
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("threads", b, 64 * 17, 2 * H, 64, 128, 1, 64, 0.02, 20.0, 49)
+    rng = np.random.default_rng(H)
+    loc = rng.standard_normal((b, 17, 2 * H, 64, 128)).astype(np.float32)
+    gamma = rng.uniform(0, 1, (b, 2 * H, 17)).astype(np.float32)
+    s_h = rng.uniform(0.01, 0.05, cfg.channels).astype(np.float32)
+    want = orc.state_passing(cfg, loc, gamma, None, s_h)
+    fin, hq = torch.empty((b, 2 * H, 64, 128), device="cuda"), torch.empty(loc.shape, dtype=torch.int8, device="cuda")
+    bd.ssdi8_state_passing(bd.dims_of(cfg), gh.dev(loc), gh.dev(gamma), None, None, fin, hq, gh.dev(s_h))
+    torch.cuda.synchronize()
+    assert np.array_equal(fin.cpu().numpy(), want[1]) and np.array_equal(hq.cpu().numpy(), want[2])
