@@ -187,7 +187,7 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
     if (bmm_late && (s = launch_bmm(d, a->Cq, a->Bq, a->s_C, a->s_B, a->s_cb, cbq, a->tap_acc_cb, nullptr, a->status,
                                     st, true)) != SSDI8_OK)
       return s;
-    if ((s = launch_state_passing(d, loc, gamma, a->init_state, a->s_h, a->tap_prev, a->final_state, hq, st)) != SSDI8_OK)
+    if ((s = launch_state_passing(d, loc, gamma, a->init_state, a->s_h, a->tap_prev, a->final_state, hq, st, true)) != SSDI8_OK)
       return s;
   } else if (fused_state) {
     // both modules: the fused chunk-sequential kernel (the fp32 chunk-local states stay on chip)

@@ -111,9 +111,10 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
                                           int32_t* tap_acc, int32_t* status, bool int8_state,
                                           cudaStream_t st, uint32_t* absmax_h = nullptr);
 
+// forward: in place of the fused state kernel (codes of a NaN)
 ssdi8_status_t launch_state_passing(const Dims& d, const float* loc, const float* gamma,
                                     const float* init, const float* s_h, float* prev,
-                                    float* final_state, int8_t* hq, cudaStream_t st);
+                                    float* final_state, int8_t* hq, cudaStream_t st, bool forward = false);
 
 struct ScanTaps {
   int32_t* acc_off; float* rowmax; int8_t* Mq; int32_t* acc_diag;

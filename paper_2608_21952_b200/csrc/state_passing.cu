@@ -3,6 +3,8 @@
 // The only sequential loop of the layer (over chunks); everything else is parallel over
 // (b, h, p, n).  HBM-bound: each thread owns 4 consecutive n (16-byte loads of loc, 4-byte
 // packed stores of hq) and keeps several chunk loads in flight.
+#include <type_traits>
+
 #include "kernels.h"
 
 namespace ssdi8 {
@@ -10,7 +12,8 @@ namespace {
 
 // K chunks' loads are in flight at once; AHEAD: the next K too, requested before the present ones are used.  PREV: the entering
 // states are written; prev may be loc (or start before it): a chunk's load is ahead of the store that goes over it either way.
-template <bool PREV, int K, bool AHEAD, int THREADS>
+// FORWARD: inside a forward pass, in place of the fused state kernel, whose codes of a NaN (+127; -127 here) it takes over.
+template <bool FORWARD, bool PREV, int K, bool AHEAD, int THREADS>
 __global__ void __launch_bounds__(THREADS) state_passing_kernel(
     const float4* loc /* may alias prev: no __restrict__ */, const float* __restrict__ gamma, const float4* __restrict__ init,
     const float* __restrict__ s_h, float4* prev, float4* __restrict__ final_state,
@@ -43,9 +46,11 @@ __global__ void __launch_bounds__(THREADS) state_passing_kernel(
     }
   };
   auto step = [&](const float4& l, float g) {
-    if (hq)
-      hq[o] = pack4(rne_clamp(__fmul_rn(S.x, inv_h)), rne_clamp(__fmul_rn(S.y, inv_h)),
-                    rne_clamp(__fmul_rn(S.z, inv_h)), rne_clamp(__fmul_rn(S.w, inv_h)));
+    if (hq) {
+      const float4 v = make_float4(__fmul_rn(S.x, inv_h), __fmul_rn(S.y, inv_h), __fmul_rn(S.z, inv_h), __fmul_rn(S.w, inv_h));
+      hq[o] = FORWARD ? pack4_bits(rne_clamp_bits(v.x), rne_clamp_bits(v.y), rne_clamp_bits(v.z), rne_clamp_bits(v.w))
+                      : pack4(rne_clamp(v.x), rne_clamp(v.y), rne_clamp(v.z), rne_clamp(v.w));
+    }
     if (PREV) prev[o] = S;
     S.x = __fmaf_rn(g, S.x, l.x);
     S.y = __fmaf_rn(g, S.y, l.y);
@@ -90,7 +95,7 @@ __global__ void __launch_bounds__(THREADS) state_passing_kernel(
 
 ssdi8_status_t launch_state_passing(const Dims& d, const float* loc, const float* gamma,
                                     const float* init, const float* s_h, float* prev,
-                                    float* final_state, int8_t* hq, cudaStream_t st) {
+                                    float* final_state, int8_t* hq, cudaStream_t st, bool forward) {
   const i64 n = (i64)d.b * d.H * d.P * (d.N / 4);
   auto launch = [&](auto kernel, int threads) -> ssdi8_status_t {
     return launch_configured(kernel, dim3((unsigned)((n + threads - 1) / threads)), dim3(threads), 0, -1, false, st,
@@ -103,14 +108,18 @@ ssdi8_status_t launch_state_passing(const Dims& d, const float* loc, const float
   // next ahead: 8192 tokens x 24 heads 9.2 / 7.2, 32768 x 4 (chunks of 64) 54 / 36, but 8192 x 80 16.9 / 20.3.  Where prev is
   // written, one at a time / four / eight and the next ahead: 64 sequences of one chunk x 80 heads 89 / 118 / -, 2048 x 80 8.8 /
   // 6.8 / 7.0, 8192 x 80 38 / 36 / 33, 8192 x 24 9.1 / 11.6 / 8.5.
-  if (prev) {
-    if (d.c < 4) return launch(state_passing_kernel<true, 1, false, 256>, 256);
-    if (d.c < 16) return launch(state_passing_kernel<true, 4, false, 256>, 256);
-    return launch(state_passing_kernel<true, 8, true, 128>, 128);
-  }
-  if (d.c < 8) return launch(state_passing_kernel<false, 4, false, 256>, 256);
-  if (d.c < 16 || n > 96 * 1024) return launch(state_passing_kernel<false, 8, false, 256>, 256);
-  return launch(state_passing_kernel<false, 8, true, 128>, 128);
+  auto pick = [&](auto fwd) -> ssdi8_status_t {
+    constexpr bool F = decltype(fwd)::value;
+    if (prev) {
+      if (d.c < 4) return launch(state_passing_kernel<F, true, 1, false, 256>, 256);
+      if (d.c < 16) return launch(state_passing_kernel<F, true, 4, false, 256>, 256);
+      return launch(state_passing_kernel<F, true, 8, true, 128>, 128);
+    }
+    if (d.c < 8) return launch(state_passing_kernel<F, false, 4, false, 256>, 256);
+    if (d.c < 16 || n > 96 * 1024) return launch(state_passing_kernel<F, false, 8, false, 256>, 256);
+    return launch(state_passing_kernel<F, false, 8, true, 128>, 128);
+  };
+  return forward ? pick(std::true_type{}) : pick(std::false_type{});
 }
 
 }  // namespace ssdi8

@@ -328,3 +328,20 @@ def test_state_passing_on_either_side_of_the_thread_limit(b, H):
     bd.ssdi8_state_passing(bd.dims_of(cfg), gh.dev(loc), gh.dev(gamma), None, None, fin, hq, gh.dev(s_h))
     torch.cuda.synchronize()
     assert np.array_equal(fin.cpu().numpy(), want[1]) and np.array_equal(hq.cpu().numpy(), want[2])
+
+
+def test_a_state_that_is_not_a_number_has_the_same_codes_on_both_state_routes():
+    # 9 chunks take the two kernels, the same call with the INT8 state flag off and more heads the fused one: the codes of the
+    # first chunk's entering state are those of init_state alone
+    import gpu_harness as gh
+    few = SSDConfig("few", 1, 9 * 64, 4, 64, 64, 1, 64, 0.02, 20.0, 50)
+    many = SSDConfig("many", 1, 9 * 64, 160, 64, 64, 1, 64, 0.02, 20.0, 50)
+    hq = []
+    for cfg in (few, many):
+        q = _random_codes(cfg, 50)
+        q["init"][:] = 0.25
+        q["init"][0, 1, 7, 3:9] = np.array([0x7fc00000, 0xffc00000, 0x7f800000, 0xff800000, 0x00000000, 0x80000000],
+                                           np.uint32).view(np.float32)
+        q["s_h"][64:66] = 0.0
+        hq.append(gh.gpu_fwd(cfg, q, taps=("hq",))[2]["hq"][0, 0, :4])
+    assert np.array_equal(hq[0], hq[1])
