@@ -330,7 +330,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
         }
         if (CAL) {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) smax[CAL ? p0 + e : 0] = fabsf(__int_as_float(sv[e]));
+          for (int e = 0; e < 8; ++e) smax[CAL ? p0 + e : 0] = fmaxf(fabsf(__int_as_float(sv[e])), 0.f);   // (a NaN counts for nothing)
         }
         tmem_st8(tS + (uint32_t)p0, sv);
       }

@@ -345,3 +345,28 @@ def test_a_state_that_is_not_a_number_has_the_same_codes_on_both_state_routes():
         q["s_h"][64:66] = 0.0
         hq.append(gh.gpu_fwd(cfg, q, taps=("hq",))[2]["hq"][0, 0, :4])
     assert np.array_equal(hq[0], hq[1])
+
+
+@pytest.mark.parametrize("b,c,H,N", [(1, 3, 5, 64), (2, 1, 150, 128)])
+def test_calibration_passes_over_states_that_are_not_a_number(b, c, H, N):
+    # A NaN in init_state counts for nothing in the step size of its channel, as one anywhere else does: the step sizes are
+    # those with a zero in its place in every other channel, and finite in its own
+    import torch
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("cal_nan", b, c * 64, H, 64, N, 1, 64, 0.02, 20.0, 51)
+    q = _random_codes(cfg, 51)
+    at = ((0, 1, 7, 5), (b - 1, H - 1, 63, N - 1))
+    s_h = []
+    for bad in (0.0, np.nan):
+        init = q["init"].copy()
+        for i in at:
+            init[i] = bad
+        dv = {k: gh.dev(q[k]) for k in ("xq", "Bq", "Cq", "s_x", "s_B", "s_C", "dt", "A")}
+        s = [torch.empty(n, device="cuda") for n in (H * 64, 1, H * 64)]
+        bd.ssdi8_calibrate(bd.dims_of(cfg), bd.make_fwd_args(init_state=gh.dev(init), **dv), *s, bd.alloc_workspace(bd.dims_of(cfg)))
+        s_h.append(s[2].cpu().numpy())
+    own = np.zeros(H * 64, bool)
+    own[[h * 64 + p for _, h, p, _ in at]] = True
+    assert np.array_equal(s_h[0][~own], s_h[1][~own])
+    assert np.all(np.isfinite(s_h[1])) and np.all(s_h[1][own] <= s_h[0][own]) and np.all(s_h[1][own] > 0)
