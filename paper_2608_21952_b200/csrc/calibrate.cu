@@ -15,6 +15,7 @@ constexpr int kXsHeads = 8, kXsTokens = 64;
 __global__ void __launch_bounds__(256) absmax_xs_kernel(const int8_t* __restrict__ xq, const float* __restrict__ s_x,
                                                         const float* __restrict__ pack, uint32_t* __restrict__ absmax, Dims d) {
   __shared__ __align__(16) float lut[kXsHeads][kXsTokens];
+  __shared__ __align__(16) float sxs[kXsHeads * 64];
   __shared__ uint32_t best[8][kXsHeads * 64];
   pdl_launch_dependents();
   pdl_wait();
@@ -26,6 +27,10 @@ __global__ void __launch_bounds__(256) absmax_xs_kernel(const int8_t* __restrict
     const int hh = e / nt, i = e % nt;
     if (h0 + hh < d.H) lut[hh][i] = __ldg(pack + ((((i64)b * d.H + h0 + hh) * d.c + k) * kPackRows + PACK_LUT) * d.Q + i0 + i);
   }
+  // (by way of shared memory: ssdi8_calibrate asks for no alignment of s_x beyond a float's, and sixteen loads of one float per
+  // thread were 4 us slower)
+  for (int e = tid; e < kXsHeads * 64; e += 256)
+    if (h0 + (e >> 6) < d.H) sxs[e] = __ldg(s_x + h0 * 64 + e);
   const int hh = (tid >> 2) & 7, c = tid & 3, row = tid >> 5;   // head, 16 channels, token row of the thread
   const int h = h0 + hh;
   float mx[16];
@@ -36,7 +41,7 @@ __global__ void __launch_bounds__(256) absmax_xs_kernel(const int8_t* __restrict
     float2 sx[8];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(s_x + h * 64 + c * 16) + e);
+      const float4 v = *(reinterpret_cast<const float4*>(&sxs[hh * 64 + c * 16]) + e);
       sx[2 * e] = make_float2(v.x, v.y);
       sx[2 * e + 1] = make_float2(v.z, v.w);
     }

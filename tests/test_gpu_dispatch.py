@@ -370,3 +370,24 @@ def test_calibration_passes_over_states_that_are_not_a_number(b, c, H, N):
     own[[h * 64 + p for _, h, p, _ in at]] = True
     assert np.array_equal(s_h[0][~own], s_h[1][~own])
     assert np.all(np.isfinite(s_h[1])) and np.all(s_h[1][own] <= s_h[0][own]) and np.all(s_h[1][own] > 0)
+
+
+def test_calibration_takes_slices_of_packed_step_sizes():
+    # s_x, s_B, s_C, A and the outputs 4-byte aligned only
+    import torch
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("cal_slices", 1, 3 * 128, 9, 64, 64, 3, 128, 0.02, 20.0, 52)
+    q = _random_codes(cfg, 52)
+    dims = bd.dims_of(cfg)
+    HP, G = cfg.channels, cfg.ngroups
+    dv = {k: gh.dev(q[k]) for k in ("xq", "Bq", "Cq", "s_x", "s_B", "s_C", "dt", "A")}
+    dv["s_x"] = dv["s_x"] * torch.linspace(0.5, 2.0, HP, device="cuda")
+    got = []
+    for shift in (0, 1, 2, 3):
+        put = lambda t: torch.cat([torch.zeros(shift, device="cuda"), t])[shift:]
+        args = bd.make_fwd_args(**{k: put(v) if k in ("s_x", "s_B", "s_C", "A") else v for k, v in dv.items()})
+        s = [torch.empty(n + shift, device="cuda")[shift:] for n in (HP, G, HP)]
+        bd.ssdi8_calibrate(dims, args, *s, bd.alloc_workspace(dims))
+        got.append(torch.cat(s).cpu().numpy())
+    assert all(np.array_equal(g, got[0]) for g in got[1:])
