@@ -20,9 +20,11 @@ __global__ void __launch_bounds__(256) absmax_xs_kernel(const int8_t* __restrict
   pdl_launch_dependents();
   pdl_wait();
   const int tid = threadIdx.x;
-  const int h0 = blockIdx.x * kXsHeads, k = blockIdx.y / (d.Q / kXsTokens), b = blockIdx.z;
+  // (head blocks and token blocks in one grid dimension: a sequence of more than 4 M tokens has more than 65535 of the latter)
+  const int nhb = (d.H + kXsHeads - 1) / kXsHeads, tb = blockIdx.x / nhb, b = blockIdx.z;
+  const int h0 = (blockIdx.x - tb * nhb) * kXsHeads, k = tb / (d.Q / kXsTokens);
   constexpr int nt = kXsTokens;
-  const int i0 = (blockIdx.y % (d.Q / kXsTokens)) * nt;   // tokens of this block
+  const int i0 = (tb % (d.Q / kXsTokens)) * nt;   // tokens of this block
   for (int e = tid; e < kXsHeads * nt; e += 256) {
     const int hh = e / nt, i = e % nt;
     if (h0 + hh < d.H) lut[hh][i] = __ldg(pack + ((((i64)b * d.H + h0 + hh) * d.c + k) * kPackRows + PACK_LUT) * d.Q + i0 + i);
@@ -105,7 +107,9 @@ __global__ void finalize_scales(float* s, int n, float* q, int nq, const float* 
 
 ssdi8_status_t launch_absmax_xs(const Dims& d, const int8_t* xq, const float* s_x, const float* pack, uint32_t* absmax,
                                 cudaStream_t st) {
-  const dim3 grid((d.H + kXsHeads - 1) / kXsHeads, d.c * (d.Q / kXsTokens), d.b);
+  const i64 blocks = (i64)((d.H + kXsHeads - 1) / kXsHeads) * d.c * (d.Q / kXsTokens);
+  if (blocks > 0x7fffffff) return SSDI8_ERR_SHAPE;
+  const dim3 grid((unsigned)blocks, 1, d.b);
   return launch_configured(absmax_xs_kernel, grid, dim3(256), 0, kStreamCarveout, false, st, xq, s_x, pack, absmax, d);
 }
 

@@ -391,3 +391,25 @@ def test_calibration_takes_slices_of_packed_step_sizes():
         bd.ssdi8_calibrate(dims, args, *s, bd.alloc_workspace(dims))
         got.append(torch.cat(s).cpu().numpy())
     assert all(np.array_equal(g, got[0]) for g in got[1:])
+
+
+def test_calibration_on_a_sequence_of_more_than_four_million_tokens():
+    # s_xs and s_cb do not depend on how the chunks are shared out among batch elements
+    import torch
+    from paper_2608_21952_b200 import binding as bd
+    g = torch.Generator(device="cuda").manual_seed(53)
+    T = 256 * 5 * 3277
+    i8 = lambda: torch.randint(-127, 128, (T, 64), generator=g, device="cuda", dtype=torch.int8)
+    q = dict(xq=i8(), Bq=i8(), Cq=i8(), dt=0.01 + 0.1 * torch.rand(T, 1, generator=g, device="cuda"),
+             A=torch.full((1,), -0.5, device="cuda"), s_x=0.01 + torch.rand(64, generator=g, device="cuda"),
+             s_B=torch.full((1,), 0.03, device="cuda"), s_C=torch.full((1,), 0.03, device="cuda"))
+    got = []
+    for b in (1, 5):
+        dims = bd.Dims(b, T // b, 1, 64, 64, 1, 256)
+        s = [torch.empty(n, device="cuda") for n in (64, 1, 64)]
+        ws = bd.alloc_workspace(dims)
+        bd.ssdi8_calibrate(dims, bd.make_fwd_args(**q), *s, ws)
+        got.append([t.cpu().numpy() for t in s])
+        del ws
+    assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
+    assert np.all(np.isfinite(got[0][2])) and np.all(got[0][2] > 0)
