@@ -272,6 +272,7 @@ ssdi8_status_t ssdi8_chunk_scan_fwd_static(const ssdi8_dims_t* dims, const ssdi8
  *   on two copy streams while the kernels of a slice run, so both directions of the host link stay
  *   busy.  scratch: DEVICE, 256-byte aligned, ssdi8_layer_fwd_host_scratch_bytes(dims, flags) bytes
  *   (three stages of one slice's tensors).
+ *   Calls from several threads, each with its stream and scratch, are enqueued one after the other.
  * Layouts as in ssdi8_fwd_args_t; D, corr, init_state, final_state, status may be NULL.  Both calls
  * return once everything is enqueued and leave `stream` waiting for the last piece of work, so
  * synchronising `stream` completes them.  flags: any of SSDI8_FLAG_INT8_STATE, SSDI8_FLAG_Y_FP16,

@@ -112,9 +112,12 @@ Layout make_layout(const ssdi8_dims_t& d, const Cut& c, uint8_t* base, uint32_t 
   return lo;
 }
 
-// copy streams and events of the host-buffer entry point, made once per device and kept for the life of the process
+// Copy streams and events of the host-buffer entry point, made once per device and kept for the life of the process.  All
+// calls on a device share them, so a call holds `enqueue` while it enqueues: a wait for an event means the last record ahead
+// of it, and two calls whose records and waits mixed would wait for each other's kernels instead of their own.
 struct Plumbing {
   bool ready = false;
+  std::mutex enqueue;
   cudaStream_t s_in = nullptr, s_out = nullptr;
   cudaEvent_t start = nullptr, in_done[kStages] = {}, cmp_done[kStages] = {}, out_done[kStages] = {}, blk_done[kBlocks] = {},
               gate[2] = {};
@@ -255,6 +258,7 @@ ssdi8_status_t ssdi8_layer_fwd_host(const ssdi8_dims_t* dims, const ssdi8_layer_
   Plumbing* p = nullptr;
   ssdi8_status_t s = get_plumbing(&p);
   if (s != SSDI8_OK) return s;
+  std::lock_guard<std::mutex> lock(p->enqueue);
   cudaStream_t s_cmp = static_cast<cudaStream_t>(stream);
   const size_t L = dims->seqlen, D = (size_t)dims->nheads * dims->headdim, H = dims->nheads;
   const size_t GN = (size_t)dims->ngroups * dims->dstate, nstate = D * dims->dstate;   // state of an element

@@ -413,3 +413,52 @@ def test_calibration_on_a_sequence_of_more_than_four_million_tokens():
         del ws
     assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
     assert np.all(np.isfinite(got[0][2])) and np.all(got[0][2] > 0)
+
+
+def test_host_pipeline_calls_from_several_threads():
+    # each thread with its stream, scratch, buffers and inputs; slices in one piece per call and in many
+    import threading
+    import torch
+    from paper_2608_21952_b200 import binding as bd
+
+    def setup(seed, b, c, H):
+        cfg = SSDConfig("threads", b, c * 128, H, 64, 64, 1, 128, 0.02, 20.0, seed)
+        dims = bd.dims_of(cfg)
+        g = torch.Generator().manual_seed(seed)
+        T, HP = cfg.tokens, cfg.channels
+        r = lambda *s: torch.randn(*s, generator=g)
+        host = {"x": r(T, HP), "B": r(T, 64), "C": r(T, 64), "dt": torch.nn.functional.softplus(r(T, H) - 3.0)}
+        host = {k: v.pin_memory() for k, v in host.items()}
+        par = {"A": -torch.exp(r(H)), "D": r(H), "s_x": torch.full((HP,), 0.03), "s_B": torch.full((1,), 0.03),
+               "s_C": torch.full((1,), 0.03), "s_xs": torch.full((HP,), 0.002), "s_cb": torch.full((1,), 0.4),
+               "s_h": torch.full((HP,), 0.02)}
+        par = {k: v.cuda() for k, v in par.items()}
+        y, fin = torch.empty(T, HP, device="cuda"), torch.empty(b, H, 64, 64, device="cuda")
+        ws = torch.empty(bd.ssdi8_layer_fwd_workspace_bytes(dims, 0), dtype=torch.uint8, device="cuda")
+        bd.ssdi8_layer_fwd(dims, bd.make_layer_args(y=y, final_state=fin, **{k: v.cuda() for k, v in host.items()}, **par), ws)
+        torch.cuda.synchronize()
+        scratch = torch.empty(bd.ssdi8_layer_fwd_host_scratch_bytes(dims, 0), dtype=torch.uint8, device="cuda")
+        return dims, host, par, scratch, y.cpu(), fin.cpu()
+
+    work = [setup(60, 2, 12, 40), setup(61, 9, 1, 80), setup(62, 1, 9, 200)]
+    wrong = []
+
+    def run(dims, host, par, scratch, y, fin):
+        try:
+            stream = torch.cuda.Stream()
+            for _ in range(8):
+                yh = torch.full(y.shape, float("nan")).pin_memory()
+                fh = torch.full(fin.shape, float("nan")).pin_memory()
+                bd.ssdi8_layer_fwd_host(dims, bd.make_host_args(y=yh, final_state=fh, **host, **par), scratch, stream=stream)
+                stream.synchronize()
+                if not (torch.equal(yh, y) and torch.equal(fh, fin)):
+                    wrong.append(dims.nheads)
+        except BaseException as e:   # noqa: BLE001 (a thread's exception would not fail the test)
+            wrong.append(e)
+
+    threads = [threading.Thread(target=run, args=w) for w in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
