@@ -147,6 +147,19 @@ ssdi8_status_t get_plumbing(Plumbing** out) {
   return SSDI8_OK;
 }
 
+// Leaves the caller's stream behind the copy streams when a call ends early: copies that it has enqueued still read
+// and write the caller's buffers.
+struct JoinOnError {
+  Plumbing* p;
+  cudaStream_t st;
+  bool armed = true;
+  ~JoinOnError() {
+    if (!armed) return;
+    for (cudaStream_t side : {p->s_in, p->s_out})
+      if (cudaEventRecord(p->start, side) == cudaSuccess) (void)cudaStreamWaitEvent(st, p->start, 0);
+  }
+};
+
 struct LayerWs {
   int8_t *xq, *Bq, *Cq;
   void* ws;
@@ -268,6 +281,7 @@ ssdi8_status_t ssdi8_layer_fwd_host(const ssdi8_dims_t* dims, const ssdi8_layer_
   SSDI8_CUDA_CHECK(cudaEventRecord(p->start, s_cmp));
   SSDI8_CUDA_CHECK(cudaStreamWaitEvent(p->s_in, p->start, 0));
   SSDI8_CUDA_CHECK(cudaStreamWaitEvent(p->s_out, p->start, 0));
+  JoinOnError join{p, s_cmp};
 
   struct Slice {
     size_t b0, t0, nb, Lt, tok0, T;   // first element, first token in it, elements, tokens of each; the same over all tokens
@@ -345,6 +359,7 @@ ssdi8_status_t ssdi8_layer_fwd_host(const ssdi8_dims_t* dims, const ssdi8_layer_
   // the caller's stream ends after the last copies (one stream, in order: its last event covers all)
   SSDI8_CUDA_CHECK(cudaEventRecord(p->start, p->s_out));
   SSDI8_CUDA_CHECK(cudaStreamWaitEvent(s_cmp, p->start, 0));
+  join.armed = false;
   if (a->status)
     SSDI8_CUDA_CHECK(cudaMemcpyAsync(a->status, lo.status, sizeof(int32_t), cudaMemcpyDeviceToHost, s_cmp));
   return SSDI8_OK;

@@ -462,3 +462,30 @@ def test_host_pipeline_calls_from_several_threads():
     for t in threads:
         t.join()
     assert not wrong
+
+
+def test_host_pipeline_that_ends_early_leaves_the_stream_behind_its_copies():
+    # an initial state that is not 16-byte aligned is refused by the first slice's kernels, with the slice's copies on their way:
+    # after the caller's stream they are complete
+    import torch
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("early", 1, 24 * 128, 80, 64, 64, 1, 128, 0.02, 20.0, 63)
+    dims = bd.dims_of(cfg)
+    T, HP = cfg.tokens, cfg.channels
+    pin = lambda *s: torch.randn(*s).pin_memory()
+    x, y = pin(T, HP), torch.empty(T, HP).pin_memory()
+    c = lambda n: torch.ones(n, device="cuda")
+    init = torch.zeros(80 * 64 * 64 + 1, device="cuda")[1:]
+    scratch = torch.zeros(bd.ssdi8_layer_fwd_host_scratch_bytes(dims, 0), dtype=torch.uint8, device="cuda")
+    args = bd.make_host_args(x=x, B=pin(T, 64), C=pin(T, 64), dt=torch.rand(T, 80).pin_memory(), A=-c(80), y=y, init_state=init,
+                             s_x=c(HP), s_B=c(1), s_C=c(1), s_xs=c(HP), s_cb=c(1), s_h=c(HP))
+    torch.cuda.synchronize()
+    with pytest.raises(bd.SSDi8Error) as e:
+        bd.ssdi8_layer_fwd_host(dims, args, scratch)
+    first = scratch[:128 * HP * 4].clone()   # x of the first chunk, at the start of the scratch
+    assert e.value.code == bd.ERR_ALIGN
+    assert torch.equal(first.view(torch.float32).cpu(), x[:128].reshape(-1))
+    args.init_state = 0
+    bd.ssdi8_layer_fwd_host(dims, args, scratch)
+    torch.cuda.synchronize()
+    assert torch.isfinite(y).all()
