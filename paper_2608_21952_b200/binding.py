@@ -71,6 +71,9 @@ class LayerArgs(C.Structure):
     _fields_ = [(k, C.c_void_p) for k in _LAYER_FIELDS]
 
 
+_m.init(Dims, FwdArgs, LayerArgs, C.Structure.__base__, C.ArgumentError)
+
+
 _lib.ssdi8_status_string.restype = C.c_char_p
 _lib.ssdi8_status_string.argtypes = [C.c_int32]
 _lib.ssdi8_workspace_bytes.restype = C.c_size_t

@@ -1,6 +1,6 @@
 // Argument marshalling of the Python binding (paper_2608_21952_b200/binding.py): torch tensors and ctypes structures
 // to the pointers the C entry points take, the current stream, the call with the interpreter lock released.  No
-// arithmetic and no checks beyond the ones a pointer needs (a contiguous CUDA tensor).
+// arithmetic and no checks beyond the ones a pointer needs (a contiguous CUDA tensor, the right ctypes structure).
 // Why native: through ctypes a call with a dozen tensors took 9 to 13 us of host time (0.25 us per tensor for
 // its type checks and address, 3.4 us for the stream object) ahead of a launch of 3 us, more than the device time of
 // a decode step of one sequence (7 us for its three calls); from here a call takes 3.5 to 4 us, launch included, and
@@ -52,10 +52,24 @@ float real(PyObject* o) {
   return (float)v;
 }
 
+// The binding's ctypes types, given once at its import (init): a structure of another type, or any other object with a
+// buffer, would be read as pointers and sizes that it does not hold.  The errors are those of ctypes' byref and argtypes.
+struct Types {
+  PyObject *dims = nullptr, *fwd = nullptr, *layer = nullptr, *ctypes_base = nullptr, *argument_error = nullptr;
+} g_types;
+
 // the memory of a ctypes structure
 struct Struct {
   Py_buffer b{};
-  Struct(PyObject* o, size_t bytes) {
+  Struct(PyObject* o, PyObject* type, size_t bytes) {
+    const auto is_a = [o](PyObject* t) { return t != nullptr && PyObject_TypeCheck(o, reinterpret_cast<PyTypeObject*>(t)); };
+    if (!is_a(type)) {
+      if (is_a(g_types.ctypes_base))
+        PyErr_Format(g_types.argument_error, "expected %R instead of %R", type, reinterpret_cast<PyObject*>(Py_TYPE(o)));
+      else
+        PyErr_Format(PyExc_TypeError, "a ctypes structure is expected, not '%s'", Py_TYPE(o)->tp_name);
+      throw BadArgument{};
+    }
     if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) throw BadArgument{};
     if ((size_t)b.len < bytes) {
       PyBuffer_Release(&b);
@@ -68,15 +82,15 @@ struct Struct {
   Struct& operator=(const Struct&) = delete;
 };
 struct DimsArg : Struct {
-  explicit DimsArg(PyObject* o) : Struct(o, sizeof(ssdi8_dims_t)) {}
+  explicit DimsArg(PyObject* o) : Struct(o, g_types.dims, sizeof(ssdi8_dims_t)) {}
   const ssdi8_dims_t* get() const { return static_cast<const ssdi8_dims_t*>(b.buf); }
 };
 struct FwdArg : Struct {
-  explicit FwdArg(PyObject* o) : Struct(o, sizeof(ssdi8_fwd_args_t)) {}
+  explicit FwdArg(PyObject* o) : Struct(o, g_types.fwd, sizeof(ssdi8_fwd_args_t)) {}
   const ssdi8_fwd_args_t* get() const { return static_cast<const ssdi8_fwd_args_t*>(b.buf); }
 };
 struct LayerArg : Struct {
-  explicit LayerArg(PyObject* o) : Struct(o, sizeof(ssdi8_layer_args_t)) {}
+  explicit LayerArg(PyObject* o) : Struct(o, g_types.layer, sizeof(ssdi8_layer_args_t)) {}
   const ssdi8_layer_args_t* get() const { return static_cast<const ssdi8_layer_args_t*>(b.buf); }
 };
 
@@ -120,6 +134,18 @@ PyObject* entry(Py_ssize_t n, F f) {
 
 #define ENTRY(NAME, N) PyObject* NAME(PyObject*, PyObject* const* a, Py_ssize_t n) { return entry<N>(n, [&]() -> PyObject*
 #define END ); }
+
+ENTRY(init, 5) {   // Dims, FwdArgs, LayerArgs, the base type of ctypes objects, ctypes.ArgumentError
+  for (int i = 0; i < 5; ++i) {
+    if (!PyType_Check(a[i])) {
+      PyErr_SetString(PyExc_TypeError, "a type is expected");
+      throw BadArgument{};
+    }
+    Py_INCREF(a[i]);   // (kept for the life of the process, like the module)
+  }
+  g_types = {a[0], a[1], a[2], a[3], a[4]};
+  Py_RETURN_NONE;
+} END
 
 ENTRY(quantize_act, 8) {   // inp, R, Ch, I, scale, mode, out, stream
   const float* in = ptr_as<const float>(a[0]);
@@ -239,7 +265,7 @@ ENTRY(softplus_dt, 6) {   // dt_raw, dt_bias, rows, H, dt, stream
 #undef END
 
 #define METHOD(NAME) {#NAME, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(NAME)), METH_FASTCALL, nullptr}
-PyMethodDef kMethods[] = {METHOD(quantize_act), METHOD(quantize_entry), METHOD(chunk_scan_fwd), METHOD(chunk_scan_fwd_static),
+PyMethodDef kMethods[] = {METHOD(init), METHOD(quantize_act), METHOD(quantize_entry), METHOD(chunk_scan_fwd), METHOD(chunk_scan_fwd_static),
                           METHOD(layer_fwd), METHOD(layer_fwd_host), METHOD(calibrate), METHOD(mean_correction),
                           METHOD(state_passing), METHOD(ssd_step), METHOD(softplus_dt), {nullptr, nullptr, 0, nullptr}};
 #undef METHOD

@@ -196,3 +196,39 @@ def test_host_side_argument_errors_of_the_layer_and_entry_calls():
     assert q(4096, 3, 16, 64, 1, 16, 4096, 4096, 4096, 4096, 4096, 4096, None) == bd.ERR_UNSUPPORTED
     assert q(4096, 0, 16, 62, 1, 16, 4096, 4096, 4096, 4096, 4096, 4096, None) == bd.ERR_SHAPE
     assert q(4096 + 4, 0, 16, 64, 1, 16, 4096, 4096, 4096, 4096, 4096, 4096, None) == bd.ERR_ALIGN
+
+
+def test_binding_refuses_other_structures():
+    """A structure of another type or another object with a buffer is refused before its memory is read as pointers, by the
+    errors of ctypes; the right type and its subclasses pass on to the next argument."""
+    import numpy as np
+    from paper_2608_21952_b200 import binding as bd
+    d, f, a = bd.Dims(), bd.FwdArgs(), bd.LayerArgs()
+    big = np.zeros(4096, np.uint8)
+
+    class Sub(bd.Dims):
+        pass
+
+    calls = [lambda x, y: bd.ssdi8_chunk_scan_fwd(x, y, None), lambda x, y: bd.ssdi8_chunk_scan_fwd_static(x, y, flags="none"),
+             lambda x, y: bd.ssdi8_calibrate(x, y, None, None, None, None),
+             lambda x, y: bd.ssdi8_layer_fwd(x, y, None), lambda x, y: bd.ssdi8_layer_fwd_host(x, y, None)]
+    for call, right, wrong in zip(calls, (f, f, f, a, a), (a, a, a, f, f)):
+        for bad in (wrong, d, C.c_int(3), C.pointer(right)):
+            with pytest.raises(C.ArgumentError):
+                call(d, bad)
+        for bad in (right, wrong):
+            with pytest.raises(C.ArgumentError):
+                call(bad, right)
+        for bad in (None, b"0" * 4096, bytearray(4096), big, 4096, C.byref(d)):
+            with pytest.raises(TypeError):
+                call(d, bad)
+            with pytest.raises(TypeError):
+                call(bad, right)
+        for dims in (d, Sub()):
+            with pytest.raises(TypeError, match="workspace|integer"):
+                call(dims, right)
+    for call in (lambda x: bd.ssdi8_state_passing(x, *[None] * 7), lambda x: bd.ssdi8_ssd_step(x, *[None] * 12)):
+        with pytest.raises(C.ArgumentError):
+            call(f)
+        with pytest.raises(TypeError):
+            call(big)
