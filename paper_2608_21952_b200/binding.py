@@ -23,7 +23,13 @@ if not os.path.exists(_LIB_PATH):
 _lib = C.CDLL(_LIB_PATH)
 if not os.path.exists(_build.MARSHAL):
     raise ImportError(f"{_build.MARSHAL} is missing: build it with `python -m paper_2608_21952_b200.build`")
-from . import _marshal as _m  # noqa: E402  (linked against the library loaded above)
+_REBUILD = "build it again for the installed torch with `python -m paper_2608_21952_b200.build`"
+try:
+    from . import _marshal as _m  # noqa: E402  (linked against the library loaded above)
+except ImportError as e:
+    raise ImportError(f"{_build.MARSHAL} does not load with torch {torch.__version__}: {_REBUILD}") from e
+if _m.TORCH_VERSION != torch.__version__:   # (it reads torch's C++ objects, whose layout is that of one torch build)
+    raise ImportError(f"{_build.MARSHAL} was compiled against torch {_m.TORCH_VERSION}, not {torch.__version__}: {_REBUILD}")
 
 OK = 0
 ERR_NULL, ERR_SHAPE, ERR_ALIGN, ERR_WORKSPACE, ERR_ARCH, ERR_CUDA, ERR_DEVICE_TIMEOUT, ERR_UNSUPPORTED = \

@@ -274,4 +274,9 @@ PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, kMethods,
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__marshal() { return PyModule_Create(&kModule); }
+PyMODINIT_FUNC PyInit__marshal() {
+  PyObject* m = PyModule_Create(&kModule);
+  // the torch whose C++ classes this was compiled against: the binding compares it with the torch that is loaded
+  if (m && PyModule_AddStringConstant(m, "TORCH_VERSION", SSDI8_TORCH_VERSION) != 0) Py_CLEAR(m);
+  return m;
+}

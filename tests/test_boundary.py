@@ -232,3 +232,30 @@ def test_binding_refuses_other_structures():
             call(f)
         with pytest.raises(TypeError):
             call(big)
+
+
+def test_marshalling_module_belongs_to_one_torch(monkeypatch, tmp_path):
+    """build() compiles the marshalling module again for another torch, not for the same one; the binding refuses one that was
+    compiled against another."""
+    import subprocess
+    import sys
+    from paper_2608_21952_b200 import build
+    build.build()
+    stamp = tmp_path / "built_for"
+    stamp.write_text(open(build.MARSHAL_STAMP).read())
+    monkeypatch.setattr(build, "MARSHAL_STAMP", str(stamp))
+    ran = []
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, check: ran.append(cmd))
+    build.build_marshal()
+    assert not ran
+    good = stamp.read_text()
+    stamp.write_text(good.replace("torch ", "torch 0."))
+    build.build_marshal()
+    assert len(ran) == 1 and stamp.read_text() == good
+    stamp.unlink()
+    build.build_marshal()
+    assert len(ran) == 2
+    code = "import torch; torch.__version__ = '0.0'; from paper_2608_21952_b200 import binding"
+    monkeypatch.undo()
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode != 0 and "ImportError" in r.stderr and "build it again" in r.stderr
