@@ -50,7 +50,7 @@ struct Workspace {
   size_t pack, gamma, cbq, loc, hq, total;
 };
 
-Workspace layout(const Dims& d, bool fp16_operand = false) {
+Workspace layout(const Dims& d) {
   Workspace w;
   size_t o = 0;
   const size_t nst = (size_t)d.b * d.c * d.H * d.P * d.N;
@@ -59,7 +59,6 @@ Workspace layout(const Dims& d, bool fp16_operand = false) {
   w.cbq = o;   o = align_up(o + (size_t)d.b * d.c * d.G * d.Q * d.Q, 256);
   w.loc = o;   o = align_up(o + sizeof(float) * nst, 256);
   w.hq = o;    o = align_up(o + nst, 256);
-  (void)fp16_operand;   // the FP16 operand needs no scratch of its own
   w.total = o;
   return w;
 }
@@ -85,7 +84,7 @@ const char* ssdi8_status_string(ssdi8_status_t s) {
 
 size_t ssdi8_workspace_bytes(const ssdi8_dims_t* dims, uint32_t flags) {
   if ((flags & ~kFwdFlags) != 0 || !dims_supported(dims, true)) return 0;
-  return layout(make_dims(dims), (flags & SSDI8_FLAG_FP16_OPERAND) != 0).total;
+  return layout(make_dims(dims)).total;
 }
 
 ssdi8_status_t ssdi8_quantize_act(const float* in, int64_t R, int64_t Ch, int64_t I, float* scale,
@@ -111,12 +110,6 @@ ssdi8_status_t ssdi8_chunk_scan_fwd(const ssdi8_dims_t* dims, const ssdi8_fwd_ar
 }  // extern "C"
 
 namespace ssdi8 {
-void workspace_pack_gamma(const Dims& d, void* workspace, float** pack, float** gamma) {
-  const Workspace w = layout(d);
-  *pack = reinterpret_cast<float*>(static_cast<char*>(workspace) + w.pack);
-  *gamma = reinterpret_cast<float*>(static_cast<char*>(workspace) + w.gamma);
-}
-
 ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, uint32_t flags, void* workspace,
                           size_t workspace_bytes, void* stream, bool clear_status) {
   if (!dims || !a) return SSDI8_ERR_NULL;
@@ -144,7 +137,7 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
     if (p && !aligned16(p)) return SSDI8_ERR_ALIGN;
   if (reinterpret_cast<uintptr_t>(workspace) & 255u) return SSDI8_ERR_ALIGN;
   const Dims d = make_dims(dims);
-  const Workspace w = layout(d, f16op);
+  const Workspace w = layout(d);
   if (workspace_bytes < w.total) return SSDI8_ERR_WORKSPACE;
   ssdi8_status_t s = check_arch();
   if (s != SSDI8_OK) return s;

@@ -5,11 +5,10 @@
 //   loc[p,n]    = fmul(float(acc_st), fmul(s_xs[h,p], s_B[g]))                         (Eq. 4 rescale)
 //   hq[k][p,n]  = rne(fmul(S[p,n], fdiv(1, s_h[h,p])))     (state entering chunk k, int8 for ChunkScan1)
 //   S[p,n]      = fmaf(Gamma_k, S[p,n], loc[p,n])                                      (Eq. 6)
-// and final_state = S after the last chunk.  The running state lives in registers: the
-// accumulator has the state index n on the TMEM lanes, so thread (lane n) keeps S[., n] for its
-// 32 channels p; the state itself is kept in tensor memory beside the accumulator (64 more columns,
-// read and written 8 columns at a time), which leaves the threads with few registers so that three CTAs
-// fit an SM: the kernel is a chain of short dependent steps per chunk, and what fills an SM is other
+// and final_state = S after the last chunk.  The accumulator has the state index n on the TMEM lanes, so thread
+// (lane n) works on S[., n] of its 32 channels p; the running state is kept in tensor memory beside the
+// accumulator (64 more columns, read and written 8 columns at a time), which leaves the threads with few
+// registers so that three CTAs fit an SM: the kernel is a chain of short dependent steps per chunk, and what fills an SM is other
 // CTAs' chains.  Three warps re-quantise the xq rows up to two chunks ahead, a fourth issues the MMAs
 // and requests the tiles by TMA: xq double-buffered across chunks, Bq single-buffered (requested
 // when the MMAs of the chunk before have finished); hq leaves through
@@ -36,8 +35,7 @@ struct FusedArgs {
   const float* gamma; const float* init; float* final_state;
   float* tap_loc; float* tap_prev; int8_t* tap_Xsq; int32_t* tap_acc; int32_t* status; uint32_t* absmax_h;
   Dims d;
-  int n_full;  // CTAs below this index own a whole (batch, head); the rest own one part of one
-  int split;   // parts per (batch, head) of the rest: 2 (halves of 32 channels) or 4 (quarters of 16)
+  int n_full;  // CTAs below this index own a whole (batch, head); the rest own a quarter (16 channels) of one
 };
 
 constexpr int kStateThreads = 256;   // warps 0-7: running state, hq and its TMA stores
@@ -166,7 +164,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
   if (warp >= kStateThreads / 32) {
     // ------------------------------------------------------------ Q(X_scaled), one chunk ahead of the state warps
     const int qt = tid - kStateThreads;
-    constexpr int lq = ncq == 4 ? 2 : ncq == 2 ? 1 : 0;  // log2(chunks per row in this CTA's range)
+    constexpr int lq = ncq == 4 ? 2 : 0;  // log2(chunks per row in this CTA's range)
     const int c = c0 + (qt & (ncq - 1));  // 16-byte chunk (16 channels) of every row this thread visits
     float rx[16];
 #pragma unroll
@@ -179,7 +177,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     float rxm = 0.f;
 #pragma unroll
     for (int e = 0; e < 16; ++e) rxm = fmaxf(rxm, fabsf(rx[e]));
-    if (ncq >= 2) rxm = fmaxf(rxm, __shfl_xor_sync(0xffffffffu, rxm, 1));
+    if (ncq == 4) rxm = fmaxf(rxm, __shfl_xor_sync(0xffffffffu, rxm, 1));
     if (ncq == 4) rxm = fmaxf(rxm, __shfl_xor_sync(0xffffffffu, rxm, 2));
     const float b127 = __fmul_rn(127.0f, rxm);
     // Three of the warps share the live rows of a chunk evenly, up to two chunks ahead; the fourth requests the tiles, the
@@ -489,18 +487,14 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
 }
 
 // Column range of a CTA: 16-channel chunks c0 .. c0 + ncq - 1 of one head.  Whole heads first, then
-// the heads of a nearly empty last wave, split in halves or quarters so that they spread over the
-// free slots (operand tiles and the MMA stay full width: only the re-quantisation, the state
-// update and the hq rows are restricted to the range).
+// heads in quarters, for a short remainder or a small workload (see the launcher; operand tiles and the MMA stay
+// full width: only the re-quantisation, the state update and the hq rows are restricted to the range).
 template <bool I8S, bool TAPS, bool CAL>
 __global__ void __launch_bounds__(kThreads, CAL ? 2 : 3)
 chunk_state_pass_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__ CUtensorMap tm_x,
                     const __grid_constant__ CUtensorMap tm_hq, const FusedArgs a) {
   if ((int)blockIdx.x < a.n_full) {
     fused_body<I8S, TAPS, CAL, 4>(tm_B, tm_x, tm_hq, a, (int)blockIdx.x, 0);
-  } else if (a.split == 2) {
-    const int r = (int)blockIdx.x - a.n_full;
-    fused_body<I8S, TAPS, CAL, 2>(tm_B, tm_x, tm_hq, a, a.n_full + (r >> 1), 2 * (r & 1));
   } else {
     const int r = (int)blockIdx.x - a.n_full;
     fused_body<I8S, TAPS, CAL, 1>(tm_B, tm_x, tm_hq, a, a.n_full + (r >> 2), r & 3);
@@ -536,10 +530,8 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
     uint32_t box[2] = {(uint32_t)d.N, 16};
     if (!encode_tensor_map(&tm_hq, hq, 1, 2, dims, str, box, 0)) return SSDI8_ERR_CUDA;
   }
-  // (batch, head) units over the CTA slots of the device (3 CTAs per SM): whole waves of whole
-  // units, and the units of a last, partly filled wave as four quarter-width CTAs each, which pack
-  // into that wave's free slots (a quarter costs about a third of a whole unit: the operand tiles
-  // and the MMA stay full width)
+  // (batch, head) units over the CTA slots of the device, 3 per SM.  (The calibration instance has two per SM; it follows
+  // the same rule, whose lines were measured on the others.)
   const int sms = sm_count();
   if (sms == 0) return SSDI8_ERR_CUDA;
   const int units = d.H * d.b, slots = 3 * sms;
@@ -552,13 +544,12 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
   // 128 43.8 / 40.4, 1024 x 80 36.6 / 35.5; but with one or two chunks 3 x 256 x 37 24.4 / 26.0, 512 x 100 29.9 / 30.5, and
   // 2048 x 111 55.8 / 56.7).
   int n_full = units / slots * slots;
-  int split = 4;
   const bool quarters = 8 * (units - n_full) <= slots || (n_full == 0 && d.c >= 4 && 4 * units <= slots - slots / 10);
   if (!quarters) n_full = units;
   FusedArgs a = {s_x, s_xs, s_B, s_h, pack, gamma, init, final_state, tap_loc, tap_prev, tap_Xsq, tap_acc,
-                 status, absmax_h, d, n_full, split};
+                 status, absmax_h, d, n_full};
   const size_t smem = SMEM_BYTES;
-  const unsigned grid = (unsigned)(n_full + split * (units - n_full));
+  const unsigned grid = (unsigned)(n_full + 4 * (units - n_full));
   const bool taps = tap_loc || tap_prev || tap_Xsq || tap_acc;
   auto launch = [&](auto kernel) -> ssdi8_status_t {
     return launch_configured(kernel, dim3(grid), dim3(kThreads), smem, -1, true, st, tm_B, tm_x, tm_hq, a);

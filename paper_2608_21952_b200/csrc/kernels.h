@@ -78,9 +78,6 @@ ssdi8_status_t launch_quantize_entry(const void* xBC, int dtype, i64 T_, int D, 
 ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, uint32_t flags, void* workspace,
                           size_t workspace_bytes, void* stream, bool clear_status);
 
-// where ChunkCumsum's outputs live inside a workspace of ssdi8_workspace_bytes
-void workspace_pack_gamma(const Dims& d, void* workspace, float** pack, float** gamma);
-
 // pack [b,H,c,6,Q], gamma [b,H,c], tap_cs [b,H,c,Q] or NULL; clear_status: a status word the kernel sets to 0, or NULL
 // softplus: dt is the raw time step, dt = softplus(dt + dt_bias[h]) is applied first (dt_bias may be NULL)
 ssdi8_status_t launch_cumsum(const Dims& d, const float* dt, const float* A, float* pack,

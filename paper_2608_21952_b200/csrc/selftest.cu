@@ -71,7 +71,7 @@ __global__ void bounded_wait_expires(int32_t* status) {
   if (threadIdx.x == 0) {
     mbar_init(&bar, 1);
     fence_mbar_init();
-    mbar_wait_slow<48>(&bar, 0, status, 0u);
+    mbar_wait_slow<48>(&bar, 0, status);
   }
 }
 

@@ -40,18 +40,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// One look at the barrier without suspending: has the phase of that parity completed?
-__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.b32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
 // Bounded wait.  Every try_wait blocks for up to its suspend-time hint, so the cap is of the
 // order of a second.  On expiry the caller's status word is set and the wait returns; once
 // the word is set, every later wait of the grid gives up after a few polls, so the kernel runs
@@ -62,24 +50,15 @@ constexpr uint32_t kWaitCap = 1u << 17;
 // (CAP is a template parameter only so that the library's self-test can run this very loop with a
 // cap of a few dozen polls on a barrier nobody arrives on; every kernel of the layer uses kWaitCap.)
 template <uint32_t CAP = kWaitCap>
-static __device__ __noinline__ void mbar_wait_slow(uint64_t* bar, uint32_t parity, int32_t* status,
-                                                   uint32_t sleep_ns) {
+static __device__ __noinline__ void mbar_wait_slow(uint64_t* bar, uint32_t parity, int32_t* status) {
   for (uint32_t it = 0; it < CAP; ++it) {
     if (mbar_try_wait(bar, parity)) return;
-    if (sleep_ns) __nanosleep(sleep_ns);
     if ((it & 255u) == 255u && status && *reinterpret_cast<volatile int32_t*>(status) != 0) return;
   }
   if (status) atomicExch(status, (int32_t)SSDI8_ERR_DEVICE_TIMEOUT);
 }
 __device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, int32_t* status) {
-  if (!mbar_try_wait(bar, parity)) mbar_wait_slow(bar, parity, status, 0u);
-}
-
-// The same bounded wait for warps whose wait is long and off the critical path (producers waiting
-// for a free slot, epilogue warps waiting for an accumulator): a failed poll is followed by a short
-// sleep, so the polling loop leaves the issue slots to the warps that compute.
-__device__ __forceinline__ void mbar_wait_relaxed(uint64_t* bar, uint32_t parity, int32_t* status) {
-  if (!mbar_try_wait(bar, parity)) mbar_wait_slow(bar, parity, status, 256u);
+  if (!mbar_try_wait(bar, parity)) mbar_wait_slow(bar, parity, status);
 }
 
 // named barrier among `nthreads` threads (whole warps) of the CTA; id 0 is __syncthreads
@@ -95,7 +74,7 @@ __device__ __forceinline__ void drain_after_timeout(const int32_t* status) {
     for (int i = 0; i < 50; ++i) __nanosleep(1000);
 }
 
-// Inline forms of both waits, for kernels with few wait sites and no registers to spare around a call.
+// Inline form of the wait (SLEEP_NS: a short sleep after a failed poll), for kernels with few wait sites and no registers to spare around a call.
 template <uint32_t SLEEP_NS>
 __device__ __forceinline__ void mbar_wait_inline(uint64_t* bar, uint32_t parity, int32_t* status) {
   for (uint32_t it = 0; it < kWaitCap; ++it) {
@@ -159,10 +138,6 @@ __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk
 __device__ __forceinline__ void tma_store_wait_read() {
   asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
-// all but the most recent bulk store of this thread have finished reading shared memory
-__device__ __forceinline__ void tma_store_wait_read1() {
-  asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-}
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* tm) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
 }
@@ -190,15 +165,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, int (&v)[32]) {
         "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
         "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
         "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, int (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr)
       : "memory");
 }
