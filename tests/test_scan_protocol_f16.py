@@ -1,13 +1,14 @@
 """The barrier protocol of the FP16-operand ChunkScan kernel (csrc/chunk_scan_f16.cu) on the host-side model of
 test_scan_protocol_model.py: one CBq buffer and one xq buffer whose barriers come in pairs by the parity of the chunk, xq
 rows expanded by the mask group behind its first tile.  Every wait is decided by parity alone and checked against the true
-phase counts."""
+phase counts, and the two single buffers are watched: a load must not start while the tile before is still read.  `broken` names
+variants that the model has to report."""
 import pytest
 
 from test_scan_protocol_model import Bar, Sim
 
 
-def build(sim, ntiles, ntpu, speed):
+def build(sim, ntiles, ntpu, speed, broken=None):
     rng = sim.rng
     B = lambda name, count, n: [Bar(f"{name}{i}", count) for i in range(n)]
     cb_full, cb_free, mq = B("CB_FULL", 1, 4), B("CB_FREE", 8, 4), B("MQ", 8, 4)
@@ -24,28 +25,44 @@ def build(sim, ntiles, ntpu, speed):
     full = lambda bar, use: ("wait", bar, use & 1, use + 1)
     free = lambda bar, use: ("wait", bar, (use & 1) ^ 1, use)
 
+    held = {}   # single buffer -> whose contents are being read
+
+    def fill(name, who):
+        assert held.get(name) is None, f"{name}: filled for {who} while {held[name]} is read"
+        held[name] = who
+
+    one_ch = broken == "one Cq/hq barrier pair"
+
     def prod_cb():
         for n in range(ntiles):
             ci = cb_index(n)
             yield free(tok_free[n & 3], n >> 2)
             yield ("async", t("load"), [(tok_full[n & 3], 1)])
             if ntpu == 2 and it_of(n) == 0:
-                if n > 0:
+                if broken == "first CBq by its own pair":
+                    yield free(cb_free[ci], n >> 2)
+                elif n > 0:
                     yield full(cb_free[ci ^ 1], (n - 2) >> 2)
+                fill("CB1", n)
             else:
                 yield free(cb_free[ci], n >> 2)
             yield ("async", t("load"), [(cb_full[ci], 1)])
             yield ("work", t("producer"))
 
     def prod_ch():
+        fill("XRAW", 0)
         yield ("async", t("load"), [(x_raw[0], 1)])
         for n in range(ntiles):
-            if n > 0:
+            if one_ch:
+                yield free(ch_free[0], n)
+            elif n > 0:
                 yield full(ch_free[(n - 1) & 1], (n - 1) >> 1)
-            yield ("async", t("load"), [(ch_full[n & 1], 1)])
+            yield ("async", t("load"), [(ch_full[0 if one_ch else n & 1], 1)])
             if it_of(n) == 0 and n + ntpu < ntiles:
                 u = unit(n)
-                yield full(raw_free, u)
+                if broken != "xq codes without RAW_FREE":
+                    yield full(raw_free, u)
+                fill("XRAW", u + 1)
                 yield ("async", t("load"), [(x_raw[(u + 1) & 1], 1)])
             yield ("work", t("producer"))
 
@@ -53,9 +70,9 @@ def build(sim, ntiles, ntpu, speed):
         for n in range(par, ntiles, 2):
             u = unit(n)
             yield free(acc_free[n & 1], n >> 1)
-            yield full(ch_full[par], n >> 1)
+            yield full(ch_full[0], n) if one_ch else full(ch_full[par], n >> 1)
             yield ("work", t("mma"))
-            yield ("async", t("mma"), [(ch_free[par], 1)])
+            yield ("async", t("mma"), [(ch_free[0 if one_ch else par], 1)])
             yield full(x_full[u & 1], u >> 1)
             yield full(mq[cb_index(n)], n >> 2)
             yield ("work", t("mma"))
@@ -71,11 +88,14 @@ def build(sim, ntiles, ntpu, speed):
             yield free(afree[n & 1], n >> 1)
             yield ("work", t("mask") * (1 + 2 * it_of(n)))
             yield ("arrive", mq[cb_index(n)], 8)
+            if ntpu == 2 and it_of(n) == 0:
+                held["CB1"] = None
             yield ("arrive", cb_free[cb_index(n)], 8)
             if it_of(n) == 0:
                 yield full(x_raw[u & 1], u >> 1)
                 yield free(x_free[u & 1], u >> 1)
                 yield ("work", t("mask"))
+                held["XRAW"] = None
                 yield ("arrive", x_full[u & 1], 8)
                 yield ("arrive", raw_free, 8)
 
@@ -109,3 +129,22 @@ def test_every_wait_is_sound_at_random_and_extreme_speeds(ntpu, units):
             speed = {r: 100.0 if r == ROLES[seed] else 0.01 for r in ROLES}
         build(sim, units * ntpu, ntpu, speed)
         sim.run()
+
+
+@pytest.mark.parametrize("broken,where", [("first CBq by its own pair", "CB1"), ("one Cq/hq barrier pair", "CH_FULL"),
+                                          ("xq codes without RAW_FREE", "XRAW")])
+def test_broken_variants_are_reported(broken, where):
+    """The first tiles' one CBq buffer guarded by the chunk before the last only; the odd tiles' MMA issuer on a barrier pair
+    shared with the even ones', which polls the parity of phase 1 before phase 0 has completed; the xq codes of the next chunk
+    requested without waiting for the mask group that expands the present ones."""
+    hit = 0
+    for seed in range(24):
+        sim = Sim(seed)
+        speed = {r: 10.0 ** sim.rng.uniform(-2, 2) for r in ROLES}
+        build(sim, 36, 2, speed, broken)
+        try:
+            sim.run()
+        except AssertionError as e:
+            assert where in str(e) or "deadlock" in str(e), e
+            hit += 1
+    assert hit > 0

@@ -1,13 +1,14 @@
 """The barrier protocol of the int8 ChunkScan kernel (csrc/chunk_scan.cu) on the host-side model of
 test_scan_protocol_model.py: two producers (one per tile of a chunk), one issuer per contraction, two mask groups, two
 epilogue groups that hand xq back before they wait for the accumulators.  Every wait is decided by parity alone and checked
-against the true phase counts: none is lapped, none passes early, every role finishes."""
+against the true phase counts: none is lapped, none passes early, every role finishes.  `broken` names variants that the model
+has to report."""
 import pytest
 
 from test_scan_protocol_model import Bar, Sim
 
 
-def build(sim, ntiles, ntpu, speed):
+def build(sim, ntiles, ntpu, speed, broken=None):
     rng = sim.rng
     B = lambda name, count, n: [Bar(f"{name}{i}", count) for i in range(n)]
     cb_full, cb_free, mq = B("CB_FULL", 1, 4), B("CB_FREE", 1, 4), B("MQ", 8, 4)
@@ -16,7 +17,7 @@ def build(sim, ntiles, ntpu, speed):
     row_full, row_free = B("ROW_FULL", 9, 8), B("ROW_FREE", 4, 8)
     c_full, c_free = Bar("C_FULL", 1), Bar("C_FREE", 1)
     h_full, h_free = B("H_FULL", 1, 2), B("H_FREE", 1, 2)
-    x_full, x_free = B("X_FULL", 1, 2), B("X_FREE", (4 if ntpu == 1 else 8) + 1, 2)
+    x_full, x_free = B("X_FULL", 1, 2), B("X_FREE", (4 if ntpu == 1 else 8) + (broken != "x_free without the MMAs"), 2)
 
     it_of = lambda n: n % ntpu
     unit = lambda n: n // ntpu
@@ -64,7 +65,8 @@ def build(sim, ntiles, ntpu, speed):
             yield full(x_full[u & 1], u >> 1)
             yield full(mq[cb_index(n)], n >> 2)
             yield ("work", t("mma"))
-            done = [(cb_free[cb_index(n)], 1), (acc[n & 3], 1)] + ([(x_free[u & 1], 1)] if it_of(n) + 1 == ntpu else [])
+            done = [(cb_free[cb_index(n)], 1), (acc[n & 3], 1)] + (
+                [(x_free[u & 1], 1)] if it_of(n) + 1 == ntpu and broken != "x_free without the MMAs" else [])
             yield ("async", t("mma"), done)
 
     def mask(g):
@@ -87,6 +89,8 @@ def build(sim, ntiles, ntpu, speed):
             yield full(x_full[u & 1], u >> 1)
             yield ("arrive", x_free[u & 1], 4)
             yield full(acc[n & 3], n >> 2)
+            if broken == "epilogue waits on MQ":
+                yield full(mq[cb_index(n)], n >> 2)
             yield full(row_full[n & 7], n >> 3)
             yield ("work", t("epilogue"))
             yield ("arrive", acc_free[n & 3], 4)
@@ -110,3 +114,22 @@ def test_every_wait_is_sound_at_random_and_extreme_speeds(ntpu, units):
             speed = {r: 100.0 if r == ROLES[seed] else 0.01 for r in ROLES}
         build(sim, units * ntpu, ntpu, speed)
         sim.run()
+
+
+@pytest.mark.parametrize("broken,barrier", [("epilogue waits on MQ", "MQ"), ("x_free without the MMAs", "X_F")])
+def test_broken_variants_are_reported(broken, barrier):
+    """The mask barrier of a CBq buffer may complete for tile n + 4 while the epilogue group of tile n is busy with tile n - 2:
+    nothing the epilogue releases stands between the two.  And an xq buffer that the epilogue alone hands back is filled again
+    ahead of the MMAs that wait for its contents."""
+    hit = 0
+    for seed in range(24):
+        sim = Sim(seed)
+        speed = dict(load=0.1, producer=0.01, mma=0.01, mask=0.01, epilogue=5.0) if seed % 2 else \
+            dict(load=0.1, producer=0.01, mma=5.0, mask=5.0, epilogue=0.01)
+        build(sim, 36, 2, speed, broken)
+        try:
+            sim.run()
+        except AssertionError as e:
+            assert barrier in str(e) or "deadlock" in str(e)
+            hit += 1
+    assert hit > 0
