@@ -52,10 +52,13 @@ constexpr uint32_t OFF_BAR = OFF_COL + 768;
 constexpr uint32_t SMEM_BYTES = OFF_BAR + 64;     // 76 608 bytes: three CTAs per SM
 constexpr uint32_t kTmemCols = 128;               // accumulator in columns 0..63, running state in 64..127
 
-enum { B_XFULL = 0, B_BFULL = 2, B_MMA = 3, B_ACC_FREE = 4, B_XQ = 5, B_COUNT = 7 };
+enum { B_XFULL = 0, B_BFULL = 2, B_MMA = 3, B_ACC_FREE = 4, B_COUNT = 5 };
 
 __device__ __forceinline__ void named_bar(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+__device__ __forceinline__ void named_bar_arrive(int id, int nthreads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
 
 // TAPS: any of the intermediate-tensor taps is requested (tests); the production instance carries no tap code
@@ -125,8 +128,6 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
       mbar_init(&bars[B_BFULL], 1);
       mbar_init(&bars[B_MMA], 1);
       mbar_init(&bars[B_ACC_FREE], kStateThreads / 32);
-      mbar_init(&bars[B_XQ], kRowWarps);
-      mbar_init(&bars[B_XQ + 1], kRowWarps);
       fence_mbar_init();
       tma_prefetch_desc(&tm_B);
       tma_prefetch_desc(&tm_x);
@@ -185,8 +186,10 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     // whole slabs dealt out by position the warp that had most of them was the time of a chunk, and with all of xq
     // and Bq loaded (48 KB per chunk and CTA) the loads of three CTAs took 1.4 us.  The row warps only arrive at
     // the barrier that releases the MMAs, one of two in turn: they are held back by the xq tile of the chunk after next,
-    // which is requested when this chunk's MMAs have finished.  (An mbarrier, whose wait is bounded like every other: once waits
-    // give up, the row warps get ahead of the issuing one, and a hardware barrier that they had overrun would never fill.)
+    // which is requested when this chunk's MMAs have finished.  A row warp whose wait for a tile
+    // has given up is no longer held back by it: from then on it only waits at the barrier, since one that is overrun never
+    // fills, and nothing bounds that wait.  (An mbarrier in its place, with a bounded wait, costs 0.14 us per chunk of a lone chain:
+    // 2 x 8192 tokens x 7 heads with INT8 states 66.8 -> 71.4 us.)
     // (Batch 8 x 2048 x 80 heads: 48.9 us with slabs dealt out by position, 41.0 this way, 38.7 with the first tiles requested
     // ahead of all other set-up and s_x / s_xs divided once per channel; 4 x 8192 x 128 151, 118, 115.)
     const int qw = warp - kStateThreads / 32, nsl = Q / 32;
@@ -227,9 +230,9 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
       for (int k = 0; k < d.c; ++k) {
         Lut v = {};
         if (k + 2 < d.c) v = lut_of_lane(lut0 + (k + 2) * lut_step);     // (its latency under the waits)
+        named_bar(2 + (k & 1), kQuantThreads);                           // the rows are re-quantised
         mbar_wait_inline<0>(&bars[B_ACC_FREE], (k & 1) ^ 1, a.status);   // the state warps have read the accumulator of chunk k-1
         mbar_wait_inline<0>(&bars[B_BFULL], k & 1, a.status);            // the chunk's Bq rows have landed
-        mbar_wait_inline<0>(&bars[B_XQ + (k & 1)], (k >> 1) & 1, a.status);   // the rows are re-quantised (mostly the last to come)
         tc_fence_after();
         const uint32_t sBa = smem_u32(smem + OFF_B), sXa = smem_u32(smem + OFF_X + (k & 1) * XSTAGE);
         if (elect_one()) {
@@ -252,13 +255,14 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
         }
       }
     } else {
+    int k = 0;
 #pragma unroll 1
-    for (int k = 0; k < d.c; ++k) {
+    for (; k < d.c; ++k) {
       const int s = k & 1;
       uint8_t* sX = smem + OFF_X + s * XSTAGE;
       float* lut = reinterpret_cast<float*>(smem + OFF_LUT) + s * 256;
       const i64 tok0 = (i64)b * d.L + (i64)k * Q;
-      mbar_wait_inline<256>(&bars[B_XFULL + s], (k >> 1) & 1, a.status);
+      if (__any_sync(0xffffffffu, !mbar_wait_inline<256>(&bars[B_XFULL + s], (k >> 1) & 1, a.status))) break;
       const uint32_t lm = live_slabs(lut_of_lane(lut));   // (every warp computes the same mask)
       const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
       if (TAPS && a.tap_Xsq) {
@@ -301,9 +305,9 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
         if (TAPS && a.tap_Xsq) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = v;
       }
       fence_async_smem();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bars[B_XQ + s]);
+      named_bar_arrive(2 + s, kQuantThreads);
     }
+    for (; k < d.c; ++k) named_bar(2 + (k & 1), kQuantThreads);   // (a wait has given up)
     }
   } else {
     // ------------------------------------------------------------ state warps

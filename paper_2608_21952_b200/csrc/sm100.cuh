@@ -75,14 +75,16 @@ __device__ __forceinline__ void drain_after_timeout(const int32_t* status) {
 }
 
 // Inline form of the wait (SLEEP_NS: a short sleep after a failed poll), for kernels with few wait sites and no registers to spare around a call.
+// Returns false if it gave up.
 template <uint32_t SLEEP_NS>
-__device__ __forceinline__ void mbar_wait_inline(uint64_t* bar, uint32_t parity, int32_t* status) {
+__device__ __forceinline__ bool mbar_wait_inline(uint64_t* bar, uint32_t parity, int32_t* status) {
   for (uint32_t it = 0; it < kWaitCap; ++it) {
-    if (mbar_try_wait(bar, parity)) return;
+    if (mbar_try_wait(bar, parity)) return true;
     if (SLEEP_NS) __nanosleep(SLEEP_NS);
-    if ((it & 255u) == 255u && status && *reinterpret_cast<volatile int32_t*>(status) != 0) return;
+    if ((it & 255u) == 255u && status && *reinterpret_cast<volatile int32_t*>(status) != 0) return false;
   }
   if (status) atomicExch(status, (int32_t)SSDI8_ERR_DEVICE_TIMEOUT);
+  return false;
 }
 
 // One lane of the (converged) warp.  Issue loops run with the whole warp and elect the issuing lane only around
