@@ -117,7 +117,6 @@ __device__ __forceinline__ uint32_t pack4_bits(uint32_t a, uint32_t b, uint32_t 
 struct Step4 {
   float2 y01, y23, n01, n23;   // reciprocals and negatives of four step sizes
   float4 lim;                  // 127.25 of them
-  float neg0;                  // -0.0
   bool usable;
 };
 __device__ __forceinline__ Step4 step4(const float4& a) {
@@ -128,14 +127,14 @@ __device__ __forceinline__ Step4 step4(const float4& a) {
   s.n01 = make_float2(-a.x, -a.y);
   s.n23 = make_float2(-a.z, -a.w);
   s.lim = make_float4(__fmul_rn(a.x, 127.25f), __fmul_rn(a.y, 127.25f), __fmul_rn(a.z, 127.25f), __fmul_rn(a.w, 127.25f));
-  s.neg0 = __fmul_rn(-a.x, 0.0f);   // (a product, so that the sum in code4 stays: a.x might not be finite)
   s.usable = normal(a.x) && normal(a.y) && normal(a.z) && normal(a.w);
   return s;
 }
 __device__ __forceinline__ uint32_t code4(const float4& v, const Step4& s) {
-  // v - 0 is v, and a NaN of either sign becomes the positive one that a division gives: its code is +127
-  const float2 z = make_float2(s.neg0, s.neg0);
-  float2 v01 = __fadd2_rn(make_float2(v.x, v.y), z), v23 = __fadd2_rn(make_float2(v.z, v.w), z);
+  // v - 0 is v, and a NaN of either sign becomes the positive one that a division gives: its code is +127.  (The zero as a
+  // product that the compiler cannot know: the step size might not be finite.)
+  const float2 z = make_float2(0.f, 0.f);
+  float2 v01 = __ffma2_rn(s.n01, z, make_float2(v.x, v.y)), v23 = __ffma2_rn(s.n23, z, make_float2(v.z, v.w));
   // min(|v|, lim) with the sign of v
   asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(v01.x) : "f"(v01.x), "f"(s.lim.x));
   asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(v01.y) : "f"(v01.y), "f"(s.lim.y));

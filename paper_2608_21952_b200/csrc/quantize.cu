@@ -125,10 +125,8 @@ __global__ void __launch_bounds__(128, 8) quant_jobs(const QuantJobs a) {
       for (int u = 0; u < QROWS; ++u) out[e + u * stride] = code4_by_division(in[e + u * stride], s);
     }
   }
-  for (; left > 0; --left, e += stride) {
-    const float4 v = __ldcs(in + e);
-    out[e] = st.usable ? code4(v, st) : code4_by_division(v, s);
-  }
+  // (a layer's token count is a multiple of 64, which leaves no rest; the short form keeps the registers from spilling)
+  for (; left > 0; --left, e += stride) out[e] = code4_by_division(__ldcs(in + e), s);
 }
 
 // ---- quantise, I % 4 == 0: 4 consecutive elements share a channel
