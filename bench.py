@@ -304,7 +304,7 @@ class Layer:
 
     def e2e_step(self):
         """The same step through the host-buffer entry point of the C-ABI: pinned fp32 x, B, C, dt in,
-        fp32 y out, copies pipelined against the kernels batch element by batch element."""
+        fp32 y out, copies pipelined against the kernels a few chunks at a time."""
         if self.host_args is None:
             bd, torch = self.bd, self.torch
             self.host_scratch = torch.empty(bd.ssdi8_layer_fwd_host_scratch_bytes(self.dims), dtype=torch.uint8,
@@ -618,9 +618,10 @@ def run_ours(args):
                     "peak_source": peaks["source"], "algorithmic_bytes": head["chunk_scan_hbm"]["algorithmic_bytes"],
                     "launch_ms": kernel_ms["chunk_scan"], "traffic": ncu.get("traffic"),
                     "traffic_source": ncu.get("source"), "slowest_module": dom,
-                    "limiter": "instruction issue of the CUDA cores that build the int8 masked operand and the "
-                               "fp32 output around the MMAs (neither DRAM nor the tensor pipe is saturated); "
-                               "HBM is the roof the bytes of this kernel set"}
+                    "limiter": "the epilogue groups that form y, then the mask groups, the round trip of the one Cq "
+                               "buffer and the DRAM writes of y, each within 15 % of the pace (issue slots two thirds "
+                               "used; neither DRAM nor the tensor pipe saturated); HBM is the roof the bytes of this "
+                               "kernel set"}
         roofline_tensor = dict(head["chunk_scan_int8"])
         roofline_tensor.update({"int8_tops_measured": int8_peak, "tensor_active_pct": ncu.get("tensor_active_pct"),
                                 "tensor_active_source": ncu.get("source")})
@@ -660,7 +661,7 @@ def run_ours(args):
                 "e2e": {"value": ranks.whole_job_tokens_per_s(cfg.tokens, world, ms_e2e), "unit": UNIT,
                         "h2d_bytes_per_step": layer_h2d, "d2h_bytes_per_step": layer_d2h,
                         "ms_per_step": ms_e2e, "rounds": e2e_rounds,
-                        "api": "ssdi8_layer_fwd_host (pinned host buffers; copies pipelined per batch element)"},
+                        "api": "ssdi8_layer_fwd_host (pinned host buffers; copies pipelined in slices of a few chunks)"},
                 "gpu_launches": Layer.LAUNCHES_PER_STEP * args.steps * head["rounds"],
                 "gpu_launches_per_step": Layer.LAUNCHES_PER_STEP,
                 "parity": parity,

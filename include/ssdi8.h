@@ -266,19 +266,20 @@ ssdi8_status_t ssdi8_chunk_scan_fwd_static(const ssdi8_dims_t* dims, const ssdi8
  *   ssdi8_layer_fwd_workspace_bytes(dims, flags) bytes (the int8 tensors plus ssdi8_workspace_bytes).
  * ssdi8_layer_fwd_host: x, B, C, dt, y, final_state, status are HOST pointers (page-locked memory, or
  *   the copies neither overlap nor run asynchronously), the rest DEVICE pointers.  One slice at a
- *   time, a slice being a run of whole chunks of one batch element (2 to 8 MB of x; its final state is
- *   the next slice's initial state) or several whole elements where they are smaller: the
+ *   time, a slice being a run of whole chunks of one batch element, at least one (aiming at a twelfth of the
+ *   call's x, and 2 to 8 MB; its final state is the next slice's initial state), or one or several whole
+ *   elements where that comes close: the
  *   host->device copies of the next slices and the device->host copies of y of the ones before run
  *   on two copy streams while the kernels of a slice run, so both directions of the host link stay
  *   busy.  scratch: DEVICE, 256-byte aligned, ssdi8_layer_fwd_host_scratch_bytes(dims, flags) bytes
  *   (three stages of one slice's tensors).
- *   Calls from several threads, each with its stream and scratch, are enqueued one after the other.
  * Layouts as in ssdi8_fwd_args_t; D, corr, init_state, final_state, status may be NULL.  Both calls
  * return once everything is enqueued and leave `stream` waiting for the last piece of work, so
  * synchronising `stream` completes them.  flags: any of SSDI8_FLAG_INT8_STATE, SSDI8_FLAG_Y_FP16,
  * SSDI8_FLAG_Y_BF16 (`y` then points to 16-bit elements), SSDI8_FLAG_FP16_OPERAND.  The copy streams and
- * events of ssdi8_layer_fwd_host are created at the first call on each device and shared by later calls:
- * calls of ssdi8_layer_fwd_host on one device must not overlap in time.  Errors: as ssdi8_quantize_act / ssdi8_chunk_scan_fwd, plus
+ * events of ssdi8_layer_fwd_host are created at the first call on each device and shared by later calls: calls from
+ * several threads, each with its own stream and scratch, are enqueued one after the other.  A call that ends with an error
+ * leaves `stream` behind the copies it has enqueued.  Errors: as ssdi8_quantize_act / ssdi8_chunk_scan_fwd, plus
  * SSDI8_ERR_WORKSPACE for a short workspace or scratch. */
 typedef struct {
   const float* x; const float* B; const float* C; const float* dt;   /* [B,L,H,P], [B,L,G,N] x2, [B,L,H] */
@@ -301,7 +302,8 @@ ssdi8_status_t ssdi8_layer_fwd_host(const ssdi8_dims_t* dims, const ssdi8_layer_
  *   s_cb[g]   = absmax over the causal half of |acc_cb| * fmul(s_C, s_B) / 127
  *   s_h[h,p]  = absmax over init_state and every S_k, all b and n, / 127
  * (each 1 if its absmax is 0).  Reads xq, Bq, Cq, s_x, s_B, s_C, dt, A, init_state of `args`;
- * ignores its other members.  Writes s_xs [H*P], s_cb [G], s_h [H*P]. */
+ * ignores its other members; xq, Bq, Cq, dt and init_state are 16-byte aligned, the rest needs a float's
+ * alignment.  A NaN counts for nothing.  Writes s_xs [H*P], s_cb [G], s_h [H*P]. */
 ssdi8_status_t ssdi8_calibrate(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* args,
                                float* s_xs, float* s_cb, float* s_h, void* workspace,
                                size_t workspace_bytes, void* stream);

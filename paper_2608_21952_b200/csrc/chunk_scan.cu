@@ -17,11 +17,12 @@
 // tiles) and an 8-deep ring for what the mask warps hand to the epilogue keep the mask and the MMAs
 // of the next tiles independent of the epilogue of the current ones.  Every buffer has its own
 // "free" barrier, released by whoever reads it last (tcgen05.commit for MMA operands), so loads run
-// several tiles ahead.  What bounds the kernel is instruction issue (78 M warp instructions, 66 % of the
-// slots with binary32 y at batch 8 x 2048 x 80 heads, 0.113 ms; 0.104 ms with 16-bit y), so it is
-// written to issue little: in each group one warp polls the mbarriers and the others wait at a hardware
-// barrier, the wait loop is one out-of-line function, the tile walk has no divisions, and the code is kept
-// small enough for the instruction cache (every role executes different code at the same time).
+// several tiles ahead.  What bounds the kernel (0.113 ms with binary32 y at batch 8 x 2048 x 80 heads, 0.103 with 16-bit
+// y) are the epilogue groups, busy 85 to 90 % of the time, and close behind them the mask groups, the round trip of the one
+// Cq buffer and the DRAM writes of y: without the mask 0.111 ms, without mask and y stores 0.0725.  Issue slots are two
+// thirds used (78 M warp instructions), so it is written to issue little all the same: in each group one warp polls the
+// mbarriers and the others wait at a hardware barrier, the wait loop is one out-of-line function, the tile walk has no
+// divisions, and the code is kept small enough for the instruction cache (every role executes different code).
 // The pipeline around it is built so that no role waits for another's order: a timeline of one CTA had the
 // mask groups waiting 2.6 us of every 6.6 for CBq buffers, which waited for in-order MMAs, which waited for
 // xq, whose buffer the epilogue gave back last; with the loads of the two tiles of a chunk on
@@ -465,7 +466,8 @@ chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ 
     // ------------------------------------------------------------ mask warps.  With two tiles per chunk, group g
     // takes the chunks c = g, g + 2, ... of this CTA, both tiles: warp w builds the 16-row block w of the
     // first tile and block 7 - w of the second, which is the same number of 16-column sub-blocks for every
-    // warp (the causal rows grow with the row index).  With one tile per chunk the groups alternate tiles.
+    // warp over a chunk (the causal rows grow with the row index); the group meets once per tile, though, so each
+    // tile lasts as long as its slowest warp.  With one tile per chunk the groups alternate tiles.
     const int g = (warp - kMaskWarp0) / kGroupWarps;
     const int w = (warp - kMaskWarp0) % kGroupWarps;
     Tile t = *first_tile;

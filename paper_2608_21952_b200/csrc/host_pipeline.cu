@@ -22,7 +22,8 @@ constexpr uint32_t kLayerFlags = SSDI8_FLAG_FP16_OPERAND | SSDI8_FLAG_INT8_STATE
 
 inline size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-// How the host pipeline cuts a call.  The pipeline fills with two slices' copies in and drains with two slices'
+// How the host pipeline cuts a call.  (Measured at one size, below; the limits of 2 and 8 MB are not, beyond the results being
+// right on both sides of them.)  The pipeline fills with two slices' copies in and drains with two slices'
 // copies out exposed, so slices are small; but a slice's kernels are a chain of about 30 us whatever its size, and a
 // copy costs a few microseconds beside its bytes, so they are not smaller than kMinSlice of x.  Measured on PCIe 5
 // x16 at 3 x 1024 tokens x 80 heads (63 MB of x in and of y out, 1.15 ms each way with the link to itself): a

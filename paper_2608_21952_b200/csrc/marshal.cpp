@@ -4,7 +4,7 @@
 // Why native: through ctypes a call with a dozen tensors took 9 to 13 us of host time (0.25 us per tensor for
 // its type checks and address, 3.4 us for the stream object) ahead of a launch of 3 us, more than the device time of
 // a decode step of one sequence (7 us for its three calls); from here a call takes 3.5 to 4 us, launch included, and
-// that decode step 8.1 instead of 29 us.
+// that decode step 8.1 to 9.3 us, by the machine, instead of 29.
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <c10/cuda/CUDAStream.h>
