@@ -93,6 +93,21 @@ def test_quantiser_gives_all_zero_channels_a_step_of_one(R, Ch, I):
     assert np.array_equal(q.reshape(-1), np.asarray(qr).reshape(-1))
 
 
+@pytest.mark.parametrize("Q,N,H", [(256, 128, 5), (256, 64, 148), (256, 128, 149), (128, 128, 3)])
+def test_scan_with_one_chunk_per_cta(Q, N, H):
+    # As many chunks as SMs, one more, and few: the mask groups take a tile each where a CTA has one chunk
+    import gpu_harness as gh
+    cfg = SSDConfig("one", 1, Q, H, 64, N, 1, Q, 0.02, 20.0, 47)
+    q = orc.prepare_quantized(cfg, inputs.make_prefill(cfg))
+    y, fin, taps = gh.gpu_fwd(cfg, q, taps=("Mq", "acc_diag"))
+    _, fin_ref, ref = orc.ssdi8_fwd(cfg, q["xq"], q["Bq"], q["Cq"], q["s_x"], q["s_B"], q["s_C"], q["dt"], q["A"], q["D"], None,
+                                    q["s_xs"], q["s_cb"], q["s_h"], taps=("Mq", "acc_diag"))
+    assert np.array_equal(fin, fin_ref)
+    for name in taps:
+        assert np.array_equal(taps[name], ref[name]), name
+    assert np.array_equal(y, gh.gpu_fwd(cfg, q, taps=())[0])
+
+
 @pytest.mark.parametrize("b,c,H,G", [(9, 1, 80, 1), (5, 2, 129, 1), (2, 7, 130, 2), (6, 3, 40, 8), (1, 9, 256, 1), (14, 1, 8, 1)],
                          ids=lambda v: str(v))
 @pytest.mark.parametrize("flags", [0, 2 | 4], ids=["default", "int8_state_y_fp16"])
