@@ -17,8 +17,8 @@ __global__ void __launch_bounds__(256) absmax_xs_kernel(const int8_t* __restrict
   __shared__ __align__(16) float lut[kXsHeads][kXsTokens];
   __shared__ __align__(16) float sxs[kXsHeads * 64];
   __shared__ uint32_t best[8][kXsHeads * 64];
-  pdl_launch_dependents();
   pdl_wait();
+  pdl_launch_dependents();   // (after the wait: ChunkBMM, launched next, does not wait for this kernel)
   const int tid = threadIdx.x;
   // (head blocks and token blocks in one grid dimension: a sequence of more than 4 M tokens has more than 65535 of the latter)
   const int nhb = (d.H + kXsHeads - 1) / kXsHeads, tb = blockIdx.x / nhb, b = blockIdx.z;
@@ -81,25 +81,24 @@ __global__ void __launch_bounds__(256) absmax_xs_kernel(const int8_t* __restrict
   }
 }
 
-__global__ void clear_words(uint32_t* a, int na, uint32_t* b, int nb, uint32_t* c, int nc) {
+__global__ void clear_words(uint32_t* a, int n) {
   pdl_launch_dependents();
   pdl_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < na) a[e] = 0u;
-  if (e < nb) b[e] = 0u;
-  if (e < nc) c[e] = 0u;
+  if (e < n) a[e] = 0u;
 }
 
-// s[k] holds a binary32 absmax, q[g] an int32 absmax of acc_cb; both become step sizes in place:
-// s = fdiv(s, 127), q = fdiv(fmul(float(q), fmul(s_C, s_B)), 127), 1 where the maximum is 0
-__global__ void finalize_scales(float* s, int n, float* q, int nq, const float* s_C, const float* s_B) {
+// step sizes from maxima: s_h = fdiv(max_h, 127), s_cb = fdiv(fmul(float(max_cb), fmul(s_C, s_B)), 127), 1 where the
+// maximum is 0
+__global__ void finalize_scales(const uint32_t* max_h, float* s_h, int n, const uint32_t* max_cb, float* s_cb, int nq,
+                                const float* s_C, const float* s_B) {
   pdl_launch_dependents();
   pdl_wait();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n) s[k] = __float_as_uint(s[k]) == 0u ? 1.0f : __fdiv_rn(s[k], 127.0f);
+  if (k < n) s_h[k] = step_of_max(max_h[k]);
   if (k < nq) {
-    const int v = __float_as_int(q[k]);
-    q[k] = v == 0 ? 1.0f : __fdiv_rn(__fmul_rn((float)v, __fmul_rn(s_C[k], s_B[k])), 127.0f);
+    const int v = (int)max_cb[k];
+    s_cb[k] = v == 0 ? 1.0f : __fdiv_rn(__fmul_rn((float)v, __fmul_rn(s_C[k], s_B[k])), 127.0f);
   }
 }
 
@@ -113,17 +112,16 @@ ssdi8_status_t launch_absmax_xs(const Dims& d, const int8_t* xq, const float* s_
   return launch_configured(absmax_xs_kernel, grid, dim3(256), 0, kStreamCarveout, false, st, xq, s_x, pack, absmax, d);
 }
 
-ssdi8_status_t launch_clear_words(void* a, i64 na, void* b, i64 nb, void* c, i64 nc, cudaStream_t st) {
-  const i64 n = na > nb ? (na > nc ? na : nc) : (nb > nc ? nb : nc);
+ssdi8_status_t launch_clear_words(void* a, i64 n, cudaStream_t st) {
   return launch_configured(clear_words, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, -1, false, st,
-                           static_cast<uint32_t*>(a), (int)na, static_cast<uint32_t*>(b), (int)nb, static_cast<uint32_t*>(c),
-                           (int)nc);
+                           static_cast<uint32_t*>(a), (int)n);
 }
 
-ssdi8_status_t launch_finalize_scales(float* s, i64 n, float* q, i64 nq, const float* s_C, const float* s_B, cudaStream_t st) {
+ssdi8_status_t launch_finalize_scales(const uint32_t* max_h, float* s_h, i64 n, const uint32_t* max_cb, float* s_cb, i64 nq,
+                                      const float* s_C, const float* s_B, cudaStream_t st) {
   const i64 m = n > nq ? n : nq;
-  return launch_configured(finalize_scales, dim3((unsigned)((m + 255) / 256)), dim3(256), 0, -1, false, st, s, (int)n, q,
-                           (int)nq, s_C, s_B);
+  return launch_configured(finalize_scales, dim3((unsigned)((m + 255) / 256)), dim3(256), 0, -1, false, st, max_h, s_h, (int)n,
+                           max_cb, s_cb, (int)nq, s_C, s_B);
 }
 
 }  // namespace ssdi8

@@ -33,7 +33,7 @@ using namespace sm100;
 struct FusedArgs {
   const float* s_x; const float* s_xs; const float* s_B; const float* s_h; const float* pack;
   const float* gamma; const float* init; float* final_state;
-  float* tap_loc; float* tap_prev; int8_t* tap_Xsq; int32_t* tap_acc; int32_t* status; uint32_t* absmax_h;
+  float* tap_loc; float* tap_prev; int8_t* tap_Xsq; int32_t* tap_acc; int32_t* status; uint32_t* absmax_h; float* s_xs_out;
   Dims d;
   int n_full;  // CTAs below this index own a whole (batch, head); the rest own a quarter (16 channels) of one
 };
@@ -144,8 +144,13 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     issue_x(0, (1u << (Q / 32)) - 1u);
     issue_B(0, (1u << (Q / 32)) - 1u);
   }
+  auto step_xs = [&](int p) -> float {   // (the calibration pass is given the maxima of |X_scaled|)
+    const float v = a.s_xs[h * P + p];
+    return CAL ? step_of_max(__float_as_uint(v)) : v;
+  };
   if (tid < 64) {
-    const float sxb = __fmul_rn(a.s_xs[h * P + tid], a.s_B[g]);
+    const float sx = step_xs(tid), sxb = __fmul_rn(sx, a.s_B[g]);
+    if (CAL && b == 0 && tid >= 16 * c0 && tid < 16 * (c0 + ncq)) a.s_xs_out[h * P + tid] = sx;
     if (CAL) {
       col_scale[tid] = sxb;
       col_invh[tid] = 0.f;               // running maximum of the channel
@@ -155,7 +160,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
       col_invh[tid] = __fdiv_rn(1.0f, sh);
     }
   } else if (tid < 128) {
-    col_rx[tid - 64] = __fdiv_rn(a.s_x[h * P + tid - 64], a.s_xs[h * P + tid - 64]);
+    col_rx[tid - 64] = __fdiv_rn(a.s_x[h * P + tid - 64], step_xs(tid - 64));
   }
   tc_fence_before();
   __syncthreads();
@@ -513,7 +518,7 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
                                           const float* init, int8_t* hq, float* final_state,
                                           float* tap_loc, float* tap_prev, int8_t* tap_Xsq,
                                           int32_t* tap_acc, int32_t* status, bool int8_state,
-                                          cudaStream_t st, uint32_t* absmax_h) {
+                                          cudaStream_t st, uint32_t* absmax_h, float* s_xs_out) {
   const uint64_t T = (uint64_t)d.b * d.L;
   CUtensorMap tm_B, tm_x, tm_hq;
   {
@@ -551,7 +556,7 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
   const bool quarters = 8 * (units - n_full) <= slots || (n_full == 0 && d.c >= 4 && 4 * units <= slots - slots / 10);
   if (!quarters) n_full = units;
   FusedArgs a = {s_x, s_xs, s_B, s_h, pack, gamma, init, final_state, tap_loc, tap_prev, tap_Xsq, tap_acc,
-                 status, absmax_h, d, n_full};
+                 status, absmax_h, s_xs_out, d, n_full};
   const size_t smem = SMEM_BYTES;
   const unsigned grid = (unsigned)(n_full + 4 * (units - n_full));
   const bool taps = tap_loc || tap_prev || tap_Xsq || tap_acc;

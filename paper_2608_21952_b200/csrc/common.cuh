@@ -197,6 +197,9 @@ __device__ __forceinline__ float softplus_dt(float dt_raw, float bias) {
   return (float)__dadd_rn(v > 0.0 ? v : 0.0, lp);
 }
 
+// step size of a channel from the bits of its largest magnitude (Eq. 1; an all-zero channel gets 1)
+__device__ __forceinline__ float step_of_max(uint32_t bits) { return bits == 0u ? 1.0f : __fdiv_rn(__uint_as_float(bits), 127.0f); }
+
 // Programmatic dependent launch.  Every kernel of the layer lets its successor in the stream be
 // scheduled early (launch_dependents at its start) and itself waits for its predecessor's completion
 // and memory flush (pdl_wait) before its first access to global memory, so only work that touches no

@@ -50,18 +50,26 @@ __device__ __forceinline__ void st_row(float* p, const float (&v)[TPL], uint64_t
 
 // TPL: tokens per lane, Q / 32.  SOFTPLUS: dt holds the raw time step and dt = softplus(dt + dt_bias[h])
 // (dt_bias may be NULL) is applied as the values are staged (Algorithm 2 module 1 starts there).
+// CLEAR: nclear words are set to 0 as well (calibration).
 // status: the caller's status word, cleared here (this is the first kernel of a forward pass), or NULL.
-template <int TPL, bool SOFTPLUS>
+template <int TPL, bool SOFTPLUS, bool CLEAR>
 __global__ void __launch_bounds__(32 * kMaxHeads) cumsum_kernel(const float* __restrict__ dt, const float* __restrict__ A,
                                                                 float* __restrict__ pack, float* __restrict__ gamma,
                                                                 float* __restrict__ tap_cs, Dims d,
-                                                                const float* __restrict__ dt_bias, int32_t* status) {
+                                                                const float* __restrict__ dt_bias, int32_t* status,
+                                                                uint32_t* clear, int nclear) {
   constexpr int Q = 32 * TPL, LD = Q + 4;
   __shared__ __align__(16) float dts[kMaxHeads * LD];
   // The wait comes first: a successor that needs nothing of this kernel (the layer step's quantiser of x, B
   // and C) is launched without a wait of its own at its start, so by the time it may be scheduled everything
   // that precedes this kernel in the stream must have completed.
   pdl_wait();
+  if (CLEAR) {   // (words that kernels behind the next one use, not all of which wait for this one: cleared ahead of the trigger)
+    const int nb = (int)(gridDim.x * gridDim.y * gridDim.z), blk = (int)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x);
+    for (int i = blk * (int)blockDim.x + (int)threadIdx.x; i < nclear; i += nb * (int)blockDim.x) clear[i] = 0u;
+    __threadfence();
+    __syncthreads();
+  }
   pdl_launch_dependents();
   const int hpb = (int)(blockDim.x >> 5), lh = 31 - __clz(hpb);   // heads of this block (a power of two)
   const int h0 = blockIdx.x * hpb, k = blockIdx.y, b = blockIdx.z;
@@ -235,7 +243,8 @@ ssdi8_status_t launch_softplus_dt(const float* dt_raw, const float* dt_bias, flo
 }
 
 ssdi8_status_t launch_cumsum(const Dims& d, const float* dt, const float* A, float* pack, float* gamma, float* tap_cs,
-                             cudaStream_t st, const float* dt_bias, bool softplus, int32_t* clear_status) {
+                             cudaStream_t st, const float* dt_bias, bool softplus, int32_t* clear_status,
+                             uint32_t* clear, int nclear) {
   const int sms = sm_count();
   if (sms == 0) return SSDI8_ERR_CUDA;
   // a grid that leaves SMs empty takes half the heads per block: one warp per scheduler, twice the SMs
@@ -244,15 +253,19 @@ ssdi8_status_t launch_cumsum(const Dims& d, const float* dt, const float* A, flo
   const dim3 grid((d.H + hpb - 1) / hpb, d.c, d.b);
   auto launch = [&](auto kernel) -> ssdi8_status_t {
     return launch_configured(kernel, grid, dim3(32 * hpb), 0, kStreamCarveout, false, st, dt, A, pack, gamma, tap_cs, d,
-                             dt_bias, clear_status);
+                             dt_bias, clear_status, clear, nclear);
+  };
+  if (nclear && softplus) return SSDI8_ERR_UNSUPPORTED;   // (calibration takes the positive time step)
+  auto pick = [&](auto sp, auto plain, auto clearing) -> ssdi8_status_t {
+    return softplus ? launch(sp) : nclear ? launch(clearing) : launch(plain);
   };
   ssdi8_status_t ls;
   if (d.Q == 256)
-    ls = softplus ? launch(cumsum_kernel<8, true>) : launch(cumsum_kernel<8, false>);
+    ls = pick(cumsum_kernel<8, true, false>, cumsum_kernel<8, false, false>, cumsum_kernel<8, false, true>);
   else if (d.Q == 128)
-    ls = softplus ? launch(cumsum_kernel<4, true>) : launch(cumsum_kernel<4, false>);
+    ls = pick(cumsum_kernel<4, true, false>, cumsum_kernel<4, false, false>, cumsum_kernel<4, false, true>);
   else
-    ls = softplus ? launch(cumsum_kernel<2, true>) : launch(cumsum_kernel<2, false>);
+    ls = pick(cumsum_kernel<2, true, false>, cumsum_kernel<2, false, false>, cumsum_kernel<2, false, true>);
   if (ls != SSDI8_OK) return ls;
   SSDI8_LAUNCH_CHECK();
   return SSDI8_OK;

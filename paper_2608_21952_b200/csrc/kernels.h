@@ -78,17 +78,19 @@ ssdi8_status_t launch_quantize_entry(const void* xBC, int dtype, i64 T_, int D, 
 ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, uint32_t flags, void* workspace,
                           size_t workspace_bytes, void* stream, bool clear_status);
 
-// pack [b,H,c,6,Q], gamma [b,H,c], tap_cs [b,H,c,Q] or NULL; clear_status: a status word the kernel sets to 0, or NULL
+// pack [b,H,c,6,Q], gamma [b,H,c], tap_cs [b,H,c,Q] or NULL; clear_status: a status word the kernel sets to 0, or NULL;
+// clear: so many words that it sets to 0 before the next kernel may be scheduled
 // softplus: dt is the raw time step, dt = softplus(dt + dt_bias[h]) is applied first (dt_bias may be NULL)
 ssdi8_status_t launch_cumsum(const Dims& d, const float* dt, const float* A, float* pack,
                              float* gamma, float* tap_cs, cudaStream_t st, const float* dt_bias = nullptr,
-                             bool softplus = false, int32_t* clear_status = nullptr);
+                             bool softplus = false, int32_t* clear_status = nullptr, uint32_t* clear = nullptr,
+                             int nclear = 0);
 ssdi8_status_t launch_softplus_dt(const float* dt_raw, const float* dt_bias, float* out, i64 rows, int H,
                                   cudaStream_t st);
 
 // acc_cb (tap, may be NULL), CBq (may be NULL when s_cb is NULL), absmax_acc: per-group
 // running max of |acc_cb| over the causal half (calibration; may be NULL).  after_state_kernel: the launch
-// directly follows launch_chunk_state_passing in the same stream and may run beside it (see bmm.cu)
+// directly follows launch_chunk_state_passing (or launch_absmax_xs) in the same stream and may run beside it (see bmm.cu)
 ssdi8_status_t launch_bmm(const Dims& d, const int8_t* Cq, const int8_t* Bq, const float* s_C,
                           const float* s_B, const float* s_cb, int8_t* CBq, int32_t* tap_acc,
                           uint32_t* absmax_acc, int32_t* status, cudaStream_t st, bool after_state_kernel = false);
@@ -99,14 +101,15 @@ ssdi8_status_t launch_chunk_state(const Dims& d, const int8_t* xq, const int8_t*
                                   int32_t* tap_acc, int32_t* status, cudaStream_t st);
 
 // ChunkState and StatePassing in one chunk-sequential kernel (loc never leaves the chip).  absmax_h (calibration):
-// per-channel running max (binary32 bits) of |S| over init and every S_k; no other output is written then
+// per-channel running max (binary32 bits) of |S| over init and every S_k; s_xs then holds the maxima of |X_scaled|, whose step
+// sizes go to s_xs_out, and no other output is written
 ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const int8_t* Bq,
                                           const float* s_x, const float* s_xs, const float* s_B,
                                           const float* s_h, const float* pack, const float* gamma,
                                           const float* init, int8_t* hq, float* final_state,
                                           float* tap_loc, float* tap_prev, int8_t* tap_Xsq,
                                           int32_t* tap_acc, int32_t* status, bool int8_state,
-                                          cudaStream_t st, uint32_t* absmax_h = nullptr);
+                                          cudaStream_t st, uint32_t* absmax_h = nullptr, float* s_xs_out = nullptr);
 
 // forward: in place of the fused state kernel (codes of a NaN)
 ssdi8_status_t launch_state_passing(const Dims& d, const float* loc, const float* gamma,
@@ -147,11 +150,12 @@ ssdi8_status_t launch_int8_mma_peak(int nbatch, int32_t* status, int* ctas, cuda
 int int8_mma_peak_batch();
 ssdi8_status_t launch_bounded_wait_expires(int32_t* status, cudaStream_t st);
 
-// calibration (calibrate.cu): per-channel running max of |X_scaled|; three arrays of words set to 0; step sizes from
-// maxima in place (s: binary32 absmax; q: int32 absmax of acc_cb, times s_C s_B), 1 where a maximum is 0
+// calibration (calibrate.cu): per-channel running max of |X_scaled|; words set to 0; step sizes from maxima (s_h: binary32
+// absmax; s_cb: int32 absmax of acc_cb, times s_C s_B), 1 where a maximum is 0
 ssdi8_status_t launch_absmax_xs(const Dims& d, const int8_t* xq, const float* s_x, const float* pack, uint32_t* absmax,
                                 cudaStream_t st);
-ssdi8_status_t launch_clear_words(void* a, i64 na, void* b, i64 nb, void* c, i64 nc, cudaStream_t st);
-ssdi8_status_t launch_finalize_scales(float* s, i64 n, float* q, i64 nq, const float* s_C, const float* s_B, cudaStream_t st);
+ssdi8_status_t launch_clear_words(void* a, i64 na, cudaStream_t st);
+ssdi8_status_t launch_finalize_scales(const uint32_t* max_h, float* s_h, i64 n, const uint32_t* max_cb, float* s_cb, i64 nq,
+                                      const float* s_C, const float* s_B, cudaStream_t st);
 
 }  // namespace ssdi8

@@ -93,6 +93,19 @@ def test_quantiser_gives_all_zero_channels_a_step_of_one(R, Ch, I):
     assert np.array_equal(q.reshape(-1), np.asarray(qr).reshape(-1))
 
 
+@pytest.mark.parametrize("R", [1, 3, 15, 17, 31, 33, 63, 2051])
+@pytest.mark.parametrize("Ch", [4, 508, 516])
+def test_absmax_takes_every_row_into_account(R, Ch):
+    # The largest value of each channel in a row of its own: remainders of the rows in flight, the row groups and the blocks
+    import gpu_harness as gh
+    v = np.random.default_rng(R).uniform(-1, 1, (R, Ch, 1)).astype(np.float32)
+    v[np.arange(Ch) * 7 % R, np.arange(Ch), 0] = -(2.0 + np.arange(Ch, dtype=np.float32))
+    q, s = gh.gpu_quantize(v, R, Ch, 1)
+    qr, sr = orc.quantize(v, R, Ch, 1, mode=1)
+    assert np.array_equal(s, sr)
+    assert np.array_equal(q.reshape(-1), np.asarray(qr).reshape(-1))
+
+
 @pytest.mark.parametrize("Q,N,H", [(256, 128, 5), (256, 64, 148), (256, 128, 149), (128, 128, 3)])
 def test_scan_with_one_chunk_per_cta(Q, N, H):
     # As many chunks as SMs, one more, and few: the mask groups take a tile each where a CTA has one chunk
