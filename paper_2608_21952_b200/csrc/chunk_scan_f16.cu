@@ -16,8 +16,7 @@
 // One factor per 16-column sub-block as in chunk_scan.cu: own sub-block by the running product of
 // per-token decays, earlier ones woff_j f with f the row's decay to the end of the sub-block before its own
 // times ChunkCumsum's tabulated block-to-block decay; a sub-block whose bound
-// says every |value| < 2^-25 (half of the smallest FP16 subnormal) is zero, and so is every
-// farther one where cs does not increase (p127, see cumsum.cu).  No multicast; bounded waits.
+// says every |value| < 2^-25 (half of the smallest FP16 subnormal) is zero.  No multicast; bounded waits.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -56,7 +55,7 @@ constexpr uint32_t OFF_X = 122880;      // ring of 2 x [256][64] fp16 (128-byte 
 constexpr uint32_t X_BYTES = 32768;
 constexpr uint32_t OFF_TOK = OFF_X + 2 * X_BYTES;   // ring of 4 x (5 Q floats: cs, dt, woff, atok, bounds)
 constexpr uint32_t TOK_BYTES = 6144;
-constexpr uint32_t TOK_SCAL = 5888;   // two scalars of the tile: s_C of the group, D of the head
+constexpr uint32_t TOK_SCAL = 5888;   // scalars of the tile: s_C of the group, D of the head, s_cb of the group
 constexpr uint32_t TOK_COLS = 5120;   // byte offset of the head's s_x, s_h and correction vectors ([64] each) in a slot
 constexpr uint32_t OFF_YST = OFF_TOK + 4 * TOK_BYTES;  // 8 warps x [32][64 B] y staging
 constexpr uint32_t OFF_BAR = OFF_YST + 16384;
@@ -98,24 +97,37 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, int b_mn_major) {
 }
 
 // ---- the FP16 operand of one tile, written to tensor memory.  A warp owns 32 rows (lane = row =
-// TMEM lane, warp index mod 4 = lane quarter) and the 16-column chunks of one parity q2; every
-// chunk of that parity in the contraction range gets one collective store of 8 packed words per
-// row (zeros where the chunk lies after the row's own, is skipped, or the row is idle).
+// TMEM lane, warp index mod 4 = lane quarter), which are two sub-blocks a16 and a16 + 1 of 16 tokens, and the 16-column
+// chunks of one parity q2; every chunk of that parity in the contraction range gets one collective store of 8 packed words per
+// row.  One chunk of the warp touches the diagonal: straight-line code, own sub-block for the rows that have it there, column
+// weights for the others.  Of the chunks ahead of both sub-blocks one ballot names those that hold a value of 2^-25 or more in some row
+// (bounds by ChunkCumsum, one chunk per lane; fmul is monotone, so the bound with the largest decay of a sub-block's rows is
+// at least every row's); the rest are stored as zeros.
+// (Before, every row tested its chunks one after the other inside the walk: 600 cycles each, most of them the latency of
+// that chain.  The paper's formats at batch 8 x 2048 x 80 heads, all kernels: 266.6 -> 259.1 us.)
 __device__ __forceinline__ void mask_tile_f16(const uint8_t* sCB, const float* tokbuf, uint32_t a_tmem, int rq,
                                               int q2, int lane, int TM, uint32_t RBQ, const Tile& t,
                                               const ScanArgs& a) {
   const int Q = a.d.Q;
+  const int nch = t.KJ >> 4;         // 16-column chunks in the contraction range
+  const uint32_t lane_addr = a_tmem + ((uint32_t)(rq * 32) << 16);
+  const uint32_t zero8[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+  if (rq * 32 >= TM) {               // idle rows (whole warps: TM is a multiple of 32)
+#pragma unroll 1
+    for (int c = q2; c < nch; c += 2) tmem_st8(lane_addr + (uint32_t)(c * 8), zero8);
+    tmem_st_wait();
+    return;
+  }
   const float* cs_s = tokbuf;
   const float* dt_s = tokbuf + Q;
   const float* woff_s = tokbuf + 2 * Q;
   const float* atok_s = tokbuf + 3 * Q;
   const float* b127_s = tokbuf + 4 * Q;
-  const float* p127_s = b127_s + 16;
+  const float scb = tokbuf[TOK_SCAL / 4 + 2];
   const int r = rq * 32 + lane;
-  const bool row_ok = r < TM;
   const int i = t.it * TM + r;       // row within the chunk
-  const int I16 = i >> 4, ri = i & 15;
-  const int nch = t.KJ >> 4;         // 16-column chunks in the contraction range
+  const int a16 = (t.it * TM + rq * 32) >> 4;
+  const int I16 = a16 + (lane >> 4), ri = lane & 15;
   const uint32_t cshift = RBQ == 128 ? 3u : 2u;  // log2(chunks per panel row)
   const uint8_t* const rowbase = sCB + (RBQ == 128 ? (uint32_t)r * 128u : (uint32_t)r * 64u);
   const uint32_t rx = RBQ == 128 ? ((uint32_t)r & 7u) : (((uint32_t)r >> 1) & 3u);  // swizzle term of the row
@@ -123,24 +135,57 @@ __device__ __forceinline__ void mask_tile_f16(const uint8_t* sCB, const float* t
     const uint32_t pn = (uint32_t)c >> cshift, cc = (uint32_t)c & ((1u << cshift) - 1u);
     return reinterpret_cast<const uint4*>(rowbase + pn * PANEL + ((cc ^ rx) << 4));
   };
-  const float cs_i = row_ok ? cs_s[i] : 0.f;
-  const float scb = a.s_cb[t.h / a.w.hpg];
   // decay to an earlier chunk c: the row's decay to the end of the chunk before its own, times the
   // tabulated decay from there to the end of chunk c (1 for c = I16 - 1)
-  const float ri_dec = I16 > 0 ? exp32(__fsub_rn(cs_i, cs_s[I16 * 16 - 1])) : 0.f;
+  const float dec = I16 > 0 ? exp32(__fsub_rn(cs_s[i], cs_s[I16 * 16 - 1])) : 0.f;
   const float* const gtab = b127_s + 32 + ((I16 * (I16 - 1)) >> 1);
   const float kTiny = 2.9e-8f;       // below 2^-25 = 2.98e-8: rounds to zero in FP16
-  const uint32_t lane_addr = a_tmem + ((uint32_t)(rq * 32) << 16);
-  bool done = !row_ok;               // this row has nothing (more) to contribute
-  // The row's own sub-block, right to left: E[i,i] = 1, E[i,j] = fmul(E[i,j+1], a_{j+1}).  Straight-line
-  // code ahead of the walk: a step that a row does not take multiplies by 1 (exact), a column past the
-  // diagonal is selected to 0, so the 32 rows of the warp (two sub-blocks, every diagonal position) do
-  // not diverge; the walk below only picks the result up when it reaches the sub-block.
-  uint32_t own[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-  {
-    const uint4 w4 = row_ok ? *chunk_ptr(I16) : make_uint4(0u, 0u, 0u, 0u);
+  // eight packed words of chunk c < I16 (zeros where the row's bound says so)
+  auto earlier = [&](int c, const uint4& w4, uint32_t (&w8)[8]) {
+    const float g = __fmul_rn(__fmul_rn(dec, gtab[c]), scb);
+    const bool live = __fmul_rn(b127_s[c], g) >= kTiny;
+    const float2 g2 = make_float2(g, g);
     const uint32_t ww[4] = {w4.x ^ 0x80808080u, w4.y ^ 0x80808080u, w4.z ^ 0x80808080u, w4.w ^ 0x80808080u};
-    const int i0 = row_ok ? I16 * 16 : 0;
+    const float4* wo = reinterpret_cast<const float4*>(woff_s + c * 16);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      const float4 fo = wo[w];
+      const uint32_t lo = half2_bits(__fmul2_rn(__fmul2_rn(unpack2(ww[w], 0), make_float2(fo.x, fo.y)), g2));
+      const uint32_t hi = half2_bits(__fmul2_rn(__fmul2_rn(unpack2(ww[w], 2), make_float2(fo.z, fo.w)), g2));
+      w8[2 * w] = live ? lo : 0u;
+      w8[2 * w + 1] = live ? hi : 0u;
+    }
+  };
+  // the chunks ahead of the warp's rows that are not all zeros
+  uint32_t m = 0;
+  {
+    float R = dec;                     // largest of the 16 rows of a sub-block
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) R = fmaxf(R, __shfl_xor_sync(0xffffffffu, R, o));
+    const float Ra = __shfl_sync(0xffffffffu, R, 0), Rb = __shfl_sync(0xffffffffu, R, 16);
+    bool live = false;
+    if (lane < a16 && (lane & 1) == q2) {
+      const float* const ga = b127_s + 32 + ((a16 * (a16 - 1)) >> 1);   // (row a16 + 1 of the table follows a16 entries on)
+      const float b = b127_s[lane];
+      live = __fmul_rn(b, __fmul_rn(__fmul_rn(Ra, ga[lane]), scb)) >= kTiny ||
+             __fmul_rn(b, __fmul_rn(__fmul_rn(Rb, ga[a16 + lane]), scb)) >= kTiny;
+    }
+    m = __ballot_sync(0xffffffffu, live);
+  }
+  const int cd = (a16 & 1) == q2 ? a16 : a16 + 1;   // the warp's chunk on the diagonal
+#pragma unroll 1
+  for (int c = q2; c < nch; c += 2)
+    if (c != cd && !((m >> c) & 1u)) tmem_st8(lane_addr + (uint32_t)(c * 8), zero8);
+  int c = m ? 31 - __clz(m) : -1;
+  uint4 w4 = *chunk_ptr(c >= 0 ? c : cd);   // (a chunk ahead of its use)
+  // The row's own sub-block, right to left: E[i,i] = 1, E[i,j] = fmul(E[i,j+1], a_{j+1}).  Straight-line code: a step that
+  // a row does not take multiplies by 1 (exact), a column past the diagonal is selected to 0, so the 32 rows of the warp (two
+  // sub-blocks, every diagonal position) do not diverge.
+  {
+    const uint4 w4d = *chunk_ptr(cd);
+    uint32_t own[8];
+    const uint32_t ww[4] = {w4d.x ^ 0x80808080u, w4d.y ^ 0x80808080u, w4d.z ^ 0x80808080u, w4d.w ^ 0x80808080u};
+    const int i0 = I16 * 16;
     const float2 scb2 = make_float2(scb, scb);
     float E = 1.0f;
 #pragma unroll
@@ -167,34 +212,27 @@ __device__ __forceinline__ void mask_tile_f16(const uint8_t* sCB, const float* t
         own[e >> 1] = half2_bits(make_float2(k <= rr ? t2.x : 0.f, k + 1 <= rr ? t2.y : 0.f));
       }
     }
+    if (cd == a16) {                   // the upper sub-block's rows have it next to their own
+      uint32_t near8[8];
+      earlier(a16, w4d, near8);        // (of the lower rows' gtab: entry a16 of row a16, the next row's first; not used)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) own[e] = lane < 16 ? own[e] : near8[e];
+    } else {                           // the lower sub-block's rows end ahead of it
+#pragma unroll
+      for (int e = 0; e < 8; ++e) own[e] = lane < 16 ? 0u : own[e];
+    }
+    tmem_st8(lane_addr + (uint32_t)(cd * 8), own);
   }
 #pragma unroll 1
-  for (int c = ((nch - 1 - q2) & ~1) + q2; c >= 0; c -= 2) {
-    uint32_t w8[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-    if (!done && c == I16) {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) w8[e] = own[e];
-    } else if (!done && c < I16) {
-      {
-        const float g = __fmul_rn(__fmul_rn(ri_dec, gtab[c]), scb);
-        if (__fmul_rn(p127_s[c], g) < kTiny) {
-          done = true;               // this chunk and every farther one round to zero
-        } else if (__fmul_rn(b127_s[c], g) >= kTiny) {
-          const float2 g2 = make_float2(g, g);
-          const uint4 w4 = *chunk_ptr(c);
-          const uint32_t ww[4] = {w4.x ^ 0x80808080u, w4.y ^ 0x80808080u, w4.z ^ 0x80808080u, w4.w ^ 0x80808080u};
-          const float4* wo = reinterpret_cast<const float4*>(woff_s + c * 16);
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            const float4 fo = wo[w];
-            w8[2 * w] = half2_bits(__fmul2_rn(__fmul2_rn(unpack2(ww[w], 0), make_float2(fo.x, fo.y)), g2));
-            w8[2 * w + 1] = half2_bits(__fmul2_rn(__fmul2_rn(unpack2(ww[w], 2), make_float2(fo.z, fo.w)), g2));
-          }
-        }
-      }
-    }
-    __syncwarp();
+  while (c >= 0) {
+    m ^= 1u << c;
+    const int cn = m ? 31 - __clz(m) : -1;
+    uint32_t w8[8];
+    const uint4 wn = *chunk_ptr(cn >= 0 ? cn : c);
+    earlier(c, w4, w8);
     tmem_st8(lane_addr + (uint32_t)(c * 8), w8);
+    c = cn;
+    w4 = wn;
   }
   tmem_st_wait();
 }
@@ -295,6 +333,7 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
           float* sc = reinterpret_cast<float*>(slot + TOK_SCAL);
           sc[0] = a.s_C[tg];
           sc[1] = a.D ? a.D[t.h] : 0.f;
+          sc[2] = a.s_cb[tg];
         }
         mbar_expect_tx(&bars[B_TOK_FULL + t3], (uint32_t)(5 * Q * 4 + (CORR ? 3 : 2) * P * 4));
         bulk_load(slot, a.pack + t.unit * kPackRows * Q, (uint32_t)(5 * Q * 4), &bars[B_TOK_FULL + t3]);
