@@ -111,7 +111,7 @@ ssdi8_status_t ssdi8_chunk_scan_fwd(const ssdi8_dims_t* dims, const ssdi8_fwd_ar
 
 namespace ssdi8 {
 ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, uint32_t flags, void* workspace,
-                          size_t workspace_bytes, void* stream, bool clear_status) {
+                          size_t workspace_bytes, void* stream, bool clear_status, const LayerInputs* layer) {
   if (!dims || !a) return SSDI8_ERR_NULL;
   if ((flags & ~kFwdFlags) != 0) return SSDI8_ERR_UNSUPPORTED;
   const bool i8s = (flags & SSDI8_FLAG_INT8_STATE) != 0;
@@ -153,7 +153,11 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
   int32_t* const to_clear = clear_status ? a->status : nullptr;
   if (to_clear && !(ph & SSDI8_PHASE_CUMSUM)) SSDI8_CUDA_CHECK(cudaMemsetAsync(to_clear, 0, sizeof(int32_t), st));
 
-  if ((ph & SSDI8_PHASE_CUMSUM) && (s = launch_cumsum(d, a->dt, a->A, pack, gamma, a->tap_cs, st, a->dt_bias,
+  if (layer) {
+    if ((s = launch_lead(d, *layer, a->dt, a->A, pack, gamma, a->s_x, a->s_B, a->s_C, const_cast<int8_t*>(a->xq),
+                         const_cast<int8_t*>(a->Bq), const_cast<int8_t*>(a->Cq), to_clear, st)) != SSDI8_OK)
+      return s;
+  } else if ((ph & SSDI8_PHASE_CUMSUM) && (s = launch_cumsum(d, a->dt, a->A, pack, gamma, a->tap_cs, st, a->dt_bias,
                                                      (flags & SSDI8_FLAG_DT_SOFTPLUS) != 0, to_clear)) != SSDI8_OK)
     return s;
   // ChunkBMM depends on neither ChunkCumsum nor the state kernels and is needed by ChunkScan only.  When both

@@ -187,33 +187,17 @@ ssdi8_status_t layer_step(const ssdi8_dims_t& d, const ssdi8_layer_args_t& a, co
                           const float* C, const float* dt, const float* init, float* y, float* fin,
                           int32_t* status, int8_t* xq, int8_t* Bq, int8_t* Cq, void* ws, size_t ws_bytes,
                           uint32_t flags, cudaStream_t st, bool clear_status) {
-  const int64_t T = (int64_t)d.batch * d.seqlen;
   ssdi8_fwd_args_t f = {};
   f.xq = xq; f.Bq = Bq; f.Cq = Cq;
   f.s_x = a.s_x; f.s_B = a.s_B; f.s_C = a.s_C;
   f.dt = dt; f.A = a.A; f.D = a.D; f.corr = a.corr;
   f.s_xs = a.s_xs; f.s_cb = a.s_cb; f.s_h = a.s_h;
   f.init_state = init; f.y = y; f.final_state = fin; f.status = status;
-  const uint32_t fl = flags & kLayerFlags;
-  ssdi8_status_t s;
   // (the three quantisers are one launch: it needs a power-of-two N, which every supported N is, and 16-byte
   // aligned tensors, which the entry points have checked or provide themselves)
   if ((d.dstate & (d.dstate - 1)) != 0) return SSDI8_ERR_UNSUPPORTED;
-  // ChunkCumsum (it reads dt and A only) and the quantisers need nothing of each other.  ChunkCumsum goes
-  // first and lets its successor be scheduled once its own wait for the work ahead of the layer is over;
-  // the quantisers' launch then starts without a wait and runs beside it, with the wait at the end of its
-  // last block (see quant_jobs), so that the state kernel, which waits for the quantisers' launch, has
-  // ChunkCumsum complete as well.  One stream, no events.  Measured per step, this chain / ChunkCumsum on a
-  // side stream / ChunkCumsum's blocks inside the quantisers' grid: 0.286 / 0.293 / 0.287 ms at batch
-  // 8 x 2048 x 80 heads, 0.056 / 0.062 / 0.062 ms at 2048 x 24 heads.
-  if ((s = fwd_phases(&d, &f, fl | SSDI8_PHASE_CUMSUM, ws, ws_bytes, st, clear_status)) != SSDI8_OK) return s;
-  if ((s = launch_quantize_xbc(x, B, C, T, d.nheads * d.headdim, d.ngroups, d.dstate, a.s_x, a.s_B, a.s_C, xq, Bq, Cq, st,
-                               true)) != SSDI8_OK)
-    return s;
-  // the rest, chained by programmatic dependent launch: the fused state kernel, ChunkBMM (needed by ChunkScan
-  // only: launched behind the state kernel, it works beside that kernel's last wave), ChunkScan
-  return fwd_phases(&d, &f, fl | SSDI8_PHASE_BMM | SSDI8_PHASE_CHUNK_STATE | SSDI8_PHASE_STATE_PASSING | SSDI8_PHASE_SCAN,
-                    ws, ws_bytes, st, false);
+  const LayerInputs in = {x, B, C};
+  return fwd_phases(&d, &f, flags & kLayerFlags, ws, ws_bytes, st, clear_status, &in);
 }
 
 bool layer_args_ok(const ssdi8_layer_args_t* a) {

@@ -55,13 +55,14 @@ constexpr int kStreamCarveout = 28;
 ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* scale, int mode,
                                int8_t* out, cudaStream_t st);
 
-// the layer's three static quantisers as one launch: x [T][D] with D step sizes, B and C [T][G N] with G
-// step sizes each (N a power of two, D and N multiples of 4).
-// after_cumsum: the launch directly follows launch_cumsum of the same layer in the same stream and runs beside
-// it (see quant_jobs).
-ssdi8_status_t launch_quantize_xbc(const float* x, const float* B, const float* C, i64 T_, int D, int G, int N,
-                                   const float* s_x, const float* s_B, const float* s_C, int8_t* xq, int8_t* Bq,
-                                   int8_t* Cq, cudaStream_t st, bool after_cumsum = false);
+// The head of a layer step: ChunkCumsum, and the three static quantisers (x [T][H P] with H P step sizes, B and C [T][G N] with G
+// step sizes each), as one launch or two.  clear_status: a status word that is set to 0, or NULL.
+struct LayerInputs {
+  const float* x; const float* B; const float* C;
+};
+ssdi8_status_t launch_lead(const Dims& d, const LayerInputs& in, const float* dt, const float* A, float* pack, float* gamma,
+                           const float* s_x, const float* s_B, const float* s_C, int8_t* xq, int8_t* Bq, int8_t* Cq,
+                           int32_t* clear_status, cudaStream_t st);
 
 // Per-(batch, head, chunk) pack of kPackRows rows of Q floats: cs, dt, woff, atok, wmax, lut (see
 // cumsum.cu); element (u, row, i) at pack[(u * kPackRows + row) * Q + i], u = (b*H + h)*c + k.
@@ -73,10 +74,10 @@ ssdi8_status_t launch_quantize_entry(const void* xBC, int dtype, i64 T_, int D, 
                                      const float* s_B, const float* s_C, int8_t* xq, int8_t* Bq, int8_t* Cq,
                                      cudaStream_t st);
 
-// ssdi8_chunk_scan_fwd's body; clear_status = false leaves the status word alone (callers that run
-// the modules as several calls clear it once themselves)
+// ssdi8_chunk_scan_fwd's body; clear_status = false leaves the status word alone (the host pipeline clears it once for all
+// its slices).  layer: the layer step, which quantises these (16-byte aligned) into a->xq, Bq and Cq first; all modules run then
 ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, uint32_t flags, void* workspace,
-                          size_t workspace_bytes, void* stream, bool clear_status);
+                          size_t workspace_bytes, void* stream, bool clear_status, const LayerInputs* layer = nullptr);
 
 // pack [b,H,c,6,Q], gamma [b,H,c], tap_cs [b,H,c,Q] or NULL; clear_status: a status word the kernel sets to 0, or NULL;
 // clear: so many words that it sets to 0 before the next kernel may be scheduled

@@ -2,7 +2,7 @@
 // of the view in[R][Ch][I].  HBM-bound: 16-byte loads, 4-byte packed stores, every warp
 // instruction fully coalesced; absmax by per-thread running maxima, warp shuffles and
 // one order-independent atomicMax on the (non-negative) binary32 bit pattern.
-#include "kernels.h"
+#include "cumsum.cuh"
 
 namespace ssdi8 {
 namespace {
@@ -73,21 +73,7 @@ struct QuantJobs {
   int late_wait;   // 1: launched right behind ChunkCumsum of the same layer, which it does not depend on (see the kernel)
 };
 
-__global__ void __launch_bounds__(128, 8) quant_jobs(const QuantJobs a) {
-  pdl_launch_dependents();
-  // Programmatic dependent launch.  Normally: wait for the predecessor before the first global access.
-  // Launched right behind ChunkCumsum (which waits for ITS predecessor before it lets this kernel be
-  // scheduled, and whose outputs this kernel does not touch), the blocks start at once and work beside
-  // that kernel.  The wait moves to the end of the grid's last block (one waiting block is enough, and a
-  // wait in every block would keep the early ones resident until ChunkCumsum has finished): it keeps
-  // "this kernel complete" implying "ChunkCumsum complete" for the state kernel that follows, and by then
-  // it returns at once.
-  if (!a.late_wait) pdl_wait();
-  struct LateWait {
-    bool on;
-    __device__ ~LateWait() { if (on) pdl_wait(); }
-  } late_wait_at_exit{a.late_wait != 0 && blockIdx.x == gridDim.x - 1};
-  const int blk = (int)blockIdx.x;
+__device__ __forceinline__ void quant_block(const QuantJobs& a, const int blk) {
   const int jb = blk >= a.job[2].first_block ? 2 : blk >= a.job[1].first_block ? 1 : 0;
   const QuantJob& j = a.job[jb];
   const int rel = blk - j.first_block;
@@ -127,6 +113,40 @@ __global__ void __launch_bounds__(128, 8) quant_jobs(const QuantJobs a) {
   }
   // (a layer's token count is a multiple of 64, which leaves no rest; the short form keeps the registers from spilling)
   for (; left > 0; --left, e += stride) out[e] = code4_by_division(__ldcs(in + e), s);
+}
+
+__global__ void __launch_bounds__(128, 8) quant_jobs(const QuantJobs a) {
+  pdl_launch_dependents();
+  // Programmatic dependent launch.  Normally: wait for the predecessor before the first global access.
+  // Launched right behind ChunkCumsum (which waits for ITS predecessor before it lets this kernel be
+  // scheduled, and whose outputs this kernel does not touch), the blocks start at once and work beside
+  // that kernel.  The wait moves to the end of the grid's last block (one waiting block is enough, and a
+  // wait in every block would keep the early ones resident until ChunkCumsum has finished): it keeps
+  // "this kernel complete" implying "ChunkCumsum complete" for the state kernel that follows, and by then
+  // it returns at once.
+  if (!a.late_wait) pdl_wait();
+  struct LateWait {
+    bool on;
+    __device__ ~LateWait() { if (on) pdl_wait(); }
+  } late_wait_at_exit{a.late_wait != 0 && blockIdx.x == gridDim.x - 1};
+  quant_block(a, (int)blockIdx.x);
+}
+
+// ---- ChunkCumsum and the three quantisers of a layer as one launch: the first ncum blocks take four heads of a chunk each
+// (hblocks blocks to a chunk).  See launch_lead for where it is taken.
+template <int TPL>
+__global__ void __launch_bounds__(128, 8) lead_kernel(const QuantJobs a, const cumsum::Args c, int ncum, int hblocks) {
+  __shared__ __align__(16) float dts[4 * (32 * TPL + 4)];
+  pdl_wait();
+  pdl_launch_dependents();
+  const int blk = (int)blockIdx.x;
+  if (blk >= ncum) {
+    quant_block(a, blk - ncum);
+    return;
+  }
+  if (c.status && blk == 0 && threadIdx.x == 0) *c.status = 0;
+  const int bk = blk / hblocks;
+  cumsum::chunk_of_heads<TPL, false>(dts, 4, (blk - bk * hblocks) * 4, bk % c.d.c, bk / c.d.c, c);
 }
 
 // ---- quantise, I % 4 == 0: 4 consecutive elements share a channel
@@ -283,12 +303,12 @@ ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* sca
                            (uint32_t)(I / 4), (uint32_t)Ch);
 }
 
-ssdi8_status_t launch_quantize_xbc(const float* x, const float* B, const float* C, i64 T_, int D, int G, int N,
-                                   const float* s_x, const float* s_B, const float* s_C, int8_t* xq, int8_t* Bq,
-                                   int8_t* Cq, cudaStream_t st, bool after_cumsum) {
-  if (T_ == 0) return SSDI8_OK;
-  if (T_ * D / 4 >= ((i64)1 << 31) || T_ * G * N / 4 >= ((i64)1 << 31)) return SSDI8_ERR_UNSUPPORTED;
-  QuantJobs a;
+namespace {
+
+// the jobs of a layer; returns the number of blocks, 0 where an index would not fit
+int make_jobs(QuantJobs& a, const float* x, const float* B, const float* C, i64 T_, int D, int G, int N, const float* s_x,
+              const float* s_B, const float* s_C, int8_t* xq, int8_t* Bq, int8_t* Cq) {
+  if (T_ * D / 4 >= ((i64)1 << 31) || T_ * G * N / 4 >= ((i64)1 << 31)) return 0;
   a.R = T_;
   int shift = 0;
   while ((1 << shift) < N) ++shift;   // N is a power of two here (the caller checks)
@@ -309,8 +329,45 @@ ssdi8_status_t launch_quantize_xbc(const float* x, const float* B, const float* 
   };
   int nb = fill(a.job[0], B, s_B, Bq, G * N, shift, 0);
   nb = fill(a.job[1], C, s_C, Cq, G * N, shift, nb);
-  nb = fill(a.job[2], x, s_x, xq, D, 0, nb);
-  a.late_wait = after_cumsum ? 1 : 0;
+  return fill(a.job[2], x, s_x, xq, D, 0, nb);
+}
+
+}  // namespace
+
+ssdi8_status_t launch_lead(const Dims& d, const LayerInputs& in, const float* dt, const float* A, float* pack, float* gamma,
+                           const float* s_x, const float* s_B, const float* s_C, int8_t* xq, int8_t* Bq, int8_t* Cq,
+                           int32_t* clear_status, cudaStream_t st) {
+  QuantJobs a;
+  const i64 T = (i64)d.b * d.L;
+  const int nb = make_jobs(a, in.x, in.B, in.C, T, d.H * d.P, d.G, d.N, s_x, s_B, s_C, xq, Bq, Cq);
+  if (nb == 0) return SSDI8_ERR_UNSUPPORTED;
+  a.late_wait = 0;
+  const int hblocks = (d.H + 3) / 4;
+  const i64 ncum = (i64)hblocks * d.c * d.b;
+  // One launch or two, by tokens x heads.  One saves a launch, which is what the smallest layers consist of, and where the blocks of
+  // both fill the device a few times over ChunkCumsum's run in the gaps of the quantisers'; in between ChunkCumsum is on the
+  // critical path and its own launch has the shorter chain (eight warps a block, more registers), and with many waves the
+  // quantisers alone keep the memory busier.  Layer, us, two launches / one: 512 x 4 (chunks of 64) 16.6 / 16.0; 512 x 24 18.9 /
+  // 19.7, 2048 x 24 28.4 / 29.2, 1024 x 80 31.3 / 32.3; 2048 x 80 48.1 / 46.5, 8 x 1024 x 20 (chunks of 128) 56.7 / 52.1, 3 x 1408 x
+  // 50 (chunks of 128) 68.9 / 64.7, 4 x 1024 x 80 71.9 / 70.1, 8192 x 60 126.2 / 125.7; 12 x 1024 x 100 221 / 227, 8 x 2048 x 80
+  // 230 / 237.
+  const i64 th = T * d.H;
+  if (th <= 4096 || (th >= 128 * 1024 && th <= 512 * 1024)) {
+    const cumsum::Args c = {dt, A, pack, gamma, nullptr, nullptr, clear_status, d};
+    auto launch = [&](auto kernel) -> ssdi8_status_t {
+      return launch_configured(kernel, dim3((unsigned)(nb + ncum)), dim3(128), 0, kStreamCarveout, false, st, a, c, (int)ncum, hblocks);
+    };
+    return d.Q == 256 ? launch(lead_kernel<8>) : d.Q == 128 ? launch(lead_kernel<4>) : launch(lead_kernel<2>);
+  }
+  // ChunkCumsum (it reads dt and A only) and the quantisers need nothing of each other.  ChunkCumsum goes
+  // first and lets its successor be scheduled once its own wait for the work ahead of the layer is over;
+  // the quantisers' launch then starts without a wait and runs beside it, with the wait at the end of its
+  // last block (see quant_jobs), so that the state kernel, which waits for the quantisers' launch, has
+  // ChunkCumsum complete as well.  One stream, no events.  (ChunkCumsum on a side stream instead: 0.293 against 0.286 ms at
+  // batch 8 x 2048 x 80 heads.)
+  const ssdi8_status_t s = launch_cumsum(d, dt, A, pack, gamma, nullptr, st, nullptr, false, clear_status);
+  if (s != SSDI8_OK) return s;
+  a.late_wait = 1;
   return launch_configured(quant_jobs, dim3((unsigned)nb), dim3(128), 0, kStreamCarveout, false, st, a);
 }
 

@@ -106,6 +106,43 @@ def test_absmax_takes_every_row_into_account(R, Ch):
     assert np.array_equal(q.reshape(-1), np.asarray(qr).reshape(-1))
 
 
+@pytest.mark.parametrize("b,L,H,N,G,Q", [(1, 64, 1, 64, 1, 64), (1, 128, 7, 128, 1, 128), (2, 256, 8, 64, 2, 256), (1, 256, 17, 128, 1, 256),
+                                         (2, 1024, 63, 64, 1, 128), (5, 1280, 21, 64, 3, 256), (4, 1024, 129, 64, 1, 64)])
+def test_layer_head_in_one_launch_and_in_two(b, L, H, N, G, Q):
+    # On either side of the lines of the dispatch, head counts that leave a block of four heads partly idle: the layer call
+    # gives the bits of the separate calls, whose ChunkCumsum and quantisers are launches of their own
+    import torch
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("lead", b, L, H, 64, N, G, Q, 0.02, 20.0, 48)
+    t = inputs.make_prefill(cfg)
+    T, HP = b * L, H * 64
+    s = {"s_x": np.full(HP, 0.05), "s_B": np.full(G, 0.03), "s_C": np.full(G, 0.03), "s_xs": np.full(HP, 0.002),
+         "s_cb": np.full(G, 0.4), "s_h": np.full(HP, 0.02)}
+    s = {k: gh.dev(v.astype(np.float32)) for k, v in s.items()}
+    dv = {k: gh.dev(np.asarray(v, np.float32)) for k, v in t.items()}
+    codes = {k: torch.empty(n, dtype=torch.int8, device="cuda") for k, n in (("xq", (T, HP)), ("Bq", (T, G * N)), ("Cq", (T, G * N)))}
+    bd.ssdi8_quantize_act(dv["x"], T, HP, 1, s["s_x"], 0, codes["xq"])
+    bd.ssdi8_quantize_act(dv["B"], T, G, N, s["s_B"], 0, codes["Bq"])
+    bd.ssdi8_quantize_act(dv["C"], T, G, N, s["s_C"], 0, codes["Cq"])
+    dims = bd.dims_of(cfg)
+    out = []
+    for layer in (False, True):
+        y = torch.full((b, L, H, 64), float("nan"), device="cuda")
+        fin = torch.full((b, H, 64, N), float("nan"), device="cuda")
+        status = torch.full((1,), 5, dtype=torch.int32, device="cuda")
+        rest = dict(dt=dv["dt"], A=dv["A"], D=dv["D"], y=y, final_state=fin, status=status, **s)
+        if layer:
+            ws = torch.empty(bd.ssdi8_layer_fwd_workspace_bytes(dims), dtype=torch.uint8, device="cuda")
+            bd.ssdi8_layer_fwd(dims, bd.make_layer_args(x=dv["x"], B=dv["B"], C=dv["C"], **rest), ws)
+        else:
+            bd.ssdi8_chunk_scan_fwd(dims, bd.make_fwd_args(**codes, **rest), bd.alloc_workspace(dims))
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        out.append((y, fin))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
 @pytest.mark.parametrize("Q,N,H", [(256, 128, 5), (256, 64, 148), (256, 128, 149), (128, 128, 3)])
 def test_scan_with_one_chunk_per_cta(Q, N, H):
     # As many chunks as SMs, one more, and few: the mask groups take a tile each where a CTA has one chunk
