@@ -306,6 +306,26 @@ def test_output_does_not_depend_on_the_pace_of_the_epilogue(Q, taps):
         assert np.array_equal(y, want[0]) and np.array_equal(fin, want[1])
 
 
+@pytest.mark.parametrize("flag", ["INT8", "FP16"])
+@pytest.mark.parametrize("Q", [128, 256])
+def test_few_heads_give_the_bits_of_the_same_heads_among_many(Q, flag):
+    # One chunk per CTA (its mask groups take a tile each) against several
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    flags = bd.FLAG_FP16_OPERAND if flag == "FP16" else 0
+    many = SSDConfig("many", 1, Q, 320, 64, 128, 1, Q, 0.02, 20.0, 49)
+    q = _random_codes(many, 49)
+    want = gh.gpu_fwd(many, q, taps=(), flags=flags)[:2]
+    few = SSDConfig("few", 1, Q, 7, 64, 128, 1, Q, 0.02, 20.0, 49)
+    cut = dict(q)
+    for k in ("xq", "dt", "A", "D", "s_x", "s_xs", "s_h", "init"):
+        v = np.asarray(q[k])
+        axis = [n for n, size in enumerate(v.shape) if size in (320, 320 * 64)][0]
+        cut[k] = np.ascontiguousarray(np.take(v, np.arange(v.shape[axis] // 320 * 7), axis=axis))
+    y, fin, _ = gh.gpu_fwd(few, cut, taps=(), flags=flags)
+    assert np.array_equal(y, want[0][:, :, :7]) and np.array_equal(fin, want[1][:, :7])
+
+
 @pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
 @pytest.mark.parametrize("Q", [64, 256])
 def test_a_time_step_that_is_not_finite_does_not_reach_earlier_tokens(Q, value):
