@@ -20,7 +20,7 @@ struct BmmArgs {
   int32_t* tap_acc; uint32_t* absmax_acc; int32_t* status;
   Dims d;
   int store;  // 0: calibration pass (no CBq written)
-  int late_wait;  // 1: launched right after the fused state kernel, which it does not depend on (see below)
+  int late_wait;  // 1: launched right after a kernel that it does not depend on, the fused state kernel or the calibration's pass over xq (see below)
 };
 
 constexpr int kThreads = 512;   // 16 warps: warp w reads TMEM lane quarter w % 4 (rows) and every fourth 32-column piece from w / 4
