@@ -260,7 +260,7 @@ ssdi8_status_t ssdi8_chunk_scan_fwd_static(const ssdi8_dims_t* dims, const ssdi8
  * ssdi8_layer_fwd: every pointer is a DEVICE pointer.  The three quantisers are one launch (x, B and C
  *   must be 16-byte aligned like every other tensor: SSDI8_ERR_ALIGN otherwise, before anything is
  *   enqueued); all kernels run on `stream`, chained by programmatic dependent launch: ChunkCumsum (reads
- *   dt and A only) first, the quantisers' launch beside it (or both as one launch, by size), then the state kernel,
+ *   dt and A only) first, the quantisers' launch beside it (or both as one launch, by chunk length and size), then the state kernel,
  *   ChunkBMM beside the state kernel's last wave, and ChunkScan; no other stream, no event.  The call may be captured into a
  *   CUDA graph.  workspace: 256-byte aligned,
  *   ssdi8_layer_fwd_workspace_bytes(dims, flags) bytes (the int8 tensors plus ssdi8_workspace_bytes).

@@ -346,20 +346,25 @@ ssdi8_status_t launch_lead(const Dims& d, const LayerInputs& in, const float* dt
   a.late_wait = 0;
   const int hblocks = (d.H + 3) / 4;
   const i64 ncum = (i64)hblocks * d.c * d.b;
-  // One launch or two, by tokens x heads.  One saves a launch, which is what the smallest layers consist of, and where the blocks of
-  // both fill the device a few times over ChunkCumsum's run in the gaps of the quantisers'; in between ChunkCumsum is on the
-  // critical path and its own launch has the shorter chain (eight warps a block, more registers), and with many waves the
-  // quantisers alone keep the memory busier.  Layer, us, two launches / one: 512 x 4 (chunks of 64) 16.6 / 16.0; 512 x 24 18.9 /
-  // 19.7, 2048 x 24 28.4 / 29.2, 1024 x 80 31.3 / 32.3; 2048 x 80 48.1 / 46.5, 8 x 1024 x 20 (chunks of 128) 56.7 / 52.1, 3 x 1408 x
-  // 50 (chunks of 128) 68.9 / 64.7, 4 x 1024 x 80 71.9 / 70.1, 8192 x 60 126.2 / 125.7; 12 x 1024 x 100 221 / 227, 8 x 2048 x 80
-  // 230 / 237.
+  // One launch or two, by chunk length and tokens x heads.  One saves a launch, which is what the smallest layers consist of,
+  // and where the blocks of both fill the device a few times over ChunkCumsum's run in the gaps of the quantisers'; in between
+  // ChunkCumsum is on the critical path and its own launch has the shorter chain (eight warps a block, more registers), and with
+  // many waves the quantisers alone keep the memory busier.  Chunks of 256 have two everywhere: eight tokens a lane do not
+  // fit the 64 registers that the quantisers leave a thread.  Layer calls in a row, us, two launches / one:
+  //   chunks of 64:  512 x 4 17.2 / 16.7, 256 x 8 16.3 / 15.5, 1024 x 4 18.0 / 18.1; one chunk x 6 heads 13.3 / 13.7; 1024 x 8 19.7 / 21.3;
+  //     2 x 1024 x 64 (N 128) 73.6 / 71.8, 4 x 3392 x 28 195.6 / 181.8, 3 x 1408 x 50 102.8 / 101.8 (N 128: 100.3 / 103.6, the one loss beyond
+  //     the noise of 70 sizes), 8 x 1024 x 80 190.3 / 190.3
+  //   chunks of 128: 512 x 4 17.0 / 16.4, 256 x 8 15.4 / 15.7, 1024 x 8 19.7 / 19.4, 512 x 24 19.6 / 20.0; 8 x 1024 x 20 56.8 / 53.0,
+  //     3 x 1408 x 50 72.2 / 70.8, 4 x 1024 x 64 70.9 / 70.5, 8 x 1024 x 80 140.2 / 140.8
+  //   chunks of 256: 1024 x 4 18.6 / 18.9, 256 x 16 17.9 / 19.1; with N 128 2048 x 80 51.2 / 50.2, but 8 x 1024 x 20 49.2 / 52.4, 4 x 1024 x 40 51.8 / 54.4,
+  //     4 x 1024 x 64 64.2 / 66.0
   const i64 th = T * d.H;
-  if (th <= 4096 || (th >= 128 * 1024 && th <= 512 * 1024)) {
+  if (d.Q <= 128 && ((d.c >= 3 && th <= 4096) || (th >= 128 * 1024 && th <= 512 * 1024))) {
     const cumsum::Args c = {dt, A, pack, gamma, nullptr, nullptr, clear_status, d};
     auto launch = [&](auto kernel) -> ssdi8_status_t {
       return launch_configured(kernel, dim3((unsigned)(nb + ncum)), dim3(128), 0, kStreamCarveout, false, st, a, c, (int)ncum, hblocks);
     };
-    return d.Q == 256 ? launch(lead_kernel<8>) : d.Q == 128 ? launch(lead_kernel<4>) : launch(lead_kernel<2>);
+    return d.Q == 128 ? launch(lead_kernel<4>) : launch(lead_kernel<2>);
   }
   // ChunkCumsum (it reads dt and A only) and the quantisers need nothing of each other.  ChunkCumsum goes
   // first and lets its successor be scheduled once its own wait for the work ahead of the layer is over;

@@ -107,7 +107,9 @@ def test_absmax_takes_every_row_into_account(R, Ch):
 
 
 @pytest.mark.parametrize("b,L,H,N,G,Q", [(1, 64, 1, 64, 1, 64), (1, 128, 7, 128, 1, 128), (2, 256, 8, 64, 2, 256), (1, 256, 17, 128, 1, 256),
-                                         (2, 1024, 63, 64, 1, 128), (5, 1280, 21, 64, 3, 256), (4, 1024, 129, 64, 1, 64)])
+                                         (2, 1024, 63, 64, 1, 128), (5, 1280, 21, 64, 3, 256), (4, 1024, 129, 64, 1, 64),
+                                         (1, 192, 1, 64, 1, 64), (3, 256, 5, 128, 1, 64), (2, 384, 5, 128, 1, 128), (4, 1024, 33, 64, 3, 64),
+                                         (2, 1024, 65, 128, 5, 128), (3, 1408, 50, 64, 2, 128)])
 def test_layer_head_in_one_launch_and_in_two(b, L, H, N, G, Q):
     # On either side of the lines of the dispatch, head counts that leave a block of four heads partly idle: the layer call
     # gives the bits of the separate calls, whose ChunkCumsum and quantisers are launches of their own
@@ -141,6 +143,38 @@ def test_layer_head_in_one_launch_and_in_two(b, L, H, N, G, Q):
         assert int(status.item()) == 0
         out.append((y, fin))
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("b,L,H,Q,head", [(1, 128, 4, 64, 2), (1, 192, 4, 64, 1), (1, 1024, 4, 64, 1), (1, 1088, 4, 64, 2), (2, 1024, 63, 64, 2),
+                                          (2, 1024, 64, 64, 1), (4, 1024, 128, 64, 1), (4, 1024, 129, 64, 2), (8, 256, 1, 128, 2), (1, 384, 8, 128, 1),
+                                          (1, 1152, 4, 128, 2), (2, 1024, 64, 128, 1), (4, 1024, 129, 128, 2), (1, 1024, 4, 256, 2),
+                                          (2, 1024, 64, 256, 2), (4, 1024, 128, 256, 2)])
+def test_launches_of_the_layer_head(b, L, H, Q, head):
+    # ChunkCumsum and the quantisers are one launch for chunks of up to 128, three or more of them with at most 4096 tokens x heads,
+    # or 128 to 512 thousand: a layer call then has as many kernels as Algorithm 2 alone, elsewhere one more
+    import torch
+    rt = pytest.importorskip("cuda.bindings.runtime")
+    from paper_2608_21952_b200 import binding as bd
+    T, HP = b * L, H * 64
+    dims = bd.Dims(b, L, H, 64, 64, 1, Q)
+    new = lambda *n: torch.ones(*n, device="cuda")  # noqa: E731
+    s = {"s_x": new(HP), "s_B": new(1), "s_C": new(1), "s_xs": new(HP), "s_cb": new(1), "s_h": new(HP)}
+    rest = dict(dt=new(T, H), A=-new(H), D=new(H), y=new(b, L, H, 64), final_state=new(b, H, 64, 64), **s)
+    codes = {k: torch.ones(n, dtype=torch.int8, device="cuda") for k, n in (("xq", (T, HP)), ("Bq", (T, 64)), ("Cq", (T, 64)))}
+    fwd, layer = bd.make_fwd_args(**codes, **rest), bd.make_layer_args(x=new(T, HP), B=new(T, 64), C=new(T, 64), **rest)
+    ws = bd.alloc_workspace(dims)
+    layer_ws = torch.empty(bd.ssdi8_layer_fwd_workspace_bytes(dims), dtype=torch.uint8, device="cuda")
+
+    def kernels(call):
+        g = torch.cuda.CUDAGraph(keep_graph=True)
+        with torch.cuda.graph(g):
+            call()
+        err, _, n = rt.cudaGraphGetNodes(g.raw_cuda_graph())
+        assert int(err) == 0
+        return n
+
+    alone = kernels(lambda: bd.ssdi8_chunk_scan_fwd(dims, fwd, ws))
+    assert kernels(lambda: bd.ssdi8_layer_fwd(dims, layer, layer_ws)) == alone + head - 1
 
 
 @pytest.mark.parametrize("Q,N,H", [(256, 128, 5), (256, 64, 148), (256, 128, 149), (128, 128, 3)])
