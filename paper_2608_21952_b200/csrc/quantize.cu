@@ -261,9 +261,10 @@ ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* sca
     if (I == 1) {
       int ch4 = (int)(Ch / 4);
       int gx = (ch4 + 127) / 128;
-      // one wave of blocks, each with as many rows as that leaves it (at least a few rounds of loads)
-      i64 want = (148 * 3) / gx;
-      if (want < 1) want = 1;
+      // one wave of blocks, each with as many rows as that leaves it (at least a few rounds of loads); where the columns alone
+      // are more than half a wave, several waves, the last of which is a small part (128 rows x 230400 channels 44.0 us as
+      // one block per 512 channels, 39.8 as six; 1024 rows 355 and 325)
+      const i64 want = gx > (148 * 3) / 2 ? 6 : (148 * 3) / gx;
       i64 rows = (R + want - 1) / want;
       if (rows < 2 * AROWS * AGROUPS) rows = 2 * AROWS * AGROUPS;
       rows = (rows + AROWS * AGROUPS - 1) / (AROWS * AGROUPS) * (AROWS * AGROUPS);

@@ -93,8 +93,7 @@ def test_quantiser_gives_all_zero_channels_a_step_of_one(R, Ch, I):
     assert np.array_equal(q.reshape(-1), np.asarray(qr).reshape(-1))
 
 
-@pytest.mark.parametrize("R", [1, 3, 15, 17, 31, 33, 63, 2051])
-@pytest.mark.parametrize("Ch", [4, 508, 516])
+@pytest.mark.parametrize("R,Ch", [(R, Ch) for R in (1, 3, 15, 17, 31, 33, 63, 2051) for Ch in (4, 508, 516)] + [(227, 113664), (227, 113668)])
 def test_absmax_takes_every_row_into_account(R, Ch):
     # The largest value of each channel in a row of its own: remainders of the rows in flight, the row groups and the blocks
     import gpu_harness as gh
