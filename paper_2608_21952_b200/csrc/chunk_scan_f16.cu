@@ -221,6 +221,7 @@ __device__ __forceinline__ void mask_tile_f16(const uint8_t* sCB, const float* t
 #pragma unroll
       for (int e = 0; e < 8; ++e) own[e] = lane < 16 ? 0u : own[e];
     }
+    __syncwarp();                      // (the store is collective; what precedes it depends on the lane)
     tmem_st8(lane_addr + (uint32_t)(cd * 8), own);
   }
 #pragma unroll 1
@@ -230,6 +231,7 @@ __device__ __forceinline__ void mask_tile_f16(const uint8_t* sCB, const float* t
     uint32_t w8[8];
     const uint4 wn = *chunk_ptr(cn >= 0 ? cn : c);
     earlier(c, w4, w8);
+    __syncwarp();
     tmem_st8(lane_addr + (uint32_t)(c * 8), w8);
     c = cn;
     w4 = wn;

@@ -360,16 +360,19 @@ def test_few_heads_give_the_bits_of_the_same_heads_among_many(Q, flag):
 
 
 @pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
-@pytest.mark.parametrize("Q", [64, 256])
-def test_a_time_step_that_is_not_finite_does_not_reach_earlier_tokens(Q, value):
+@pytest.mark.parametrize("Q", [64, 128, 256])
+@pytest.mark.parametrize("flag", ["INT8", "FP16"])
+def test_a_time_step_that_is_not_finite_does_not_reach_earlier_tokens(Q, value, flag):
     import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    flags = bd.FLAG_FP16_OPERAND if flag == "FP16" else 0
     cfg = SSDConfig("causal", 1, 2 * Q, 3, 64, 64, 1, Q, 0.02, 20.0, 47)
     q = _random_codes(cfg, 47)
-    want = gh.gpu_fwd(cfg, q, taps=())[0]
+    want = gh.gpu_fwd(cfg, q, taps=(), flags=flags)[0]
     for j in (0, 5, 15, Q - 1, Q + 8, 2 * Q - 10):
         dt = q["dt"].copy()
         dt[j, 1] = value
-        y = gh.gpu_fwd(cfg, dict(q, dt=dt), taps=())[0]
+        y = gh.gpu_fwd(cfg, dict(q, dt=dt), taps=(), flags=flags)[0]
         assert np.array_equal(y[:, :j], want[:, :j]), j
         assert np.array_equal(y[:, :, ::2], want[:, :, ::2])
 
