@@ -68,10 +68,7 @@ struct QuantJob {
   int first_block;  // of this job in the grid
   int rows;         // rows per block
 };
-struct QuantJobs {
-  QuantJob job[3]; i64 R;
-  int late_wait;   // 1: launched right behind ChunkCumsum of the same layer, which it does not depend on (see the kernel)
-};
+struct QuantJobs { QuantJob job[3]; i64 R; };
 
 __device__ __forceinline__ void quant_block(const QuantJobs& a, const int blk) {
   const int jb = blk >= a.job[2].first_block ? 2 : blk >= a.job[1].first_block ? 1 : 0;
@@ -117,19 +114,14 @@ __device__ __forceinline__ void quant_block(const QuantJobs& a, const int blk) {
 
 __global__ void __launch_bounds__(128, 8) quant_jobs(const QuantJobs a) {
   pdl_launch_dependents();
-  // Programmatic dependent launch.  Normally: wait for the predecessor before the first global access.
-  // Launched right behind ChunkCumsum (which waits for ITS predecessor before it lets this kernel be
-  // scheduled, and whose outputs this kernel does not touch), the blocks start at once and work beside
-  // that kernel.  The wait moves to the end of the grid's last block (one waiting block is enough, and a
+  // Programmatic dependent launch, right behind ChunkCumsum of the same layer, which waits for ITS predecessor before
+  // it lets this kernel be scheduled, and whose outputs this kernel does not touch: the blocks start at once and work
+  // beside it.  The wait stands at the end of the grid's last block (one waiting block is enough, and a
   // wait in every block would keep the early ones resident until ChunkCumsum has finished): it keeps
   // "this kernel complete" implying "ChunkCumsum complete" for the state kernel that follows, and by then
   // it returns at once.
-  if (!a.late_wait) pdl_wait();
-  struct LateWait {
-    bool on;
-    __device__ ~LateWait() { if (on) pdl_wait(); }
-  } late_wait_at_exit{a.late_wait != 0 && blockIdx.x == gridDim.x - 1};
   quant_block(a, (int)blockIdx.x);
+  if (blockIdx.x == gridDim.x - 1) pdl_wait();
 }
 
 // ---- ChunkCumsum and the three quantisers of a layer as one launch: the first ncum blocks take four heads of a chunk each
@@ -344,7 +336,6 @@ ssdi8_status_t launch_lead(const Dims& d, const LayerInputs& in, const float* dt
   const i64 T = (i64)d.b * d.L;
   const int nb = make_jobs(a, in.x, in.B, in.C, T, d.H * d.P, d.G, d.N, s_x, s_B, s_C, xq, Bq, Cq);
   if (nb == 0) return SSDI8_ERR_UNSUPPORTED;
-  a.late_wait = 0;
   const int hblocks = (d.H + 3) / 4;
   const i64 ncum = (i64)hblocks * d.c * d.b;
   // One launch or two, by chunk length and tokens x heads.  One saves a launch, which is what the smallest layers consist of,
@@ -375,7 +366,6 @@ ssdi8_status_t launch_lead(const Dims& d, const LayerInputs& in, const float* dt
   // batch 8 x 2048 x 80 heads.)
   const ssdi8_status_t s = launch_cumsum(d, dt, A, pack, gamma, nullptr, st, nullptr, false, clear_status);
   if (s != SSDI8_OK) return s;
-  a.late_wait = 1;
   return launch_configured(quant_jobs, dim3((unsigned)nb), dim3(128), 0, kStreamCarveout, false, st, a);
 }
 
