@@ -111,7 +111,7 @@ __device__ __forceinline__ uint32_t pack4_rn_product(float2 a, float2 b, float2 
 // sub-block with bound[c] R <= 1 raises no row maximum, and with R = the warp's largest dec_i inv_i one
 // with bound[c] R < 1/2 rounds to zero in every row; both with a slack of 1e-5, far above the few
 // binary32 roundings (and the approximate reciprocal) on either side.  One ballot so names the sub-blocks
-// to visit.  Where cs increases somewhere in the chunk (p127 is +inf then) dec_i and gtab are not
+// to visit.  Where cs increases somewhere in the chunk (b127[16] is +inf then) dec_i and gtab are not
 // bounded by 1, products may leave the binary32 range, and every sub-block is visited.
 // (Against a walk that tested one sub-block after the other, nearest first, 16 columns per thread: 86.5 against 97.1 M
 // warp instructions, 0.125 against 0.139 ms at batch 8 x 2048 x 80 heads.)
@@ -470,7 +470,7 @@ chunk_scan_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ 
     // tile lasts as long as its slowest warp.  With one tile per chunk the groups alternate tiles.
     const int g = (warp - kMaskWarp0) / kGroupWarps;
     const int w = (warp - kMaskWarp0) % kGroupWarps;
-    // A CTA of one chunk (a launch of no more chunks than SMs): a tile each.  One group after the other tile kept the second group
+    // A CTA of one chunk (all of them where there are no more chunks than SMs): a tile each.  One group after the other tile kept the second group
     // idle: prefill of 256 tokens x 24 heads 24.8 -> 23.5 us.
     const bool one = ntpu == 2 && n_end == 2;
     Tile t = *first_tile;

@@ -6,7 +6,7 @@
 namespace ssdi8 {
 namespace cumsum {
 
-constexpr int kTieWindow = 512;   // binary64 units around a binary32 rounding boundary (see above)
+constexpr int kTieWindow = 512;   // binary64 units around a binary32 rounding boundary (see cumsum.cu)
 
 template <int TPL>
 __device__ __forceinline__ void st_row(float* p, const float (&v)[TPL], uint64_t pol) {
@@ -146,22 +146,14 @@ __device__ __forceinline__ void chunk_of_heads(float* dts, const int hpb, const 
   }
   st_row<TPL>(p + PACK_LUT * Q, v, pol);
 
-  // the bounds row: 127 wmax of sub-block c in lane c and in lane 16 + c, their running maximum by a scan over
-  // each half of the warp
+  // the bounds row: 127 wmax of sub-block c in lane c; in lane 16 whether cs increases (the lanes beyond fill the sector)
   float* const bounds = a.pack + un * (kPackRows * Q) + PACK_WMAX * Q;
 #pragma unroll
   for (int o = 1; o < LPS; o <<= 1) wm = fmaxf(wm, __shfl_xor_sync(kAll, wm, o));
   const int c16 = lane & 15;
   float m = __shfl_sync(kAll, wm, (c16 * LPS) & 31);
   m = c16 < NSB ? __fmul_rn(127.0f, m) : 0.f;
-  float pm = m;
-#pragma unroll
-  for (int o = 1; o < 16; o <<= 1) {
-    const float y = __shfl_up_sync(kAll, pm, o, 16);
-    if (c16 >= o) pm = fmaxf(pm, y);
-  }
-  pm = mono ? __fmul_rn(pm, 1.00001f) : __int_as_float(0x7f800000);
-  bounds[lane] = lane < 16 ? m : c16 < NSB ? pm : 0.f;
+  bounds[lane] = lane >= 16 && !mono ? __int_as_float(0x7f800000) : m;
   // block-to-block decays G[I][c], c < I (triangular: 120 entries for 16 sub-blocks)
 #pragma unroll
   for (int r = 0; r < (NTRI + 31) / 32; ++r) {
