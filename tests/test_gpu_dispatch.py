@@ -178,7 +178,8 @@ def test_launches_of_the_layer_head(b, L, H, Q, head):
 
 @pytest.mark.parametrize("Q,N,H", [(256, 128, 5), (256, 64, 148), (256, 128, 149), (128, 128, 3)])
 def test_scan_with_one_chunk_per_cta(Q, N, H):
-    # As many chunks as SMs, one more, and few: the mask groups take a tile each where a CTA has one chunk
+    # As many chunks as SMs, one more, and few: with two tiles per chunk the mask groups take one each where a CTA has one chunk (with
+    # chunks of 128, a tile each as it is, one group has all the work)
     import gpu_harness as gh
     cfg = SSDConfig("one", 1, Q, H, 64, N, 1, Q, 0.02, 20.0, 47)
     q = orc.prepare_quantized(cfg, inputs.make_prefill(cfg))
@@ -342,7 +343,8 @@ def test_output_does_not_depend_on_the_pace_of_the_epilogue(Q, taps):
 @pytest.mark.parametrize("flag", ["INT8", "FP16"])
 @pytest.mark.parametrize("Q", [128, 256])
 def test_few_heads_give_the_bits_of_the_same_heads_among_many(Q, flag):
-    # One chunk per CTA (its mask groups take a tile each) against several
+    # One chunk per CTA against several; with chunks of 256 its mask groups take a tile each there, with chunks of 128 (one tile) the
+    # first group has it
     import gpu_harness as gh
     from paper_2608_21952_b200 import binding as bd
     flags = bd.FLAG_FP16_OPERAND if flag == "FP16" else 0

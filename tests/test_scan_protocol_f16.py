@@ -25,6 +25,8 @@ def build(sim, ntiles, ntpu, speed, broken=None):
     full = lambda bar, use: ("wait", bar, use & 1, use + 1)
     free = lambda bar, use: ("wait", bar, (use & 1) ^ 1, use)
 
+    one = ntpu == 2 and ntiles == 2           # a CTA of one chunk: the mask groups take a tile each
+    reading = [set() for _ in range(4)]       # the groups that read a slot of the scalar pack
     held = {}   # single buffer -> whose contents are being read
 
     def fill(name, who):
@@ -36,7 +38,9 @@ def build(sim, ntiles, ntpu, speed, broken=None):
     def prod_cb():
         for n in range(ntiles):
             ci = cb_index(n)
-            yield free(tok_free[n & 3], n >> 2)
+            if broken != "scalar pack without TOK_FREE":
+                yield free(tok_free[n & 3], n >> 2)
+            assert not reading[n & 3], f"TOK{n & 3}: filled for tile {n} while it is read"
             yield ("async", t("load"), [(tok_full[n & 3], 1)])
             if ntpu == 2 and it_of(n) == 0:
                 if broken == "first CBq by its own pair":
@@ -81,12 +85,14 @@ def build(sim, ntiles, ntpu, speed, broken=None):
     def mask(g):
         for n in range(ntiles):
             u = unit(n)
-            if (u & 1) != g:
+            if ((n if one else u) & 1) != g:
                 continue
             yield full(tok_full[n & 3], n >> 2)
+            reading[n & 3].add(g)
             yield full(cb_full[cb_index(n)], n >> 2)
             yield free(afree[n & 1], n >> 1)
             yield ("work", t("mask") * (1 + 2 * it_of(n)))
+            reading[n & 3].discard(g)
             yield ("arrive", mq[cb_index(n)], 8)
             if ntpu == 2 and it_of(n) == 0:
                 held["CB1"] = None
@@ -105,7 +111,9 @@ def build(sim, ntiles, ntpu, speed, broken=None):
             yield full(acc[n & 1], n >> 1)
             yield full(x_full[u & 1], u >> 1)
             yield full(tok_full[n & 3], n >> 2)
+            reading[n & 3].add("epi")
             yield ("work", t("epilogue"))
+            reading[n & 3].discard("epi")
             yield ("arrive", acc_free[n & 1], 8)
             yield ("arrive", tok_free[n & 3], 8)
             if it_of(n) + 1 == ntpu:
@@ -132,11 +140,12 @@ def test_every_wait_is_sound_at_random_and_extreme_speeds(ntpu, units):
 
 
 @pytest.mark.parametrize("broken,where", [("first CBq by its own pair", "CB1"), ("one Cq/hq barrier pair", "CH_FULL"),
-                                          ("xq codes without RAW_FREE", "XRAW")])
+                                          ("xq codes without RAW_FREE", "XRAW"), ("scalar pack without TOK_FREE", "TOK")])
 def test_broken_variants_are_reported(broken, where):
     """The first tiles' one CBq buffer guarded by the chunk before the last only; the odd tiles' MMA issuer on a barrier pair
     shared with the even ones', which polls the parity of phase 1 before phase 0 has completed; the xq codes of the next chunk
-    requested without waiting for the mask group that expands the present ones."""
+    requested without waiting for the mask group that expands the present ones; a slot of the scalar pack filled while a group
+    reads it."""
     hit = 0
     for seed in range(24):
         sim = Sim(seed)

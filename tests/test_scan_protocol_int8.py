@@ -25,12 +25,16 @@ def build(sim, ntiles, ntpu, speed, broken=None):
     t = lambda role: rng.expovariate(1.0) * speed[role]
     full = lambda bar, use: ("wait", bar, use & 1, use + 1)
     free = lambda bar, use: ("wait", bar, (use & 1) ^ 1, use)
+    one = ntpu == 2 and ntiles == 2           # a CTA of one chunk: the mask groups take a tile each
+    reading = [set() for _ in range(4)]       # the mask groups that read a slot of the scalar pack
 
     def producer(mine):
         for n0 in range(0, ntiles, ntpu):
             u = unit(n0)
             if mine == 0:
-                yield free(tok_free[u & 3], u >> 2)
+                if broken != "scalar pack without TOK_FREE":
+                    yield free(tok_free[u & 3], u >> 2)
+                assert not reading[u & 3], f"TOK{u & 3}: filled for chunk {u} while it is read"
                 yield ("async", t("load"), [(tok_full[u & 3], 1)])
                 yield free(h_free[u & 1], u >> 1)
                 yield ("async", t("load"), [(h_full[u & 1], 1)])
@@ -72,12 +76,14 @@ def build(sim, ntiles, ntpu, speed, broken=None):
     def mask(g):
         for n in range(ntiles):
             u = unit(n)
-            if (u & 1) != g:
+            if ((n if one else u) & 1) != g:
                 continue
             yield full(tok_full[u & 3], u >> 2)
+            reading[u & 3].add(g)
             yield full(cb_full[cb_index(n)], n >> 2)
             yield free(row_free[n & 7], n >> 3)
             yield ("work", t("mask") * (1 + 2 * it_of(n)))
+            reading[u & 3].discard(g)
             yield ("arrive", mq[cb_index(n)], 8)
             yield ("arrive", row_full[n & 7], 8)
             if it_of(n) + 1 == ntpu:
@@ -116,17 +122,18 @@ def test_every_wait_is_sound_at_random_and_extreme_speeds(ntpu, units):
         sim.run()
 
 
-@pytest.mark.parametrize("broken,barrier", [("epilogue waits on MQ", "MQ"), ("x_free without the MMAs", "X_F")])
-def test_broken_variants_are_reported(broken, barrier):
+@pytest.mark.parametrize("broken,barrier,ntpu", [("epilogue waits on MQ", "MQ", 2), ("x_free without the MMAs", "X_F", 2),
+                                                 ("scalar pack without TOK_FREE", "TOK", 1)])
+def test_broken_variants_are_reported(broken, barrier, ntpu):
     """The mask barrier of a CBq buffer may complete for tile n + 4 while the epilogue group of tile n is busy with tile n - 2:
     nothing the epilogue releases stands between the two.  And an xq buffer that the epilogue alone hands back is filled again
-    ahead of the MMAs that wait for its contents."""
+    ahead of the MMAs that wait for its contents.  And a slot of the scalar pack is filled while the slower mask group reads it."""
     hit = 0
     for seed in range(24):
         sim = Sim(seed)
         speed = dict(load=0.1, producer=0.01, mma=0.01, mask=0.01, epilogue=5.0) if seed % 2 else \
             dict(load=0.1, producer=0.01, mma=5.0, mask=5.0, epilogue=0.01)
-        build(sim, 36, 2, speed, broken)
+        build(sim, 36, ntpu, speed, broken)
         try:
             sim.run()
         except AssertionError as e:
