@@ -31,20 +31,22 @@
 // heads (the shortest a block can take), 17 against 32 us with it at batch 8 x 2048 x 80 heads.
 #include "cumsum.cuh"
 
+#include <type_traits>
+
 namespace ssdi8 {
 namespace {
-
-constexpr int kMaxHeads = 8;      // heads (warps) per block: 8 heads of a token are one 32-byte sector of dt
 
 // TPL: tokens per lane, Q / 32.  SOFTPLUS: dt holds the raw time step and dt = softplus(dt + dt_bias[h])
 // (dt_bias may be NULL) is applied as the values are staged (Algorithm 2 module 1 starts there).
 // CLEAR: nclear words are set to 0 as well (calibration).
 // status: the caller's status word, cleared here (this is the first kernel of a forward pass), or NULL.
-// Three blocks per SM: left to itself the compiler takes 60 registers for eight tokens a lane with the softplus, and the prefill
-// of 5 x 1792 tokens x 80 heads 126.2 us (four blocks per SM) instead of 123.8 (80 registers); with two blocks 126.9.
-template <int TPL, bool SOFTPLUS, bool CLEAR>
-__global__ void __launch_bounds__(32 * kMaxHeads, 3) cumsum_kernel(const cumsum::Args a, uint32_t* clear, int nclear) {
-  __shared__ __align__(16) float dts[kMaxHeads * (32 * TPL + 4)];
+// HEADS: heads (warps) per block, 8 (of a token one 32-byte sector of dt) or, for the few blocks of a small grid, 4.  Blocks
+// of 8 three to an SM: left to itself the compiler takes 60 registers for eight tokens a lane with the softplus, and the prefill
+// of 5 x 1792 tokens x 80 heads 126.2 us (four blocks per SM) instead of 123.8 (80 registers); with two blocks 126.9.  Blocks of 4
+// take the registers that the shortest chain wants, 102 (layer of 2048 tokens x 24 heads 31.2 us with 80, 29.4).
+template <int TPL, bool SOFTPLUS, bool CLEAR, int HEADS>
+__global__ void __launch_bounds__(32 * HEADS, HEADS == 8 ? 3 : 1) cumsum_kernel(const cumsum::Args a, uint32_t* clear, int nclear) {
+  __shared__ __align__(16) float dts[HEADS * (32 * TPL + 4)];
   // The wait comes first: a successor that needs nothing of this kernel (the layer step's quantiser of x, B
   // and C) is launched without a wait of its own at its start, so by the time it may be scheduled everything
   // that precedes this kernel in the stream must have completed.
@@ -57,8 +59,7 @@ __global__ void __launch_bounds__(32 * kMaxHeads, 3) cumsum_kernel(const cumsum:
   }
   pdl_launch_dependents();
   if (a.status && threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) *a.status = 0;
-  const int hpb = (int)(blockDim.x >> 5);
-  cumsum::chunk_of_heads<TPL, SOFTPLUS>(dts, hpb, (int)blockIdx.x * hpb, (int)blockIdx.y, (int)blockIdx.z, a);
+  cumsum::chunk_of_heads<TPL, SOFTPLUS>(dts, HEADS, (int)blockIdx.x * HEADS, (int)blockIdx.y, (int)blockIdx.z, a);
 }
 
 // dt = softplus(dt_raw + dt_bias[h]) alone (for callers that calibrate on the positive time step)
@@ -89,7 +90,7 @@ ssdi8_status_t launch_cumsum(const Dims& d, const float* dt, const float* A, flo
   const int sms = sm_count();
   if (sms == 0) return SSDI8_ERR_CUDA;
   // a grid that leaves SMs empty takes half the heads per block: one warp per scheduler, twice the SMs
-  int hpb = kMaxHeads;
+  int hpb = 8;
   if ((i64)((d.H + hpb - 1) / hpb) * d.c * d.b <= sms) hpb /= 2;
   const dim3 grid((d.H + hpb - 1) / hpb, d.c, d.b);
   auto launch = [&](auto kernel) -> ssdi8_status_t {
@@ -97,16 +98,18 @@ ssdi8_status_t launch_cumsum(const Dims& d, const float* dt, const float* A, flo
                              cumsum::Args{dt, A, pack, gamma, tap_cs, dt_bias, clear_status, d}, clear, nclear);
   };
   if (nclear && softplus) return SSDI8_ERR_UNSUPPORTED;   // (calibration takes the positive time step)
-  auto pick = [&](auto sp, auto plain, auto clearing) -> ssdi8_status_t {
-    return softplus ? launch(sp) : nclear ? launch(clearing) : launch(plain);
+  auto pick = [&](auto tpl, auto heads) -> ssdi8_status_t {
+    constexpr int T = decltype(tpl)::value, N = decltype(heads)::value;
+    return softplus ? launch(cumsum_kernel<T, true, false, N>)
+           : nclear ? launch(cumsum_kernel<T, false, true, N>)
+                    : launch(cumsum_kernel<T, false, false, N>);
   };
-  ssdi8_status_t ls;
-  if (d.Q == 256)
-    ls = pick(cumsum_kernel<8, true, false>, cumsum_kernel<8, false, false>, cumsum_kernel<8, false, true>);
-  else if (d.Q == 128)
-    ls = pick(cumsum_kernel<4, true, false>, cumsum_kernel<4, false, false>, cumsum_kernel<4, false, true>);
-  else
-    ls = pick(cumsum_kernel<2, true, false>, cumsum_kernel<2, false, false>, cumsum_kernel<2, false, true>);
+  auto by_chunk = [&](auto heads) -> ssdi8_status_t {
+    return d.Q == 256   ? pick(std::integral_constant<int, 8>{}, heads)
+           : d.Q == 128 ? pick(std::integral_constant<int, 4>{}, heads)
+                        : pick(std::integral_constant<int, 2>{}, heads);
+  };
+  const ssdi8_status_t ls = hpb == 8 ? by_chunk(std::integral_constant<int, 8>{}) : by_chunk(std::integral_constant<int, 4>{});
   if (ls != SSDI8_OK) return ls;
   SSDI8_LAUNCH_CHECK();
   return SSDI8_OK;
