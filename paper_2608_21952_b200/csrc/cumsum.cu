@@ -40,13 +40,17 @@ namespace {
 // (dt_bias may be NULL) is applied as the values are staged (Algorithm 2 module 1 starts there).
 // CLEAR: nclear words are set to 0 as well (calibration).
 // status: the caller's status word, cleared here (this is the first kernel of a forward pass), or NULL.
-// HEADS: heads (warps) per block, 8 (of a token one 32-byte sector of dt) or, for the few blocks of a small grid, 4.  Blocks
-// of 8 three to an SM: left to itself the compiler takes 60 registers for eight tokens a lane with the softplus, and the prefill
-// of 5 x 1792 tokens x 80 heads 126.2 us (four blocks per SM) instead of 123.8 (80 registers); with two blocks 126.9.  Blocks of 4
-// take the registers that the shortest chain wants, 102 (layer of 2048 tokens x 24 heads 31.2 us with 80, 29.4).
-template <int TPL, bool SOFTPLUS, bool CLEAR, int HEADS>
-__global__ void __launch_bounds__(32 * HEADS, HEADS == 8 ? 3 : 1) cumsum_kernel(const cumsum::Args a, uint32_t* clear, int nclear) {
-  __shared__ __align__(16) float dts[HEADS * (32 * TPL + 4)];
+// FEW: a grid of four heads per block for up to half of the SMs, which may take the registers that the shortest chain wants (102 for eight
+// tokens a lane).  A larger grid takes eight or four heads per block and few registers, because the quantisers of a layer work
+// beside it, but with the softplus three blocks per SM: left to itself the compiler takes 60 registers for it, and the prefill of
+// 5 x 1792 tokens x 80 heads 126.2 us (four blocks per SM) instead of 123.8 (80 registers); with two blocks 126.9.  Layer calls, us, 62
+// registers / 102: 1024 tokens x 48 heads 29.9 / 28.4, 2048 x 24 32.4 / 32.0, 6 x 1024 x 24 (144 blocks) 47.4 / 48.2, 11 x 1536 x 13
+// (264) 64.7 / 66.3.
+template <int TPL, bool SOFTPLUS, bool CLEAR, bool FEW>
+__global__ void __launch_bounds__(FEW ? 128 : 256, FEW ? 1 : SOFTPLUS ? 3 : 0) cumsum_kernel(const cumsum::Args a, uint32_t* clear,
+                                                                                          int nclear) {
+  constexpr int kHeads = FEW ? 4 : 8;   // (8 heads of a token are one 32-byte sector of dt)
+  __shared__ __align__(16) float dts[kHeads * (32 * TPL + 4)];
   // The wait comes first: a successor that needs nothing of this kernel (the layer step's quantiser of x, B
   // and C) is launched without a wait of its own at its start, so by the time it may be scheduled everything
   // that precedes this kernel in the stream must have completed.
@@ -59,7 +63,8 @@ __global__ void __launch_bounds__(32 * HEADS, HEADS == 8 ? 3 : 1) cumsum_kernel(
   }
   pdl_launch_dependents();
   if (a.status && threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) *a.status = 0;
-  cumsum::chunk_of_heads<TPL, SOFTPLUS>(dts, HEADS, (int)blockIdx.x * HEADS, (int)blockIdx.y, (int)blockIdx.z, a);
+  const int hpb = FEW ? 4 : (int)(blockDim.x >> 5);
+  cumsum::chunk_of_heads<TPL, SOFTPLUS>(dts, hpb, (int)blockIdx.x * hpb, (int)blockIdx.y, (int)blockIdx.z, a);
 }
 
 // dt = softplus(dt_raw + dt_bias[h]) alone (for callers that calibrate on the positive time step)
@@ -93,23 +98,21 @@ ssdi8_status_t launch_cumsum(const Dims& d, const float* dt, const float* A, flo
   int hpb = 8;
   if ((i64)((d.H + hpb - 1) / hpb) * d.c * d.b <= sms) hpb /= 2;
   const dim3 grid((d.H + hpb - 1) / hpb, d.c, d.b);
+  const bool few = hpb == 4 && (i64)grid.x * d.c * d.b * 2 <= sms;
   auto launch = [&](auto kernel) -> ssdi8_status_t {
     return launch_configured(kernel, grid, dim3(32 * hpb), 0, kStreamCarveout, false, st,
                              cumsum::Args{dt, A, pack, gamma, tap_cs, dt_bias, clear_status, d}, clear, nclear);
   };
   if (nclear && softplus) return SSDI8_ERR_UNSUPPORTED;   // (calibration takes the positive time step)
-  auto pick = [&](auto tpl, auto heads) -> ssdi8_status_t {
-    constexpr int T = decltype(tpl)::value, N = decltype(heads)::value;
-    return softplus ? launch(cumsum_kernel<T, true, false, N>)
-           : nclear ? launch(cumsum_kernel<T, false, true, N>)
-                    : launch(cumsum_kernel<T, false, false, N>);
+  auto pick = [&](auto tpl) -> ssdi8_status_t {
+    constexpr int T = decltype(tpl)::value;
+    if (softplus) return few ? launch(cumsum_kernel<T, true, false, true>) : launch(cumsum_kernel<T, true, false, false>);
+    if (nclear) return few ? launch(cumsum_kernel<T, false, true, true>) : launch(cumsum_kernel<T, false, true, false>);
+    return few ? launch(cumsum_kernel<T, false, false, true>) : launch(cumsum_kernel<T, false, false, false>);
   };
-  auto by_chunk = [&](auto heads) -> ssdi8_status_t {
-    return d.Q == 256   ? pick(std::integral_constant<int, 8>{}, heads)
-           : d.Q == 128 ? pick(std::integral_constant<int, 4>{}, heads)
-                        : pick(std::integral_constant<int, 2>{}, heads);
-  };
-  const ssdi8_status_t ls = hpb == 8 ? by_chunk(std::integral_constant<int, 8>{}) : by_chunk(std::integral_constant<int, 4>{});
+  const ssdi8_status_t ls = d.Q == 256   ? pick(std::integral_constant<int, 8>{})
+                            : d.Q == 128 ? pick(std::integral_constant<int, 4>{})
+                                         : pick(std::integral_constant<int, 2>{});
   if (ls != SSDI8_OK) return ls;
   SSDI8_LAUNCH_CHECK();
   return SSDI8_OK;

@@ -361,6 +361,30 @@ def test_few_heads_give_the_bits_of_the_same_heads_among_many(Q, flag):
     assert np.array_equal(y, want[0][:, :, :7]) and np.array_equal(fin, want[1][:, :7])
 
 
+@pytest.mark.parametrize("softplus", [False, True])
+@pytest.mark.parametrize("Q", [64, 128, 256])
+def test_cumsum_of_a_chunk_does_not_depend_on_the_number_of_chunks(Q, softplus):
+    # Blocks of four heads for up to half of the SMs (74 blocks of a B200: 37 chunks of 5 heads), for more of them, and blocks of
+    # eight: cs and y of the first chunks are the same
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("long", 1, 149 * Q, 5, 64, 64, 1, Q, 0.02, 20.0, 50)
+    q = _random_codes(cfg, 50)
+    bias = np.linspace(-4, -2, 5).astype(np.float32) if softplus else None
+    flags = bd.FLAG_DT_SOFTPLUS if softplus else 0
+    runs = []
+    for c in (37, 38, 149):
+        short = SSDConfig("short", 1, c * Q, 5, 64, 64, 1, Q, 0.02, 20.0, 50)
+        cut = {k: np.ascontiguousarray(v[:c * Q]) if k in ("xq", "Bq", "Cq", "dt") else v for k, v in q.items()}
+        y, _, taps = gh.gpu_fwd(short, cut, taps=("cs",), flags=flags, dt_bias=bias)
+        runs.append((y[:, :37 * Q], taps["cs"][:, :, :37]))
+    for y, cs in runs[1:]:
+        assert np.array_equal(y, runs[0][0]) and np.array_equal(cs, runs[0][1])
+    if not softplus:
+        ref = np.cumsum((q["dt"][:37 * Q].astype(np.float64) * q["A"].astype(np.float64)).reshape(37, Q, 5), axis=1).astype(np.float32)
+        assert np.array_equal(runs[0][1][0], ref.transpose(2, 0, 1))
+
+
 @pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
 @pytest.mark.parametrize("Q", [64, 128, 256])
 @pytest.mark.parametrize("flag", ["INT8", "FP16"])
