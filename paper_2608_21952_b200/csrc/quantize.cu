@@ -338,25 +338,27 @@ ssdi8_status_t launch_lead(const Dims& d, const LayerInputs& in, const float* dt
   if (nb == 0) return SSDI8_ERR_UNSUPPORTED;
   const int hblocks = (d.H + 3) / 4;
   const i64 ncum = (i64)hblocks * d.c * d.b;
-  // One launch or two, by chunk length and tokens x heads.  One saves a launch, which is what the smallest layers consist of,
-  // and where the blocks of both fill the device a few times over ChunkCumsum's run in the gaps of the quantisers'; in between
-  // ChunkCumsum is on the critical path and its own launch has the shorter chain (eight warps a block, more registers), and with
-  // many waves the quantisers alone keep the memory busier.  Chunks of 256 have two everywhere: eight tokens a lane do not
-  // fit the 64 registers that the quantisers leave a thread.  Layer calls in a row, us, two launches / one:
-  //   chunks of 64:  512 x 4 17.2 / 16.7, 256 x 8 16.3 / 15.5, 1024 x 4 18.0 / 18.1; one chunk x 6 heads 13.3 / 13.7; 1024 x 8 19.7 / 21.3;
-  //     2 x 1024 x 64 (N 128) 73.6 / 71.8, 4 x 3392 x 28 195.6 / 181.8, 3 x 1408 x 50 102.8 / 101.8 (N 128: 100.3 / 103.6, the one loss beyond
-  //     the noise of 70 sizes), 8 x 1024 x 80 190.3 / 190.3
-  //   chunks of 128: 512 x 4 17.0 / 16.4, 256 x 8 15.4 / 15.7, 1024 x 8 19.7 / 19.4, 512 x 24 19.6 / 20.0; 8 x 1024 x 20 56.8 / 53.0,
-  //     3 x 1408 x 50 72.2 / 70.8, 4 x 1024 x 64 70.9 / 70.5, 8 x 1024 x 80 140.2 / 140.8
-  //   chunks of 256: 1024 x 4 18.6 / 18.9, 256 x 16 17.9 / 19.1; with N 128 2048 x 80 51.2 / 50.2, but 8 x 1024 x 20 49.2 / 52.4, 4 x 1024 x 40 51.8 / 54.4,
-  //     4 x 1024 x 64 64.2 / 66.0
+  // One launch or two, by tokens x heads.  One saves a launch, which is what the smallest layers consist of, and where the blocks of
+  // both fill the device a few times over ChunkCumsum's run in the gaps of the quantisers'; in between ChunkCumsum is on the
+  // critical path and its own launch has the shorter chain (more warps a block, more registers), and with many waves the
+  // quantisers alone keep the memory busier.  Of the smallest, one or two chunks and chunks of 256 have two: there the chain of
+  // ChunkCumsum is what the state kernel waits for.  Layer calls in a row, inputs changing, us, two launches / one (G = 1 where
+  // not stated):
+  //   smallest, chunks of 64:  256 tokens x 4 heads 15.8 / 15.1, 512 x 4 17.0 / 16.6, 1024 x 4 18.1 / 18.2; one chunk x 6 13.3 / 13.7;
+  //     1024 x 8 19.7 / 21.3.  Of 128: 512 x 4 16.8 / 16.4, 256 x 4 15.1 / 15.3, 1024 x 4 18.4 / 18.2, 512 x 24 19.6 / 20.0.  Of 256:
+  //     256 x 4 17.0 / 18.0, 1024 x 4 18.4 / 18.5, 256 x 16 18.0 / 19.2
+  //   128 to 512 thousand, chunks of 64:  2 x 2688 x 38 96.4 / 96.0, 5 x 6784 x 8 (G 4) 208.2 / 206.9, 4 x 3392 x 28 195.6 / 181.8, 8 x 1024 x
+  //     80 (beyond) 190.3 / 190.3, but 3 x 1408 x 50 (N 128) 100.3 / 103.6.  Of 128: 7 x 2816 x 9 67.6 / 66.8, 3 x 5376 x 16 (G 8) 143.2 / 142.1,
+  //     3 x 1408 x 50 72.2 / 70.8, 8 x 1024 x 80 (beyond) 140.2 / 140.8.  Of 256: 2 x 2048 x 40 51.7 / 51.3, 4 x 8192 x 7 73.8 / 72.8, 8 x 256 x 64
+  //     (G 8) 49.2 / 47.6, 2 x 8192 x 16 (G 4) 97.1 / 95.8, but 6 x 1536 x 20 60.0 / 61.5, 8 x 1024 x 20 53.9 / 54.6, 2 x 8192 x 8 with INT8 states
+  //     68.6 / 74.8; 8 x 1024 x 80 (beyond) 126.6 / 127.6.  In the mean of 68 drawn sizes one launch is 0.9 % faster, 63 of them gain.
   const i64 th = T * d.H;
-  if (d.Q <= 128 && ((d.c >= 3 && th <= 4096) || (th >= 128 * 1024 && th <= 512 * 1024))) {
+  if ((d.Q <= 128 && d.c >= 3 && th <= 4096) || (th >= 128 * 1024 && th <= 512 * 1024)) {
     const cumsum::Args c = {dt, A, pack, gamma, nullptr, nullptr, clear_status, d};
     auto launch = [&](auto kernel) -> ssdi8_status_t {
       return launch_configured(kernel, dim3((unsigned)(nb + ncum)), dim3(128), 0, kStreamCarveout, false, st, a, c, (int)ncum, hblocks);
     };
-    return d.Q == 128 ? launch(lead_kernel<4>) : launch(lead_kernel<2>);
+    return d.Q == 256 ? launch(lead_kernel<8>) : d.Q == 128 ? launch(lead_kernel<4>) : launch(lead_kernel<2>);
   }
   // ChunkCumsum (it reads dt and A only) and the quantisers need nothing of each other.  ChunkCumsum goes
   // first and lets its successor be scheduled once its own wait for the work ahead of the layer is over;

@@ -147,10 +147,10 @@ def test_layer_head_in_one_launch_and_in_two(b, L, H, N, G, Q):
 @pytest.mark.parametrize("b,L,H,Q,head", [(1, 128, 4, 64, 2), (1, 192, 4, 64, 1), (1, 1024, 4, 64, 1), (1, 1088, 4, 64, 2), (2, 1024, 63, 64, 2),
                                           (2, 1024, 64, 64, 1), (4, 1024, 128, 64, 1), (4, 1024, 129, 64, 2), (8, 256, 1, 128, 2), (1, 384, 8, 128, 1),
                                           (1, 1152, 4, 128, 2), (2, 1024, 64, 128, 1), (4, 1024, 129, 128, 2), (1, 1024, 4, 256, 2),
-                                          (2, 1024, 64, 256, 2), (4, 1024, 128, 256, 2)])
+                                          (2, 1024, 63, 256, 2), (2, 1024, 64, 256, 1), (4, 1024, 128, 256, 1), (4, 1024, 129, 256, 2)])
 def test_launches_of_the_layer_head(b, L, H, Q, head):
-    # ChunkCumsum and the quantisers are one launch for chunks of up to 128, three or more of them with at most 4096 tokens x heads,
-    # or 128 to 512 thousand: a layer call then has as many kernels as Algorithm 2 alone, elsewhere one more
+    # ChunkCumsum and the quantisers are one launch for three or more chunks of up to 128 with at most 4096 tokens x heads, and for
+    # 128 to 512 thousand: a layer call then has as many kernels as Algorithm 2 alone, elsewhere one more
     import torch
     rt = pytest.importorskip("cuda.bindings.runtime")
     from paper_2608_21952_b200 import binding as bd
