@@ -104,7 +104,8 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, int b_mn_major) {
 // (bounds by ChunkCumsum, one chunk per lane; fmul is monotone, so the bound with the largest decay of a sub-block's rows is
 // at least every row's); the rest are stored as zeros.
 // (Before, every row tested its chunks one after the other inside the walk: 600 cycles each, most of them the latency of
-// that chain.  The paper's formats at batch 8 x 2048 x 80 heads, all kernels: 266.6 -> 259.1 us.)
+// that chain.  The paper's formats at batch 8 x 2048 x 80 heads, all kernels, calls in a row:
+// 270 -> 259.5 us; no gain with chunks of 64 and 128.)
 __device__ __forceinline__ void mask_tile_f16(const uint8_t* sCB, const float* tokbuf, uint32_t a_tmem, int rq,
                                               int q2, int lane, int TM, uint32_t RBQ, const Tile& t,
                                               const ScanArgs& a) {
@@ -444,7 +445,7 @@ chunk_scan_f16_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constan
     const int wg = (warp - kMaskWarp0) % kGroupWarps;
     const int rq = warp & 3;               // TMEM lane quarter of this warp = row quarter of the tile
     const int q2 = wg >> 2;                // chunk parity of this warp
-    const bool one = ntpu == 2 && n_end == 2;   // a CTA of one chunk: a tile each (256 tokens x 80 heads 25.9 -> 25.0 us)
+    const bool one = ntpu == 2 && n_end == 2;   // a CTA of one chunk: a tile each (prefill of 256 tokens x 80 heads 27.9 -> 27.3 us, calls in a row)
     Tile t = decode_unit((int)blockIdx.x, d, TM);
 #pragma unroll 1
     for (int n = 0; n < n_end; ++n, next_tile(t, d, a.w, TM, ntpu)) {

@@ -155,7 +155,7 @@ ssdi8_status_t launch_bounded_wait_expires(int32_t* status, cudaStream_t st);
 // absmax; s_cb: int32 absmax of acc_cb, times s_C s_B), 1 where a maximum is 0
 ssdi8_status_t launch_absmax_xs(const Dims& d, const int8_t* xq, const float* s_x, const float* pack, uint32_t* absmax,
                                 cudaStream_t st);
-ssdi8_status_t launch_clear_words(void* a, i64 na, cudaStream_t st);
+ssdi8_status_t launch_clear_words(void* a, i64 n, cudaStream_t st);
 ssdi8_status_t launch_finalize_scales(const uint32_t* max_h, float* s_h, i64 n, const uint32_t* max_cb, float* s_cb, i64 nq,
                                       const float* s_C, const float* s_B, cudaStream_t st);
 

@@ -169,7 +169,9 @@ __global__ void __launch_bounds__(QT) quant_inner(const float4* __restrict__ in,
 
 // ---- absmax, I == 1.  A thread owns 4 channels and every fourth row of the block's, with AROWS loads in flight; the four
 // threads of a channel meet in shared memory, so that a block of many rows leaves one atomic per channel (an atomic per thread of
-// 24 rows: 171 on each of 5120 addresses at 4096 rows; the calibration of 2 x 2048 x 80 heads 95.3 against 89.5 us).  The loads
+// 24 rows: 171 on each of 5120 addresses at 4096 rows; the calibration of 2 x 2048 x 80 heads 91.5 against 88.0 us, of 5 x 2304 x 16
+// 105.3 against 84.3, calls in a row; this kernel alone at 65536 rows x 64 channels 53 against 19, at 16384 x 5120 120.8 against
+// 115.5).  The loads
 // leave their lines in L2 for the quantiser that follows.
 constexpr int AROWS = 4, AGROUPS = 4;
 __global__ void __launch_bounds__(128 * AGROUPS, 3) absmax_ch_fastest(const float4* __restrict__ in,
@@ -281,8 +283,8 @@ ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* sca
     const int ch4 = (int)(Ch / 4);
     const int gx = (ch4 + 127) / 128;
     // slabs of rows: enough blocks to fill the machine several times over, at least 16 rows each (at least 32 left 2560 to 5120
-    // channels of a few thousand rows on one wave and a bit: calibration of 5 x 2304 x 16 heads 79.2 against 72.1 us, 2 x 2048 x
-    // 80 82.3 against 80.9)
+    // channels of a few thousand rows on one wave and a bit: calibration of 5 x 2304 x 16 heads 84.3 against 79.1 us, 2 x 2048 x
+    // 80 88.0 against 86.4, calls in a row)
     i64 want = (148 * 32 + gx - 1) / gx;
     i64 rows = (R + want - 1) / want;
     if (rows < 16) rows = 16;
@@ -342,7 +344,7 @@ ssdi8_status_t launch_lead(const Dims& d, const LayerInputs& in, const float* dt
   // both fill the device a few times over ChunkCumsum's run in the gaps of the quantisers'; in between ChunkCumsum is on the
   // critical path and its own launch has the shorter chain (more warps a block, more registers), and with many waves the
   // quantisers alone keep the memory busier.  Of the smallest, one or two chunks and chunks of 256 have two: there the chain of
-  // ChunkCumsum is what the state kernel waits for.  Layer calls in a row, inputs changing, us, two launches / one (G = 1 where
+  // ChunkCumsum is what the state kernel waits for.  Layer calls in a row, us, two launches / one (G = 1 where
   // not stated):
   //   smallest, chunks of 64:  256 tokens x 4 heads 15.8 / 15.1, 512 x 4 17.0 / 16.6, 1024 x 4 18.1 / 18.2; one chunk x 6 13.3 / 13.7;
   //     1024 x 8 19.7 / 21.3.  Of 128: 512 x 4 16.8 / 16.4, 256 x 4 15.1 / 15.3, 1024 x 4 18.4 / 18.2, 512 x 24 19.6 / 20.0.  Of 256:
