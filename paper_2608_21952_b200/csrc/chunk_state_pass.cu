@@ -1,19 +1,23 @@
 // ChunkState + StatePassing fused, chunk-sequential per (batch, head): the fp32 chunk-local
 // state never goes to HBM.  For chunk k = 0 .. c-1 of one (b, h):
 //   Xs_q[i,p]   = rne(fmul(fmul(float(xq[i,p]), fdiv(s_x, s_xs)), LUT_state[i]))       (Eq. 3)
-//   acc_st[n,p] = sum_i Bq[i,n] Xs_q[i,p]            INT8 MMA over the chunk's tokens, INT32 in TMEM
+//   acc_st[p,n] = sum_i Xs_q[i,p] Bq[i,n]            INT8 MMA over the chunk's tokens, INT32 in TMEM
 //   loc[p,n]    = fmul(float(acc_st), fmul(s_xs[h,p], s_B[g]))                         (Eq. 4 rescale)
 //   hq[k][p,n]  = rne(fmul(S[p,n], fdiv(1, s_h[h,p])))     (state entering chunk k, int8 for ChunkScan1)
 //   S[p,n]      = fmaf(Gamma_k, S[p,n], loc[p,n])                                      (Eq. 6)
-// and final_state = S after the last chunk.  The accumulator has the state index n on the TMEM lanes, so thread
-// (lane n) works on S[., n] of its 32 channels p; the running state is kept in tensor memory beside the
-// accumulator (64 more columns, read and written 8 columns at a time), which leaves the threads with few
-// registers so that three CTAs fit an SM: the kernel is a chain of short dependent steps per chunk, and what fills an SM is other
-// CTAs' chains.  Three warps re-quantise the xq rows up to two chunks ahead, a fourth issues the MMAs
-// and requests the tiles by TMA: xq double-buffered across chunks, Bq single-buffered (requested
-// when the MMAs of the chunk before have finished); hq leaves through
-// a shared-memory tile and one TMA store per chunk.  Same arithmetic, operation for operation,
-// as the separate kernels (chunk_state.cu, state_passing.cu).
+// and final_state = S after the last chunk.  The kernel is bound by instruction issue where every SM holds three CTAs and by the
+// chain of a chunk (MMAs -> accumulator -> update) where it holds one, so both are kept short:
+//   * The accumulator has the 64 channels on its rows (M = 64, 16 tensor-memory lanes per warp quarter) and is read in the
+//     16 x 256-bit form, which gives all 32 threads of a warp work: a thread has two channels and pairs of neighbouring n.  The
+//     running state stays in registers (32 of them at N = 128), the scales of a channel too, and codes leave two at a time.
+//   * Tokens arrive in slabs of 64 (xq, Bq and LUT_state of each), live slabs only, through a ring of four or six, so that tiles
+//     are requested and re-quantised ahead of the chain; LUT_state of the chunks reaches the loading warp four chunks ahead (read
+//     from global memory a chunk ahead, its latency was the time of a chunk of a lone CTA).
+// (Against n on the lanes, the state in tensor memory, a byte store per code, a shared-memory load per scale and whole chunks
+// of xq and Bq, ncu, us and million warp instructions: 8 x 2048 x 80 heads 43.3 -> 40.2, 25.3 -> 16.8; 4 x 8192 x 128 121 -> 107;
+// 3 x 1408 x 50 22.8 -> 18.7; calibration of 2 x 2048 x 80 22.2 -> 18.2.  Calls: 229.4 -> 225, 816 -> 797, 65.7 -> 53.2, 81.4 -> 75.7.)
+// Roles: eight state warps, which also form Q(X_scaled), in place, or two warps for that (see Geo), MMA issue, TMA loads.  hq leaves through two shared-memory tiles, one
+// TMA store per chunk.  Same arithmetic, operation for operation, as the separate kernels (chunk_state.cu, state_passing.cu).
 // I8S = true selects the paper's own state format (Section 4.2, Eq. 4 and Eq. 7): the state is an
 // int8 code with the one per-(H,P) scale s_h, the chunk-local state goes INT32 -> INT8 in
 // registers, and the recurrence is integer with a fixed-point decay:
@@ -21,7 +25,9 @@
 //   Sq   = sat(locq + ((Gq * Sq + 64) >> 7));  hq[k] = Sq before the update;  final = fmul(float(Sq), s_h)
 // CAL = true is the calibration pass: no codes are formed; the largest |S| of every channel over init_state and
 // every S_k goes into absmax_h (binary32 bits, one atomic per channel and CTA).  (Against separate ChunkState and
-// StatePassing passes over 42 MB of chunk-local states in HBM, 28 + 7 us at batch 2 x 2048 x 80 heads, this takes 22.)
+// StatePassing passes over 42 MB of chunk-local states in HBM, 28 + 7 us at batch 2 x 2048 x 80 heads, this takes 18.)
+#include <type_traits>
+
 #include "kernels.h"
 #include "sm100.cuh"
 
@@ -35,122 +41,228 @@ struct FusedArgs {
   const float* gamma; const float* init; float* final_state;
   float* tap_loc; float* tap_prev; int8_t* tap_Xsq; int32_t* tap_acc; int32_t* status; uint32_t* absmax_h; float* s_xs_out;
   Dims d;
-  int n_full;  // CTAs below this index own a whole (batch, head); the rest own a quarter (16 channels) of one
+  int n_full;  // CTAs below this index own a whole (batch, head); the rest own `slice` columns of the state of one
+  int slice;   // 32 or 64
 };
 
-constexpr int kStateThreads = 256;   // warps 0-7: running state, hq and its TMA stores
-constexpr int kQuantThreads = 128;   // warps 8-10: Q(X_scaled), up to two chunks ahead; warp 11: MMA issue, TMA loads
-constexpr int kThreads = kStateThreads + kQuantThreads;
-constexpr int kRowWarps = 3;
-constexpr uint32_t XSTAGE = 16384;                // xq rows [Q][64] of one chunk
-constexpr uint32_t OFF_X = 0;                     // two stages
-constexpr uint32_t OFF_B = 2 * XSTAGE;            // Bq rows [Q][N] of one chunk (single buffer)
-constexpr uint32_t OFF_HQ = OFF_B + 32768;        // [64 p][N] int8 staging of hq
-constexpr uint32_t OFF_LUT = OFF_HQ + 8192;       // 2 x [256] floats
-constexpr uint32_t OFF_COL = OFF_LUT + 2048;      // [64] loc scale, [64] 1 / s_h, [64] s_x / s_xs
-constexpr uint32_t OFF_BAR = OFF_COL + 768;
-constexpr uint32_t SMEM_BYTES = OFF_BAR + 64;     // 76 608 bytes: three CTAs per SM
-constexpr uint32_t kTmemCols = 128;               // accumulator in columns 0..63, running state in 64..127
+constexpr int kStateWarps = 8, kStateThreads = 32 * kStateWarps;
+constexpr int kSlab = 64;                         // tokens of a slab
+constexpr int kLutAhead = 4;                      // LUT_state of so many chunks is under way to the loading warp
+enum { SLAB_LAST = 1 };                           // of its chunk (the word also has the slab's index from bit 8, the chunk's from 16)
 
-enum { B_XFULL = 0, B_BFULL = 2, B_MMA = 3, B_ACC_FREE = 4, B_COUNT = 5 };
-
-__device__ __forceinline__ void named_bar(int id, int nthreads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-__device__ __forceinline__ void named_bar_arrive(int id, int nthreads) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
+// FEW: up to two CTAs per SM.  A CTA alone on its SM is a chain of latencies, the longest where decay is slow and most slabs live: the
+// state warps quantise Q(X_scaled) themselves, all eight at a slab, one chunk ahead, behind a ring of six slabs.  With three
+// CTAs per SM what counts is that the chains overlap: two warps of their own quantise, and the ring has four slabs (all of a
+// chunk of 256).  Layer calls, us, eight state warps / two of their own: 3 x 1408 x 50 56.5 / 58.8, calibration of 2 x 2048 x 80 heads
+// 77.4 / 79.7, but 8 x 2048 x 80 228.7 / 224.8, 4 x 8192 x 128 803 / 791, 5 x 1792 x 80 119.3 / 118.7.
+template <bool FEW>
+struct Geo {
+  static constexpr int kRowWarps = FEW ? 0 : 2, kSlots = FEW ? 6 : 4;
+  static constexpr int kMmaWarp = kStateWarps + kRowWarps, kLoadWarp = kMmaWarp + 1, kThreads = 32 * (kLoadWarp + 1);
+  static constexpr uint32_t OFF_X = 0;                             // kSlots x [kSlab][64]   xq rows
+  static constexpr uint32_t OFF_B = OFF_X + kSlots * kSlab * 64;   // kSlots x [kSlab][NS]   Bq rows (NS: state columns of the CTA)
+  static constexpr uint32_t OFF_HQ = OFF_B + kSlots * kSlab * 128; // 2 x [64 p][NS] int8 staging of hq
+  static constexpr uint32_t OFF_LUT = OFF_HQ + 2 * 8192;           // kSlots x [kSlab] floats
+  static constexpr uint32_t OFF_COL = OFF_LUT + kSlots * kSlab * 4;   // [64] loc scale, [64] 1 / s_h, [64] s_x / s_xs
+  static constexpr uint32_t OFF_CHUNK = OFF_COL + 768;             // kLutAhead x [Q] floats: LUT_state of whole chunks, for the loading warp
+  static constexpr uint32_t OFF_INFO = OFF_CHUNK + kLutAhead * 1024;   // kSlots words by the loading warp
+  static constexpr uint32_t OFF_BAR = OFF_INFO + 32;
+  enum { B_FULL = 0, B_READY = kSlots, B_FREE = 2 * kSlots, B_ACC = 3 * kSlots, B_ACC_FREE = B_ACC + 2, B_LUT = B_ACC_FREE + 2,
+         B_COUNT = B_LUT + kLutAhead };
+  static constexpr uint32_t SMEM_BYTES = OFF_BAR + 8 * B_COUNT + 16;   // 97 584 bytes, two CTAs per SM; 71 792, three
+};
+// More than half of an SM's shared memory, asked for where there is a CTA per SM or less: the scheduler, which starts CTAs beside those of the
+// kernel before wherever these have left room, would put up to three on one SM, each of them slower for it.  (Likewise the ring of six:
+// 3 x 1408 x 50 56.5 us with three to an SM, 53.4 with two; 3 x 2048 x 80 98.7 / 94.7, 1 x 1024 x 128 (G 8) 41.3 / 40.7.)
+constexpr uint32_t kSmemAlone = 120 * 1024;
+// position in a ring of slabs
+template <int SLOTS>
+struct Ring {
+  int slot = 0;
+  uint32_t phase = 0;
+  __device__ __forceinline__ void next() {
+    if (++slot == SLOTS) {
+      slot = 0;
+      phase ^= 1u;
+    }
+  }
+};
 
 // TAPS: any of the intermediate-tensor taps is requested (tests); the production instance carries no tap code
-// NCQ: 16-channel chunks of the head this CTA owns (4 = the whole head, 1 = one quarter)
-template <bool I8S, bool TAPS, bool CAL, int NCQ>
+// N: state columns of a head; NS: of this CTA (all, or a slice from n_base on)
+template <bool I8S, bool TAPS, bool CAL, bool FEW, int N, int NS>
 __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtensorMap& tm_x, const CUtensorMap& tm_hq,
-                                           const FusedArgs& a, const int unit, const int c0) {
-  // (no padding for the 1024-byte alignment the swizzled tiles need: three CTAs fill the SM's shared
-  // memory to the last kilobyte; the launcher checks that the kernel uses no static shared memory, so
-  // the dynamic part starts at the window's base, and the kernel checks the address itself)
+                                           const FusedArgs& a, const int unit, const int n_base) {
+  // (no padding for the 1024-byte alignment the swizzled tiles need: the launcher checks that the kernel uses no static
+  // shared memory, so the dynamic part starts at the window's base, and the kernel checks the address itself)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  constexpr int ncq = NCQ;
+  using G = Geo<FEW>;
+  constexpr int kMmaWarp = G::kMmaWarp, kLoadWarp = G::kLoadWarp, kThreads = G::kThreads;
+  constexpr uint32_t OFF_X = G::OFF_X, OFF_B = G::OFF_B, OFF_LUT = G::OFF_LUT;
+  constexpr int B_FULL = G::B_FULL, B_READY = G::B_READY, B_FREE = G::B_FREE, B_ACC = G::B_ACC, B_ACC_FREE = G::B_ACC_FREE, B_LUT = G::B_LUT;
+  using Pos = Ring<G::kSlots>;
   uint8_t* smem = smem_raw;
   if ((smem_u32(smem) & 1023u) != 0) {
     if (threadIdx.x == 0 && a.status) atomicExch(a.status, (int32_t)SSDI8_ERR_ALIGN);
     return;
   }
+  constexpr int NA = NS == 128 ? 1 : 2;                 // accumulators: two where they fit beside those of two more CTAs
+  constexpr uint32_t kTmemCols = NS * NA;
   const Dims& d = a.d;
-  const int Q = d.Q, N = d.N, P = d.P;
+  const int Q = d.Q, P = d.P;
   const int h = unit % d.H, b = unit / d.H;
   const int g = h / (d.H / d.G);
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // (the shuffle: uniform for the compiler)
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + OFF_BAR);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + B_COUNT);
-  uint8_t* sHQ = smem + OFF_HQ;
-  float* col_scale = reinterpret_cast<float*>(smem + OFF_COL);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + G::OFF_BAR);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + G::B_COUNT);
+  volatile int* info = reinterpret_cast<volatile int*>(smem + G::OFF_INFO);
+  float* col_scale = reinterpret_cast<float*>(smem + G::OFF_COL);
   float* col_invh = col_scale + 64;
   float* col_rx = col_invh + 64;
   const i64 bh = (i64)b * d.H + h;
   const i64 unit0 = bh * d.c;
+  const int nsl = Q / kSlab, tpl = Q / 32;     // slabs of a chunk; tokens of a lane that holds LUT_state of a chunk
 
-  // One warp: the slabs of 32 tokens named by m of the xq rows (with LUT_state of the chunk: a global
-  // load there would sit on the re-quantisation group's critical path) or of the Bq rows of chunk k
-  auto issue_x = [&](int k, uint32_t m) {
-    const int s = k & 1;
-    const int tok0 = (int)((i64)b * d.L + (i64)k * Q);
-    if (elect_one()) {
-      mbar_expect_tx(&bars[B_XFULL + s], (uint32_t)(__popc(m) * 32 * 64 + Q * 4));
-      bulk_load(smem + OFF_LUT + s * 1024, a.pack + ((unit0 + k) * kPackRows + PACK_LUT) * Q, (uint32_t)(Q * 4),
-                &bars[B_XFULL + s]);
-#pragma unroll 1
-      for (; m; m &= m - 1) {
-        const int i0 = (__ffs((int)m) - 1) * 32;
-        tma_load_3d(smem + OFF_X + s * XSTAGE + i0 * 64, &tm_x, &bars[B_XFULL + s], 0, h, tok0 + i0);
+  // LUT_state of a chunk: tpl consecutive tokens per lane, 32 / nsl lanes per slab
+  struct Lut { float4 a, b; };
+  auto lut_of_lane = [&](int k) -> Lut {
+    Lut v = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    const float* l = reinterpret_cast<const float*>(smem + G::OFF_CHUNK) + (k % kLutAhead) * 256 + lane * tpl;
+    if (tpl == 2) {
+      const float2 u = *reinterpret_cast<const float2*>(l);
+      v.a.x = u.x;
+      v.a.y = u.y;
+    } else {
+      v.a = reinterpret_cast<const float4*>(l)[0];
+      if (tpl == 8) v.b = reinterpret_cast<const float4*>(l)[1];
+    }
+    return v;
+  };
+  // the loading warp: slab sl of chunk k into a slot: the copies, and LUT_state of the slab, from the registers of the
+  // chunk's, with the arrival (which may come after the copies' bytes)
+  auto copy = [&](int slot, int k, int sl) {
+    const int tok = (int)((i64)b * d.L + (i64)k * Q) + kSlab * sl;
+    tma_load_3d(smem + OFF_X + slot * (kSlab * 64), &tm_x, &bars[B_FULL + slot], 0, h, tok);
+    tma_load_3d(smem + OFF_B + slot * (kSlab * NS), &tm_B, &bars[B_FULL + slot], n_base, g, tok);
+  };
+  auto describe = [&](int slot, int k, int sl, const Lut& v, bool last, bool copies) {
+    const int rel = lane * tpl - kSlab * sl;   // of this lane's tokens in the slab
+    if ((uint32_t)rel < (uint32_t)kSlab) {
+      float* l = reinterpret_cast<float*>(smem + OFF_LUT) + slot * kSlab + rel;
+      if (tpl == 2) {
+        *reinterpret_cast<float2*>(l) = make_float2(v.a.x, v.a.y);
+      } else {
+        reinterpret_cast<float4*>(l)[0] = v.a;
+        if (tpl == 8) reinterpret_cast<float4*>(l)[1] = v.b;
       }
     }
     __syncwarp();
-  };
-  auto issue_B = [&](int k, uint32_t m) {   // once the MMAs of chunk k - 1 have finished
-    const int tok0 = (int)((i64)b * d.L + (i64)k * Q);
     if (elect_one()) {
-      mbar_expect_tx(&bars[B_BFULL], (uint32_t)(__popc(m) * 32 * N));
-#pragma unroll 1
-      for (; m; m &= m - 1) {
-        const int i0 = (__ffs((int)m) - 1) * 32;
-        tma_load_3d(smem + OFF_B + i0 * N, &tm_B, &bars[B_BFULL], 0, g, tok0 + i0);
-      }
+      info[slot] = (last ? SLAB_LAST : 0) | (sl << 8) | (TAPS ? k << 16 : 0);
+      mbar_expect_tx(&bars[B_FULL + slot], kSlab * 64 + kSlab * NS);   // (an arrival: releases the stores above)
+      if (copies) copy(slot, k, sl);
     }
     __syncwarp();
   };
 
-  constexpr int kLoadWarp = kStateThreads / 32 + kRowWarps;
   if (warp == kLoadWarp) {
     if (lane == 0) {
-      mbar_init(&bars[B_XFULL], 1);
-      mbar_init(&bars[B_XFULL + 1], 1);
-      mbar_init(&bars[B_BFULL], 1);
-      mbar_init(&bars[B_MMA], 1);
-      mbar_init(&bars[B_ACC_FREE], kStateThreads / 32);
+      for (int s = 0; s < G::kSlots; ++s) {
+        mbar_init(&bars[B_FULL + s], 1);
+        mbar_init(&bars[B_READY + s], FEW ? kStateWarps : G::kRowWarps);
+        mbar_init(&bars[B_FREE + s], 1);
+      }
+      for (int s = 0; s < kLutAhead; ++s) mbar_init(&bars[B_LUT + s], 1);
+      for (int s = 0; s < 2; ++s) {
+        mbar_init(&bars[B_ACC + s], 1);
+        mbar_init(&bars[B_ACC_FREE + s], kStateWarps);
+      }
       fence_mbar_init();
       tma_prefetch_desc(&tm_B);
       tma_prefetch_desc(&tm_x);
       tma_prefetch_desc(&tm_hq);
     }
     __syncwarp();
+    asm volatile("bar.arrive 2, %0;" ::"n"(kThreads) : "memory");   // (its set-up for the others)
   }
   if (warp == 1) tmem_alloc(tmem_slot, kTmemCols);
+  if (warp == 2 && lane < 8) {   // the head's vectors into L2 (which touches no value), two lines of each
+    const float* const v = lane < 2 ? a.s_x : lane < 4 ? a.s_xs : lane < 6 ? a.s_h : nullptr;
+    if (v) asm volatile("prefetch.global.L2 [%0];" ::"l"(v + h * P + 32 * (lane & 1)));
+  }
   pdl_wait();   // everything below reads global memory
   // (after the wait, not before it: ChunkBMM, launched next, reads and writes global memory without waiting
   // for this kernel, so it must not be scheduled before this kernel's predecessors have completed)
   pdl_launch_dependents();
-  if (warp == kLoadWarp) {   // all slabs of the first chunk: its LUT_state would have to come first
-    issue_x(0, (1u << (Q / 32)) - 1u);
-    issue_B(0, (1u << (Q / 32)) - 1u);
-  }
   auto step_xs = [&](int p) -> float {   // (the calibration pass is given the maxima of |X_scaled|)
     const float v = a.s_xs[h * P + p];
     return CAL ? step_of_max(__float_as_uint(v)) : v;
   };
+  auto alive = [](float bound, float l) { return !(__fmul_rn(bound, fabsf(l)) < 0.5f); };
+  // Rows that re-quantise to zero (the sparsity Eq. 3 rests on: LUT_state decays towards the start
+  // of a chunk).  fmul is monotone, so with rxm >= |rx| of every channel,
+  // fmul(fmul(127, rxm), |LUT_state[i]|) < 1/2 implies |fmul(fmul(x, rx), LUT_state[i])| < 1/2 for every
+  // code x: row i of Q(X_scaled) is all zeros, exactly.  Such a row is stored as zeros without the
+  // arithmetic, and a slab of such rows is left out altogether: no loads, no MMA.  A
+  // chunk without a live slab opens the accumulator with its last one, all rows of it stored as zeros.
+  auto row_bound = [&](float rx0, float rx1) -> float {   // the channels of the head, two per lane
+    return __fmul_rn(127.0f, __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fmaxf(0.f, fabsf(rx0)), fabsf(rx1))))));
+  };
+
+  if (warp == kLoadWarp) {
+    // ------------------------------------------------------------ loads, as many slabs ahead as the ring has places.  This warp
+    // forms the bound itself and does not wait for the others' set-up; the last slab of the first chunk, the likeliest to
+    // live, is under way before its LUT_state is known.
+    auto fetch_lut = [&](int k) {
+      if (k < d.c && elect_one()) {
+        mbar_expect_tx(&bars[B_LUT + k % kLutAhead], (uint32_t)(Q * 4));
+        bulk_load(smem + G::OFF_CHUNK + (k % kLutAhead) * 1024, a.pack + ((unit0 + k) * kPackRows + PACK_LUT) * Q, (uint32_t)(Q * 4),
+                  &bars[B_LUT + k % kLutAhead]);
+      }
+      __syncwarp();
+    };
+    const float sx0 = a.s_x[h * P + lane], sx1 = a.s_x[h * P + 32 + lane], xs0 = step_xs(lane), xs1 = step_xs(32 + lane);
+    fetch_lut(0);
+    if (elect_one()) copy(0, 0, nsl - 1);
+    __syncwarp();
+    for (int k = 1; k < kLutAhead; ++k) fetch_lut(k);
+    const float bound = row_bound(__fdiv_rn(sx0, xs0), __fdiv_rn(sx1, xs1));
+    auto live_slabs = [&](const Lut& v) -> uint32_t {
+      if (TAPS) return (1u << nsl) - 1u;
+      const bool any = alive(bound, v.a.x) | alive(bound, v.a.y) | alive(bound, v.a.z) | alive(bound, v.a.w) | alive(bound, v.b.x) |
+                       alive(bound, v.b.y) | alive(bound, v.b.z) | alive(bound, v.b.w);
+      const uint32_t bal = __ballot_sync(0xffffffffu, any);
+      const int lps = 32 / nsl;
+      return __ballot_sync(0xffffffffu, lane < nsl && ((bal >> ((lane * lps) & 31)) & ((1u << lps) - 1u)) != 0);
+    };
+    Pos at;
+    bool on = true;
+#pragma unroll 1
+    for (int k = 0; k < d.c; ++k) {
+      on = __all_sync(0xffffffffu, mbar_wait_inline<0>(&bars[B_LUT + k % kLutAhead], (k / kLutAhead) & 1, a.status));
+      if (!on) break;
+      const Lut v = lut_of_lane(k);
+      uint32_t m = live_slabs(v);
+      const uint32_t top = 1u << (nsl - 1);
+      if (k == 0 || m == 0) m |= top;
+      bool issued = k == 0;                         // (slab `top` then comes first)
+#pragma unroll 1
+      while (m) {
+        const int sl = issued ? nsl - 1 : __ffs((int)m) - 1;
+        m &= ~(1u << sl);
+        on = __all_sync(0xffffffffu, mbar_wait_inline<0>(&bars[B_FREE + at.slot], at.phase ^ 1, a.status));
+        if (!on) break;
+        describe(at.slot, k, sl, v, m == 0, !issued);
+        issued = false;
+        at.next();
+      }
+      if (!on) break;
+      fetch_lut(k + kLutAhead);                     // (every lane's values have gone into the mask and the slabs)
+    }
+  } else {
   if (tid < 64) {
     const float sx = step_xs(tid), sxb = __fmul_rn(sx, a.s_B[g]);
-    if (CAL && b == 0 && tid >= 16 * c0 && tid < 16 * (c0 + ncq)) a.s_xs_out[h * P + tid] = sx;
+    if (CAL && b == 0 && n_base == 0) a.s_xs_out[h * P + tid] = sx;
     if (CAL) {
       col_scale[tid] = sxb;
       col_invh[tid] = 0.f;               // running maximum of the channel
@@ -163,350 +275,248 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     col_rx[tid - 64] = __fdiv_rn(a.s_x[h * P + tid - 64], step_xs(tid - 64));
   }
   tc_fence_before();
-  __syncthreads();
+  named_bar_sync(2, kThreads);
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp >= kStateThreads / 32) {
-    // ------------------------------------------------------------ Q(X_scaled), one chunk ahead of the state warps
-    const int qt = tid - kStateThreads;
-    constexpr int lq = ncq == 4 ? 2 : 0;  // log2(chunks per row in this CTA's range)
-    const int c = c0 + (qt & (ncq - 1));  // 16-byte chunk (16 channels) of every row this thread visits
-    float rx[16];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) rx[e] = col_rx[c * 16 + e];
-    // Rows that re-quantise to zero (the sparsity Eq. 3 rests on: LUT_state decays towards the start
-    // of a chunk).  fmul is monotone, so with rxm >= |rx| of every channel of this CTA's range,
-    // fmul(fmul(127, rxm), |LUT_state[i]|) < 1/2 implies |fmul(fmul(x, rx), LUT_state[i])| < 1/2 for every
-    // code x: row i of Q(X_scaled) is all zeros, exactly.  Such a row is stored as zeros without the
-    // arithmetic, and a 32-token slab of such rows is left out altogether (no MMA).
-    float rxm = 0.f;
-#pragma unroll
-    for (int e = 0; e < 16; ++e) rxm = fmaxf(rxm, fabsf(rx[e]));
-    if (ncq == 4) rxm = fmaxf(rxm, __shfl_xor_sync(0xffffffffu, rxm, 1));
-    if (ncq == 4) rxm = fmaxf(rxm, __shfl_xor_sync(0xffffffffu, rxm, 2));
-    const float b127 = __fmul_rn(127.0f, rxm);
-    // Three of the warps share the live rows of a chunk evenly, up to two chunks ahead; the fourth requests the tiles, the
-    // live slabs of them only, and issues the MMAs.  The live slabs are the last ones of a chunk, often two or three: with
-    // whole slabs dealt out by position the warp that had most of them was the time of a chunk, and with all of xq
-    // and Bq loaded (48 KB per chunk and CTA) the loads of three CTAs took 1.4 us.  The row warps only arrive at
-    // the barrier that releases the MMAs, one of two in turn: they are held back by the xq tile of the chunk after next,
-    // which is requested when this chunk's MMAs have finished.  A row warp whose wait for a tile
-    // has given up is no longer held back by it: from then on it only waits at the barrier, since one that is overrun never
-    // fills, and nothing bounds that wait.  (An mbarrier in its place, with a bounded wait, costs 0.14 us per chunk of a lone chain:
-    // 2 x 8192 tokens x 7 heads with INT8 states 66.8 -> 71.4 us.)
-    // (Batch 8 x 2048 x 80 heads: 48.9 us with slabs dealt out by position, 41.0 this way, 38.7 with the first tiles requested
-    // ahead of all other set-up and s_x / s_xs divided once per channel; 4 x 8192 x 128 151, 118, 115.)
-    const int qw = warp - kStateThreads / 32, nsl = Q / 32;
-    // live slabs of a chunk from its LUT_state: nsl consecutive tokens per lane, 32 / nsl lanes per slab.  A chunk
-    // without a live slab opens the accumulator with its last one, all rows of it stored as zeros.
-    struct Lut { float4 a, b; };
-    auto lut_of_lane = [&](const float* l) -> Lut {
-      Lut v = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-      if (nsl == 2) {
-        const float2 u = reinterpret_cast<const float2*>(l)[lane];
-        v.a.x = u.x;
-        v.a.y = u.y;
-      } else {
-        v.a = reinterpret_cast<const float4*>(l + lane * nsl)[0];
-        if (nsl == 8) v.b = reinterpret_cast<const float4*>(l + lane * nsl)[1];
-      }
-      return v;
-    };
-    auto live_slabs = [&](const Lut& v) -> uint32_t {
-      auto alive = [&](float l) { return !(__fmul_rn(b127, fabsf(l)) < 0.5f); };
-      const bool any = alive(v.a.x) | alive(v.a.y) | alive(v.a.z) | alive(v.a.w) | alive(v.b.x) | alive(v.b.y) | alive(v.b.z) | alive(v.b.w);
-      const uint32_t bal = __ballot_sync(0xffffffffu, any);
-      const int lps = 32 / nsl;
-      const uint32_t m = __ballot_sync(0xffffffffu, lane < nsl && ((bal >> ((lane * lps) & 31)) & ((1u << lps) - 1u)) != 0);
-      return m ? m : 1u << (nsl - 1);
-    };
-    constexpr int kRowStep = 32 * kRowWarps >> lq;
-    const float* const lut0 = a.pack + (unit0 * kPackRows + PACK_LUT) * Q;   // LUT_state of chunk 0; the next one kPackRows Q floats on
-    const i64 lut_step = (i64)kPackRows * Q;
-    if (qw == kRowWarps) {
-      uint32_t cur = live_slabs(lut_of_lane(lut0)), next = 0;
-      if (d.c > 1) {
-        next = live_slabs(lut_of_lane(lut0 + lut_step));
-        issue_x(1, next);
-      }
-      const uint32_t idesc = idesc_s8(N, 64, 1, 1);
-#pragma unroll 1
-      for (int k = 0; k < d.c; ++k) {
-        Lut v = {};
-        if (k + 2 < d.c) v = lut_of_lane(lut0 + (k + 2) * lut_step);     // (its latency under the waits)
-        named_bar(2 + (k & 1), kQuantThreads);                           // the rows are re-quantised
-        mbar_wait_inline<0>(&bars[B_ACC_FREE], (k & 1) ^ 1, a.status);   // the state warps have read the accumulator of chunk k-1
-        mbar_wait_inline<0>(&bars[B_BFULL], k & 1, a.status);            // the chunk's Bq rows have landed
-        tc_fence_after();
-        const uint32_t sBa = smem_u32(smem + OFF_B), sXa = smem_u32(smem + OFF_X + (k & 1) * XSTAGE);
-        if (elect_one()) {
-#pragma unroll 1
-          for (uint32_t m = cur; m; m &= m - 1) {
-            const int sl = __ffs((int)m) - 1;
-            mma_s8_ss(tmem, tile_desc(sBa + 32 * sl * N, (uint32_t)N), tile_desc(sXa + 32 * sl * 64, 64), idesc, m != cur);
-          }
-          mma_commit(&bars[B_MMA]);
-        }
-        __syncwarp();
-        if (k + 1 < d.c) {
-          mbar_wait_inline<0>(&bars[B_MMA], k & 1, a.status);   // the MMAs of chunk k have read the Bq buffer and its xq stage
-          issue_B(k + 1, next);
-          cur = next;
-          if (k + 2 < d.c) {
-            next = live_slabs(v);
-            issue_x(k + 2, next);
-          }
-        }
-      }
-    } else {
-    int k = 0;
-#pragma unroll 1
-    for (; k < d.c; ++k) {
-      const int s = k & 1;
-      uint8_t* sX = smem + OFF_X + s * XSTAGE;
-      float* lut = reinterpret_cast<float*>(smem + OFF_LUT) + s * 256;
-      const i64 tok0 = (i64)b * d.L + (i64)k * Q;
-      if (__any_sync(0xffffffffu, !mbar_wait_inline<256>(&bars[B_XFULL + s], (k >> 1) & 1, a.status))) break;
-      const uint32_t lm = live_slabs(lut_of_lane(lut));   // (every warp computes the same mask)
-      const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
-      if (TAPS && a.tap_Xsq) {
-        for (int i = qt >> lq; i < Q; i += kRowStep)
-          if (!((lm >> (i >> 5)) & 1u)) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = zero4;
-      }
-#pragma unroll 1
-      for (int r = qt >> lq, m = (int)lm;; r += kRowStep) {   // r: row among the live ones
-        for (; r >= 32; r -= 32) m &= m - 1;
-        if (m == 0) break;
-        const int i = (__ffs(m) - 1) * 32 + r;
-        uint4* ptr = reinterpret_cast<uint4*>(sX + swz_off((uint32_t)i, (uint32_t)c, 64));
-        const float l = lut[i];
-        if (__fmul_rn(b127, fabsf(l)) < 0.5f) {
-          *ptr = zero4;
-          if (TAPS && a.tap_Xsq) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = zero4;
-          continue;
-        }
-        const uint4 w4 = *ptr;
-        const uint32_t ww[4] = {w4.x ^ 0x80808080u, w4.y ^ 0x80808080u, w4.z ^ 0x80808080u, w4.w ^ 0x80808080u};
-        const float2 l2 = make_float2(l, l);
-        uint32_t o[4];
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          uint32_t q4[4];
-#pragma unroll
-          for (int e = 0; e < 4; e += 2) {
-            const float2 xf = __fadd2_rn(
-                make_float2(__uint_as_float(__byte_perm(ww[w], 0x4B400000u, 0x7650u + e)),
-                            __uint_as_float(__byte_perm(ww[w], 0x4B400000u, 0x7651u + e))),
-                make_float2(-kMagicIn, -kMagicIn));
-            const uint2 c2 = rne_clamp_bits2(__fmul2_rn(__fmul2_rn(xf, make_float2(rx[w * 4 + e], rx[w * 4 + e + 1])), l2));
-            q4[e] = c2.x;
-            q4[e + 1] = c2.y;
-          }
-          o[w] = pack4_bits(q4[0], q4[1], q4[2], q4[3]);
-        }
-        const uint4 v = make_uint4(o[0], o[1], o[2], o[3]);
-        *ptr = v;
-        if (TAPS && a.tap_Xsq) *reinterpret_cast<uint4*>(a.tap_Xsq + ((tok0 + i) * d.H + h) * P + c * 16) = v;
-      }
-      fence_async_smem();
-      named_bar_arrive(2 + s, kQuantThreads);
+  // row `row` of a slab, 16 channels (those of lane % 4) of it
+  auto quantise_rows = [&](int slot, int inf, int row, float bound) {
+    const int c = lane & 3;
+    const float l = reinterpret_cast<const float*>(smem + OFF_LUT)[slot * kSlab + row];
+    uint4* ptr = reinterpret_cast<uint4*>(smem + OFF_X + slot * (kSlab * 64) + swz_off((uint32_t)row, (uint32_t)c, 64));
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (alive(bound, l)) {
+      const uint4 w4 = *ptr;
+      const float2 l2 = make_float2(l, l);
+      auto four = [&](uint32_t word, int j) -> uint32_t {
+        const uint32_t ww = word ^ 0x80808080u;
+        const float4 rx = *reinterpret_cast<const float4*>(col_rx + c * 16 + 4 * j);
+        auto pair = [&](int e, const float2& r) -> uint2 {
+          const float2 xf = __fadd2_rn(make_float2(__uint_as_float(__byte_perm(ww, 0x4B400000u, 0x7650u + e)),
+                                                   __uint_as_float(__byte_perm(ww, 0x4B400000u, 0x7651u + e))),
+                                       make_float2(-kMagicIn, -kMagicIn));
+          return rne_clamp_bits2(__fmul2_rn(__fmul2_rn(xf, r), l2));
+        };
+        const uint2 q0 = pair(0, make_float2(rx.x, rx.y)), q1 = pair(2, make_float2(rx.z, rx.w));
+        return pack4_bits(q0.x, q0.y, q1.x, q1.y);
+      };
+      v = make_uint4(four(w4.x, 0), four(w4.y, 1), four(w4.z, 2), four(w4.w, 3));
     }
-    for (; k < d.c; ++k) named_bar(2 + (k & 1), kQuantThreads);   // (a wait has given up)
+    *ptr = v;
+    if (TAPS && a.tap_Xsq)
+      *reinterpret_cast<uint4*>(a.tap_Xsq + (((i64)b * d.L + (i64)(inf >> 16) * Q + ((inf >> 8) & 255) * kSlab + row) * d.H + h) * P +
+                                c * 16) = v;
+  };
+
+  if (warp == kMmaWarp) {
+    // ------------------------------------------------------------ MMA issue
+    const uint32_t idesc = idesc_s8(64, NS, 1, 1);
+    const uint32_t sxa = smem_u32(smem + OFF_X), sba = smem_u32(smem + OFF_B);
+    uint32_t open = 0;                     // the chunk's accumulator has been opened
+    Pos at;
+#pragma unroll 1
+    for (int k = 0; k < d.c; at.next()) {
+      const int slot = at.slot;
+      if (__any_sync(0xffffffffu, !mbar_wait_inline<0>(&bars[B_READY + slot], at.phase, a.status))) break;
+      const int inf = info[slot];
+      const bool last = (inf & SLAB_LAST) != 0;
+      const uint32_t ai = NA == 1 ? 0u : (uint32_t)k & 1u;
+      if (!open) mbar_wait_inline<0>(&bars[B_ACC_FREE + ai], ((k / NA) & 1) ^ 1, a.status);   // the state warps have read the chunk that had it
+      tc_fence_after();
+      if (elect_one()) {
+        const uint64_t da = tile_desc(sxa + slot * (kSlab * 64), 64), db = tile_desc(sba + slot * (kSlab * NS), NS);
+        mma_s8_ss(tmem + ai * NS, da, db, idesc, open);
+        mma_s8_ss(tmem + ai * NS, da + ((32 * 64) >> 4), db + ((32 * NS) >> 4), idesc, 1);
+        mma_commit(&bars[B_FREE + slot]);
+        if (last) mma_commit(&bars[B_ACC + ai]);
+      }
+      __syncwarp();
+      open = last ? 0u : 1u;
+      k += last ? 1 : 0;
+    }
+  } else if (!FEW && warp >= kStateWarps) {
+    // ------------------------------------------------------------ Q(X_scaled) of the slabs, in place: eight rows of a slab at a time
+    const float bound = row_bound(col_rx[lane], col_rx[lane + 32]);
+    Pos at;
+#pragma unroll 1
+    for (int k = 0; k < d.c; at.next()) {
+      const int slot = at.slot;
+      if (__any_sync(0xffffffffu, !mbar_wait_inline<256>(&bars[B_FULL + slot], at.phase, a.status))) break;
+      const int inf = info[slot];
+#pragma unroll 1
+      for (int row = 8 * (warp - kStateWarps) + (lane >> 2); row < kSlab; row += 8 * G::kRowWarps) quantise_rows(slot, inf, row, bound);
+      fence_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars[B_READY + slot]);
+      k += inf & SLAB_LAST;
     }
   } else {
-    // ------------------------------------------------------------ state warps
-    // M = 128: accumulator row n on TMEM lane n; M = 64: row n on lane (n % 16) + 32 (n / 16),
-    // i.e. the first 16 lanes of each warp's quarter
+    // ------------------------------------------------------------ state warps.  Accumulator row p on TMEM lane (p % 16) + 32 (p / 16);
+    // 16 x 256 bit loads: registers 0, 1 of a group of eight columns hold row lane / 4, columns 2 (lane % 4) and the next,
+    // registers 2, 3 the same columns of row lane / 4 + 8
+    constexpr int NC = NS / 2, NG = NC / 8;        // columns of a warp, groups of eight
     const int q = warp & 3, ch = warp >> 2;
-    constexpr int npp = 8 * ncq;             // channels per thread
-    const int cb = 16 * c0 + ch * npp;       // first channel of this thread
-    const bool ok = (N == 128) || (lane < 16);
-    const int n = (N == 128) ? q * 32 + lane : q * 16 + lane;
-    // the running state S[p, n]: fp32, or (I8S) the integer code, in tensor-memory columns 64 + p of lane n
-    const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16);
-    const uint32_t tS = tlane + 64u + (uint32_t)cb;
-    float smax[CAL ? 32 : 1];   // CAL: running maxima of |S[p, n]| over the chunks
+    const int p0 = 16 * q + (lane >> 2);           // this thread's channels: p0 and p0 + 8
+    const int n0 = n_base + ch * NC + 2 * (lane & 3);
+    const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * NC);
+    const float2 cs0 = make_float2(col_scale[p0], col_scale[p0]), cs1 = make_float2(col_scale[p0 + 8], col_scale[p0 + 8]);
+    const float2 ih0 = make_float2(col_invh[p0], col_invh[p0]), ih1 = make_float2(col_invh[p0 + 8], col_invh[p0 + 8]);
+    // the running state S[p, n]: fp32, or (I8S) the integer code
+    float2 S[2 * NG];
+    float smax0 = 0.f, smax1 = 0.f;                // CAL: running maxima of |S[p, n]| (a NaN counts for nothing)
+    auto code2 = [&](const float2& v, const float2& ih) -> uint2 {
+      return I8S ? make_uint2(__float_as_uint(v.x), __float_as_uint(v.y)) : rne_clamp_bits2(__fmul2_rn(v, ih));
+    };
 #pragma unroll
-    for (int p0 = 0; p0 < 32; p0 += 8) {
-      if (p0 < npp) {
-        int sv[8];
+    for (int i = 0; i < NG; ++i) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float v = (a.init && ok) ? a.init[(bh * P + cb + p0 + e) * N + n] : 0.f;
-          sv[e] = I8S ? (int)(int8_t)(rne_clamp_bits(__fmul_rn(v, col_invh[(cb + p0 + e) & 63])) & 0xffu) : __float_as_int(v);
+      for (int r = 0; r < 2; ++r) {
+        float2 v = a.init ? *reinterpret_cast<const float2*>(a.init + (bh * P + p0 + 8 * r) * N + n0 + 8 * i) : make_float2(0.f, 0.f);
+        if (I8S) {
+          const uint2 cd = rne_clamp_bits2(__fmul2_rn(v, r ? ih1 : ih0));
+          v = make_float2(__int_as_float((int)(int8_t)(cd.x & 0xffu)), __int_as_float((int)(int8_t)(cd.y & 0xffu)));
         }
-        if (CAL) {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) smax[CAL ? p0 + e : 0] = fmaxf(fabsf(__int_as_float(sv[e])), 0.f);   // (a NaN counts for nothing)
-        }
-        tmem_st8(tS + (uint32_t)p0, sv);
+        if (CAL) (r ? smax1 : smax0) = fmaxf(fmaxf(r ? smax1 : smax0, fabsf(v.x)), fabsf(v.y));
+        S[2 * i + r] = v;
       }
     }
-    tmem_st_wait();
+    // codes go to row p0 of the staging tile, swizzled for the TMA store: chunk of 16 columns ^ a term of the row that is the same for p0 + 8
+    constexpr int kRowShift = NS == 128 ? 0 : NS == 64 ? 1 : 2, kRowMask = NS / 16 - 1;
+    const uint32_t hoff = (uint32_t)p0 * NS + ((uint32_t)(((ch * NC / 16) ^ ((p0 >> kRowShift) & kRowMask)) << 4)) + 2u * (lane & 3);
+    // ---- (FEW) Q(X_scaled) of a chunk's slabs, in place, one chunk ahead: a warp takes eight rows of each
+    const float bound = FEW ? row_bound(col_rx[lane], col_rx[lane + 32]) : 0.f;
+    Pos at;
+    auto quantise_chunk = [&]() {
+#pragma unroll 1
+      for (int more = 1; more; at.next()) {
+        const int slot = at.slot;
+        if (__any_sync(0xffffffffu, !mbar_wait_inline<0>(&bars[B_FULL + slot], at.phase, a.status))) return;
+        const int inf = info[slot];
+        quantise_rows(slot, inf, 8 * warp + (lane >> 2), bound);
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars[B_READY + slot]);
+        more = (inf & SLAB_LAST) ^ SLAB_LAST;
+      }
+    };
+    if (FEW) quantise_chunk();
 #pragma unroll 1
     for (int k = 0; k < d.c; ++k) {
       const float gam = a.gamma[unit0 + k];
-      if (tid < ncq && k > 0) tma_store_wait_read();  // last chunk's hq store has read the staging tile
-      named_bar(1, kStateThreads);  // also: every state thread has read the accumulator of chunk k-1
-      // ---- hq[k] = codes of the state entering this chunk (and the prev tap).  They are formed here, ahead
-      // of the wait for the chunk's MMAs, from a second read of the state; forming them in the update pass of
-      // the chunk before, while the new values are in registers, puts them behind that wait on the chain of
-      // the chunk and was measured slower (0.0568 against 0.0536 ms at batch 8 x 2048 x 80 heads).
+      if (FEW && k + 1 < d.c) quantise_chunk();
+      const uint32_t ai = NA == 1 ? 0u : (uint32_t)k & 1u;
+      // ---- hq[k] = codes of the state entering this chunk (and the prev tap), ahead of the wait for the chunk's MMAs
+      uint8_t* const hq = smem + G::OFF_HQ + (k & 1) * 8192;
       if (!CAL) {
-        const i64 obase = (((((i64)b * d.c + k) * d.H + h) * P) + cb) * N + n;
-        // batches of 8: all loads of a batch before its byte stores (a byte store may alias anything,
-        // so interleaving them would serialise the loop on shared-memory latency).  The tensor-memory
-        // loads are warp-wide; lanes without a state row (N = 64) skip what follows them.
 #pragma unroll
-        for (int p0 = 0; p0 < 32; p0 += 8) {
-          if (p0 < npp) {
-            int sv[8];
-            tmem_ld8(tS + (uint32_t)p0, sv);
-            tmem_ld_wait();
-            if (ok) {
-              uint32_t code[8];
-              // (cb is a multiple of 8: the eight reciprocals are two 16-byte loads)
-              const float4 i0 = *reinterpret_cast<const float4*>(col_invh + cb + p0);
-              const float4 i1 = *reinterpret_cast<const float4*>(col_invh + cb + p0 + 4);
-              const float ih[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
-#pragma unroll
-              for (int e = 0; e < 8; e += 2) {
-                if (I8S) {
-                  code[e] = (uint32_t)sv[e];
-                  code[e + 1] = (uint32_t)sv[e + 1];
-                } else {
-                  const uint2 c2 = rne_clamp_bits2(__fmul2_rn(make_float2(__int_as_float(sv[e]), __int_as_float(sv[e + 1])),
-                                                              make_float2(ih[e], ih[e + 1])));
-                  code[e] = c2.x;
-                  code[e + 1] = c2.y;
-                }
-              }
-              uint8_t* hrow = sHQ + (cb + p0) * N + n;
-#pragma unroll
-              for (int e = 0; e < 8; ++e, hrow += N) *hrow = (uint8_t)code[e];
-              if (TAPS && !I8S && a.tap_prev) {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) a.tap_prev[obase + (i64)(p0 + e) * N] = __int_as_float(sv[e]);
-              }
-            }
-          }
+        for (int i = 0; i < NG; ++i) {
+          uint8_t* const at = hq + ((hoff ^ (uint32_t)((i >> 1) << 4)) + 8 * (i & 1));
+          const uint2 c0 = code2(S[2 * i], ih0), c1 = code2(S[2 * i + 1], ih1);
+          *reinterpret_cast<uint16_t*>(at) = (uint16_t)__byte_perm(c0.x, c0.y, 0x0040u);
+          *reinterpret_cast<uint16_t*>(at + 8 * NS) = (uint16_t)__byte_perm(c1.x, c1.y, 0x0040u);
         }
+        if (TAPS && !I8S && a.tap_prev) {
+#pragma unroll
+          for (int i = 0; i < 2 * NG; ++i)
+            *reinterpret_cast<float2*>(a.tap_prev + (((((i64)b * d.c + k) * d.H + h) * P) + p0 + 8 * (i & 1)) * N + n0 + 8 * (i >> 1)) = S[i];
+        }
+        fence_async_smem();
+        if (tid == 0) tma_store_wait_read();     // the store of chunk k - 1: its tile is written again in chunk k + 1
       }
-      fence_async_smem();
       // one warp polls for the MMAs of this chunk; the barrier passes their completion on to the others
-      if (warp == 0) mbar_wait_inline<256>(&bars[B_MMA], k & 1, a.status);
-      named_bar(1, kStateThreads);
-      // ---- hq[k] leaves by TMA
-      if (tid < ncq && !CAL) {
-        const int j = c0 + tid;              // 16 channels (rows of hq) per store
-        tma_store_2d(&tm_hq, sHQ + 16 * j * N, 0, (int)(((((i64)b * d.c + k) * d.H + h) * P) + 16 * j));
+      if (warp == 0) mbar_wait_inline<256>(&bars[B_ACC + ai], (k / NA) & 1, a.status);
+      named_bar_sync(1, kStateThreads);
+      if (tid == 0 && !CAL) {                    // hq[k] leaves by TMA
+        tma_store_2d(&tm_hq, hq, n_base, (int)((((i64)b * d.c + k) * d.H + h) * P));
         tma_store_commit();
       }
-      // ---- epilogue of the MMA: S = fmaf(Gamma_k, S, loc), 8 channels at a time
+      // ---- epilogue of the MMA: S = fmaf(Gamma_k, S, loc), 16 columns at a time
       tc_fence_after();
+      const float2 g2 = make_float2(gam, gam);
+      const int Gq = I8S ? __float2int_rn(__fmul_rn(gam, 128.0f)) : 0;
 #pragma unroll
-      for (int hf = 0; hf < 4; ++hf) {       // 8 channels at a time
-        if (hf < ncq) {
-        int acc[8], sv[8];
-        tmem_ld8(tlane + (uint32_t)(cb + hf * 8), acc);
-        tmem_ld8(tS + (uint32_t)(hf * 8), sv);
+      for (int i0 = 0; i0 < NG; i0 += 2) {
+        int acc[8];
+        tmem_ld_16x256_x2(tacc + ai * NS + 8 * i0, acc);
         tmem_ld_wait();
-        if (ok) {
-          const i64 obase = (((((i64)b * d.c + k) * d.H + h) * P) + cb + hf * 8) * N + n;
-          const float4 c0v = *reinterpret_cast<const float4*>(col_scale + cb + hf * 8);
-          const float4 c1v = *reinterpret_cast<const float4*>(col_scale + cb + hf * 8 + 4);
-          const float cscale[8] = {c0v.x, c0v.y, c0v.z, c0v.w, c1v.x, c1v.y, c1v.z, c1v.w};
-#pragma unroll
-          for (int e = 0; e < 8; e += 2) {
-            const float2 af = __fadd2_rn(make_float2(__int_as_float(acc[e] + 0x4B400000), __int_as_float(acc[e + 1] + 0x4B400000)),
-                                         make_float2(-kMagicOut, -kMagicOut));   // exact for |acc| < 2^22
-            const float2 l2 = __fmul2_rn(af, make_float2(cscale[e], cscale[e + 1]));
-            if (TAPS && a.tap_acc) {
-              a.tap_acc[obase + (i64)e * N] = acc[e];
-              a.tap_acc[obase + (i64)(e + 1) * N] = acc[e + 1];
-            }
-            if (I8S) {
-              const int Gq = __float2int_rn(__fmul_rn(gam, 128.0f));
-#pragma unroll
-              for (int j = 0; j < 2; ++j) {
-                const int locq = (int)(int8_t)(rne_clamp_bits(j ? l2.y : l2.x) & 0xffu);
-                const int Sn = locq + ((Gq * sv[e + j] + 64) >> 7);
-                sv[e + j] = max(-127, min(127, Sn));
-              }
-            } else {
-              if (TAPS && a.tap_loc) {
-                a.tap_loc[obase + (i64)e * N] = l2.x;
-                a.tap_loc[obase + (i64)(e + 1) * N] = l2.y;
-              }
-              const float2 s2 = __ffma2_rn(make_float2(gam, gam),
-                                           make_float2(__int_as_float(sv[e]), __int_as_float(sv[e + 1])), l2);
-              sv[e] = __float_as_int(s2.x);
-              sv[e + 1] = __float_as_int(s2.y);
-              if (CAL) {
-                smax[CAL ? hf * 8 + e : 0] = fmaxf(smax[CAL ? hf * 8 + e : 0], fabsf(s2.x));
-                smax[CAL ? hf * 8 + e + 1 : 0] = fmaxf(smax[CAL ? hf * 8 + e + 1 : 0], fabsf(s2.y));
-              }
-            }
-          }
+        if (i0 + 2 == NG) {                        // this warp has read the accumulator
+          tc_fence_before();
+          if (lane == 0) mbar_arrive(&bars[B_ACC_FREE + ai]);
         }
-        tmem_st8(tS + (uint32_t)(hf * 8), sv);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {              // two columns of one row each
+          const int i = i0 + (j >> 1);
+          const float2 af = __fadd2_rn(make_float2(__int_as_float(acc[2 * j] + 0x4B400000), __int_as_float(acc[2 * j + 1] + 0x4B400000)),
+                                       make_float2(-kMagicOut, -kMagicOut));   // exact for |acc| < 2^22
+          const float2 l2 = __fmul2_rn(af, j & 1 ? cs1 : cs0);
+          float2& sv = S[2 * i + (j & 1)];
+          if (TAPS) {
+            const i64 o = (((((i64)b * d.c + k) * d.H + h) * P) + p0 + 8 * (j & 1)) * N + n0 + 8 * i;
+            if (a.tap_acc) *reinterpret_cast<int2*>(a.tap_acc + o) = make_int2(acc[2 * j], acc[2 * j + 1]);
+            if (!I8S && a.tap_loc) *reinterpret_cast<float2*>(a.tap_loc + o) = l2;
+          }
+          if (I8S) {
+            const uint2 lq = rne_clamp_bits2(l2);     // 0x4B400000 + locq
+            auto next = [&](float s, uint32_t l) -> float {
+              return __int_as_float(max(-127, min(127, (int)l + ((Gq * __float_as_int(s) + 64) >> 7) - 0x4B400000)));
+            };
+            sv = make_float2(next(sv.x, lq.x), next(sv.y, lq.y));
+          } else {
+            sv = __ffma2_rn(g2, sv, l2);
+          }
+          if (CAL) (j & 1 ? smax1 : smax0) = fmaxf(fmaxf(j & 1 ? smax1 : smax0, fabsf(sv.x)), fabsf(sv.y));
+        }
       }
-      }
-      tmem_st_wait();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bars[B_ACC_FREE]);  // this warp has read the accumulator of chunk k
     }
     if (CAL) {
 #pragma unroll
-      for (int p = 0; p < 32; ++p) {
-        if (p < npp) {
-          const uint32_t m = __reduce_max_sync(0xffffffffu, ok ? __float_as_uint(smax[CAL ? p : 0]) : 0u);
-          if (lane == (p & 31)) atomicMax(reinterpret_cast<uint32_t*>(col_invh) + cb + p, m);
-        }
+      for (int o = 1; o < 4; o <<= 1) {
+        smax0 = fmaxf(smax0, __shfl_xor_sync(0xffffffffu, smax0, o));
+        smax1 = fmaxf(smax1, __shfl_xor_sync(0xffffffffu, smax1, o));
       }
-      named_bar(1, kStateThreads);
+      if ((lane & 3) == 0) {
+        atomicMax(reinterpret_cast<uint32_t*>(col_invh) + p0, __float_as_uint(smax0));
+        atomicMax(reinterpret_cast<uint32_t*>(col_invh) + p0 + 8, __float_as_uint(smax1));
+      }
+      named_bar_sync(1, kStateThreads);
       if (tid < 64) atomicMax(a.absmax_h + h * P + tid, reinterpret_cast<const uint32_t*>(col_invh)[tid]);
     }
     if (!CAL && a.final_state) {
+      const float sh0 = I8S ? a.s_h[h * P + p0] : 0.f, sh1 = I8S ? a.s_h[h * P + p0 + 8] : 0.f;
 #pragma unroll
-      for (int p0 = 0; p0 < 32; p0 += 8) {
-        if (p0 < npp) {
-          int sv[8];
-          tmem_ld8(tS + (uint32_t)p0, sv);
-          tmem_ld_wait();
-          if (ok) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-              a.final_state[(bh * P + cb + p0 + e) * N + n] =
-                  I8S ? __fmul_rn((float)sv[e], a.s_h[h * P + cb + p0 + e]) : __int_as_float(sv[e]);
-          }
-        }
+      for (int i = 0; i < 2 * NG; ++i) {
+        float2 v = S[i];
+        if (I8S) v = make_float2(__fmul_rn((float)__float_as_int(v.x), i & 1 ? sh1 : sh0), __fmul_rn((float)__float_as_int(v.y), i & 1 ? sh1 : sh0));
+        *reinterpret_cast<float2*>(a.final_state + (bh * P + p0 + 8 * (i & 1)) * N + n0 + 8 * (i >> 1)) = v;
       }
     }
-    if (tid < ncq) tma_store_wait_read();
+    if (tid == 0 && !CAL) tma_store_wait_read();
+  }
+  tc_fence_before();
   }
   drain_after_timeout(a.status);
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, kTmemCols);
+    tmem_dealloc(*tmem_slot, kTmemCols);
   }
 }
 
-// Column range of a CTA: 16-channel chunks c0 .. c0 + ncq - 1 of one head.  Whole heads first, then
-// heads in quarters, for a short remainder or a small workload (see the launcher; operand tiles and the MMA stay
-// full width: only the re-quantisation, the state update and the hq rows are restricted to the range).
-template <bool I8S, bool TAPS, bool CAL>
-__global__ void __launch_bounds__(kThreads, CAL ? 2 : 3)
+// Whole heads first, then heads in slices of 32 or 64 state columns, for a short remainder or a small workload (see the launcher; a
+// slice re-quantises all channels of the head itself and has the MMA, the state update and the hq columns of its own columns only).
+template <bool I8S, bool TAPS, bool CAL, bool FEW, int N>
+__global__ void __launch_bounds__(Geo<FEW>::kThreads, FEW ? 2 : 3)
 chunk_state_pass_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__ CUtensorMap tm_x,
-                    const __grid_constant__ CUtensorMap tm_hq, const FusedArgs a) {
+                    const __grid_constant__ CUtensorMap tm_hq, const __grid_constant__ CUtensorMap tm_Bs,
+                    const __grid_constant__ CUtensorMap tm_hqs, const FusedArgs a) {
   if ((int)blockIdx.x < a.n_full) {
-    fused_body<I8S, TAPS, CAL, 4>(tm_B, tm_x, tm_hq, a, (int)blockIdx.x, 0);
+    fused_body<I8S, TAPS, CAL, FEW, N, N>(tm_B, tm_x, tm_hq, a, (int)blockIdx.x, 0);
   } else {
     const int r = (int)blockIdx.x - a.n_full;
-    fused_body<I8S, TAPS, CAL, 1>(tm_B, tm_x, tm_hq, a, a.n_full + (r >> 2), r & 3);
+    if (N == 128 && a.slice == 64)
+      fused_body<I8S, TAPS, CAL, FEW, N, 64>(tm_Bs, tm_x, tm_hqs, a, a.n_full + r / (N / 64), r % (N / 64) * 64);
+    else
+      fused_body<I8S, TAPS, CAL, FEW, N, 32>(tm_Bs, tm_x, tm_hqs, a, a.n_full + r / (N / 32), r % (N / 32) * 32);
   }
 }
 
@@ -520,56 +530,71 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
                                           int32_t* tap_acc, int32_t* status, bool int8_state,
                                           cudaStream_t st, uint32_t* absmax_h, float* s_xs_out) {
   const uint64_t T = (uint64_t)d.b * d.L;
-  CUtensorMap tm_B, tm_x, tm_hq;
-  {
+  CUtensorMap tm_B, tm_x, tm_hq, tm_Bs, tm_hqs;   // (the last two: of a slice)
+  auto maps = [&](CUtensorMap& mB, CUtensorMap& mh, int cols) -> bool {
     uint64_t dims[3] = {(uint64_t)d.N, (uint64_t)d.G, T};
     uint64_t str[2] = {(uint64_t)d.N, (uint64_t)d.G * d.N};
-    uint32_t box[3] = {(uint32_t)d.N, 1, 32};
-    if (!encode_tensor_map(&tm_B, Bq, 1, 3, dims, str, box, d.N)) return SSDI8_ERR_CUDA;
-  }
+    uint32_t box[3] = {(uint32_t)cols, 1, kSlab};
+    uint64_t hdims[2] = {(uint64_t)d.N, (uint64_t)d.b * d.c * d.H * d.P};
+    uint64_t hstr[1] = {(uint64_t)d.N};
+    uint32_t hbox[2] = {(uint32_t)cols, 64};
+    return encode_tensor_map(&mB, Bq, 1, 3, dims, str, box, cols) && encode_tensor_map(&mh, hq, 1, 2, hdims, hstr, hbox, cols);
+  };
   {
     uint64_t dims[3] = {(uint64_t)d.P, (uint64_t)d.H, T};
     uint64_t str[2] = {(uint64_t)d.P, (uint64_t)d.H * d.P};
-    uint32_t box[3] = {64, 1, 32};
+    uint32_t box[3] = {64, 1, kSlab};
     if (!encode_tensor_map(&tm_x, xq, 1, 3, dims, str, box, 64)) return SSDI8_ERR_CUDA;
   }
-  {
-    uint64_t dims[2] = {(uint64_t)d.N, (uint64_t)d.b * d.c * d.H * d.P};
-    uint64_t str[1] = {(uint64_t)d.N};
-    uint32_t box[2] = {(uint32_t)d.N, 16};
-    if (!encode_tensor_map(&tm_hq, hq, 1, 2, dims, str, box, 0)) return SSDI8_ERR_CUDA;
-  }
-  // (batch, head) units over the CTA slots of the device, 3 per SM.  (The calibration instance has two per SM; it follows
-  // the same rule, whose lines were measured on the others.)
+  // (batch, head) units over the CTA slots of the device, 3 per SM.
   const int sms = sm_count();
   if (sms == 0) return SSDI8_ERR_CUDA;
   const int units = d.H * d.b, slots = 3 * sms;
-  // Whole (batch, head) units wherever the device is filled: a partly filled last wave of whole units runs faster per
-  // CTA and costs less than the same units cut into more CTAs (592 units on 444 slots: 36.7 us whole, 41.9 with the last
-  // 148 in quarters).  Quarter-width CTAs have the shorter chain per chunk (a quarter of the state per thread), so they
-  // take a remainder of less than an eighth of a wave (512 tokens x 24 heads: 5.1 us, 7.1 whole) and, where all
-  // of them fit the device beside the next kernel's first CTAs and a chain has four chunks or more, the whole workload
-  // (Algorithm 2, us, whole / quarters: 2048 tokens x 80 heads 50.4 / 47.6, 2 x 2048 x 50 54.0 / 52.0, 1408 x 70 in chunks of
-  // 128 43.8 / 40.4, 1024 x 80 36.6 / 35.5; but with one or two chunks 3 x 256 x 37 24.4 / 26.0, 512 x 100 29.9 / 30.5, and
-  // 2048 x 111 55.8 / 56.7).
-  int n_full = units / slots * slots;
-  const bool quarters = 8 * (units - n_full) <= slots || (n_full == 0 && d.c >= 4 && 4 * units <= slots - slots / 10);
-  if (!quarters) n_full = units;
+  // Whole heads wherever the device is filled; a remainder of less than an eighth of a wave goes in slices of 32 columns, whose
+  // chain per chunk is shorter.  Few units go in slices of 64, the longest chains of them in 32 (Algorithm 2, us, whole / slices
+  // of 64 / of 32): N 128: 512 tokens x 24 heads 18.9 / 18.1 / 19.9, 1024 x 32 22.2 / 21.1 / 20.9, 1024 x 96 34.6 / 33.7 / 37.2, 3 x 512 x 12
+  // 22.1 / 20.6 / 23.3, 256 x 64 23.2 / 22.8 / 22.5, 2048 x 80 48.7 / 48.1 / 54.7, 2 x 8192 x 8 (INT8 states) 78.3 / 68.0 / 64.6; but 4096 x
+  // 100 even, 512 x 60 22.1 / 22.4 / 22.6, 2 x 2048 x 128 98.9 / 108 / 118.  N 64, from four chunks on: 768 x 60 28.7 / - / 27.9, 256 x 32 (chunks
+  // of 64) 16.4 / - / 15.6, 2048 x 60 44.9 / - / 44.6, but 256 x 36 (chunks of 128) 16.4 / - / 18.1.
+  int n_full = units / slots * slots, slice = 32;
+  const int last = units - n_full;
+  if (n_full > 0) {
+    if (8 * last > slots) n_full = units;
+  } else if (d.N == 128 && 3 * units <= 2 * sms) {
+    slice = d.c >= 12 && 4 * units <= sms ? 32 : 64;
+  } else if (!(d.N == 64 && d.c >= 4 && 2 * units <= sms)) {
+    n_full = units;
+  }
+  if (!maps(tm_B, tm_hq, d.N)) return SSDI8_ERR_CUDA;
+  if (n_full == units) {
+    tm_Bs = tm_B;
+    tm_hqs = tm_hq;
+  } else if (!maps(tm_Bs, tm_hqs, slice)) {
+    return SSDI8_ERR_CUDA;
+  }
   FusedArgs a = {s_x, s_xs, s_B, s_h, pack, gamma, init, final_state, tap_loc, tap_prev, tap_Xsq, tap_acc,
-                 status, absmax_h, s_xs_out, d, n_full};
-  const size_t smem = SMEM_BYTES;
-  const unsigned grid = (unsigned)(n_full + 4 * (units - n_full));
+                 status, absmax_h, s_xs_out, d, n_full, slice};
+  const unsigned grid = (unsigned)(n_full + d.N / slice * (units - n_full));
   const bool taps = tap_loc || tap_prev || tap_Xsq || tap_acc;
-  auto launch = [&](auto kernel) -> ssdi8_status_t {
-    return launch_configured(kernel, dim3(grid), dim3(kThreads), smem, -1, true, st, tm_B, tm_x, tm_hq, a);
+  const bool few = (int)grid <= 2 * sms;
+  auto launch = [&](auto few_c, auto kernel) -> ssdi8_status_t {
+    using G = Geo<decltype(few_c)::value>;
+    const size_t smem = (int)grid <= sms ? kSmemAlone : G::SMEM_BYTES;
+    return launch_sized(kernel, dim3(grid), dim3(G::kThreads), smem, decltype(few_c)::value ? kSmemAlone : smem, 100, true, st, tm_B, tm_x, tm_hq,
+                        tm_Bs, tm_hqs, a);
   };
-  ssdi8_status_t ls;
-  if (absmax_h)
-    ls = launch(chunk_state_pass_tc<false, false, true>);
-  else if (int8_state)
-    ls = taps ? launch(chunk_state_pass_tc<true, true, false>) : launch(chunk_state_pass_tc<true, false, false>);
-  else
-    ls = taps ? launch(chunk_state_pass_tc<false, true, false>) : launch(chunk_state_pass_tc<false, false, false>);
+  auto pick = [&](auto few_c, auto n) -> ssdi8_status_t {
+    constexpr bool F = decltype(few_c)::value;
+    constexpr int N = decltype(n)::value;
+    if (absmax_h) return launch(few_c, chunk_state_pass_tc<false, false, true, F, N>);
+    if (int8_state)
+      return taps ? launch(few_c, chunk_state_pass_tc<true, true, false, F, N>) : launch(few_c, chunk_state_pass_tc<true, false, false, F, N>);
+    return taps ? launch(few_c, chunk_state_pass_tc<false, true, false, F, N>) : launch(few_c, chunk_state_pass_tc<false, false, false, F, N>);
+  };
+  auto pick_n = [&](auto few_c) -> ssdi8_status_t {
+    return d.N == 128 ? pick(few_c, std::integral_constant<int, 128>{}) : pick(few_c, std::integral_constant<int, 64>{});
+  };
+  const ssdi8_status_t ls = few ? pick_n(std::true_type{}) : pick_n(std::false_type{});
   if (ls != SSDI8_OK) return ls;
   SSDI8_LAUNCH_CHECK();
   return SSDI8_OK;

@@ -30,17 +30,23 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 // kernel uses static shared memory (kernels that need their dynamic part at the window's base).
 cudaError_t kernel_ready(const void* kernel, size_t smem, int carveout, bool check_static);
 void kernel_forget(const void* kernel);   // the device was reset under us: set the attributes again
+// (smem_most: the largest that any launch of the kernel asks for)
 template <typename... KArgs, typename... Args>
-inline ssdi8_status_t launch_configured(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, int carveout,
-                                        bool check_static, cudaStream_t st, Args&&... args) {
+inline ssdi8_status_t launch_sized(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, size_t smem_most, int carveout,
+                                   bool check_static, cudaStream_t st, Args&&... args) {
   const void* k = reinterpret_cast<const void*>(kernel);
   for (int attempt = 0; attempt < 2; ++attempt) {
-    if (kernel_ready(k, smem, carveout, check_static) != cudaSuccess) break;
+    if (kernel_ready(k, smem_most, carveout, check_static) != cudaSuccess) break;
     if (launch_pdl(kernel, grid, block, smem, st, args...) == cudaSuccess) return SSDI8_OK;
     kernel_forget(k);
   }
   (void)cudaGetLastError();
   return SSDI8_ERR_CUDA;
+}
+template <typename... KArgs, typename... Args>
+inline ssdi8_status_t launch_configured(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, int carveout,
+                                        bool check_static, cudaStream_t st, Args&&... args) {
+  return launch_sized(kernel, grid, block, smem, smem, carveout, check_static, st, std::forward<Args>(args)...);
 }
 int sm_count();   // of the current device (0 on failure)
 

@@ -12,7 +12,7 @@ struct Slot {
   std::atomic<const void*> kernel{nullptr};
   std::atomic<uint64_t> devices{0};
 };
-constexpr int kSlots = 128;   // the library has about ninety kernels, most of them with attributes
+constexpr int kSlots = 128;   // the library has about a hundred kernels, most of them with attributes
 Slot g_slots[kSlots];
 
 Slot* find_slot(const void* kernel) {

@@ -177,6 +177,15 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, int (&v)[8]) {
       : "r"(taddr)
       : "memory");
 }
+// 16 lanes x 16 consecutive columns (.16x256b.x2), for accumulators of 64 rows, which take the first 16 lanes of every quarter:
+// thread t receives of each group of eight columns the columns 2 (t % 4), 2 (t % 4) + 1 of lane t / 4, then of lane t / 4 + 8
+__device__ __forceinline__ void tmem_ld_16x256_x2(uint32_t taddr, int (&v)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+      : "r"(taddr)
+      : "memory");
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // 32 lanes x 8 consecutive 32-bit columns, registers -> tensor memory (thread t writes lane base + t)
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const int (&v)[8]) {
@@ -198,11 +207,11 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo_bytes
          ((uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32) | (1ull << 46) | ((uint64_t)swizzle << 61);
 }
 
-// Operand tile whose rows are `row_bytes` (64 or 128) long and swizzled at that width: rows are
+// Operand tile whose rows are `row_bytes` (32, 64 or 128) long and swizzled at that width: rows are
 // the M/N index for a K-major operand and the K index for an MN-major operand.  Groups of 8
 // rows are `8 * row_bytes` apart (the stride byte offset) in both cases.
 __device__ __forceinline__ uint64_t tile_desc(uint32_t saddr, uint32_t row_bytes) {
-  return smem_desc(saddr, 16, 8 * row_bytes, row_bytes == 128 ? SWZ_128B : SWZ_64B);
+  return smem_desc(saddr, 16, 8 * row_bytes, row_bytes == 128 ? SWZ_128B : row_bytes == 64 ? SWZ_64B : SWZ_32B);
 }
 
 // Instruction descriptor for kind::i8: signed 8-bit A and B, 32-bit integer accumulator.
@@ -239,6 +248,6 @@ __device__ __forceinline__ uint32_t swz_off(uint32_t r, uint32_t c, uint32_t row
 // false if the driver entry point is unavailable or the encode fails.
 bool encode_tensor_map(CUtensorMap* out, const void* base, int elem_bytes, int rank, const uint64_t* dims,
                        const uint64_t* strides_bytes /* rank-1 entries */, const uint32_t* box,
-                       int swizzle_bytes /* 0, 64, 128 */);
+                       int swizzle_bytes /* 0, 32, 64, 128 */);
 
 }  // namespace ssdi8

@@ -255,6 +255,32 @@ def test_state_kernels_on_both_sides_of_the_dispatch(cfg, fast):
     check_fwd(cfg, init=inputs.make_init_state(cfg, 0.5), mutate=decay if fast else None)
 
 
+@pytest.mark.parametrize("cfg", [SSDConfig("whole_few", 2, 3 * 128, 50, 64, 128, 2, 128, 0.02, 20.0, 51),
+                                 SSDConfig("whole_alone", 1, 2 * 64, 101, 64, 128, 1, 64, 0.02, 20.0, 52),
+                                 SSDConfig("slices_64", 1, 3 * 256, 9, 64, 128, 3, 256, 0.02, 20.0, 53),
+                                 SSDConfig("slices_32", 1, 13 * 64, 5, 64, 128, 1, 64, 0.02, 20.0, 54),
+                                 SSDConfig("slices_n64", 1, 5 * 128, 7, 64, 64, 1, 128, 0.02, 20.0, 55),
+                                 SSDConfig("many", 3, 2 * 256, 100, 64, 64, 2, 256, 0.02, 20.0, 56),
+                                 SSDConfig("slices_last", 5, 2 * 64, 90, 64, 128, 1, 64, 0.02, 20.0, 57)], ids=lambda c: c.name)
+@pytest.mark.parametrize("decay", [0.002, 1.0, 60.0])
+def test_fused_state_kernel_with_few_and_many_sequences(cfg, decay):
+    # Up to two CTAs per SM (whole heads, slices of 32 and of 64 state columns), three, and a last wave in slices; decay rates
+    # at which every slab of every chunk is live, some are, and none is.  INT8 states always take this kernel, and the codes of
+    # the states that enter the chunks and the final state are all that it writes (the taps' instance is another kernel).
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    t = inputs.make_prefill(cfg)
+    t["A"] *= np.float32(decay)
+    init = inputs.make_init_state(cfg, 0.5)
+    q = orc.prepare_quantized(cfg, t, init)
+    for gpu_flags, flags in ((0, 0), (bd.FLAG_INT8_STATE, orc.FLAG_INT8_STATE)):
+        _, fin_ref, ref = orc.ssdi8_fwd(cfg, q["xq"], q["Bq"], q["Cq"], q["s_x"], q["s_B"], q["s_C"], q["dt"], q["A"], q["D"], None,
+                                        q["s_xs"], q["s_cb"], q["s_h"], init, taps=("hq",), flags=flags)
+        _, fin, got = gh.gpu_fwd(cfg, q, taps=("hq",), flags=gpu_flags)
+        assert np.array_equal(got["hq"], ref["hq"])
+        assert np.array_equal(fin, fin_ref)
+
+
 def _near_ties():
     # Pairs (v, alpha) whose quotient lies within 8 / alpha's significand of the midpoint between k + 1/2 and a neighbour
     # in binary32: where a quotient formed from a reciprocal could fall on the other side.

@@ -1,7 +1,7 @@
 """The handshake of the fused state kernel (csrc/chunk_state_pass.cu) on the host-side model of test_scan_protocol_model.py:
-three row warps, the warp that issues MMAs and loads, the state warps.  Every wait is decided by parity alone and checked against
-the true phase counts.  A second model lets arrivals go missing and waits run out: every role must still come to its end.
-`broken` is the form in which the row warps go on as if their waits had not given up."""
+the loading warp, the ring of slabs, the warps that re-quantise (the state warps themselves or two of their own), the issuing warp,
+the state warps.  Every wait is decided by parity alone and checked against the true phase counts.  A second model lets arrivals
+go missing and waits run out: every role must still come to its end."""
 import heapq
 
 import pytest
@@ -62,67 +62,94 @@ class StateSim(Sim):
         return ok
 
 
-def build(sim, chunks, speed, broken=False):
+def build(sim, chunks, speed, few, na, slabs=None):
+    """few: the eight state warps re-quantise, one chunk ahead, behind a ring of six; else two row warps behind a ring of four.
+    na accumulators.  slabs: live slabs of every chunk (of up to four; drawn if not given)."""
     rng = sim.rng
-    xfull, bfull, mma = [Bar("XFULL0", 1), Bar("XFULL1", 1)], Bar("BFULL", 1), Bar("MMA", 1)
-    acc_free = Bar("ACC_FREE", 8)
-    named = [Named(4), Named(4)]
+    slots, rows = (6, 8) if few else (4, 2)
+    bars = lambda name, n, count: [Bar(f"{name}{i}", count) for i in range(n)]
+    fulls, ready, freed = bars("FULL", slots, 1), bars("READY", slots, rows), bars("FREE", slots, 1)
+    accs, acc_free = bars("ACC", na, 1), bars("ACC_FREE", na, 8)
+    meet = Named(8)
+    slabs = slabs or [rng.randint(1, 4) for _ in range(chunks)]
+    first = [sum(slabs[:k]) for k in range(chunks)]
     t = lambda role: rng.expovariate(1.0) * speed[role]
-    full = lambda bar, use: ("wait", bar, use & 1, use + 1)
-    free = lambda bar, use: ("wait", bar, (use & 1) ^ 1, use)
+    full = lambda ring, i, lost: ("wait", ring[i % len(ring)], i // len(ring) & 1, i // len(ring) + 1, lost)
+    free = lambda ring, i, lost: ("wait", ring[i % len(ring)], (i // len(ring) & 1) ^ 1, i // len(ring), lost)
 
-    def row_warp():
-        lost = []   # filled when a wait gives up
-        for k in range(chunks):
-            if broken or not lost:
-                yield (*full(xfull[k & 1], k >> 1), lost)
-            if broken or not lost:
-                yield ("work", t("rows"))
-                yield ("hw_arrive", named[k & 1])
-            else:
-                yield ("hw_sync", named[k & 1])
+    def loader():
+        lost = []   # filled when a wait gives up: the role ends
+        for i in range(sum(slabs)):
+            yield free(freed, i, lost)
+            if lost:
+                return
+            yield ("async", t("load"), [(fulls[i % slots], 1)])
 
     def issuer():
-        yield ("async", t("load"), [(xfull[0], 1)])
-        yield ("async", t("load"), [(bfull, 1)])
-        if chunks > 1:
-            yield ("async", t("load"), [(xfull[1], 1)])
+        lost = []
         for k in range(chunks):
-            yield ("hw_sync", named[k & 1])
-            yield free(acc_free, k)
-            yield full(bfull, k)
-            yield ("work", t("mma") * 0.2)
-            yield ("async", t("mma"), [(mma, 1)])
-            if k + 1 < chunks:
-                yield full(mma, k)
-                yield ("async", t("load"), [(bfull, 1)])
-                if k + 2 < chunks:
-                    yield ("async", t("load"), [(xfull[k & 1], 1)])
+            for i in range(first[k], first[k] + slabs[k]):
+                yield full(ready, i, lost)
+                if lost:
+                    return
+                if i == first[k]:
+                    yield free(acc_free, k, [])   # (gives up, goes on)
+                yield ("work", t("mma") * 0.2)
+                last = i + 1 == first[k] + slabs[k]
+                yield ("async", t("mma"), [(freed[i % slots], 1)] + ([(accs[k % na], 1)] if last else []))
 
-    def state_warps():   # (eight warps that meet at hardware barriers of their own, in step)
+    def quantise(k, lost):
+        for i in range(first[k], first[k] + slabs[k]):
+            yield full(fulls, i, lost)
+            if lost:
+                return
+            yield ("work", t("rows"))
+            yield ("arrive", ready[i % slots], 1)
+
+    def row_warp():
+        lost = []
         for k in range(chunks):
-            yield ("work", t("state"))
-            yield full(mma, k)
-            yield ("work", t("state"))
-            yield ("arrive", acc_free, 8)
+            yield from quantise(k, lost)
+            if lost:
+                return
 
-    for i in range(3):
-        sim.spawn(f"row{i}", row_warp())
+    def state_warp(w):
+        lost = []
+        if few:
+            yield from quantise(0, lost)
+        for k in range(chunks):
+            if few and k + 1 < chunks and not lost:
+                yield from quantise(k + 1, lost)
+            yield ("work", t("state"))
+            if w == 0:
+                yield full(accs, k, [])
+            yield ("hw_sync", meet)
+            yield ("work", t("state"))
+            yield ("arrive", acc_free[k % na], 1)
+
+    sim.spawn("load", loader())
     sim.spawn("issue", issuer())
-    sim.spawn("state", state_warps())
+    for w in range(0 if few else rows):
+        sim.spawn(f"row{w}", row_warp())
+    for w in range(8):
+        sim.spawn(f"state{w}", state_warp(w))
 
 
 ROLES = ("load", "rows", "mma", "state")
 
 
+FORMS = [(True, 1), (True, 2), (False, 1), (False, 2)]
+
+
+@pytest.mark.parametrize("few,na", FORMS)
 @pytest.mark.parametrize("chunks", [1, 2, 3, 4, 5, 8, 33])
-def test_every_wait_is_sound_at_random_and_extreme_speeds(chunks):
+def test_every_wait_is_sound_at_random_and_extreme_speeds(chunks, few, na):
     for seed in range(24):
         sim = StateSim(seed)
         speed = {r: 10.0 ** sim.rng.uniform(-2, 2) for r in ROLES}
         if seed < len(ROLES):
             speed = {r: 100.0 if r == ROLES[seed] else 0.01 for r in ROLES}
-        build(sim, chunks, speed)
+        build(sim, chunks, speed, few, na, slabs=[4] * chunks if seed % 3 == 0 else None)
         sim.run()
 
 
@@ -178,23 +205,13 @@ SPEED = dict(load=1.0, rows=1.0, mma=0.3, state=1.0)
 
 
 @pytest.mark.parametrize("rest", [False, True])
-@pytest.mark.parametrize("chunks", [1, 2, 3, 5, 8])
-def test_every_role_ends_when_arrivals_go_missing(chunks, rest):
+@pytest.mark.parametrize("few,na", FORMS)
+@pytest.mark.parametrize("chunks", [1, 2, 3, 5])
+def test_every_role_ends_when_arrivals_go_missing(chunks, few, na, rest):
     gave_up = 0
-    for drop in range(1, 4 * chunks):
-        for seed in range(4):
-            sim = LossySim(seed, drop, rest)
-            build(sim, chunks, SPEED)
-            assert sim.run(), (drop, seed)
-            gave_up += sim.gave_up
+    for drop in range(1, 6 * chunks):
+        sim = LossySim(drop, drop, rest)
+        build(sim, chunks, SPEED, few, na)
+        assert sim.run(), drop
+        gave_up += sim.gave_up
     assert gave_up > 0
-
-
-def test_row_warps_that_go_on_would_not_let_them():
-    # the row warps give up one wait per chunk, the issuing warp two: they overrun the barrier
-    stuck = 0
-    for drop in range(1, 20):
-        sim = LossySim(drop, drop, rest=True)
-        build(sim, 8, SPEED, broken=True)
-        stuck += not sim.run()
-    assert stuck > 0
