@@ -164,37 +164,55 @@ __device__ __forceinline__ int sx8(uint32_t w, int k) { return (int)(int8_t)((w 
 // binary32 result is defined bit for bit: v = (double)fadd(dt_raw, bias); u = exp(-|v|) by Cody-Waite
 // reduction and a degree-13 Taylor polynomial; log(1 + u) = 2 atanh(u / (2 + u)) by its odd series up
 // to the 27th power; dt = (float)(max(v, 0) + log(1 + u)).
-__device__ __forceinline__ float softplus_dt(float dt_raw, float bias) {
-  const double v = (double)__fadd_rn(dt_raw, bias);
-  const double a = fabs(v);
-  double u = 0.0;
-  if (a <= 700.0) {
-    const double LOG2E = 0x1.71547652b82fep+0, LN2_HI = 0x1.62e42fee00000p-1, LN2_LO = 0x1.a39ef35793c76p-33;
-    const double n = rint(__dmul_rn(-a, LOG2E));
-    double r = __fma_rn(n, -LN2_HI, -a);
-    r = __fma_rn(n, -LN2_LO, r);
-    double p = 1.0 / 6227020800.0;
-    p = __fma_rn(p, r, 1.0 / 479001600.0);
-    p = __fma_rn(p, r, 1.0 / 39916800.0);
-    p = __fma_rn(p, r, 1.0 / 3628800.0);
-    p = __fma_rn(p, r, 1.0 / 362880.0);
-    p = __fma_rn(p, r, 1.0 / 40320.0);
-    p = __fma_rn(p, r, 1.0 / 5040.0);
-    p = __fma_rn(p, r, 1.0 / 720.0);
-    p = __fma_rn(p, r, 1.0 / 120.0);
-    p = __fma_rn(p, r, 1.0 / 24.0);
-    p = __fma_rn(p, r, 1.0 / 6.0);
-    p = __fma_rn(p, r, 0.5);
-    p = __fma_rn(p, r, 1.0);
-    p = __fma_rn(p, r, 1.0);
-    u = __longlong_as_double(__double_as_longlong(p) + ((long long)__double2int_rn(n) << 52));
-  }
-  const double s = __ddiv_rn(u, __dadd_rn(2.0, u)), z = __dmul_rn(s, s);
-  double q = 1.0 / 27.0;
+// W values side by side, step by step: each binary64 operation waits for the one before it, and a coefficient is two moves (one
+// value after the other takes 120 instructions each, 43 of them binary64; prefill of 256 tokens x 24 heads 23.85 us, two side by
+// side 23.25, four 22.7, all eight of a lane 22.55; 5 x 1792 x 80 122.9 and 121.7).
+template <int W>
+__device__ __forceinline__ void softplus_dt(const float* dt_raw, float bias, float* dt) {
+  const double LOG2E = 0x1.71547652b82fep+0, LN2_HI = 0x1.62e42fee00000p-1, LN2_LO = 0x1.a39ef35793c76p-33;
+  const double kExp[14] = {1.0 / 6227020800.0, 1.0 / 479001600.0, 1.0 / 39916800.0, 1.0 / 3628800.0, 1.0 / 362880.0,
+                           1.0 / 40320.0,      1.0 / 5040.0,      1.0 / 720.0,      1.0 / 120.0,     1.0 / 24.0,
+                           1.0 / 6.0,          0.5,               1.0,              1.0};
+  double v[W], r[W], p[W], s[W];
+  int n[W];
 #pragma unroll
-  for (int k = 12; k >= 0; --k) q = __fma_rn(q, z, 1.0 / (double)(2 * k + 1));
-  const double lp = __dmul_rn(__dmul_rn(2.0, s), q);
-  return (float)__dadd_rn(v > 0.0 ? v : 0.0, lp);
+  for (int i = 0; i < W; ++i) {
+    v[i] = (double)__fadd_rn(dt_raw[i], bias);
+    const double a = fabs(v[i]) <= 700.0 ? fabs(v[i]) : 0.0;   // (beyond, u is 0: below)
+    const double nd = rint(__dmul_rn(-a, LOG2E));
+    n[i] = __double2int_rn(nd);
+    r[i] = __fma_rn(nd, -LN2_HI, -a);
+    r[i] = __fma_rn(nd, -LN2_LO, r[i]);
+    p[i] = kExp[0];
+  }
+#pragma unroll
+  for (int k = 1; k < 14; ++k) {
+#pragma unroll
+    for (int i = 0; i < W; ++i) p[i] = __fma_rn(p[i], r[i], kExp[k]);
+  }
+#pragma unroll
+  for (int i = 0; i < W; ++i) {
+    const double e = __longlong_as_double(__double_as_longlong(p[i]) + ((long long)n[i] << 52));
+    const double u = fabs(v[i]) <= 700.0 ? e : 0.0;
+    s[i] = __ddiv_rn(u, __dadd_rn(2.0, u));
+    r[i] = __dmul_rn(s[i], s[i]);
+    p[i] = 1.0 / 27.0;
+  }
+#pragma unroll
+  for (int k = 12; k >= 0; --k) {
+#pragma unroll
+    for (int i = 0; i < W; ++i) p[i] = __fma_rn(p[i], r[i], 1.0 / (double)(2 * k + 1));
+  }
+#pragma unroll
+  for (int i = 0; i < W; ++i) {
+    const double lp = __dmul_rn(__dmul_rn(2.0, s[i]), p[i]);
+    dt[i] = (float)__dadd_rn(v[i] > 0.0 ? v[i] : 0.0, lp);
+  }
+}
+__device__ __forceinline__ float softplus_dt(float dt_raw, float bias) {
+  float dt;
+  softplus_dt<1>(&dt_raw, bias, &dt);
+  return dt;
 }
 
 // step size of a channel from the bits of its largest magnitude (Eq. 1; an all-zero channel gets 1)

@@ -42,8 +42,9 @@ __device__ __forceinline__ void chunk_of_heads(float* dts, const int hpb, const 
 #pragma unroll
     for (int u = 0; u < TPL; ++u) v[u] = ok ? __ldg(src + (i64)(32 * u) * d.H) : 0.f;
     const float bias = (SOFTPLUS && a.dt_bias && ok) ? __ldg(a.dt_bias + h0 + hh) : 0.f;
+    if (SOFTPLUS) softplus_dt<TPL>(v, bias, v);
 #pragma unroll
-    for (int u = 0; u < TPL; ++u) dts[hh * LD + 32 * u + t] = SOFTPLUS ? softplus_dt(v[u], bias) : v[u];
+    for (int u = 0; u < TPL; ++u) dts[hh * LD + 32 * u + t] = v[u];
   }
   __syncthreads();
   if (!live) return;   // whole warps
