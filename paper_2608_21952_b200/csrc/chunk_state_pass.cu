@@ -125,9 +125,9 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
 
   // LUT_state of a chunk: tpl consecutive tokens per lane, 32 / nsl lanes per slab
   struct Lut { float4 a, b; };
-  auto lut_of_lane = [&](int k) -> Lut {
+  auto lut_of_lane = [&](int place) -> Lut {
     Lut v = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-    const float* l = reinterpret_cast<const float*>(smem + G::OFF_CHUNK) + (k % kLutAhead) * 256 + lane * tpl;
+    const float* l = reinterpret_cast<const float*>(smem + G::OFF_CHUNK) + place * 256 + lane * tpl;
     if (tpl == 2) {
       const float2 u = *reinterpret_cast<const float2*>(l);
       v.a.x = u.x;
@@ -211,21 +211,38 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
 
   if (warp == kLoadWarp) {
     // ------------------------------------------------------------ loads, as many slabs ahead as the ring has places.  This warp
-    // forms the bound itself and does not wait for the others' set-up; the last slab of the first chunk, the likeliest to
-    // live, is under way before its LUT_state is known.
+    // forms the bound itself and does not wait for the others' set-up.  Where LUT_state of the first chunk is not known yet: FEW
+    // takes all slabs of that chunk (the start of the chain is what counts: 256 tokens x 24 heads 22.55 -> 22.35 us, 3 x 2048 x 80 96.5 -> 95.6), the others only the last one, the likeliest to live.
+    const float sx0 = a.s_x[h * P + lane], sx1 = a.s_x[h * P + 32 + lane], xs0 = step_xs(lane), xs1 = step_xs(32 + lane);
+    constexpr int kFirst = FEW ? 1 : 0;   // chunk from which on only live slabs are taken
     auto fetch_lut = [&](int k) {
       if (k < d.c && elect_one()) {
-        mbar_expect_tx(&bars[B_LUT + k % kLutAhead], (uint32_t)(Q * 4));
-        bulk_load(smem + G::OFF_CHUNK + (k % kLutAhead) * 1024, a.pack + ((unit0 + k) * kPackRows + PACK_LUT) * Q, (uint32_t)(Q * 4),
-                  &bars[B_LUT + k % kLutAhead]);
+        uint64_t* const bar = &bars[B_LUT + (k - kFirst) % kLutAhead];
+        mbar_expect_tx(bar, (uint32_t)(Q * 4));
+        bulk_load(smem + G::OFF_CHUNK + (k - kFirst) % kLutAhead * 1024, a.pack + ((unit0 + k) * kPackRows + PACK_LUT) * Q,
+                  (uint32_t)(Q * 4), bar);
       }
       __syncwarp();
     };
-    const float sx0 = a.s_x[h * P + lane], sx1 = a.s_x[h * P + 32 + lane], xs0 = step_xs(lane), xs1 = step_xs(32 + lane);
-    fetch_lut(0);
-    if (elect_one()) copy(0, 0, nsl - 1);
-    __syncwarp();
-    for (int k = 1; k < kLutAhead; ++k) fetch_lut(k);
+    Pos at;
+    if (FEW) {
+#pragma unroll 1
+      for (int sl = nsl - 1; sl >= 0; --sl, at.next()) {
+        if (elect_one()) {
+          info[at.slot] = (sl == 0 ? SLAB_LAST : 0) | (sl << 8);
+          mbar_expect_tx(&bars[B_FULL + at.slot], kSlab * 64 + kSlab * NS + kSlab * 4);
+          copy(at.slot, 0, sl);
+          bulk_load(smem + OFF_LUT + at.slot * (kSlab * 4), a.pack + (unit0 * kPackRows + PACK_LUT) * Q + kSlab * sl, kSlab * 4,
+                    &bars[B_FULL + at.slot]);
+        }
+        __syncwarp();
+      }
+    } else {
+      fetch_lut(0);
+      if (elect_one()) copy(0, 0, nsl - 1);
+      __syncwarp();
+    }
+    for (int k = FEW ? kFirst : 1; k < kFirst + kLutAhead; ++k) fetch_lut(k);
     const float bound = row_bound(__fdiv_rn(sx0, xs0), __fdiv_rn(sx1, xs1));
     auto live_slabs = [&](const Lut& v) -> uint32_t {
       if (TAPS) return (1u << nsl) - 1u;
@@ -235,17 +252,17 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
       const int lps = 32 / nsl;
       return __ballot_sync(0xffffffffu, lane < nsl && ((bal >> ((lane * lps) & 31)) & ((1u << lps) - 1u)) != 0);
     };
-    Pos at;
     bool on = true;
 #pragma unroll 1
-    for (int k = 0; k < d.c; ++k) {
-      on = __all_sync(0xffffffffu, mbar_wait_inline<0>(&bars[B_LUT + k % kLutAhead], (k / kLutAhead) & 1, a.status));
+    for (int k = kFirst; k < d.c; ++k) {
+      const int i = k - kFirst;
+      on = __all_sync(0xffffffffu, mbar_wait_inline<0>(&bars[B_LUT + i % kLutAhead], (i / kLutAhead) & 1, a.status));
       if (!on) break;
-      const Lut v = lut_of_lane(k);
+      const Lut v = lut_of_lane(i % kLutAhead);
       uint32_t m = live_slabs(v);
       const uint32_t top = 1u << (nsl - 1);
-      if (k == 0 || m == 0) m |= top;
-      bool issued = k == 0;                         // (slab `top` then comes first)
+      if ((!FEW && k == 0) || m == 0) m |= top;
+      bool issued = !FEW && k == 0;                 // (slab `top` then comes first)
 #pragma unroll 1
       while (m) {
         const int sl = issued ? nsl - 1 : __ffs((int)m) - 1;
@@ -551,16 +568,16 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
   if (sms == 0) return SSDI8_ERR_CUDA;
   const int units = d.H * d.b, slots = 3 * sms;
   // Whole heads wherever the device is filled; a remainder of less than an eighth of a wave goes in slices of 32 columns, whose
-  // chain per chunk is shorter.  Few units go in slices of 64, the longest chains of them in 32 (Algorithm 2, us, whole / slices
-  // of 64 / of 32): N 128: 512 tokens x 24 heads 18.9 / 18.1 / 19.9, 1024 x 32 22.2 / 21.1 / 20.9, 1024 x 96 34.6 / 33.7 / 37.2, 3 x 512 x 12
-  // 22.1 / 20.6 / 23.3, 256 x 64 23.2 / 22.8 / 22.5, 2048 x 80 48.7 / 48.1 / 54.7, 2 x 8192 x 8 (INT8 states) 78.3 / 68.0 / 64.6; but 4096 x
-  // 100 even, 512 x 60 22.1 / 22.4 / 22.6, 2 x 2048 x 128 98.9 / 108 / 118.  N 64, from four chunks on: 768 x 60 28.7 / - / 27.9, 256 x 32 (chunks
-  // of 64) 16.4 / - / 15.6, 2048 x 60 44.9 / - / 44.6, but 256 x 36 (chunks of 128) 16.4 / - / 18.1.
+  // chain per chunk is shorter.  Few units of some chunks go in slices of 64, the longest chains of them in 32 (graphs of layer calls,
+  // us, whole / slices of 64 / of 32): N 128: 1024 tokens x 32 heads 22.0 / 20.7 / 21.6, 1024 x 96 32.8 / 32.2 / 36.1, 3 x 512 x 12 (chunks of
+  // 128) 19.4 / 19.0 / 20.9, 128 x 12 (of 64) 13.6 / 12.9 / 12.8, 2048 x 80 46.8 / 45.5 / 54.7, 2 x 8192 x 8 (INT8 states) 74.7 / 66.6 / 63.1; but
+  // 256 x 64 17.7 / 18.5 / 20.1, 128 x 64 (of 128) 14.2 / 15.7 / 16.5, 192 x 80 (of 64) 18.0 / 18.7 / 19.6, 3 x 2048 x 80 92 / 101 / 112.  N 64, from
+  // four chunks on: 768 x 60 28.7 / - / 27.9, 256 x 32 (of 64) 16.4 / - / 15.6, 2048 x 60 44.9 / - / 44.6, but 256 x 36 (of 128) 16.4 / - / 18.1.
   int n_full = units / slots * slots, slice = 32;
   const int last = units - n_full;
   if (n_full > 0) {
     if (8 * last > slots) n_full = units;
-  } else if (d.N == 128 && 3 * units <= 2 * sms) {
+  } else if (d.N == 128 && (d.c >= 4 ? 3 * units <= 2 * sms : d.c >= 2 && 4 * units <= sms)) {
     slice = d.c >= 12 && 4 * units <= sms ? 32 : 64;
   } else if (!(d.N == 64 && d.c >= 4 && 2 * units <= sms)) {
     n_full = units;
