@@ -242,6 +242,138 @@ __global__ void __launch_bounds__(QT) absmax_inner(const float4* __restrict__ in
   }
 }
 
+// ---- calibrate mode in one launch: a cluster of eight CTAs holds all rows of a column block (I == 1: 8 float4 wide) or of a channel
+// (I % 4 == 0) in shared memory, its CTAs exchange their largest magnitudes, and the codes are formed from shared memory: a tensor is read
+// once, in one launch instead of three (clear, absmax, codes).  It pays where the whole grid is resident at once and no CTA has much to
+// hold; otherwise the three launches, which overlap, use the memory better.  ssdi8_quantize_act, us, three launches / one: 4096 rows
+// x 512 channels 12.6 / 7.4, 4096 x 1024 13.9 / 8.0, 512 x 512 7.2 / 4.2, 12800 x 512 25.2 / 19.2, but 12800 x 1024 25.2 / 30.4, 4096 x 5120 27.5 / 28.9,
+// 8192 x 5120 55 / 84; channels of 128 elements: 256 rows x 1 7.6 / 3.3, 1024 x 1 7.2 / 5.1, 1024 x 8 9.2 / 6.4, 1024 x 32 12.6 / 7.9, but 2048 x 1
+// 7.4 / 8.7, 4096 x 1 9.1 / 14.4.
+constexpr int kCluster = 8, kHeldRows = 1600;   // CTAs; rows of a column block that one of them holds at most (200 KB)
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float remote_float(const float* own, int rank) {   // that of another CTA of the cluster
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(own);
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %0, %1;" : "+r"(a) : "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(QT)
+calibrate_ch_fastest(const float4* __restrict__ in, float* __restrict__ scale, uint32_t* __restrict__ out, i64 R, int ch4, int rows) {
+  extern __shared__ __align__(16) float4 tile[];   // [rows][8]; a thread reads what it has copied itself
+  __shared__ float part[QT / 32][32], mine[32], step[32];
+  pdl_launch_dependents();
+  pdl_wait();
+  const int tid = threadIdx.x, j = tid & 7, rank = blockIdx.x;   // (the grid is one cluster wide)
+  const int q = blockIdx.y * 8 + j;
+  const i64 r0 = (i64)rank * rows;
+  const int n = (int)(q >= ch4 || r0 >= R ? 0 : R - r0 < rows ? R - r0 : rows);
+  const float4* src = in + r0 * ch4 + q;
+  for (int r = tid >> 3; r < n; r += QT / 8) copy16(tile + r * 8 + j, src + (i64)r * ch4);
+  copies_done();
+  float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int r = tid >> 3; r < n; r += QT / 8) {
+    const float4 v = tile[r * 8 + j];
+    m.x = fmaxf(m.x, fabsf(v.x)); m.y = fmaxf(m.y, fabsf(v.y));
+    m.z = fmaxf(m.z, fabsf(v.z)); m.w = fmaxf(m.w, fabsf(v.w));
+  }
+#pragma unroll
+  for (int o = 8; o < 32; o <<= 1) {
+    m.x = fmaxf(m.x, __shfl_xor_sync(0xffffffffu, m.x, o)); m.y = fmaxf(m.y, __shfl_xor_sync(0xffffffffu, m.y, o));
+    m.z = fmaxf(m.z, __shfl_xor_sync(0xffffffffu, m.z, o)); m.w = fmaxf(m.w, __shfl_xor_sync(0xffffffffu, m.w, o));
+  }
+  if ((tid & 31) < 8) *reinterpret_cast<float4*>(&part[tid >> 5][4 * j]) = m;
+  __syncthreads();
+  if (tid < 32) {
+    float a = part[0][tid];
+#pragma unroll
+    for (int w = 1; w < QT / 32; ++w) a = fmaxf(a, part[w][tid]);
+    mine[tid] = a;
+  }
+  cluster_sync();
+  if (tid < 32) {
+    float a = 0.f;
+#pragma unroll
+    for (int c = 0; c < kCluster; ++c) a = fmaxf(a, remote_float(&mine[tid], c));
+    const float al = step_of_max(__float_as_uint(a));
+    step[tid] = al;
+    if (rank == 0 && blockIdx.y * 32 + tid < ch4 * 4) scale[blockIdx.y * 32 + tid] = al;
+  }
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");   // (this CTA has read the others' maxima)
+  const float4 a4 = *reinterpret_cast<const float4*>(&step[4 * j]);
+  const Step4 st = step4(a4);
+  uint32_t* dst = out + r0 * ch4 + q;
+  for (int r = tid >> 3; r < n; r += QT / 8)
+    __stcs(dst + (i64)r * ch4, st.usable ? code4(tile[r * 8 + j], st) : code4_by_division(tile[r * 8 + j], a4));
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
+
+constexpr int kInnerThreads = 1024, kInnerHeld = 8;   // threads of a CTA, float4 of each at most
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kInnerThreads)
+calibrate_inner(const float4* __restrict__ in, float* __restrict__ scale, uint32_t* __restrict__ out, int R, int Ch, int I4, int rows) {
+  extern __shared__ __align__(16) float4 tile[];   // [<= kInnerHeld][kInnerThreads]; a thread reads what it has copied itself
+  __shared__ float part[kInnerThreads / 32], mine, step;
+  pdl_launch_dependents();
+  pdl_wait();
+  const int tid = threadIdx.x, rank = blockIdx.x, ch = blockIdx.y;
+  const int r0 = rank * rows, r1 = min(R, r0 + rows);
+  // element tid + u kInnerThreads of the CTA's rows of this channel is float4 i of row r
+  const int dr = kInnerThreads / I4, di = kInnerThreads % I4;
+  auto walk = [&](auto&& f) {
+    int r = r0 + tid / I4, i = tid % I4;
+    for (int u = 0; r < r1; ++u) {
+      f(u, ((i64)r * Ch + ch) * I4 + i);
+      r += dr;
+      i += di;
+      if (i >= I4) {
+        i -= I4;
+        ++r;
+      }
+    }
+  };
+  walk([&](int u, i64 e) { copy16(tile + u * kInnerThreads + tid, in + e); });
+  copies_done();
+  float m = 0.f;
+  walk([&](int u, i64) {
+    const float4 v = tile[u * kInnerThreads + tid];
+    m = fmaxf(fmaxf(fmaxf(m, fabsf(v.x)), fmaxf(fabsf(v.y), fabsf(v.z))), fabsf(v.w));
+  });
+  auto largest = [](float v) { return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v))); };   // v >= 0
+  m = largest(m);
+  if ((tid & 31) == 0) part[tid >> 5] = m;
+  __syncthreads();
+  if (tid < 32) {
+    m = largest(part[tid]);
+    if (tid == 0) mine = m;
+  }
+  cluster_sync();
+  if (tid < 32) {
+    m = largest(tid < kCluster ? remote_float(&mine, tid) : 0.f);
+    if (tid == 0) {
+      step = step_of_max(__float_as_uint(m));
+      if (rank == 0) scale[ch] = step;
+    }
+  }
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
+  const float al = step;
+  const float4 a4 = make_float4(al, al, al, al);
+  const Step4 st = step4(a4);
+  walk([&](int u, i64 e) {
+    const float4 v = tile[u * kInnerThreads + tid];
+    out[e] = st.usable ? code4(v, st) : code4_by_division(v, a4);
+  });
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
+
 }  // namespace
 
 ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* scale, int mode,
@@ -250,6 +382,21 @@ ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* sca
   if (n4 == 0) return SSDI8_OK;
   uint32_t* bits = reinterpret_cast<uint32_t*>(scale);
   ssdi8_status_t ls;
+  if (mode == 1) {
+    const int sms = sm_count();
+    if (sms == 0) return SSDI8_ERR_CUDA;
+    const i64 rows = (R + kCluster - 1) / kCluster, held = (rows * (I / 4) + kInnerThreads - 1) / kInnerThreads;
+    const i64 per_sm = rows <= kHeldRows ? (224 * 1024) / (rows * 128 + 4 * 1024) : 0;
+    if (I == 1 && 10 * (Ch / 4) <= 9 * sms * (per_sm < 4 ? per_sm : 4)) {
+      const int ch4 = (int)(Ch / 4);
+      return launch_sized(calibrate_ch_fastest, dim3(kCluster, (unsigned)((ch4 + 7) / 8)), dim3(QT), (size_t)rows * 128, (size_t)kHeldRows * 128,
+                          -1, false, st, reinterpret_cast<const float4*>(in), scale, reinterpret_cast<uint32_t*>(out), R, ch4, (int)rows);
+    }
+    if (I > 1 && (held <= 4 ? kCluster * Ch <= 2 * sms : held <= kInnerHeld && Ch >= 4 && kCluster * Ch <= sms))
+      return launch_sized(calibrate_inner, dim3(kCluster, (unsigned)Ch), dim3(kInnerThreads), (size_t)held * kInnerThreads * 16,
+                          (size_t)kInnerHeld * kInnerThreads * 16, -1, false, st, reinterpret_cast<const float4*>(in), scale,
+                          reinterpret_cast<uint32_t*>(out), (int)R, (int)Ch, (int)(I / 4), (int)rows);
+  }
   if (mode == 1 || mode == 2) {
     if (mode == 1 && (ls = launch_clear_words(scale, Ch, st)) != SSDI8_OK) return ls;
     if (I == 1) {

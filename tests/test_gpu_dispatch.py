@@ -93,6 +93,54 @@ def test_quantiser_gives_all_zero_channels_a_step_of_one(R, Ch, I):
     assert np.array_equal(q.reshape(-1), np.asarray(qr).reshape(-1))
 
 
+@pytest.mark.parametrize("R,Ch,I", [(1, 4, 1), (7, 36, 1), (9, 32, 1), (255, 1776, 1), (12800, 512, 1), (12801, 512, 1), (4100, 1028, 1), (300, 2400, 1),
+                                    (1, 1, 64), (13, 3, 4), (5, 7, 12), (257, 37, 128), (258, 38, 128), (1023, 1, 128), (1025, 1, 128),
+                                    (2047, 4, 128), (2049, 4, 128), (2048, 18, 64), (2048, 19, 64), (8, 2, 4096)])
+def test_calibrating_quantiser_in_one_launch_and_in_three(R, Ch, I):
+    # On either side of the lines of the dispatch; rows and columns that leave CTAs of a cluster, or threads, without any; the
+    # largest value of a channel anywhere; a channel of zeros
+    import gpu_harness as gh
+    v = np.random.default_rng(R + Ch).standard_normal((R, Ch, I)).astype(np.float32)
+    v[np.arange(Ch) * 7 % R, np.arange(Ch), np.arange(Ch) * 5 % I] = -(6.0 + np.arange(Ch, dtype=np.float32))
+    v[:, Ch // 2] = 0.0
+    q, s = gh.gpu_quantize(v, R, Ch, I)
+    qr, sr = orc.quantize(v, R, Ch, I, mode=1)
+    assert np.array_equal(s, sr)
+    assert np.array_equal(q.reshape(-1), np.asarray(qr).reshape(-1))
+
+
+@pytest.mark.parametrize("b,c,H,Q", [(1, 1, 1, 64), (2, 3, 9, 128), (1, 3, 17, 256)])
+@pytest.mark.parametrize("regime", ["fast", "slow", "codes", "mixed"])
+def test_calibration_skips_no_token_that_counts(b, c, H, Q, regime):
+    # Which tokens can raise the largest |X_scaled| is decided by LUT_state: steep and nearly flat decay, codes that make a
+    # channel's largest product sit on an early token, time steps of both signs and of zero
+    import torch
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("xs", b, c * Q, H, 64, 64, 1, Q, 0.02, 20.0, 61)
+    t = inputs.make_prefill(cfg)
+    t["A"] *= np.float32({"fast": 60.0, "slow": 0.001}.get(regime, 1.0))
+    q = orc.prepare_quantized(cfg, t, None)
+    if regime == "mixed":
+        q["dt"] = q["dt"].copy()
+        q["dt"].reshape(b, c * Q, H)[:, ::3] *= -1.0
+        q["dt"].reshape(b, c * Q, H)[:, 1::5] = 0.0
+    if regime == "codes":
+        x = (np.abs(np.arange(b * c * Q * H * 64)) % 3).astype(np.int8).reshape(b, c * Q, H, 64)
+        x[:, np.random.default_rng(1).integers(0, c * Q, 12)] = 127
+        x[:, -1] = 0
+        x[..., 5] = 0
+        q["xq"] = x.reshape(np.asarray(q["xq"]).shape)
+    want = orc.calibrate(cfg, q["xq"], q["Bq"], q["Cq"], q["s_x"], q["s_B"], q["s_C"], q["dt"], q["A"], None)
+    dims = bd.dims_of(cfg)
+    dv = {k: gh.dev(q[k]) for k in ("xq", "Bq", "Cq", "s_x", "s_B", "s_C", "dt", "A")}
+    s = [torch.full((n,), float("nan"), device="cuda") for n in (H * 64, 1, H * 64)]
+    bd.ssdi8_calibrate(dims, bd.make_fwd_args(**dv), *s, bd.alloc_workspace(dims))
+    torch.cuda.synchronize()
+    for got, ref in zip(s, want[:3]):
+        assert np.array_equal(got.cpu().numpy(), np.asarray(ref).reshape(-1))
+
+
 @pytest.mark.parametrize("R,Ch", [(R, Ch) for R in (1, 3, 15, 17, 31, 33, 63, 2051) for Ch in (4, 508, 516)] + [(227, 113664), (227, 113668)])
 def test_absmax_takes_every_row_into_account(R, Ch):
     # The largest value of each channel in a row of its own: remainders of the rows in flight, the row groups and the blocks
