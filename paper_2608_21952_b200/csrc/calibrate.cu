@@ -5,79 +5,104 @@
 namespace ssdi8 {
 namespace {
 
-// absmax_xs[h,p] = max over tokens of |fmul(fmul(float(xq), s_x), LUT_state)| (Eq. 3), as binary32 bits.  Streaming
-// over xq: a block takes 8 neighbouring heads (512 contiguous bytes of a token) and 64 tokens; a
-// thread owns 16 channels and keeps their maxima in registers, the 8 token rows of the block meet in shared
-// memory, and one atomic per channel and block leaves it.  (The ChunkState kernel did this with 16 atomics per
-// thread, all CTAs of a head on its 64 channels: 103 us at batch 2 x 2048 x 80 heads against 10.  64 tokens per
-// block instead of half a chunk: 2 us more.)
-constexpr int kXsHeads = 8, kXsTokens = 64;
-__global__ void __launch_bounds__(256) absmax_xs_kernel(const int8_t* __restrict__ xq, const float* __restrict__ s_x,
-                                                        const float* __restrict__ pack, uint32_t* __restrict__ absmax, Dims d) {
-  __shared__ __align__(16) float lut[kXsHeads][kXsTokens];
+// absmax_xs[h,p] = max over tokens of |fmul(fmul(float(xq), s_x), LUT_state)| (Eq. 3), as binary32 bits.  A block takes a
+// chunk of 8 neighbouring heads (512 contiguous bytes of a token), 32 tokens at a time from the last one on; a thread owns
+// 16 channels of four of the tokens and keeps their maxima in registers, and after a round that had anything to do the
+// token rows of the block meet in shared memory.  LUT_state decays towards the start of a chunk, so a few rounds decide the
+// maxima: a token whose 16 products cannot exceed them, |LUT_state| <= min over the channels of max / (128 |s_x|) (fmul is
+// monotone, 128 s_x is exact; a slack of 1e-5 covers the quotient), is neither loaded nor multiplied.  One atomic per channel
+// and block leaves it, if it raises what is there.  (Every token multiplied, 64 to a block,
+// calibration calls: 2 x 2048 x 80 heads 80.5 -> 78.6 us, 4 x 1024 x 128 (G 8) 125.1 -> 117.9, 12 x 512 x 64 91.1 -> 87.8, 16384 x 32 153.8 -> 145.3;
+// blocks of 512 threads 79.1, 120.1, 91.5, 151.2.)
+constexpr int kXsHeads = 8, kXsThreads = 256, kXsRows = kXsThreads / 32, kXsTokens = 4 * kXsRows;
+__global__ void __launch_bounds__(kXsThreads) absmax_xs_kernel(const int8_t* __restrict__ xq, const float* __restrict__ s_x, const float* pack,
+                                                        uint32_t* absmax, Dims d) {
+  extern __shared__ __align__(16) float lut[];    // [kXsHeads][Q]
   __shared__ __align__(16) float sxs[kXsHeads * 64];
-  __shared__ uint32_t best[8][kXsHeads * 64];
+  __shared__ uint32_t best[16][32];               // channel e of (head, 16 channels) = lane
   pdl_wait();
   pdl_launch_dependents();   // (after the wait: ChunkBMM, launched next, does not wait for this kernel)
-  const int tid = threadIdx.x;
-  // (head blocks and token blocks in one grid dimension: a sequence of more than 4 M tokens has more than 65535 of the latter)
-  const int nhb = (d.H + kXsHeads - 1) / kXsHeads, tb = blockIdx.x / nhb, b = blockIdx.z;
-  const int h0 = (blockIdx.x - tb * nhb) * kXsHeads, k = tb / (d.Q / kXsTokens);
-  constexpr int nt = kXsTokens;
-  const int i0 = (tb % (d.Q / kXsTokens)) * nt;   // tokens of this block
-  for (int e = tid; e < kXsHeads * nt; e += 256) {
-    const int hh = e / nt, i = e % nt;
-    if (h0 + hh < d.H) lut[hh][i] = __ldg(pack + ((((i64)b * d.H + h0 + hh) * d.c + k) * kPackRows + PACK_LUT) * d.Q + i0 + i);
+  const int tid = threadIdx.x, lane = tid & 31;
+  // (head blocks and chunks in one grid dimension: a sequence of more than 4 M tokens has more than 65535 of the latter)
+  const int nhb = (d.H + kXsHeads - 1) / kXsHeads, k = blockIdx.x / nhb, b = blockIdx.z;
+  const int h0 = (blockIdx.x - k * nhb) * kXsHeads;
+  const int hh = (tid >> 2) & 7, c = tid & 3, row = tid >> 5;   // head, 16 channels, token row of the thread
+  const int h = h0 + hh;
+  const bool live = h < d.H;
+  const uint4* src = reinterpret_cast<const uint4*>(xq + (((i64)b * d.L + (i64)k * d.Q + row) * d.H + h) * 64) + c;
+  const i64 stride = (i64)kXsRows * d.H * 4;   // kXsRows tokens, in 16-byte words
+  uint4 w[4];                                  // (the first round's before LUT_state is there)
+#pragma unroll
+  for (int u = 0; u < 4; ++u) w[u] = live ? __ldg(src + ((d.Q - kXsTokens) / kXsRows + u) * stride) : make_uint4(0u, 0u, 0u, 0u);
+  const int lq = 31 - __clz(d.Q) - 2;          // LUT_state, 16 bytes at a time
+  for (int e = tid; e < (kXsHeads << lq); e += kXsThreads) {
+    const int hl = e >> lq, i = (e - (hl << lq)) * 4;
+    if (h0 + hl < d.H)
+      *reinterpret_cast<float4*>(lut + hl * d.Q + i) =
+          *reinterpret_cast<const float4*>(pack + ((((i64)b * d.H + h0 + hl) * d.c + k) * kPackRows + PACK_LUT) * d.Q + i);
   }
   // (by way of shared memory: ssdi8_calibrate asks for no alignment of s_x beyond a float's, and sixteen loads of one float per
   // thread were 4 us slower)
-  for (int e = tid; e < kXsHeads * 64; e += 256)
-    if (h0 + (e >> 6) < d.H) sxs[e] = __ldg(s_x + h0 * 64 + e);
-  const int hh = (tid >> 2) & 7, c = tid & 3, row = tid >> 5;   // head, 16 channels, token row of the thread
-  const int h = h0 + hh;
+  for (int e = tid; e < kXsHeads * 64; e += kXsThreads) {
+    sxs[e] = h0 + (e >> 6) < d.H ? __ldg(s_x + h0 * 64 + e) : 0.f;
+    best[e >> 5][e & 31] = 0u;
+  }
   float mx[16];
 #pragma unroll
   for (int e = 0; e < 16; ++e) mx[e] = 0.f;
   __syncthreads();
-  if (h < d.H) {
-    float2 sx[8];
+  float2 sx[8];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float4 v = *(reinterpret_cast<const float4*>(&sxs[hh * 64 + c * 16]) + e);
-      sx[2 * e] = make_float2(v.x, v.y);
-      sx[2 * e + 1] = make_float2(v.z, v.w);
-    }
-    const uint4* src = reinterpret_cast<const uint4*>(xq + (((i64)b * d.L + (i64)k * d.Q + i0 + row) * d.H + h) * 64) + c;
-    const i64 stride = (i64)8 * d.H * 4;   // 8 tokens, in 16-byte words
+  for (int e = 0; e < 4; ++e) {
+    const float4 v = *(reinterpret_cast<const float4*>(&sxs[hh * 64 + c * 16]) + e);
+    sx[2 * e] = make_float2(v.x, v.y);
+    sx[2 * e + 1] = make_float2(v.z, v.w);
+  }
+  float least = 0.f;                     // |LUT_state| up to here changes nothing
 #pragma unroll 1
-    for (int i = 0; i < nt; i += 32) {     // (four tokens per round and thread)
-      uint4 w[4];
+  for (int i0 = d.Q - kXsTokens; i0 >= 0; i0 -= kXsTokens) {
+    float l[4];
+    bool any = false;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) w[u] = __ldg(src + (i / 8 + u) * stride);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float l = lut[hh][i + 8 * u + row];
-        const float2 l2 = make_float2(l, l);
-        const uint32_t ww[4] = {w[u].x ^ 0x80808080u, w[u].y ^ 0x80808080u, w[u].z ^ 0x80808080u, w[u].w ^ 0x80808080u};
-#pragma unroll
-        for (int e = 0; e < 16; e += 2) {
-          const float2 xf = make_float2(s8_to_f32(ww[e >> 2], e & 3), s8_to_f32(ww[e >> 2], (e & 3) + 1));
-          const float2 v = __fmul2_rn(__fmul2_rn(xf, sx[e >> 1]), l2);
-          mx[e] = fmaxf(mx[e], fabsf(v.x));
-          mx[e + 1] = fmaxf(mx[e + 1], fabsf(v.y));
-        }
+    for (int u = 0; u < 4; ++u) {
+      l[u] = live ? lut[hh * d.Q + i0 + kXsRows * u + row] : 0.f;
+      if (!(fabsf(l[u]) <= least)) {
+        if (i0 != d.Q - kXsTokens) w[u] = __ldg(src + (i0 / kXsRows + u) * stride);
+        any = true;
       }
     }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (fabsf(l[u]) <= least) continue;
+      const float2 l2 = make_float2(l[u], l[u]);
+      const uint32_t ww[4] = {w[u].x ^ 0x80808080u, w[u].y ^ 0x80808080u, w[u].z ^ 0x80808080u, w[u].w ^ 0x80808080u};
+#pragma unroll
+      for (int e = 0; e < 16; e += 2) {
+        const float2 xf = make_float2(s8_to_f32(ww[e >> 2], e & 3), s8_to_f32(ww[e >> 2], (e & 3) + 1));
+        const float2 v = __fmul2_rn(__fmul2_rn(xf, sx[e >> 1]), l2);
+        mx[e] = fmaxf(mx[e], fabsf(v.x));
+        mx[e + 1] = fmaxf(mx[e + 1], fabsf(v.y));
+      }
+    }
+    if (any) {
+#pragma unroll
+      for (int e = 0; e < 16; ++e) atomicMax(&best[e][lane], __float_as_uint(mx[e]));
+    }
+    if (__syncthreads_or(any) && i0 > 0) {
+      least = __int_as_float(0x7f800000);
+#pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        mx[e] = __uint_as_float(*reinterpret_cast<volatile uint32_t*>(&best[e][lane]));
+        const float s = fabsf(e & 1 ? sx[e >> 1].y : sx[e >> 1].x);
+        least = fminf(least, __fdividef(mx[e], 128.0f * s));   // (a step size of 0 or one that is not a number bounds nothing)
+      }
+      least = least < 1e-30f ? 0.f : least * 0.99999f;
+    }
   }
-#pragma unroll
-  for (int e = 0; e < 16; ++e) best[row][hh * 64 + c * 16 + e] = __float_as_uint(mx[e]);
-  __syncthreads();
-  for (int e = tid; e < kXsHeads * 64; e += 256) {
-    if (h0 + (e >> 6) >= d.H) break;
-    uint32_t m = 0u;
-#pragma unroll
-    for (int r = 0; r < 8; ++r) m = max(m, best[r][e]);
-    atomicMax(absmax + h0 * 64 + e, m);
+  for (int e = tid; e < kXsHeads * 64; e += kXsThreads) {
+    const int hc = e & 31, ch = (hc >> 2) * 64 + (hc & 3) * 16 + (e >> 5);   // of best[e >> 5][hc]
+    const uint32_t m = best[e >> 5][hc];
+    if (h0 + (hc >> 2) < d.H && m > *reinterpret_cast<volatile uint32_t*>(absmax + h0 * 64 + ch)) atomicMax(absmax + h0 * 64 + ch, m);
   }
 }
 
@@ -106,10 +131,11 @@ __global__ void finalize_scales(const uint32_t* max_h, float* s_h, int n, const 
 
 ssdi8_status_t launch_absmax_xs(const Dims& d, const int8_t* xq, const float* s_x, const float* pack, uint32_t* absmax,
                                 cudaStream_t st) {
-  const i64 blocks = (i64)((d.H + kXsHeads - 1) / kXsHeads) * d.c * (d.Q / kXsTokens);
+  const i64 blocks = (i64)((d.H + kXsHeads - 1) / kXsHeads) * d.c;
   if (blocks > 0x7fffffff) return SSDI8_ERR_SHAPE;
   const dim3 grid((unsigned)blocks, 1, d.b);
-  return launch_configured(absmax_xs_kernel, grid, dim3(256), 0, kStreamCarveout, false, st, xq, s_x, pack, absmax, d);
+  return launch_sized(absmax_xs_kernel, grid, dim3(kXsThreads), sizeof(float) * kXsHeads * d.Q, sizeof(float) * kXsHeads * 256, kStreamCarveout,
+                      false, st, xq, s_x, pack, absmax, d);
 }
 
 ssdi8_status_t launch_clear_words(void* a, i64 n, cudaStream_t st) {
