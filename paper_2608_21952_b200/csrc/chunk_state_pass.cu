@@ -567,13 +567,13 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
   const int sms = sm_count();
   if (sms == 0) return SSDI8_ERR_CUDA;
   const int units = d.H * d.b, slots = 3 * sms;
-  // Whole heads wherever the device is filled; a remainder of less than an eighth of a wave goes in slices of 32 columns, whose
-  // chain per chunk is shorter.  Few units of some chunks go in slices of 64, the longest chains of them in 32 (graphs of layer calls,
+  // Whole heads wherever the device is filled; a remainder of less than an eighth of a wave goes in slices, whose
+  // chain per chunk is shorter (prefill of 6 x 2048 tokens x 80 heads, 36 of 480: whole 161.6 us, slices of 64 160.5, of 32 163.4).  Few units of some chunks go in slices of 64, the longest chains of them in 32 (graphs of layer calls,
   // us, whole / slices of 64 / of 32): N 128: 1024 tokens x 32 heads 22.0 / 20.7 / 21.6, 1024 x 96 32.8 / 32.2 / 36.1, 3 x 512 x 12 (chunks of
   // 128) 19.4 / 19.0 / 20.9, 128 x 12 (of 64) 13.6 / 12.9 / 12.8, 2048 x 80 46.8 / 45.5 / 54.7, 2 x 8192 x 8 (INT8 states) 74.7 / 66.6 / 63.1; but
   // 256 x 64 17.7 / 18.5 / 20.1, 128 x 64 (of 128) 14.2 / 15.7 / 16.5, 192 x 80 (of 64) 18.0 / 18.7 / 19.6, 3 x 2048 x 80 92 / 101 / 112.  N 64, from
   // four chunks on: 768 x 60 28.7 / - / 27.9, 256 x 32 (of 64) 16.4 / - / 15.6, 2048 x 60 44.9 / - / 44.6, but 256 x 36 (of 128) 16.4 / - / 18.1.
-  int n_full = units / slots * slots, slice = 32;
+  int n_full = units / slots * slots, slice = d.N == 128 ? 64 : 32;
   const int last = units - n_full;
   if (n_full > 0) {
     if (8 * last > slots) n_full = units;
