@@ -177,7 +177,21 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
       (s = launch_bmm(d, a->Cq, a->Bq, a->s_C, a->s_B, a->s_cb, cbq, a->tap_acc_cb, nullptr, a->status, st)) !=
           SSDI8_OK)
     return s;
-  if (split_state) {
+  // Eight chunks of that: both modules in one launch, a cluster of CTAs per (batch, head) (chunk_state.cu).  With fewer chunks the
+  // fused kernel is the faster one (layer calls, us, fused / clusters: 1024 tokens x 32 heads 22.8 / 23.1, 1024 x 8 19.7 / 21.0, 512 x 24
+  // 19.6 / 23.0, 3 x 512 x 12 in chunks of 128 20.7 / 21.3, 768 x 60 (N 64) in chunks of 128 25.5 / 25.3, 256 x 24 18.4 / 22.6), as it is with
+  // more sequences (2 x 2048 x 24 35.3 / 40.6).
+  const bool state_taps = a->tap_loc || a->tap_prev || a->tap_Xsq || a->tap_acc_st;
+  const bool cluster_state = split_state && d.c <= 8 && !state_taps;
+  if (cluster_state) {
+    const StatePass pass = {a->s_h, gamma, a->init_state, a->final_state, hq};
+    if ((s = launch_chunk_state(d, a->xq, a->Bq, a->s_x, a->s_xs, a->s_B, pack, nullptr, nullptr, nullptr, a->status, st, &pass)) !=
+        SSDI8_OK)
+      return s;
+    if (bmm_late && (s = launch_bmm(d, a->Cq, a->Bq, a->s_C, a->s_B, a->s_cb, cbq, a->tap_acc_cb, nullptr, a->status,
+                                    st, true)) != SSDI8_OK)
+      return s;
+  } else if (split_state) {
     if ((s = launch_chunk_state(d, a->xq, a->Bq, a->s_x, a->s_xs, a->s_B, pack, loc, a->tap_Xsq, a->tap_acc_st, a->status,
                                 st)) != SSDI8_OK)
       return s;

@@ -10,6 +10,11 @@
 // of the epilogue writes 32 consecutive n of one p: full 128-byte lines of loc[p][n].
 // The forward pass takes this kernel where there are too few (batch, head) pairs to fill the device with
 // chunk-sequential ones (see fwd_phases).
+// PASS: the chunks of a (batch, head), up to eight, are a cluster.  The chunk-local states stay in shared memory, and once all of
+// them are there each CTA takes a share of the (p, n) through all chunks (Eq. 5-6, as state_passing.cu does, operation for
+// operation), reading the others' by way of distributed shared memory: no second launch, and no 32 KB per chunk out to L2 and
+// back (layer calls: 512 tokens x 4 heads 17.0 -> 16.0 us, 2048 x 24 29.5 -> 28.4; and with the epilogue's scales in shared memory, the
+// MMAs issued from uniform registers and the pass's operands fetched under them, 14.9 and 27.95).
 #include "kernels.h"
 #include "sm100.cuh"
 
@@ -22,15 +27,19 @@ struct StateArgs {
   const float* s_x; const float* s_xs; const float* s_B; const float* pack;
   float* loc; int8_t* tap_Xsq; int32_t* tap_acc; int32_t* status;
   Dims d;
+  const float* s_h; const float* gamma; const float* init; float* final_state; int8_t* hq;   // PASS
 };
 
 constexpr int kThreads = 256;
 constexpr uint32_t OFF_B = 0;        // [Q][N]  Bq rows (token-major)
 constexpr uint32_t OFF_X = 32768;    // [Q][64] xq rows -> Xs_q in place
-constexpr uint32_t OFF_F = 49152;    // lut[256], s_x / s_xs [64], bars, tmem slot
-constexpr uint32_t SMEM_BYTES = OFF_F + 256 * 4 + 64 * 4 + 64;
+constexpr uint32_t OFF_F = 49152;    // lut[256], s_x / s_xs [64], s_xs s_B [64], bars, tmem slot
+constexpr uint32_t SMEM_BYTES = OFF_F + 256 * 4 + 128 * 4 + 64;
 
-__global__ void __launch_bounds__(kThreads, 3)
+constexpr int kMaxCluster = 8;
+
+template <bool PASS>
+__global__ void __launch_bounds__(kThreads, PASS ? 2 : 3)
 chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__ CUtensorMap tm_x,
                const StateArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -38,7 +47,7 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
   const Dims& d = a.d;
   const int Q = d.Q, N = d.N, P = d.P;
   const int TQ = Q < 128 ? Q : 128;  // rows per TMA box
-  const int h = blockIdx.x, k = blockIdx.y, b = blockIdx.z;
+  const int h = PASS ? blockIdx.y : blockIdx.x, k = PASS ? blockIdx.x : blockIdx.y, b = blockIdx.z;   // (PASS: the cluster is along x)
   const int g = h / (d.H / d.G);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const i64 tok0 = (i64)b * d.L + (i64)k * Q;
@@ -46,7 +55,8 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
   uint8_t* sX = smem + OFF_X;
   float* lut = reinterpret_cast<float*>(smem + OFF_F);
   float* rxs = lut + 256;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(rxs + 64);  // [0] operands landed, [1] MMA done
+  float* scale = rxs + 64;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(scale + 64);  // [0] operands landed, [1] MMA done
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
 
   if (tid == 0) {
@@ -74,7 +84,9 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
   if (tid < Q) lut[tid] = a.pack[((((i64)b * d.H + h) * d.c + k) * kPackRows + PACK_LUT) * Q + tid];
   if (tid >= kThreads - 64) {   // one division per channel (each thread's own sixteen were a third of the kernel's instructions)
     const int p = tid - (kThreads - 64);
-    rxs[p] = __fdiv_rn(a.s_x[h * P + p], a.s_xs[h * P + p]);
+    const float sxs = a.s_xs[h * P + p];
+    rxs[p] = __fdiv_rn(a.s_x[h * P + p], sxs);
+    scale[p] = __fmul_rn(sxs, a.s_B[g]);   // (read from global memory in the epilogue they stood behind the MMAs)
   }
   __syncthreads();
   // per-column factors of this thread's 16 channels (16-byte chunk c of every row it visits)
@@ -130,19 +142,37 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
 
   // ---- acc[n][p] = sum_i Bq[i][n] Xs_q[i][p]: A = Bq (MN-major, M = N states), B = Xs_q (MN-major)
   const uint32_t tmem = *tmem_slot;
-  if (tid == 0) {
+  if (warp == 0) {   // (the whole warp runs the loop, see elect_one)
     tc_fence_after();
     const uint32_t idesc = idesc_s8(N, 64, 1, 1);
+    const uint32_t sBa = smem_u32(sB), sXa = smem_u32(sX);
     uint32_t first = 0;
-    for (int s = 0; s < Q / 32; ++s) {
-      if (!((live >> s) & 1u)) continue;
-      mma_s8_ss(tmem, tile_desc(smem_u32(sB) + 32 * s * N, (uint32_t)N),
-                tile_desc(smem_u32(sX) + 32 * s * 64, 64), idesc, first);
-      first = 1;
+    if (elect_one()) {
+#pragma unroll 1
+      for (uint32_t m = live; m; m &= m - 1) {
+        const int s = __ffs((int)m) - 1;
+        mma_s8_ss(tmem, tile_desc(sBa + 32 * s * N, (uint32_t)N), tile_desc(sXa + 32 * s * 64, 64), idesc, first);
+        first = 1;
+      }
+      mma_commit(&bars[1]);
     }
-    mma_commit(&bars[1]);
   }
   __syncwarp();
+  // (PASS) this CTA's share of the states, four neighbouring n a thread; what the first of them needs from global memory is
+  // on its way under the MMAs
+  const int units = P * N / 4, per = (units + d.c - 1) / d.c;
+  const int u0 = k * per + tid, u1 = min(units, (k + 1) * per);
+  const i64 bh = (i64)b * d.H + h;
+  float gam[kMaxCluster], inv_h = 0.f;
+  float4 S = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (PASS) {
+#pragma unroll
+    for (int j = 0; j < kMaxCluster; ++j) gam[j] = j < d.c ? a.gamma[bh * d.c + j] : 0.f;
+    if (u0 < u1) {
+      inv_h = __fdiv_rn(1.0f, a.s_h[h * P + 4 * u0 / N]);
+      if (a.init) S = reinterpret_cast<const float4*>(a.init)[bh * units + u0];
+    }
+  }
   mbar_wait(&bars[1], 0, a.status);
   tc_fence_after();
 
@@ -155,18 +185,62 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
     tmem_ld_wait();
     const bool ok = (N == 128) || (lane < 16);
     const int n = (N == 128) ? q * 32 + lane : q * 16 + lane;
-    if (ok) {
-      const float sB_g = a.s_B[g];
+    if (PASS) {   // (over the Bq tile, which the MMAs have read)
+      float* loc = reinterpret_cast<float*>(sB) + n;
+      if (ok) {
+#pragma unroll
+        for (int pp = 0; pp < 32; ++pp) {
+          const int p = ch * 32 + pp;
+          loc[p * N] = __fmul_rn(i22_to_f32(acc[pp]), scale[p]);
+        }
+      }
+    } else if (ok) {
       const i64 obase = ((((i64)b * d.c + k) * d.H + h) * P) * N + n;
 #pragma unroll
       for (int pp = 0; pp < 32; ++pp) {
         const int p = ch * 32 + pp;
-        a.loc[obase + (i64)p * N] = __fmul_rn(i22_to_f32(acc[pp]), __fmul_rn(a.s_xs[h * P + p], sB_g));
+        a.loc[obase + (i64)p * N] = __fmul_rn(i22_to_f32(acc[pp]), scale[p]);
         if (a.tap_acc) a.tap_acc[obase + (i64)p * N] = acc[pp];
       }
     }
   }
   tc_fence_before();
+  if (PASS) {
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+    const uint32_t mine = smem_u32(sB);
+    for (int u = u0; u < u1; u += kThreads) {
+      float4 l[kMaxCluster];
+#pragma unroll
+      for (int j = 0; j < kMaxCluster; ++j) {
+        if (j < d.c) {
+          uint32_t at;
+          asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(mine + 16u * (uint32_t)u), "r"(j));
+          asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                       : "=f"(l[j].x), "=f"(l[j].y), "=f"(l[j].z), "=f"(l[j].w)
+                       : "r"(at)
+                       : "memory");
+        }
+      }
+      if (u != u0) {
+        inv_h = __fdiv_rn(1.0f, a.s_h[h * P + 4 * u / N]);
+        S = a.init ? reinterpret_cast<const float4*>(a.init)[bh * units + u] : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      uint32_t* hq = reinterpret_cast<uint32_t*>(a.hq) + ((i64)b * d.c * d.H + h) * units + u;
+#pragma unroll
+      for (int j = 0; j < kMaxCluster; ++j) {
+        if (j < d.c) {
+          hq[(i64)j * d.H * units] = pack4_bits(rne_clamp_bits(__fmul_rn(S.x, inv_h)), rne_clamp_bits(__fmul_rn(S.y, inv_h)),
+                                                rne_clamp_bits(__fmul_rn(S.z, inv_h)), rne_clamp_bits(__fmul_rn(S.w, inv_h)));
+          S.x = __fmaf_rn(gam[j], S.x, l[j].x);
+          S.y = __fmaf_rn(gam[j], S.y, l[j].y);
+          S.z = __fmaf_rn(gam[j], S.z, l[j].z);
+          S.w = __fmaf_rn(gam[j], S.w, l[j].w);
+        }
+      }
+      if (a.final_state) reinterpret_cast<float4*>(a.final_state)[bh * units + u] = S;
+    }
+    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");   // (the others have read this CTA's)
+  }
   drain_after_timeout(a.status);
   __syncthreads();
   if (warp == 1) {
@@ -180,7 +254,7 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
 ssdi8_status_t launch_chunk_state(const Dims& d, const int8_t* xq, const int8_t* Bq,
                                   const float* s_x, const float* s_xs, const float* s_B,
                                   const float* pack, float* loc, int8_t* tap_Xsq,
-                                  int32_t* tap_acc, int32_t* status, cudaStream_t st) {
+                                  int32_t* tap_acc, int32_t* status, cudaStream_t st, const StatePass* pass) {
   const int TQ = d.Q < 128 ? d.Q : 128;
   const uint64_t T = (uint64_t)d.b * d.L;
   CUtensorMap tm_B, tm_x;
@@ -196,10 +270,16 @@ ssdi8_status_t launch_chunk_state(const Dims& d, const int8_t* xq, const int8_t*
     uint32_t box[3] = {64, 1, (uint32_t)TQ};
     if (!encode_tensor_map(&tm_x, xq, 1, 3, dims, str, box, 64)) return SSDI8_ERR_CUDA;
   }
-  StateArgs a = {s_x, s_xs, s_B, pack, loc, tap_Xsq, tap_acc, status, d};
+  StateArgs a = {s_x, s_xs, s_B, pack, loc, tap_Xsq, tap_acc, status, d, nullptr, nullptr, nullptr, nullptr, nullptr};
   const size_t smem = SMEM_BYTES + 1024;
-  dim3 grid(d.H, d.c, d.b);
-  return launch_configured(chunk_state_tc, grid, dim3(kThreads), smem, -1, false, st, tm_B, tm_x, a);
+  if (!pass) return launch_configured(chunk_state_tc<false>, dim3(d.H, d.c, d.b), dim3(kThreads), smem, -1, false, st, tm_B, tm_x, a);
+  if (d.c > kMaxCluster) return SSDI8_ERR_SHAPE;
+  a.s_h = pass->s_h;
+  a.gamma = pass->gamma;
+  a.init = pass->init;
+  a.final_state = pass->final_state;
+  a.hq = pass->hq;
+  return launch_clustered(chunk_state_tc<true>, dim3(d.c, d.H, d.b), d.c, dim3(kThreads), smem, st, tm_B, tm_x, a);
 }
 
 }  // namespace ssdi8

@@ -82,7 +82,7 @@ ssdi8_status_t launch_softplus_dt(const float* dt_raw, const float* dt_bias, flo
                                   cudaStream_t st) {
   const i64 n = rows * H;
   if (n == 0) return SSDI8_OK;
-  if (launch_pdl(softplus_dt_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, dt_raw, dt_bias, out, n, H) !=
+  if (launch_pdl(softplus_dt_kernel, dim3((unsigned)((n + 255) / 256)), 0, dim3(256), 0, st, dt_raw, dt_bias, out, n, H) !=
       cudaSuccess)
     return SSDI8_ERR_CUDA;
   SSDI8_LAUNCH_CHECK();

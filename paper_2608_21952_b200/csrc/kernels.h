@@ -7,20 +7,27 @@
 namespace ssdi8 {
 
 // kernel<<<grid, block, smem, st>>>(args...) with programmatic stream serialization allowed: the
-// kernel may be scheduled while its predecessor in the stream drains (see pdl_wait in common.cuh)
+// kernel may be scheduled while its predecessor in the stream drains (see pdl_wait in common.cuh).  cluster: CTAs of a
+// cluster along x, where the kernel does not say so itself (0 or 1: none)
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int cluster, dim3 block, size_t smem, cudaStream_t st,
                               Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  if (cluster > 1) {
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cluster;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.numAttrs = 2;
+  }
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
@@ -32,16 +39,26 @@ cudaError_t kernel_ready(const void* kernel, size_t smem, int carveout, bool che
 void kernel_forget(const void* kernel);   // the device was reset under us: set the attributes again
 // (smem_most: the largest that any launch of the kernel asks for)
 template <typename... KArgs, typename... Args>
-inline ssdi8_status_t launch_sized(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, size_t smem_most, int carveout,
-                                   bool check_static, cudaStream_t st, Args&&... args) {
+inline ssdi8_status_t launch_any(void (*kernel)(KArgs...), dim3 grid, int cluster, dim3 block, size_t smem, size_t smem_most, int carveout,
+                                 bool check_static, cudaStream_t st, Args&&... args) {
   const void* k = reinterpret_cast<const void*>(kernel);
   for (int attempt = 0; attempt < 2; ++attempt) {
     if (kernel_ready(k, smem_most, carveout, check_static) != cudaSuccess) break;
-    if (launch_pdl(kernel, grid, block, smem, st, args...) == cudaSuccess) return SSDI8_OK;
+    if (launch_pdl(kernel, grid, cluster, block, smem, st, args...) == cudaSuccess) return SSDI8_OK;
     kernel_forget(k);
   }
   (void)cudaGetLastError();
   return SSDI8_ERR_CUDA;
+}
+template <typename... KArgs, typename... Args>
+inline ssdi8_status_t launch_sized(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, size_t smem_most, int carveout,
+                                   bool check_static, cudaStream_t st, Args&&... args) {
+  return launch_any(kernel, grid, 0, block, smem, smem_most, carveout, check_static, st, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline ssdi8_status_t launch_clustered(void (*kernel)(KArgs...), dim3 grid, int cluster, dim3 block, size_t smem, cudaStream_t st,
+                                       Args&&... args) {
+  return launch_any(kernel, grid, cluster, block, smem, smem, -1, false, st, std::forward<Args>(args)...);
 }
 template <typename... KArgs, typename... Args>
 inline ssdi8_status_t launch_configured(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, int carveout,
@@ -102,10 +119,14 @@ ssdi8_status_t launch_bmm(const Dims& d, const int8_t* Cq, const int8_t* Bq, con
                           const float* s_B, const float* s_cb, int8_t* CBq, int32_t* tap_acc,
                           uint32_t* absmax_acc, int32_t* status, cudaStream_t st, bool after_state_kernel = false);
 
+// pass: ChunkState and StatePassing of up to eight chunks in one launch (loc and the taps unused)
+struct StatePass {
+  const float* s_h; const float* gamma; const float* init; float* final_state; int8_t* hq;
+};
 ssdi8_status_t launch_chunk_state(const Dims& d, const int8_t* xq, const int8_t* Bq,
                                   const float* s_x, const float* s_xs, const float* s_B,
                                   const float* pack, float* loc, int8_t* tap_Xsq,
-                                  int32_t* tap_acc, int32_t* status, cudaStream_t st);
+                                  int32_t* tap_acc, int32_t* status, cudaStream_t st, const StatePass* pass = nullptr);
 
 // ChunkState and StatePassing in one chunk-sequential kernel (loc never leaves the chip).  absmax_h (calibration):
 // per-channel running max (binary32 bits) of |S| over init and every S_k; s_xs then holds the maxima of |X_scaled|, whose step

@@ -309,11 +309,16 @@ def test_state_kernels_on_both_sides_of_the_dispatch(cfg, fast):
                                  SSDConfig("slices_32", 1, 13 * 64, 5, 64, 128, 1, 64, 0.02, 20.0, 54),
                                  SSDConfig("slices_n64", 1, 5 * 128, 7, 64, 64, 1, 128, 0.02, 20.0, 55),
                                  SSDConfig("many", 3, 2 * 256, 100, 64, 64, 2, 256, 0.02, 20.0, 56),
-                                 SSDConfig("slices_last", 5, 2 * 64, 90, 64, 128, 1, 64, 0.02, 20.0, 57)], ids=lambda c: c.name)
+                                 SSDConfig("slices_last", 5, 2 * 64, 90, 64, 128, 1, 64, 0.02, 20.0, 57),
+                                 SSDConfig("cluster", 1, 8 * 64, 1, 64, 64, 1, 64, 0.02, 20.0, 58),
+                                 SSDConfig("cluster_q256", 2, 8 * 256, 3, 64, 128, 3, 256, 0.02, 20.0, 59),
+                                 SSDConfig("cluster_most", 1, 8 * 128, 37, 64, 128, 1, 128, 0.02, 20.0, 60),
+                                 SSDConfig("cluster_beyond", 1, 8 * 64, 38, 64, 64, 2, 64, 0.02, 20.0, 62)], ids=lambda c: c.name)
 @pytest.mark.parametrize("decay", [0.002, 1.0, 60.0])
 def test_fused_state_kernel_with_few_and_many_sequences(cfg, decay):
     # Up to two CTAs per SM (whole heads, slices of 32 and of 64 state columns), three, and a last wave in slices; decay rates
-    # at which every slab of every chunk is live, some are, and none is.  INT8 states always take this kernel, and the codes of
+    # at which every slab of every chunk is live, some are, and none is; eight chunks, whose binary32 states take a cluster per
+    # sequence where there are few.  INT8 states always take this kernel, and the codes of
     # the states that enter the chunks and the final state are all that it writes (the taps' instance is another kernel).
     import gpu_harness as gh
     from paper_2608_21952_b200 import binding as bd
