@@ -68,25 +68,36 @@ bmm_tc(const __grid_constant__ CUtensorMap tm_C, const __grid_constant__ CUtenso
   // scan kernel that follows.
   if (!a.late_wait) pdl_wait();
 
-  if (tid == 0) {
-    mbar_expect_tx(&bars[0], (uint32_t)(TM * N + KJ * N));
-    tma_load_3d(smem + OFF_A, &tm_C, &bars[0], 0, g, (int)(tok0 + it * TM));
-    for (int j0 = 0; j0 < KJ; j0 += TM) tma_load_3d(smem + OFF_B + j0 * N, &tm_B, &bars[0], 0, g, (int)(tok0 + j0));
+  // (the whole of warp 0 runs this, see elect_one)
+  if (warp == 0) {
+    if (elect_one()) {
+      mbar_expect_tx(&bars[0], (uint32_t)(TM * N + KJ * N));
+      tma_load_3d(smem + OFF_A, &tm_C, &bars[0], 0, g, (int)(tok0 + it * TM));
+      for (int j0 = 0; j0 < KJ; j0 += TM) tma_load_3d(smem + OFF_B + j0 * N, &tm_B, &bars[0], 0, g, (int)(tok0 + j0));
+    }
+    __syncwarp();
     mbar_wait(&bars[0], 0, a.status);
     tc_fence_after();
     const uint32_t idesc = idesc_s8(128, KJ, 0, 0);  // N = 64, 128 or 256 columns
-    for (int s = 0; s < N / 32; ++s)
-      mma_s8_ss(tmem, tile_desc(smem_u32(smem + OFF_A) + 32 * s, (uint32_t)N),
-                tile_desc(smem_u32(smem + OFF_B) + 32 * s, (uint32_t)N), idesc, s > 0);
-    mma_commit(&bars[1]);
+    const uint64_t da = tile_desc(smem_u32(smem + OFF_A), (uint32_t)N), db = tile_desc(smem_u32(smem + OFF_B), (uint32_t)N);
+    if (elect_one()) {
+      mma_s8_ss(tmem, da, db, idesc, 0);   // (descriptors advance by a constant per 32-byte K step)
+      mma_s8_ss(tmem, da + 2, db + 2, idesc, 1);
+      if (N == 128) {
+        mma_s8_ss(tmem, da + 4, db + 4, idesc, 1);
+        mma_s8_ss(tmem, da + 6, db + 6, idesc, 1);
+      }
+      mma_commit(&bars[1]);
+    }
+    __syncwarp();
   }
-  __syncwarp();
+  // (ahead of the wait, which hides its latency)
+  const float r_cb = a.s_cb ? __fdiv_rn(__fmul_rn(a.s_C[g], a.s_B[g]), a.s_cb[g]) : 0.f;
   mbar_wait(&bars[1], 0, a.status);
   tc_fence_after();
 
   // ---- epilogue: thread = row i of the tile, 32 columns at a time; the four warps that share a
   // lane quarter take alternate 32-column pieces
-  const float r_cb = a.s_cb ? __fdiv_rn(__fmul_rn(a.s_C[g], a.s_B[g]), a.s_cb[g]) : 0.f;
   const int wq = warp & 3, wc = warp >> 2;
   const int r = wq * 32 + lane;
   const int i = it * TM + r;
