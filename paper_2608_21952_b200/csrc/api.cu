@@ -166,10 +166,10 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
   const bool bmm_late = (ph & SSDI8_PHASE_BMM) && fused_state;
   // Few sequences of many chunks: the fused kernel walks a (batch, head)'s chunks one after the other, about 1.2 us
   // each however few CTAs there are, while ChunkState takes all chunks at once (states through L2) and StatePassing
-  // is a short elementwise pass.  Algorithm 2 with the fused kernel / with the two, us: 8192 tokens x 8 heads (N 64,
-  // chunks of 64) 128 / 58, 8192 x 48 98.5 / 92.5, 4096 x 48 58.8 / 57.6, 4096 x 24 44.2 / 42.7, 512 x 4 (chunks of 64)
-  // 18.0 / 16.0; but 8192 x 60 104.7 / 109.2, 8192 x 80 119 / 136, 4096 x 80 74 / 78.  With eight to eleven chunks the line
-  // lies where two CTAs per SM take all of them at once (2048 x 24: even).
+  // is a short elementwise pass.  Graphs of prefill calls with the fused kernel / with the two, us: 8192 tokens x 8 heads (N 64, chunks of
+  // 64) 109.8 / 48.4, 8192 x 36 (N 64, of 128) 112.6 / 85.0, 8192 x 20 67.7 / 53.7, 4096 x 24 44.1 / 38.3, 4096 x 48 61.5 / 58.7, 2048 x 8 29.2 /
+  // 25.3, 512 x 4 (of 64) 17.4 / 16.5; even at 8192 x 48 (96.4 / 97.2), 2048 x 36 (33.7 / 33.9), 2048 x 24 (30.5 / 30.6), and 2 x 4096 x 24 58.0
+  // / 60.0.  With eight to eleven chunks the line lies where two CTAs per SM take all of them at once.
   const int sms = fused_state ? sm_count() : 0;
   const i64 seqs = (i64)d.b * d.H;
   const bool split_state = fused_state && !i8s && (d.c >= 12 ? 3 * seqs <= sms : d.c >= 8 && seqs * d.c <= 2 * sms);
