@@ -48,7 +48,7 @@ struct FusedArgs {
 constexpr int kStateWarps = 8, kStateThreads = 32 * kStateWarps;
 constexpr int kSlab = 64;                         // tokens of a slab
 constexpr int kLutAhead = 4;                      // LUT_state of so many chunks is under way to the loading warp
-enum { SLAB_LAST = 1 };                           // of its chunk (the word also has the slab's index from bit 8, the chunk's from 16)
+enum { SLAB_LAST = 1 };                           // of its chunk (the word also has the slab's index from bit 8; the warps that need the chunk's count chunks)
 
 // FEW: up to two CTAs per SM.  A CTA alone on its SM is a chain of latencies, the longest where decay is slow and most slabs live: the
 // state warps quantise Q(X_scaled) themselves, all eight at a slab, one chunk ahead, behind a ring of six slabs.  With three
@@ -158,7 +158,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     }
     __syncwarp();
     if (elect_one()) {
-      info[slot] = (last ? SLAB_LAST : 0) | (sl << 8) | (TAPS ? k << 16 : 0);
+      info[slot] = (last ? SLAB_LAST : 0) | (sl << 8);
       mbar_expect_tx(&bars[B_FULL + slot], kSlab * 64 + kSlab * NS);   // (an arrival: releases the stores above)
       if (copies) copy(slot, k, sl);
     }
@@ -300,8 +300,8 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  // row `row` of a slab, 16 channels (those of lane % 4) of it
-  auto quantise_rows = [&](int slot, int inf, int row, float bound) {
+  // row `row` of a slab of chunk k, 16 channels (those of lane % 4) of it
+  auto quantise_rows = [&](int slot, int inf, int k, int row, float bound) {
     const int c = lane & 3;
     const float l = reinterpret_cast<const float*>(smem + OFF_LUT)[slot * kSlab + row];
     uint4* ptr = reinterpret_cast<uint4*>(smem + OFF_X + slot * (kSlab * 64) + swz_off((uint32_t)row, (uint32_t)c, 64));
@@ -325,7 +325,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     }
     *ptr = v;
     if (TAPS && a.tap_Xsq)
-      *reinterpret_cast<uint4*>(a.tap_Xsq + (((i64)b * d.L + (i64)(inf >> 16) * Q + ((inf >> 8) & 255) * kSlab + row) * d.H + h) * P +
+      *reinterpret_cast<uint4*>(a.tap_Xsq + (((i64)b * d.L + (i64)k * Q + (inf >> 8) * kSlab + row) * d.H + h) * P +
                                 c * 16) = v;
   };
 
@@ -365,7 +365,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
       if (__any_sync(0xffffffffu, !mbar_wait_inline<256>(&bars[B_FULL + slot], at.phase, a.status))) break;
       const int inf = info[slot];
 #pragma unroll 1
-      for (int row = 8 * (warp - kStateWarps) + (lane >> 2); row < kSlab; row += 8 * G::kRowWarps) quantise_rows(slot, inf, row, bound);
+      for (int row = 8 * (warp - kStateWarps) + (lane >> 2); row < kSlab; row += 8 * G::kRowWarps) quantise_rows(slot, inf, k, row, bound);
       fence_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars[B_READY + slot]);
@@ -407,24 +407,24 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     // ---- (FEW) Q(X_scaled) of a chunk's slabs, in place, one chunk ahead: a warp takes eight rows of each
     const float bound = FEW ? row_bound(col_rx[lane], col_rx[lane + 32]) : 0.f;
     Pos at;
-    auto quantise_chunk = [&]() {
+    auto quantise_chunk = [&](int k) {
 #pragma unroll 1
       for (int more = 1; more; at.next()) {
         const int slot = at.slot;
         if (__any_sync(0xffffffffu, !mbar_wait_inline<0>(&bars[B_FULL + slot], at.phase, a.status))) return;
         const int inf = info[slot];
-        quantise_rows(slot, inf, 8 * warp + (lane >> 2), bound);
+        quantise_rows(slot, inf, k, 8 * warp + (lane >> 2), bound);
         fence_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars[B_READY + slot]);
         more = (inf & SLAB_LAST) ^ SLAB_LAST;
       }
     };
-    if (FEW) quantise_chunk();
+    if (FEW) quantise_chunk(0);
 #pragma unroll 1
     for (int k = 0; k < d.c; ++k) {
       const float gam = a.gamma[unit0 + k];
-      if (FEW && k + 1 < d.c) quantise_chunk();
+      if (FEW && k + 1 < d.c) quantise_chunk(k + 1);
       const uint32_t ai = NA == 1 ? 0u : (uint32_t)k & 1u;
       // ---- hq[k] = codes of the state entering this chunk (and the prev tap), ahead of the wait for the chunk's MMAs
       uint8_t* const hq = smem + G::OFF_HQ + (k & 1) * 8192;

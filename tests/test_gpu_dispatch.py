@@ -334,6 +334,30 @@ def test_fused_state_kernel_with_few_and_many_sequences(cfg, decay):
         assert np.array_equal(fin, fin_ref)
 
 
+def test_the_tap_of_x_scaled_reaches_the_last_of_many_chunks():
+    # Q(X_scaled) of a chunk depends on nothing outside it: the same chunk 32 770 times over has the same codes 32 770 times (more
+    # chunks than 16 bits of a signed index count).  INT8 states, which take the chunk-sequential kernel at any length.
+    import torch
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    c = 32770
+    one = SSDConfig("one", 1, 64, 1, 64, 64, 1, 64, 0.02, 20.0, 64)
+    q = orc.prepare_quantized(one, inputs.make_prefill(one))
+    want = gh.dev(orc.ssdi8_fwd(one, q["xq"], q["Bq"], q["Cq"], q["s_x"], q["s_B"], q["s_C"], q["dt"], q["A"], q["D"], None, q["s_xs"],
+                                q["s_cb"], q["s_h"], None, taps=("Xsq",), flags=orc.FLAG_INT8_STATE)[2]["Xsq"]).reshape(64, 64)
+    dims = bd.Dims(1, 64 * c, 1, 64, 64, 1, 64)
+    dv = {k: gh.dev(q[k]) for k in ("s_x", "s_B", "s_C", "A", "s_xs", "s_cb", "s_h")}
+    dv.update({k: gh.dev(q[k]).reshape(64, -1).repeat(c, 1) for k in ("xq", "Bq", "Cq", "dt")})
+    tap = torch.full((c, 64, 64), 99, dtype=torch.int8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    phases = bd.PHASE_CUMSUM | bd.PHASE_CHUNK_STATE | bd.PHASE_STATE_PASSING
+    bd.ssdi8_chunk_scan_fwd(dims, bd.make_fwd_args(y=torch.empty(4, device="cuda"), tap_Xsq=tap, status=status, **dv),
+                            bd.alloc_workspace(dims, flags=bd.FLAG_INT8_STATE), flags=bd.FLAG_INT8_STATE | phases)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert torch.equal(tap, want.expand(c, 64, 64))
+
+
 def _near_ties():
     # Pairs (v, alpha) whose quotient lies within 8 / alpha's significand of the midpoint between k + 1/2 and a neighbour
     # in binary32: where a quotient formed from a reciprocal could fall on the other side.
