@@ -116,7 +116,7 @@ size_t ssdi8_workspace_bytes(const ssdi8_dims_t* dims, uint32_t flags);
  * channel of the view in[R][Ch][I]  (x: R = B*L, Ch = D, I = 1;  B and C,
  * quantised once on the group axis before any broadcast to heads, Section 4.2
  * "Quantization of B,C": R = B*L, Ch = G, I = N).
- *   alpha = fdiv(absmax, 127)  (1 if the channel is all zero)
+ *   alpha = fdiv(absmax, 127)  (1 if that is 0: an all-zero channel, or one below 9e-44)
  *   q     = rne(fdiv(v, alpha)) saturated
  * mode 0 static:    read scale[Ch], write out.
  * mode 1 calibrate: write scale[Ch] from this tensor, then write out.

@@ -127,7 +127,7 @@ void orc_exp32(const float* x, float* out, i64 n) {
 
 // ---------------------------------------------------------------------------
 // Eq. 1: uniform symmetric quantiser.  View in[R][Ch][I], one step size per Ch.
-//   alpha = absmax / 127 (1 if the channel is all zero), q = round(v / alpha),
+//   alpha = absmax / 127 (1 if that is 0 in binary32), q = round(v / alpha),
 //   quotient formed in binary32 by true division, ties to even, saturated.
 // mode 0: static (alpha given)   mode 1: calibrate (alpha written, then quantise)
 // mode 2: observe (alpha = max(alpha, absmax/127); out may be NULL)
@@ -140,12 +140,12 @@ void orc_quantize(const float* in, i64 R, i64 Ch, i64 I, float* scale, int mode,
           float a = std::fabs(in[(r * Ch + ch) * I + i]);
           if (a > m) m = a;
         }
-      float alpha = (m == 0.0f) ? 1.0f : fdiv(m, 127.0f);
+      const float alpha = fdiv(m, 127.0f);
       if (mode == 2) {
         // an all-zero observation leaves the running step size unchanged
         if (m != 0.0f && alpha > scale[ch]) scale[ch] = alpha;
       } else {
-        scale[ch] = alpha;
+        scale[ch] = alpha == 0.0f ? 1.0f : alpha;
       }
     }
   }

@@ -250,6 +250,11 @@ __global__ void __launch_bounds__(QT) absmax_inner(const float4* __restrict__ in
 // 8192 x 5120 55 / 84; channels of 128 elements: 256 rows x 1 7.6 / 3.3, 1024 x 1 7.2 / 5.1, 1024 x 8 9.2 / 6.4, 1024 x 32 12.6 / 7.9, but 2048 x 1
 // 7.4 / 8.7, 4096 x 1 9.1 / 14.4.
 constexpr int kCluster = 8, kHeldRows = 1600;   // CTAs; rows of a column block that one of them holds at most (200 KB)
+// the step size that the three launches leave: 1 where the quotient is 0, as it also is for magnitudes below 63.5 of the smallest number
+__device__ __forceinline__ float step_of_channel(float m) {
+  const float al = __fdiv_rn(m, 127.0f);
+  return al == 0.f ? 1.f : al;
+}
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
@@ -302,7 +307,7 @@ calibrate_ch_fastest(const float4* __restrict__ in, float* __restrict__ scale, u
     float a = 0.f;
 #pragma unroll
     for (int c = 0; c < kCluster; ++c) a = fmaxf(a, remote_float(&mine[tid], c));
-    const float al = step_of_max(__float_as_uint(a));
+    const float al = step_of_channel(a);
     step[tid] = al;
     if (rank == 0 && blockIdx.y * 32 + tid < ch4 * 4) scale[blockIdx.y * 32 + tid] = al;
   }
@@ -358,7 +363,7 @@ calibrate_inner(const float4* __restrict__ in, float* __restrict__ scale, uint32
   if (tid < 32) {
     m = largest(tid < kCluster ? remote_float(&mine, tid) : 0.f);
     if (tid == 0) {
-      step = step_of_max(__float_as_uint(m));
+      step = step_of_channel(m);
       if (rank == 0) scale[ch] = step;
     }
   }

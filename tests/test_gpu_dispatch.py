@@ -109,6 +109,21 @@ def test_calibrating_quantiser_in_one_launch_and_in_three(R, Ch, I):
     assert np.array_equal(q.reshape(-1), np.asarray(qr).reshape(-1))
 
 
+@pytest.mark.parametrize("R,Ch,I", [(9, 32, 1), (4100, 1028, 1), (300, 2400, 1), (13, 3, 4), (257, 37, 128), (258, 38, 128), (2049, 4, 128)])
+def test_a_channel_whose_quotient_is_zero_has_a_step_of_one(R, Ch, I):
+    # One launch and three.  63 and 64 of the smallest number lie on either side of half of it times 127
+    import gpu_harness as gh
+    v = np.random.default_rng(R).standard_normal((R, Ch, I)).astype(np.float32)
+    for ch, units in enumerate((63, 64, 7)):
+        v[:, ch] = 0.0
+        v[R // 2, ch, I // 2] = np.float32(-units * 2.0 ** -149)
+    q, s = gh.gpu_quantize(v, R, Ch, I)
+    qr, sr = orc.quantize(v, R, Ch, I, mode=1)
+    assert np.array_equal(s, sr) and np.array_equal(q.reshape(-1), np.asarray(qr).reshape(-1))
+    assert s[0] == 1.0 and s[1] == np.float32(2.0 ** -149) and s[2] == 1.0
+    assert q[R // 2, 0, I // 2] == 0 and q[R // 2, 1, I // 2] == -64
+
+
 @pytest.mark.parametrize("b,c,H,Q", [(1, 1, 1, 64), (2, 3, 9, 128), (1, 3, 17, 256)])
 @pytest.mark.parametrize("regime", ["fast", "slow", "codes", "mixed"])
 def test_calibration_skips_no_token_that_counts(b, c, H, Q, regime):
