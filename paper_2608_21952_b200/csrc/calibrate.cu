@@ -94,7 +94,8 @@ __global__ void __launch_bounds__(kXsThreads) absmax_xs_kernel(const int8_t* __r
       for (int e = 0; e < 16; ++e) {
         mx[e] = __uint_as_float(*reinterpret_cast<volatile uint32_t*>(&best[e][lane]));
         const float s = fabsf(e & 1 ? sx[e >> 1].y : sx[e >> 1].x);
-        least = fminf(least, __fdividef(mx[e], 128.0f * s));   // (a step size of 0 or one that is not a number bounds nothing)
+        const float top = 128.0f * s;
+        least = fminf(least, top >= 0x1p-126f ? __fdividef(mx[e], top) : 0.f);   // (below, the quotient's error has no bound: skip nothing)
       }
       least = least < 1e-30f ? 0.f : least * 0.99999f;
     }

@@ -156,6 +156,30 @@ def test_calibration_skips_no_token_that_counts(b, c, H, Q, regime):
         assert np.array_equal(got.cpu().numpy(), np.asarray(ref).reshape(-1))
 
 
+@pytest.mark.parametrize("step", [8e-41, 9.1e-41, 9.3e-41, 1e-39])
+def test_calibration_skips_no_token_at_step_sizes_near_the_smallest(step):
+    # 128 step sizes on either side of the normal range: the last token of the chunk has codes of 1, the one 64 before it codes of
+    # 127 and a LUT_state of nearly the same size, every other token codes of 0
+    import torch
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("tiny", 1, 256, 8, 64, 64, 1, 256, 0.02, 20.0, 63)
+    q = orc.prepare_quantized(cfg, inputs.make_prefill(cfg), None)
+    x = np.zeros((256, 8, 64), np.int8)
+    x[-1] = 1
+    x[-65] = 127
+    q.update(xq=x.reshape(np.asarray(q["xq"]).shape), s_x=np.full(512, step, np.float32), A=np.full(8, -1e-3, np.float32))
+    q["dt"] = np.full_like(q["dt"], 0.5)
+    want = orc.calibrate(cfg, q["xq"], q["Bq"], q["Cq"], q["s_x"], q["s_B"], q["s_C"], q["dt"], q["A"], None)
+    dv = {k: gh.dev(q[k]) for k in ("xq", "Bq", "Cq", "s_x", "s_B", "s_C", "dt", "A")}
+    s = [torch.full((n,), float("nan"), device="cuda") for n in (512, 1, 512)]
+    bd.ssdi8_calibrate(bd.dims_of(cfg), bd.make_fwd_args(**dv), *s, bd.alloc_workspace(bd.dims_of(cfg)))
+    torch.cuda.synchronize()
+    assert np.all(np.asarray(want[0]) > 0) and np.all(np.asarray(want[0]) < 127 * step)
+    for got, ref in zip(s, want[:3]):
+        assert np.array_equal(got.cpu().numpy(), np.asarray(ref).reshape(-1))
+
+
 @pytest.mark.parametrize("R,Ch", [(R, Ch) for R in (1, 3, 15, 17, 31, 33, 63, 2051) for Ch in (4, 508, 516)] + [(227, 113664), (227, 113668)])
 def test_absmax_takes_every_row_into_account(R, Ch):
     # The largest value of each channel in a row of its own: remainders of the rows in flight, the row groups and the blocks
