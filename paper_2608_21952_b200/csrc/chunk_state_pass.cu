@@ -75,6 +75,9 @@ struct Geo {
 // kernel before wherever these have left room, would put up to three on one SM, each of them slower for it.  (Likewise the ring of six:
 // 3 x 1408 x 50 56.5 us with three to an SM, 53.4 with two; 3 x 2048 x 80 98.7 / 94.7, 1 x 1024 x 128 (G 8) 41.3 / 40.7.)
 constexpr uint32_t kSmemAlone = 120 * 1024;
+// the lowest n of 32 bits, n from 1 on (1 << 32, of the lanes of a chunk's only slab, is not defined)
+__host__ __device__ constexpr uint32_t low_bits(int n) { return 0xffffffffu >> (32 - n); }
+static_assert(low_bits(32) == 0xffffffffu && low_bits(16) == 0xffffu && low_bits(8) == 0xffu, "a slab has 32, 16 or 8 lanes of LUT_state");
 // position in a ring of slabs
 template <int SLOTS>
 struct Ring {
@@ -254,7 +257,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
                        alive(bound, v.b.y) | alive(bound, v.b.z) | alive(bound, v.b.w);
       const uint32_t bal = __ballot_sync(0xffffffffu, any);
       const int lps = 32 / nsl;
-      return __ballot_sync(0xffffffffu, lane < nsl && ((bal >> ((lane * lps) & 31)) & ((1u << lps) - 1u)) != 0);
+      return __ballot_sync(0xffffffffu, lane < nsl && ((bal >> ((lane * lps) & 31)) & low_bits(lps)) != 0);
     };
     bool on = true;
 #pragma unroll 1
