@@ -206,7 +206,7 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
   }
   tc_fence_before();
   if (PASS) {
-    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+    cluster_sync();
     const uint32_t mine = smem_u32(sB);
     for (int u = u0; u < u1; u += kThreads) {
       float4 l[kMaxCluster];
@@ -239,7 +239,7 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
       }
       if (a.final_state) reinterpret_cast<float4*>(a.final_state)[bh * units + u] = S;
     }
-    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");   // (the others have read this CTA's)
+    cluster_sync();   // (the others have read this CTA's)
   }
   drain_after_timeout(a.status);
   __syncthreads();

@@ -242,6 +242,15 @@ __device__ __forceinline__ void st_global_hint(float* a, float4 v, uint64_t pol)
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Barrier of a cluster's CTAs in two halves.  Not the .aligned form, which needs a warp whose lanes are together: the loops and the branches
+// on the lane ahead of it do not promise that.  All threads of all CTAs arrive, also where a wait has given up; no bound of its own.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() {
+  cluster_arrive();
+  cluster_wait();
+}
+
 struct Dims {
   int b, L, H, P, N, G, Q, c;
 };

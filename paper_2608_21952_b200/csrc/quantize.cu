@@ -255,9 +255,6 @@ __device__ __forceinline__ float step_of_channel(float m) {
   const float al = __fdiv_rn(m, 127.0f);
   return al == 0.f ? 1.f : al;
 }
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
-}
 __device__ __forceinline__ float remote_float(const float* own, int rank) {   // that of another CTA of the cluster
   uint32_t a = (uint32_t)__cvta_generic_to_shared(own);
   float v;
@@ -312,13 +309,13 @@ calibrate_ch_fastest(const float4* __restrict__ in, float* __restrict__ scale, u
     if (rank == 0 && blockIdx.y * 32 + tid < ch4 * 4) scale[blockIdx.y * 32 + tid] = al;
   }
   __syncthreads();
-  asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");   // (this CTA has read the others' maxima)
+  cluster_arrive();   // (this CTA has read the others' maxima)
   const float4 a4 = *reinterpret_cast<const float4*>(&step[4 * j]);
   const Step4 st = step4(a4);
   uint32_t* dst = out + r0 * ch4 + q;
   for (int r = tid >> 3; r < n; r += QT / 8)
     __stcs(dst + (i64)r * ch4, st.usable ? code4(tile[r * 8 + j], st) : code4_by_division(tile[r * 8 + j], a4));
-  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  cluster_wait();
 }
 
 constexpr int kInnerThreads = 1024, kInnerHeld = 8;   // threads of a CTA, float4 of each at most
@@ -368,7 +365,7 @@ calibrate_inner(const float4* __restrict__ in, float* __restrict__ scale, uint32
     }
   }
   __syncthreads();
-  asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
+  cluster_arrive();
   const float al = step;
   const float4 a4 = make_float4(al, al, al, al);
   const Step4 st = step4(a4);
@@ -376,7 +373,7 @@ calibrate_inner(const float4* __restrict__ in, float* __restrict__ scale, uint32
     const float4 v = tile[u * kInnerThreads + tid];
     out[e] = st.usable ? code4(v, st) : code4_by_division(v, a4);
   });
-  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  cluster_wait();
 }
 
 }  // namespace
