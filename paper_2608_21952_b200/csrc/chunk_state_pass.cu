@@ -219,7 +219,10 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
   if (warp == kLoadWarp) {
     // ------------------------------------------------------------ loads, as many slabs ahead as the ring has places.  This warp
     // forms the bound itself and does not wait for the others' set-up.  Where LUT_state of the first chunk is not known yet: FEW
-    // takes all slabs of that chunk (the start of the chain is what counts: 256 tokens x 24 heads 22.55 -> 22.35 us, 3 x 2048 x 80 96.5 -> 95.6), the others only the last one, the likeliest to live.
+    // takes all slabs of that chunk (the start of the chain is what counts: 256 tokens x 24 heads 22.55 -> 22.35 us, 3 x 2048 x 80 96.5 -> 95.6), and of
+    // all chunks where the ring holds them, so that none of a short call waits for LUT_state and then for its tiles (graphs of layer calls: 192 tokens x 8
+    // heads in chunks of 64, N 128, 13.1 -> 12.6 us, 384 x 16 of 128 15.3 -> 14.6; live slabs only in the first chunk too: 13.2, 15.7); the
+    // others take only the last one, the likeliest to live.
     const float sx0 = a.s_x[h * P + lane], sx1 = a.s_x[h * P + 32 + lane], xs0 = step_xs(lane), xs1 = step_xs(32 + lane);
     constexpr int kFirst = FEW ? 1 : 0;   // chunk from which on only live slabs are taken
     auto fetch_lut = [&](int k) {
@@ -232,24 +235,28 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
       __syncwarp();
     };
     Pos at;
+    const bool whole = FEW && d.c * nsl <= G::kSlots;   // the ring holds the call
     if (FEW) {
 #pragma unroll 1
-      for (int sl = nsl - 1; sl >= 0; --sl, at.next()) {
-        if (elect_one()) {
-          info[at.slot] = (sl == 0 ? SLAB_LAST : 0) | (sl << 8);
-          mbar_expect_tx(&bars[B_FULL + at.slot], kSlab * 64 + kSlab * NS + kSlab * 4);
-          copy(at.slot, 0, sl);
-          bulk_load(smem + OFF_LUT + at.slot * (kSlab * 4), a.pack + (unit0 * kPackRows + PACK_LUT) * Q + kSlab * sl, kSlab * 4,
-                    &bars[B_FULL + at.slot]);
+      for (int k = 0; k < (whole ? d.c : kFirst); ++k) {
+#pragma unroll 1
+        for (int sl = nsl - 1; sl >= 0; --sl, at.next()) {
+          if (elect_one()) {
+            info[at.slot] = (sl == 0 ? SLAB_LAST : 0) | (sl << 8);
+            mbar_expect_tx(&bars[B_FULL + at.slot], kSlab * 64 + kSlab * NS + kSlab * 4);
+            copy(at.slot, k, sl);
+            bulk_load(smem + OFF_LUT + at.slot * (kSlab * 4), a.pack + ((unit0 + k) * kPackRows + PACK_LUT) * Q + kSlab * sl, kSlab * 4,
+                      &bars[B_FULL + at.slot]);
+          }
+          __syncwarp();
         }
-        __syncwarp();
       }
     } else {
       fetch_lut(0);
       if (elect_one()) copy(0, 0, nsl - 1);
       __syncwarp();
     }
-    for (int k = FEW ? kFirst : 1; k < kFirst + kLutAhead; ++k) fetch_lut(k);
+    for (int k = FEW ? kFirst : 1; k < kFirst + kLutAhead && !whole; ++k) fetch_lut(k);
     const float bound = row_bound(__fdiv_rn(sx0, xs0), __fdiv_rn(sx1, xs1));
     auto live_slabs = [&](const Lut& v) -> uint32_t {
       if (TAPS) return (1u << nsl) - 1u;
@@ -261,7 +268,7 @@ __device__ __forceinline__ void fused_body(const CUtensorMap& tm_B, const CUtens
     };
     bool on = true;
 #pragma unroll 1
-    for (int k = kFirst; k < d.c; ++k) {
+    for (int k = whole ? d.c : kFirst; k < d.c; ++k) {
       const int i = k - kFirst;
       on = __all_sync(0xffffffffu, mbar_wait_inline<0>(&bars[B_LUT + i % kLutAhead], (i / kLutAhead) & 1, a.status));
       if (!on) break;
@@ -578,13 +585,16 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
   // chain per chunk is shorter (prefill of 6 x 2048 tokens x 80 heads, 36 of 480: whole 161.6 us, slices of 64 160.5, of 32 163.4).  Few units of some chunks go in slices of 64, the longest chains of them in 32 (graphs of layer calls,
   // us, whole / slices of 64 / of 32): N 128: 1024 tokens x 32 heads 22.0 / 20.7 / 21.6, 1024 x 96 32.8 / 32.2 / 36.1, 3 x 512 x 12 (chunks of
   // 128) 19.4 / 19.0 / 20.9, 128 x 12 (of 64) 13.6 / 12.9 / 12.8, 2048 x 80 46.8 / 45.5 / 54.7, 2 x 8192 x 8 (INT8 states) 74.7 / 66.6 / 63.1; but
-  // 256 x 64 17.7 / 18.5 / 20.1, 128 x 64 (of 128) 14.2 / 15.7 / 16.5, 192 x 80 (of 64) 18.0 / 18.7 / 19.6, 3 x 2048 x 80 92 / 101 / 112.  N 64, from
-  // four chunks on: 768 x 60 28.7 / - / 27.9, 256 x 32 (of 64) 16.4 / - / 15.6, 2048 x 60 44.9 / - / 44.6, but 256 x 36 (of 128) 16.4 / - / 18.1.
+  // 256 x 64 17.7 / 18.5 / 20.1, 128 x 64 (of 128) 14.2 / 15.7 / 16.5, 3 x 2048 x 80 92 / 101 / 112.  With two or three chunks up to two units to
+  // five SMs: 768 x 36 20.8 / 18.9 / -, 384 x 42 (of 128) 17.3 / 16.4 / -, 256 x 48 (of 128) 16.2 / 15.0 / -, 512 x 12 16.6 / 16.2 / 16.8, but 128 x 54 (of 64) 13.7 /
+  // 14.4 / -, 768 x 74 24.6 / 26.8 / -, 192 x 74 (of 64) 17.4 / 18.6 / -.
+  // N 64, from four chunks on: 768 x 60 28.7 / - / 27.9, 256 x 32 (of 64) 16.4 / - / 15.6, 2048 x 60 44.9 / - / 44.6; with fewer whole heads: 128 x 60
+  // (of 64) 13.3 / - / 14.6, 256 x 74 (of 128) 16.4 / - / 17.6, 512 x 36 17.9 / - / 19.2.
   int n_full = units / slots * slots, slice = d.N == 128 ? 64 : 32;
   const int last = units - n_full;
   if (n_full > 0) {
     if (8 * last > slots) n_full = units;
-  } else if (d.N == 128 && (d.c >= 4 ? 3 * units <= 2 * sms : d.c >= 2 && 4 * units <= sms)) {
+  } else if (d.N == 128 && (d.c >= 4 ? 3 * units <= 2 * sms : d.c >= 2 && 5 * units <= 2 * sms)) {
     slice = d.c >= 12 && 4 * units <= sms ? 32 : 64;
   } else if (!(d.N == 64 && d.c >= 4 && 2 * units <= sms)) {
     n_full = units;
@@ -600,10 +610,16 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
                  status, absmax_h, s_xs_out, d, n_full, slice};
   const unsigned grid = (unsigned)(n_full + d.N / slice * (units - n_full));
   const bool taps = tap_loc || tap_prev || tap_Xsq || tap_acc;
-  const bool few = (int)grid <= 2 * sms;
+  // (FEW; but with one chunk of 256 and nearly two CTAs for every SM two warps of their own quantise faster, all four slabs of a CTA being there at once:
+  // 256 tokens x 296 heads N 128 28.3 / 26.8 us, N 64 27.1 / 25.4, 268 x N 128 25.0 / 25.2, 230 x 24.7 / 25.4)
+  const bool few = (int)grid <= 2 * sms && !(d.Q == 256 && d.c == 1 && 10 * (int)grid > 18 * sms);
+  // (kSmemAlone; not for one chunk, nor for two or three of N 128 where more than four SMs in five get a CTA: the start is what counts there, and CTAs of that
+  // size wait for the SMs that the kernel before still holds.  With / without: 256 tokens x 148 heads N 128 22.1 / 19.8 us, 64 x 100 (of 64) N 64
+  // 13.6 / 13.1, 512 x 148 N 128 29.4 / 27.4, 768 x 148 33.9 / 32.2; but 128 x 48 (of 64) N 128 14.5 / 15.3, 384 x 148 (of 128) N 64 22.3 / 22.8)
+  const bool alone = (int)grid <= sms && d.c > 1 && !(d.N == 128 && d.c <= 3 && 5 * (int)grid > 4 * sms);
   auto launch = [&](auto few_c, auto kernel) -> ssdi8_status_t {
     using G = Geo<decltype(few_c)::value>;
-    const size_t smem = (int)grid <= sms ? kSmemAlone : G::SMEM_BYTES;
+    const size_t smem = alone ? kSmemAlone : G::SMEM_BYTES;
     return launch_sized(kernel, dim3(grid), dim3(G::kThreads), smem, decltype(few_c)::value ? kSmemAlone : smem, 100, true, st, tm_B, tm_x, tm_hq,
                         tm_Bs, tm_hqs, a);
   };

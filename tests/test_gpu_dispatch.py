@@ -373,6 +373,22 @@ def test_fused_state_kernel_with_few_and_many_sequences(cfg, decay):
         assert np.array_equal(fin, fin_ref)
 
 
+@pytest.mark.parametrize("cfg", [SSDConfig("six_slabs", 1, 6 * 64, 7, 64, 64, 1, 64, 0.02, 20.0, 65),
+                                 SSDConfig("seven_slabs", 1, 7 * 64, 7, 64, 64, 1, 64, 0.02, 20.0, 66),
+                                 SSDConfig("three_of_two", 1, 3 * 128, 37, 64, 128, 1, 128, 0.02, 20.0, 67),
+                                 SSDConfig("four_of_two", 1, 4 * 128, 5, 64, 128, 1, 128, 0.02, 20.0, 68),
+                                 SSDConfig("two_of_four", 1, 2 * 256, 59, 64, 128, 1, 256, 0.02, 20.0, 69),
+                                 SSDConfig("whole_after", 1, 3 * 64, 60, 64, 128, 2, 64, 0.02, 20.0, 70),
+                                 SSDConfig("nearly_all_sms", 1, 2 * 128, 119, 64, 128, 1, 128, 0.02, 20.0, 71),
+                                 SSDConfig("nearly_two_each", 2, 256, 134, 64, 128, 1, 256, 0.02, 20.0, 72),
+                                 SSDConfig("two_each", 2, 256, 133, 64, 64, 1, 256, 0.02, 20.0, 73)], ids=lambda c: c.name)
+@pytest.mark.parametrize("decay", [0.002, 60.0])
+def test_fused_state_kernel_on_short_calls(cfg, decay):
+    # Calls whose slabs the ring of six holds at once and calls with a slab more; slices and whole heads of two and three chunks; one
+    # chunk of 256 on either side of 1.8 CTAs per SM.  Every slab live, and none
+    test_fused_state_kernel_with_few_and_many_sequences(cfg, decay)
+
+
 def test_the_tap_of_x_scaled_reaches_the_last_of_many_chunks():
     # Q(X_scaled) of a chunk depends on nothing outside it: the same chunk 32 770 times over has the same codes 32 770 times (more
     # chunks than 16 bits of a signed index count).  INT8 states, which take the chunk-sequential kernel at any length.
