@@ -156,6 +156,46 @@ def test_calibration_skips_no_token_that_counts(b, c, H, Q, regime):
         assert np.array_equal(got.cpu().numpy(), np.asarray(ref).reshape(-1))
 
 
+@pytest.mark.parametrize("R,Ch,I", [(9, 32, 1), (4100, 1028, 1), (300, 2400, 1), (13, 4, 4), (257, 37, 128), (258, 38, 128), (2049, 4, 128)])
+def test_calibrating_quantiser_on_values_that_are_not_finite(R, Ch, I):
+    # One launch and three: a NaN counts for nothing in a step size, an infinity makes it infinite (its own code is that of a NaN, all others
+    # 0), a channel of NaNs has a step of 1.  Codes are those of the static mode under the same step sizes
+    import gpu_harness as gh
+    v = np.random.default_rng(R).standard_normal((R, Ch, I)).astype(np.float32)
+    v[R // 2, 0, I // 2] = np.nan
+    v[R - 1, 1, I - 1] = np.inf
+    v[0, 2, 0], v[R - 1, 2, I - 1] = -np.inf, np.nan
+    v[:, 3] = np.nan
+    want = np.nanmax(np.abs(np.where(np.isnan(v), np.float32(0), v)), axis=(0, 2)) / np.float32(127)
+    want[3] = 1.0
+    q, s = gh.gpu_quantize(v, R, Ch, I)
+    assert np.array_equal(s, want) and np.all(np.isinf(s[1:3])) and np.isfinite(s[0])
+    assert np.array_equal(q, gh.gpu_quantize(v, R, Ch, I, scale=want, mode=0)[0])
+    finite = np.isfinite(v[:, 1])
+    assert not q.reshape(R, Ch, I)[:, 1][finite].any()
+
+
+def test_calibration_passes_over_decays_and_step_sizes_that_are_not_finite():
+    # LUT_state of a chunk with a NaN, an infinity of either sign or a very negative time step in it; step sizes of x that are infinite,
+    # a NaN and zero
+    import torch
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("odd", 1, 5 * 256, 9, 64, 64, 1, 256, 0.02, 20.0, 74)
+    q = orc.prepare_quantized(cfg, inputs.make_prefill(cfg), None)
+    q["dt"], q["s_x"] = q["dt"].copy(), q["s_x"].copy()
+    for k, bad in enumerate((np.nan, np.inf, -np.inf, -1e4)):
+        q["dt"].reshape(1280, 9)[256 * k + 200, ::2] = bad
+    q["s_x"][[5, 70, 71, 72]] = np.inf, np.nan, 0.0, np.inf
+    want = orc.calibrate(cfg, q["xq"], q["Bq"], q["Cq"], q["s_x"], q["s_B"], q["s_C"], q["dt"], q["A"], None)
+    dv = {k: gh.dev(q[k]) for k in ("xq", "Bq", "Cq", "s_x", "s_B", "s_C", "dt", "A")}
+    s = [torch.full((n,), float("nan"), device="cuda") for n in (9 * 64, 1, 9 * 64)]
+    bd.ssdi8_calibrate(bd.dims_of(cfg), bd.make_fwd_args(**dv), *s, bd.alloc_workspace(bd.dims_of(cfg)))
+    torch.cuda.synchronize()
+    for got, ref in zip(s[:2], want[:2]):
+        assert np.array_equal(got.cpu().numpy(), np.asarray(ref).reshape(-1))
+
+
 @pytest.mark.parametrize("step", [8e-41, 9.1e-41, 9.3e-41, 1e-39])
 def test_calibration_skips_no_token_at_step_sizes_near_the_smallest(step):
     # 128 step sizes on either side of the normal range: the last token of the chunk has codes of 1, the one 64 before it codes of
@@ -387,6 +427,28 @@ def test_fused_state_kernel_on_short_calls(cfg, decay):
     # Calls whose slabs the ring of six holds at once and calls with a slab more; slices and whole heads of two and three chunks; one
     # chunk of 256 on either side of 1.8 CTAs per SM.  Every slab live, and none
     test_fused_state_kernel_with_few_and_many_sequences(cfg, decay)
+
+
+@pytest.mark.parametrize("b,H", [(5, 89), (5, 99)])
+@pytest.mark.parametrize("decay", [0.002, 1.0, 60.0])
+def test_a_last_wave_of_n_64_in_slices(b, H, decay):
+    # 1 and 51 sequences beyond three per SM: state columns in slices of 32 beside whole heads, binary32 and INT8 states and the
+    # calibration of the same shape
+    import torch
+    import gpu_harness as gh
+    from paper_2608_21952_b200 import binding as bd
+    cfg = SSDConfig("slices_last_n64", b, 2 * 64, H, 64, 64, 1, 64, 0.02, 20.0, 76)
+    test_fused_state_kernel_with_few_and_many_sequences(cfg, decay)
+    t = inputs.make_prefill(cfg)
+    t["A"] *= np.float32(decay)
+    init = inputs.make_init_state(cfg, 0.5)
+    q = orc.prepare_quantized(cfg, t, init)
+    dv = {k: gh.dev(q[k]) for k in ("xq", "Bq", "Cq", "s_x", "s_B", "s_C", "dt", "A")}
+    s = [torch.full((n,), float("nan"), device="cuda") for n in (H * 64, 1, H * 64)]
+    bd.ssdi8_calibrate(bd.dims_of(cfg), bd.make_fwd_args(init_state=gh.dev(init), **dv), *s, bd.alloc_workspace(bd.dims_of(cfg)))
+    torch.cuda.synchronize()
+    for got, name in zip(s, ("s_xs", "s_cb", "s_h")):
+        assert np.array_equal(got.cpu().numpy(), np.asarray(q[name]).reshape(-1)), name
 
 
 def test_the_tap_of_x_scaled_reaches_the_last_of_many_chunks():
@@ -650,6 +712,26 @@ def test_a_state_that_is_not_a_number_has_the_same_codes_on_both_state_routes():
         q["s_h"][64:66] = 0.0
         hq.append(gh.gpu_fwd(cfg, q, taps=("hq",))[2]["hq"][0, 0, :4])
     assert np.array_equal(hq[0], hq[1])
+
+
+@pytest.mark.parametrize("N,Q", [(64, 64), (128, 256)])
+def test_a_state_that_is_not_a_number_has_the_same_codes_in_a_cluster(N, Q):
+    # Eight chunks of four heads take a cluster per head, the same heads among 160 the fused kernel: the codes of every chunk's entering
+    # state and the final state are the same, also where a NaN or an infinity goes through all chunks
+    import gpu_harness as gh
+    many = SSDConfig("many", 1, 8 * Q, 160, 64, N, 1, Q, 0.02, 20.0, 75)
+    few = SSDConfig("few", 1, 8 * Q, 4, 64, N, 1, Q, 0.02, 20.0, 75)
+    q = _random_codes(many, 75)
+    q["init"][0, 1, 7, 3:9] = np.array([0x7fc00000, 0xffc00000, 0x7f800000, 0xff800000, 0x00000000, 0x80000000], np.uint32).view(np.float32)
+    q["s_h"][64:66] = 0.0
+    q["A"][1] = -0.01   # (a decay of 0 would make NaNs of the infinities)
+    r = dict(q, init=q["init"][:, :4], A=q["A"][:4], D=q["D"][:4], **{k: np.asarray(q[k]).reshape(8 * Q, 160, -1)[:, :4] for k in ("xq", "dt")},
+             **{k: q[k][:256] for k in ("s_x", "s_xs", "s_h")})
+    _, fin, got = gh.gpu_fwd(many, q, taps=("hq",))
+    _, fin_few, got_few = gh.gpu_fwd(few, {k: np.ascontiguousarray(v) for k, v in r.items()}, taps=("hq",))
+    assert np.isnan(fin[0, 1, 7, 3]) and np.isinf(fin[0, 1, 7, 5])
+    assert np.array_equal(got_few["hq"], got["hq"][:, :, :4])
+    assert np.array_equal(fin_few, fin[:, :4], equal_nan=True)
 
 
 @pytest.mark.parametrize("b,c,H,N", [(1, 3, 5, 64), (2, 1, 150, 128)])
