@@ -544,10 +544,14 @@ chunk_state_pass_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_const
     fused_body<I8S, TAPS, CAL, FEW, N, N>(tm_B, tm_x, tm_hq, a, (int)blockIdx.x, 0);
   } else {
     const int r = (int)blockIdx.x - a.n_full;
-    if (N == 128 && a.slice == 64)
-      fused_body<I8S, TAPS, CAL, FEW, N, 64>(tm_Bs, tm_x, tm_hqs, a, a.n_full + r / (N / 64), r % (N / 64) * 64);
-    else
-      fused_body<I8S, TAPS, CAL, FEW, N, 32>(tm_Bs, tm_x, tm_hqs, a, a.n_full + r / (N / 32), r % (N / 32) * 32);
+    // (32 of 128 columns: few units only, see the launcher)
+    if constexpr (N == 64 || FEW) {
+      if (N == 64 || a.slice == 32) {
+        fused_body<I8S, TAPS, CAL, FEW, N, 32>(tm_Bs, tm_x, tm_hqs, a, a.n_full + r / (N / 32), r % (N / 32) * 32);
+        return;
+      }
+    }
+    if constexpr (N == 128) fused_body<I8S, TAPS, CAL, FEW, N, 64>(tm_Bs, tm_x, tm_hqs, a, a.n_full + r / 2, r % 2 * 64);
   }
 }
 
