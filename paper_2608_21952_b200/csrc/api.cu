@@ -182,7 +182,7 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
   // 19.6 / 23.0, 3 x 512 x 12 in chunks of 128 20.7 / 21.3, 768 x 60 (N 64) in chunks of 128 25.5 / 25.3, 256 x 24 18.4 / 22.6), as it is with
   // more sequences (2 x 2048 x 24 35.3 / 40.6).
   const bool state_taps = a->tap_loc || a->tap_prev || a->tap_Xsq || a->tap_acc_st;
-  const bool cluster_state = split_state && d.c <= 8 && !state_taps;
+  const bool cluster_state = split_state && d.c == 8 && !state_taps;
   if (cluster_state) {
     const StatePass pass = {a->s_h, gamma, a->init_state, a->final_state, hq};
     if ((s = launch_chunk_state(d, a->xq, a->Bq, a->s_x, a->s_xs, a->s_B, pack, nullptr, nullptr, nullptr, a->status, st, &pass)) !=

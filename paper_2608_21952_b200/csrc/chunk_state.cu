@@ -10,11 +10,13 @@
 // of the epilogue writes 32 consecutive n of one p: full 128-byte lines of loc[p][n].
 // The forward pass takes this kernel where there are too few (batch, head) pairs to fill the device with
 // chunk-sequential ones (see fwd_phases).
-// PASS: the chunks of a (batch, head), up to eight, are a cluster.  The chunk-local states stay in shared memory, and once all of
-// them are there each CTA takes a share of the (p, n) through all chunks (Eq. 5-6, as state_passing.cu does, operation for
+// PASS: the eight chunks of a (batch, head) are a cluster.  The chunk-local states stay in shared memory, and once all of
+// them are there each CTA takes an eighth of the (p, n) through all chunks (Eq. 5-6, as state_passing.cu does, operation for
 // operation), reading the others' by way of distributed shared memory: no second launch, and no 32 KB per chunk out to L2 and
 // back (layer calls: 512 tokens x 4 heads 17.0 -> 16.0 us, 2048 x 24 29.5 -> 28.4; and with the epilogue's scales in shared memory, the
-// MMAs issued from uniform registers and the pass's operands fetched under them, 14.9 and 27.95).
+// MMAs issued from uniform registers and the pass's operands fetched under them, 14.9 and 27.95).  The chunk count and the share of a thread
+// are constants: written for up to eight chunks it took 94 registers instead of 72, and with two CTAs on every SM ChunkBMM no longer found room beside
+// them (prefill of 1024 tokens x 37 heads 30.8 -> 26.8 us, 28.4 with two launches before; 2048 x 36 38.7 -> 33.9, 1024 x 4 18.2 -> 17.85).
 #include "kernels.h"
 #include "sm100.cuh"
 
@@ -36,7 +38,7 @@ constexpr uint32_t OFF_X = 32768;    // [Q][64] xq rows -> Xs_q in place
 constexpr uint32_t OFF_F = 49152;    // lut[256], s_x / s_xs [64], s_xs s_B [64], bars, tmem slot
 constexpr uint32_t SMEM_BYTES = OFF_F + 256 * 4 + 128 * 4 + 64;
 
-constexpr int kMaxCluster = 8;
+constexpr int kCluster = 8;   // chunks, CTAs of a cluster (PASS)
 
 template <bool PASS>
 __global__ void __launch_bounds__(kThreads, PASS ? 2 : 3)
@@ -142,7 +144,7 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
 
   // ---- acc[n][p] = sum_i Bq[i][n] Xs_q[i][p]: A = Bq (MN-major, M = N states), B = Xs_q (MN-major)
   const uint32_t tmem = *tmem_slot;
-  if (warp == 0) {   // (the whole warp runs the loop, see elect_one)
+  if (warp == 0) {   // (the descriptors are formed by the whole warp, see elect_one)
     tc_fence_after();
     const uint32_t idesc = idesc_s8(N, 64, 1, 1);
     const uint32_t sBa = smem_u32(sB), sXa = smem_u32(sX);
@@ -158,20 +160,18 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
     }
   }
   __syncwarp();
-  // (PASS) this CTA's share of the states, four neighbouring n a thread; what the first of them needs from global memory is
-  // on its way under the MMAs
-  const int units = P * N / 4, per = (units + d.c - 1) / d.c;
-  const int u0 = k * per + tid, u1 = min(units, (k + 1) * per);
+  // (PASS) this CTA's eighth of the states, four neighbouring n a thread (128 or 256 threads); what they need from global memory
+  // is on its way under the MMAs
+  const int units = P * N / 4, u = k * (units / kCluster) + tid;
+  const bool mine = PASS && tid < units / kCluster;
   const i64 bh = (i64)b * d.H + h;
-  float gam[kMaxCluster], inv_h = 0.f;
+  float gam[kCluster], inv_h = 0.f;
   float4 S = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (PASS) {
+  if (mine) {
 #pragma unroll
-    for (int j = 0; j < kMaxCluster; ++j) gam[j] = j < d.c ? a.gamma[bh * d.c + j] : 0.f;
-    if (u0 < u1) {
-      inv_h = __fdiv_rn(1.0f, a.s_h[h * P + 4 * u0 / N]);
-      if (a.init) S = reinterpret_cast<const float4*>(a.init)[bh * units + u0];
-    }
+    for (int j = 0; j < kCluster; ++j) gam[j] = a.gamma[bh * kCluster + j];
+    inv_h = __fdiv_rn(1.0f, a.s_h[h * P + 4 * u / N]);
+    if (a.init) S = reinterpret_cast<const float4*>(a.init)[bh * units + u];
   }
   mbar_wait(&bars[1], 0, a.status);
   tc_fence_after();
@@ -207,35 +207,26 @@ chunk_state_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_constant__
   tc_fence_before();
   if (PASS) {
     cluster_sync();
-    const uint32_t mine = smem_u32(sB);
-    for (int u = u0; u < u1; u += kThreads) {
-      float4 l[kMaxCluster];
+    if (mine) {
+      float4 l[kCluster];
 #pragma unroll
-      for (int j = 0; j < kMaxCluster; ++j) {
-        if (j < d.c) {
-          uint32_t at;
-          asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(mine + 16u * (uint32_t)u), "r"(j));
-          asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                       : "=f"(l[j].x), "=f"(l[j].y), "=f"(l[j].z), "=f"(l[j].w)
-                       : "r"(at)
-                       : "memory");
-        }
+      for (int j = 0; j < kCluster; ++j) {
+        uint32_t at;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(sB) + 16u * (uint32_t)u), "r"(j));
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(l[j].x), "=f"(l[j].y), "=f"(l[j].z), "=f"(l[j].w)
+                     : "r"(at)
+                     : "memory");
       }
-      if (u != u0) {
-        inv_h = __fdiv_rn(1.0f, a.s_h[h * P + 4 * u / N]);
-        S = a.init ? reinterpret_cast<const float4*>(a.init)[bh * units + u] : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      uint32_t* hq = reinterpret_cast<uint32_t*>(a.hq) + ((i64)b * d.c * d.H + h) * units + u;
+      uint32_t* hq = reinterpret_cast<uint32_t*>(a.hq) + ((i64)b * kCluster * d.H + h) * units + u;
 #pragma unroll
-      for (int j = 0; j < kMaxCluster; ++j) {
-        if (j < d.c) {
-          hq[(i64)j * d.H * units] = pack4_bits(rne_clamp_bits(__fmul_rn(S.x, inv_h)), rne_clamp_bits(__fmul_rn(S.y, inv_h)),
-                                                rne_clamp_bits(__fmul_rn(S.z, inv_h)), rne_clamp_bits(__fmul_rn(S.w, inv_h)));
-          S.x = __fmaf_rn(gam[j], S.x, l[j].x);
-          S.y = __fmaf_rn(gam[j], S.y, l[j].y);
-          S.z = __fmaf_rn(gam[j], S.z, l[j].z);
-          S.w = __fmaf_rn(gam[j], S.w, l[j].w);
-        }
+      for (int j = 0; j < kCluster; ++j) {
+        hq[(i64)j * d.H * units] = pack4_bits(rne_clamp_bits(__fmul_rn(S.x, inv_h)), rne_clamp_bits(__fmul_rn(S.y, inv_h)),
+                                              rne_clamp_bits(__fmul_rn(S.z, inv_h)), rne_clamp_bits(__fmul_rn(S.w, inv_h)));
+        S.x = __fmaf_rn(gam[j], S.x, l[j].x);
+        S.y = __fmaf_rn(gam[j], S.y, l[j].y);
+        S.z = __fmaf_rn(gam[j], S.z, l[j].z);
+        S.w = __fmaf_rn(gam[j], S.w, l[j].w);
       }
       if (a.final_state) reinterpret_cast<float4*>(a.final_state)[bh * units + u] = S;
     }
@@ -273,13 +264,13 @@ ssdi8_status_t launch_chunk_state(const Dims& d, const int8_t* xq, const int8_t*
   StateArgs a = {s_x, s_xs, s_B, pack, loc, tap_Xsq, tap_acc, status, d, nullptr, nullptr, nullptr, nullptr, nullptr};
   const size_t smem = SMEM_BYTES + 1024;
   if (!pass) return launch_configured(chunk_state_tc<false>, dim3(d.H, d.c, d.b), dim3(kThreads), smem, -1, false, st, tm_B, tm_x, a);
-  if (d.c > kMaxCluster) return SSDI8_ERR_SHAPE;
+  if (d.c != kCluster) return SSDI8_ERR_SHAPE;
   a.s_h = pass->s_h;
   a.gamma = pass->gamma;
   a.init = pass->init;
   a.final_state = pass->final_state;
   a.hq = pass->hq;
-  return launch_clustered(chunk_state_tc<true>, dim3(d.c, d.H, d.b), d.c, dim3(kThreads), smem, st, tm_B, tm_x, a);
+  return launch_clustered(chunk_state_tc<true>, dim3(kCluster, d.H, d.b), kCluster, dim3(kThreads), smem, st, tm_B, tm_x, a);
 }
 
 }  // namespace ssdi8

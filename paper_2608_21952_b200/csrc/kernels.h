@@ -119,7 +119,7 @@ ssdi8_status_t launch_bmm(const Dims& d, const int8_t* Cq, const int8_t* Bq, con
                           const float* s_B, const float* s_cb, int8_t* CBq, int32_t* tap_acc,
                           uint32_t* absmax_acc, int32_t* status, cudaStream_t st, bool after_state_kernel = false);
 
-// pass: ChunkState and StatePassing of up to eight chunks in one launch (loc and the taps unused)
+// pass: ChunkState and StatePassing of eight chunks in one launch (loc and the taps unused)
 struct StatePass {
   const float* s_h; const float* gamma; const float* init; float* final_state; int8_t* hq;
 };
