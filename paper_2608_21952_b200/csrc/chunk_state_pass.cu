@@ -614,9 +614,10 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
                  status, absmax_h, s_xs_out, d, n_full, slice};
   const unsigned grid = (unsigned)(n_full + d.N / slice * (units - n_full));
   const bool taps = tap_loc || tap_prev || tap_Xsq || tap_acc;
-  // (FEW; but with one chunk of 256 and nearly two CTAs for every SM two warps of their own quantise faster, all four slabs of a CTA being there at once:
-  // 256 tokens x 296 heads N 128 28.3 / 26.8 us, N 64 27.1 / 25.4, 268 x N 128 25.0 / 25.2, 230 x 24.7 / 25.4)
-  const bool few = (int)grid <= 2 * sms && !(d.Q == 256 && d.c == 1 && 10 * (int)grid > 18 * sms);
+  // (FEW; but of one chunk of 256 two warps of their own quantise faster where SMs have two CTAs, all four slabs of a CTA being there at once.  Layer calls in a
+  // row, FEW / two warps: 2 x 256 x 108 with 16-bit y 27.3 / 26.0 us, 2 x 256 x 130 27.2 / 25.7, 256 x 296 29.4 / 27.4, 256 x 150 23.6 / 24.3; prefill of 2 x 256 x 108
+  // 28.4 / 29.1.  Not in the calibration, which forms no codes beside it)
+  const bool few = (int)grid <= 2 * sms && !(d.Q == 256 && d.c == 1 && (int)grid > sms && !absmax_h);
   // (kSmemAlone; not for one chunk, nor for two or three of N 128 where more than four SMs in five get a CTA: the start is what counts there, and CTAs of that
   // size wait for the SMs that the kernel before still holds.  With / without: 256 tokens x 148 heads N 128 22.1 / 19.8 us, 64 x 100 (of 64) N 64
   // 13.6 / 13.1, 512 x 148 N 128 29.4 / 27.4, 768 x 148 33.9 / 32.2; but 128 x 48 (of 64) N 128 14.5 / 15.3, 384 x 148 (of 128) N 64 22.3 / 22.8)
