@@ -6,7 +6,7 @@ namespace ssdi8 {
 namespace {
 
 // absmax_xs[h,p] = max over tokens of |fmul(fmul(float(xq), s_x), LUT_state)| (Eq. 3), as binary32 bits.  A block takes a
-// chunk of 8 neighbouring heads (512 contiguous bytes of a token), 32 tokens at a time from the last one on; a thread owns
+// chunk, or 64 tokens of one, of 8 neighbouring heads (512 contiguous bytes of a token), 32 tokens at a time from the last one on; a thread owns
 // 16 channels of four of the tokens and keeps their maxima in registers, and after a round that had anything to do the
 // token rows of the block meet in shared memory.  LUT_state decays towards the start of a chunk, so a few rounds decide the
 // maxima: a token whose 16 products cannot exceed them, |LUT_state| <= min over the channels of max / (128 |s_x|) (fmul is
@@ -16,7 +16,7 @@ namespace {
 // blocks of 512 threads 79.1, 120.1, 91.5, 151.2.)
 constexpr int kXsHeads = 8, kXsThreads = 256, kXsRows = kXsThreads / 32, kXsTokens = 4 * kXsRows;
 __global__ void __launch_bounds__(kXsThreads) absmax_xs_kernel(const int8_t* __restrict__ xq, const float* __restrict__ s_x, const float* pack,
-                                                        uint32_t* absmax, Dims d) {
+                                                        uint32_t* absmax, Dims d, int parts) {
   extern __shared__ __align__(16) float lut[];    // [kXsHeads][Q]
   __shared__ __align__(16) float sxs[kXsHeads * 64];
   __shared__ uint32_t best[16][32];               // channel e of (head, 16 channels) = lane
@@ -24,22 +24,23 @@ __global__ void __launch_bounds__(kXsThreads) absmax_xs_kernel(const int8_t* __r
   pdl_launch_dependents();   // (after the wait: ChunkBMM, launched next, does not wait for this kernel)
   const int tid = threadIdx.x, lane = tid & 31;
   // (head blocks and chunks in one grid dimension: a sequence of more than 4 M tokens has more than 65535 of the latter)
-  const int nhb = (d.H + kXsHeads - 1) / kXsHeads, k = blockIdx.x / nhb, b = blockIdx.z;
-  const int h0 = (blockIdx.x - k * nhb) * kXsHeads;
+  const int nhb = (d.H + kXsHeads - 1) / kXsHeads, kp = blockIdx.x / nhb, k = kp / parts, b = blockIdx.z;
+  const int h0 = (blockIdx.x - kp * nhb) * kXsHeads;
+  const int span = d.Q / parts, first = (kp - k * parts) * span;   // tokens of the chunk that the block takes, a power of two
   const int hh = (tid >> 2) & 7, c = tid & 3, row = tid >> 5;   // head, 16 channels, token row of the thread
   const int h = h0 + hh;
   const bool live = h < d.H;
-  const uint4* src = reinterpret_cast<const uint4*>(xq + (((i64)b * d.L + (i64)k * d.Q + row) * d.H + h) * 64) + c;
+  const uint4* src = reinterpret_cast<const uint4*>(xq + (((i64)b * d.L + (i64)k * d.Q + first + row) * d.H + h) * 64) + c;
   const i64 stride = (i64)kXsRows * d.H * 4;   // kXsRows tokens, in 16-byte words
   uint4 w[4];                                  // (the first round's before LUT_state is there)
 #pragma unroll
-  for (int u = 0; u < 4; ++u) w[u] = live ? __ldg(src + ((d.Q - kXsTokens) / kXsRows + u) * stride) : make_uint4(0u, 0u, 0u, 0u);
-  const int lq = 31 - __clz(d.Q) - 2;          // LUT_state, 16 bytes at a time
+  for (int u = 0; u < 4; ++u) w[u] = live ? __ldg(src + ((span - kXsTokens) / kXsRows + u) * stride) : make_uint4(0u, 0u, 0u, 0u);
+  const int lq = 31 - __clz(span) - 2;          // LUT_state, 16 bytes at a time
   for (int e = tid; e < (kXsHeads << lq); e += kXsThreads) {
     const int hl = e >> lq, i = (e - (hl << lq)) * 4;
     if (h0 + hl < d.H)
-      *reinterpret_cast<float4*>(lut + hl * d.Q + i) =
-          *reinterpret_cast<const float4*>(pack + ((((i64)b * d.H + h0 + hl) * d.c + k) * kPackRows + PACK_LUT) * d.Q + i);
+      *reinterpret_cast<float4*>(lut + hl * span + i) =
+          *reinterpret_cast<const float4*>(pack + ((((i64)b * d.H + h0 + hl) * d.c + k) * kPackRows + PACK_LUT) * d.Q + first + i);
   }
   // (by way of shared memory: ssdi8_calibrate asks for no alignment of s_x beyond a float's, and sixteen loads of one float per
   // thread were 4 us slower)
@@ -60,14 +61,14 @@ __global__ void __launch_bounds__(kXsThreads) absmax_xs_kernel(const int8_t* __r
   }
   float least = 0.f;                     // |LUT_state| up to here changes nothing
 #pragma unroll 1
-  for (int i0 = d.Q - kXsTokens; i0 >= 0; i0 -= kXsTokens) {
+  for (int i0 = span - kXsTokens; i0 >= 0; i0 -= kXsTokens) {
     float l[4];
     bool any = false;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      l[u] = live ? lut[hh * d.Q + i0 + kXsRows * u + row] : 0.f;
+      l[u] = live ? lut[hh * span + i0 + kXsRows * u + row] : 0.f;
       if (!(fabsf(l[u]) <= least)) {
-        if (i0 != d.Q - kXsTokens) w[u] = __ldg(src + (i0 / kXsRows + u) * stride);
+        if (i0 != span - kXsTokens) w[u] = __ldg(src + (i0 / kXsRows + u) * stride);
         any = true;
       }
     }
@@ -132,11 +133,18 @@ __global__ void finalize_scales(const uint32_t* max_h, float* s_h, int n, const 
 
 ssdi8_status_t launch_absmax_xs(const Dims& d, const int8_t* xq, const float* s_x, const float* pack, uint32_t* absmax,
                                 cudaStream_t st) {
-  const i64 blocks = (i64)((d.H + kXsHeads - 1) / kXsHeads) * d.c;
+  const i64 chunks = (i64)((d.H + kXsHeads - 1) / kXsHeads) * d.c;
+  const int sms = sm_count();
+  if (sms == 0) return SSDI8_ERR_CUDA;
+  // Few chunks go 64 tokens to a block, whose rounds are a chain of loads and barriers each; with more of them ChunkBMM, which works beside this kernel,
+  // wants the room.  Calibration calls, us, whole chunks / 64 tokens: 512 tokens x 8 heads 30.6 / 28.2, 1280 x 24 43.1 / 40.7, 2048 x 32 48.6 / 46.1, but
+  // 4096 x 4 46.5 / 49.6, 8192 x 16 75.3 / 81.0.
+  const int parts = d.Q > 64 && (i64)d.b * d.c < 12 && chunks * d.b * (d.Q / 64) <= 2 * sms ? d.Q / 64 : 1;
+  const i64 blocks = chunks * parts;
   if (blocks > 0x7fffffff) return SSDI8_ERR_SHAPE;
   const dim3 grid((unsigned)blocks, 1, d.b);
   return launch_sized(absmax_xs_kernel, grid, dim3(kXsThreads), sizeof(float) * kXsHeads * d.Q, sizeof(float) * kXsHeads * 256, kStreamCarveout,
-                      false, st, xq, s_x, pack, absmax, d);
+                      false, st, xq, s_x, pack, absmax, d, parts);
 }
 
 ssdi8_status_t launch_clear_words(void* a, i64 n, cudaStream_t st) {

@@ -156,6 +156,13 @@ def test_calibration_skips_no_token_that_counts(b, c, H, Q, regime):
         assert np.array_equal(got.cpu().numpy(), np.asarray(ref).reshape(-1))
 
 
+@pytest.mark.parametrize("b,c,H,Q", [(1, 11, 9, 256), (1, 12, 9, 256), (2, 5, 24, 128), (11, 1, 9, 256), (1, 10, 70, 256)])
+@pytest.mark.parametrize("regime", ["slow", "codes"])
+def test_calibration_skips_no_token_in_whole_chunks_and_in_parts(b, c, H, Q, regime):
+    # Up to eleven chunks of few heads take 64 tokens to a block, more take the chunk
+    test_calibration_skips_no_token_that_counts(b, c, H, Q, regime)
+
+
 @pytest.mark.parametrize("R,Ch,I", [(9, 32, 1), (4100, 1028, 1), (300, 2400, 1), (13, 4, 4), (257, 37, 128), (258, 38, 128), (2049, 4, 128)])
 def test_calibrating_quantiser_on_values_that_are_not_finite(R, Ch, I):
     # One launch and three: a NaN counts for nothing in a step size, an infinity makes it infinite (its own code is that of a NaN, all others
