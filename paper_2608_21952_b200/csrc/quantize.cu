@@ -421,7 +421,9 @@ ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* sca
       i64 min_rows = (QT * 4 + I4 - 1) / I4;
       if (rows < min_rows) rows = min_rows;
       int gx = (int)((R + rows - 1) / rows);
-      ls = launch_configured(absmax_inner, dim3(gx, (unsigned)Ch), dim3(QT), 0, kStreamCarveout, false, st,
+      // (no carve-out asked for, here and for the codes: a tensor this narrow, B or C, follows x, whose clusters hold their rows in shared memory, and
+      // an SM that changes its split first has to run empty.  Calibration calls of 2048 tokens x 24 heads 50.2 -> 45.0 us, 1280 x 8 43.6 -> 38.5)
+      ls = launch_configured(absmax_inner, dim3(gx, (unsigned)Ch), dim3(QT), 0, -1, false, st,
                              reinterpret_cast<const float4*>(in), bits, R, (int)Ch, I4, (int)rows);
     }
     if (ls != SSDI8_OK) return ls;
@@ -444,7 +446,7 @@ ssdi8_status_t launch_quantize(const float* in, i64 R, i64 Ch, i64 I, float* sca
                              reinterpret_cast<float4*>(scale), reinterpret_cast<uint32_t*>(out), R, ch4, (int)rows);
   }
   const unsigned grid = (unsigned)((n4 + QT * QUNROLL - 1) / (QT * QUNROLL));
-  return launch_configured(fix ? quant_inner<true> : quant_inner<false>, dim3(grid), dim3(QT), 0, kStreamCarveout, false, st,
+  return launch_configured(fix ? quant_inner<true> : quant_inner<false>, dim3(grid), dim3(QT), 0, -1, false, st,
                            reinterpret_cast<const float4*>(in), scale, reinterpret_cast<uint32_t*>(out), (uint32_t)n4,
                            (uint32_t)(I / 4), (uint32_t)Ch);
 }
