@@ -69,7 +69,8 @@ struct Geo {
   static constexpr uint32_t OFF_BAR = OFF_INFO + 32;
   enum { B_FULL = 0, B_READY = kSlots, B_FREE = 2 * kSlots, B_ACC = 3 * kSlots, B_ACC_FREE = B_ACC + 2, B_LUT = B_ACC_FREE + 2,
          B_COUNT = B_LUT + kLutAhead };
-  static constexpr uint32_t SMEM_BYTES = OFF_BAR + 8 * B_COUNT + 16;   // 97 584 bytes, two CTAs per SM; 71 792, three
+  static constexpr uint32_t SMEM_BYTES = OFF_BAR + 8 * B_COUNT + 16;   // 96 768 bytes, two CTAs per SM; 71 632, three
+  static_assert((FEW ? 2 : 3) * (SMEM_BYTES + 1024) <= 228 * 1024, "CTAs of an SM");
 };
 // More than half of an SM's shared memory, asked for where there is a CTA per SM or less: the scheduler, which starts CTAs beside those of the
 // kernel before wherever these have left room, would put up to three on one SM, each of them slower for it.  (Likewise the ring of six:
@@ -593,12 +594,13 @@ ssdi8_status_t launch_chunk_state_passing(const Dims& d, const int8_t* xq, const
   // five SMs: 768 x 36 20.8 / 18.9 / -, 384 x 42 (of 128) 17.3 / 16.4 / -, 256 x 48 (of 128) 16.2 / 15.0 / -, 512 x 12 16.6 / 16.2 / 16.8, but 128 x 54 (of 64) 13.7 /
   // 14.4 / -, 768 x 74 24.6 / 26.8 / -, 192 x 74 (of 64) 17.4 / 18.6 / -.
   // N 64, from four chunks on: 768 x 60 28.7 / - / 27.9, 256 x 32 (of 64) 16.4 / - / 15.6, 2048 x 60 44.9 / - / 44.6; with fewer whole heads: 128 x 60
-  // (of 64) 13.3 / - / 14.6, 256 x 74 (of 128) 16.4 / - / 17.6, 512 x 36 17.9 / - / 19.2.
+  // (of 64) 13.3 / - / 14.6, 256 x 74 (of 128) 16.4 / - / 17.6, 512 x 36 17.9 / - / 19.2.  The calibration, which forms no codes, takes slices of N 128 from twelve chunks
+  // on (calls, whole / slices: 1280 x 48 43.0 / 45.3, 1024 x 32 36.0 / 38.1, 1280 x 48 (of 128) 48.3 / 51.4, but 4096 x 8 53.7 / 52.8).
   int n_full = units / slots * slots, slice = d.N == 128 ? 64 : 32;
   const int last = units - n_full;
   if (n_full > 0) {
     if (8 * last > slots) n_full = units;
-  } else if (d.N == 128 && (d.c >= 4 ? 3 * units <= 2 * sms : d.c >= 2 && 5 * units <= 2 * sms)) {
+  } else if (d.N == 128 && (!absmax_h || d.c >= 12) && (d.c >= 4 ? 3 * units <= 2 * sms : d.c >= 2 && 5 * units <= 2 * sms)) {
     slice = d.c >= 12 && 4 * units <= sms ? 32 : 64;
   } else if (!(d.N == 64 && d.c >= 4 && 2 * units <= sms)) {
     n_full = units;
