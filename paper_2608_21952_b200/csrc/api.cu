@@ -167,9 +167,10 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
   // Few sequences of many chunks: the fused kernel walks a (batch, head)'s chunks one after the other, about 1.2 us
   // each however few CTAs there are, while ChunkState takes all chunks at once (states through L2) and StatePassing
   // is a short elementwise pass.  Graphs of prefill calls with the fused kernel / with the two, us: 8192 tokens x 8 heads (N 64, chunks of
-  // 64) 109.8 / 48.4, 8192 x 36 (N 64, of 128) 112.6 / 85.0, 8192 x 20 67.7 / 53.7, 4096 x 24 44.1 / 38.3, 4096 x 48 61.5 / 58.7, 2048 x 8 29.2 /
-  // 25.3, 512 x 4 (of 64) 17.4 / 16.5; even at 8192 x 48 (96.4 / 97.2), 2048 x 36 (33.7 / 33.9), 2048 x 24 (30.5 / 30.6), and 2 x 4096 x 24 58.0
-  // / 60.0.  With eight to eleven chunks the line lies where two CTAs per SM take all of them at once.
+  // 64) 109.8 / 48.4, 8192 x 36 (N 64, of 128) 112.6 / 85.0, 8192 x 20 67.7 / 53.7, 4096 x 24 44.1 / 38.3, 4096 x 48 61.5 / 58.7; even at 8192 x 48 (96.4
+  // / 97.2), and 2 x 4096 x 24 58.0 / 60.0.  With nine to eleven chunks the line lies where two CTAs per SM take all of them at once: 2304 x 12 27.9 /
+  // 25.3, 2304 x 32 33.7 / 33.4, 2560 x 29 34.0 / 32.8, 2816 x 26 37.1 / 35.1, 1408 x 26 (of 128) 29.1 / 25.9, 640 x 4 (N 64, of 64) 17.7 / 16.8; for more than
+  // an SM's worth of N 64 in chunks of 64 the fused kernel would be even or ahead (576 x 32 21.5 / 23.2, 704 x 26 22.3 / 22.9, 704 x 20 21.8 / 21.8).
   const int sms = fused_state ? sm_count() : 0;
   const i64 seqs = (i64)d.b * d.H;
   const bool split_state = fused_state && !i8s && (d.c >= 12 ? 3 * seqs <= sms : d.c >= 8 && seqs * d.c <= 2 * sms);
@@ -177,7 +178,8 @@ ssdi8_status_t fwd_phases(const ssdi8_dims_t* dims, const ssdi8_fwd_args_t* a, u
       (s = launch_bmm(d, a->Cq, a->Bq, a->s_C, a->s_B, a->s_cb, cbq, a->tap_acc_cb, nullptr, a->status, st)) !=
           SSDI8_OK)
     return s;
-  // Eight chunks of that: both modules in one launch, a cluster of CTAs per (batch, head) (chunk_state.cu).  With fewer chunks the
+  // Eight chunks of that: both modules in one launch, a cluster of CTAs per (batch, head) (chunk_state.cu).  Graphs of prefill calls, fused / two / clusters:
+  // 2048 x 4 23.2 / 23.1 / 20.0, 2048 x 36 32.7 / 32.5 / 32.0, 1024 x 37 (of 128) 27.5 / 26.2 / 25.3, 512 x 4 (N 64, of 64) 16.7 / 16.0 / 14.4.  With fewer chunks the
   // fused kernel is the faster one (layer calls, us, fused / clusters: 1024 tokens x 32 heads 22.8 / 23.1, 1024 x 8 19.7 / 21.0, 512 x 24
   // 19.6 / 23.0, 3 x 512 x 12 in chunks of 128 20.7 / 21.3, 768 x 60 (N 64) in chunks of 128 25.5 / 25.3, 256 x 24 18.4 / 22.6), as it is with
   // more sequences (2 x 2048 x 24 35.3 / 40.6).

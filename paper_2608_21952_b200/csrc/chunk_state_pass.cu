@@ -50,7 +50,7 @@ constexpr int kSlab = 64;                         // tokens of a slab
 constexpr int kLutAhead = 4;                      // LUT_state of so many chunks is under way to the loading warp
 enum { SLAB_LAST = 1 };                           // of its chunk (the word also has the slab's index from bit 8; the warps that need the chunk's count chunks)
 
-// FEW: up to two CTAs per SM.  A CTA alone on its SM is a chain of latencies, the longest where decay is slow and most slabs live: the
+// FEW: up to two CTAs per SM (one chunk of 256: one).  A CTA alone on its SM is a chain of latencies, the longest where decay is slow and most slabs live: the
 // state warps quantise Q(X_scaled) themselves, all eight at a slab, one chunk ahead, behind a ring of six slabs.  With three
 // CTAs per SM what counts is that the chains overlap: two warps of their own quantise, and the ring has four slabs (all of a
 // chunk of 256).  Layer calls, us, eight state warps / two of their own: 3 x 1408 x 50 56.5 / 58.8, calibration of 2 x 2048 x 80 heads
@@ -72,7 +72,7 @@ struct Geo {
   static constexpr uint32_t SMEM_BYTES = OFF_BAR + 8 * B_COUNT + 16;   // 96 768 bytes, two CTAs per SM; 71 632, three
   static_assert((FEW ? 2 : 3) * (SMEM_BYTES + 1024) <= 228 * 1024, "CTAs of an SM");
 };
-// More than half of an SM's shared memory, asked for where there is a CTA per SM or less: the scheduler, which starts CTAs beside those of the
+// More than half of an SM's shared memory, asked for where there is a CTA per SM or less (and the start does not count for more, see the launcher): the scheduler, which starts CTAs beside those of the
 // kernel before wherever these have left room, would put up to three on one SM, each of them slower for it.  (Likewise the ring of six:
 // 3 x 1408 x 50 56.5 us with three to an SM, 53.4 with two; 3 x 2048 x 80 98.7 / 94.7, 1 x 1024 x 128 (G 8) 41.3 / 40.7.)
 constexpr uint32_t kSmemAlone = 120 * 1024;
