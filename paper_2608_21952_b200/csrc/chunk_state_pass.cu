@@ -545,14 +545,13 @@ chunk_state_pass_tc(const __grid_constant__ CUtensorMap tm_B, const __grid_const
     fused_body<I8S, TAPS, CAL, FEW, N, N>(tm_B, tm_x, tm_hq, a, (int)blockIdx.x, 0);
   } else {
     const int r = (int)blockIdx.x - a.n_full;
-    // (32 of 128 columns: few units only, see the launcher)
-    if constexpr (N == 64 || FEW) {
-      if (N == 64 || a.slice == 32) {
-        fused_body<I8S, TAPS, CAL, FEW, N, 32>(tm_Bs, tm_x, tm_hqs, a, a.n_full + r / (N / 32), r % (N / 32) * 32);
-        return;
-      }
+    // (32 of 128 columns: few units only, see the launcher.  Written the other way round, 32 ahead of 64, slices of 64 take 3 % longer: layer 3 x 1024 x 24 heads
+    // 29.6 -> 30.5 us, 3 x 1792 x 20 34.4 -> 35.3)
+    if (N == 128 && (!FEW || a.slice == 64)) {
+      if constexpr (N == 128) fused_body<I8S, TAPS, CAL, FEW, N, 64>(tm_Bs, tm_x, tm_hqs, a, a.n_full + r / 2, r % 2 * 64);
+    } else {
+      if constexpr (N == 64 || FEW) fused_body<I8S, TAPS, CAL, FEW, N, 32>(tm_Bs, tm_x, tm_hqs, a, a.n_full + r / (N / 32), r % (N / 32) * 32);
     }
-    if constexpr (N == 128) fused_body<I8S, TAPS, CAL, FEW, N, 64>(tm_Bs, tm_x, tm_hqs, a, a.n_full + r / 2, r % 2 * 64);
   }
 }
 
